@@ -27,6 +27,7 @@ from paper_2505_08600_b200 import binding, synth
 DEV = "cuda:0"
 LORA = dict(adapters=4, rank=16, scale=2.0)
 DISAGREE = 0.2                       # share of tokens after which draft and target name different successors
+MAMBA_VOCAB = 21128
 MAX_CTX = {"tiny": 128, "1b": 512, "7b": 2048, "13b": 8192}
 
 
@@ -107,7 +108,7 @@ def _task(case, i):
     return i % (LORA["adapters"] if case.get("adapters") else len(_models(case)[2]))
 
 
-def _load_model(ctx, model_id, dims, dtype, g, successor):
+def _load_model(ctx, model_id, dims, dtype, g, successor):         # ctx: a context, or whatever else takes tensors (exact)
     td = torch.bfloat16 if dtype == "bf16" else torch.float32
 
     def normal(shape, std):
@@ -140,12 +141,9 @@ def _load_adapters(ctx, dims, g):
                 ctx.sd_load_lora(a, l, mat, *ab)
 
 
-def _context(case, seed, g):
-    dtype, target, drafts, clf = _models(case)
-    lora = dict(lora_adapters=LORA["adapters"], lora_rank=LORA["rank"], lora_scale=LORA["scale"]) if case.get("adapters") else {}
-    gamma = case.get("gamma", 1)
-    ctx = binding.Context(target, drafts, dtype, case["batch"], MAX_CTX[case["model"]], gamma, case["temperature"], seed,
-                          clf_d_hidden=clf[1] if case.get("classifier") else 0, device=DEV, **lora)
+def _fill(ctx, case, g):
+    """Random weights of the case's models (and adapters) into ctx, drawn from g in a fixed order; the vocabulary's size."""
+    dtype, target, drafts, _ = _models(case)
     V = target["vocab"]
     successor = torch.randperm(V, generator=g, device=DEV)
     _load_model(ctx, 0, target, dtype, g, successor)
@@ -156,10 +154,47 @@ def _context(case, seed, g):
         _load_model(ctx, 1 + k, dims, dtype, g, s)
     if case.get("adapters"):
         _load_adapters(ctx, drafts[0], g)
+    return V
+
+
+def _context(case, seed, g):
+    dtype, target, drafts, clf = _models(case)
+    lora = dict(lora_adapters=LORA["adapters"], lora_rank=LORA["rank"], lora_scale=LORA["scale"]) if case.get("adapters") else {}
+    gamma = case.get("gamma", 1)
+    ctx = binding.Context(target, drafts, dtype, case["batch"], MAX_CTX[case["model"]], gamma, case["temperature"], seed,
+                          clf_d_hidden=clf[1] if case.get("classifier") else 0, device=DEV, **lora)
+    V = _fill(ctx, case, g)
     if case.get("classifier"):
         c = synth.make_classifier(*clf, seed=seed)
         ctx.sd_load_classifier(c["w1"], c["b1"], c["w2"], c["b2"])
     return ctx, V
+
+
+def _prompts(case, V, g):
+    return [torch.randint(0, V, (m,), generator=g, device=DEV, dtype=torch.int32).cpu().numpy() for m in _lengths(case)]
+
+
+def _queue(case, seed, g):
+    """The classifier's prompts: token ids one prompt after the other, and where each begins and how long it is."""
+    lens = np.random.default_rng(seed).integers(case["len_lo"], case["len_hi"] + 1, size=case["prompts"]).astype(np.int32)
+    starts = np.concatenate([[0], np.cumsum(lens)[:-1]]).astype(np.int64)
+    return torch.randint(0, MAMBA_VOCAB, (int(lens.sum()),), generator=g, device=DEV, dtype=torch.int32), starts, lens
+
+
+def _corpus(case, g):
+    """Sentence vectors in overlapping groups, and centroids as an iteration on the way has them."""
+    n, dim, k = case["n"], case["dim"], case["k"]
+    centers = torch.nn.functional.normalize(torch.randn((k, dim), generator=g, device=DEV), dim=1)
+    x = torch.randn((n, dim), generator=g, device=DEV).mul_(0.6 / math.sqrt(dim))
+    x += centers[torch.randint(0, k, (n,), generator=g, device=DEV)]
+    x /= x.norm(dim=1, keepdim=True)
+    return x, (centers + 0.2 / math.sqrt(dim) * torch.randn((k, dim), generator=g, device=DEV)).contiguous()
+
+
+def _generator(seed):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(int(seed) * 7919 + 17)
+    return g
 
 
 _streams = []
@@ -173,31 +208,21 @@ def _stream():
 
 
 def prepare(case, seed):
-    g = torch.Generator(device=DEV)
-    g.manual_seed(int(seed) * 7919 + 17)
+    g = _generator(seed)
     if case["kind"] == "classify":
-        rng = np.random.default_rng(seed)
-        vocab = 21128
-        lens = rng.integers(case["len_lo"], case["len_hi"] + 1, size=case["prompts"]).astype(np.int32)
-        starts = np.concatenate([[0], np.cumsum(lens)[:-1]]).astype(np.int64)
-        tokens = torch.randint(0, vocab, (int(lens.sum()),), generator=g, device=DEV, dtype=torch.int32)
-        clf = binding.MambaClassifier(synth.make_mamba_classifier(vocab, n_classes=case["classes"], seed=seed), DEV)
+        tokens, starts, lens = _queue(case, seed, g)
+        clf = binding.MambaClassifier(synth.make_mamba_classifier(MAMBA_VOCAB, n_classes=case["classes"], seed=seed), DEV)
         return dict(case=case, clf=clf, tokens=tokens, starts=starts, lens=lens)
     if case["kind"] == "cluster":
+        x, centroids = _corpus(case, g)
         n, dim, k = case["n"], case["dim"], case["k"]
-        centers = torch.nn.functional.normalize(torch.randn((k, dim), generator=g, device=DEV), dim=1)
-        x = torch.randn((n, dim), generator=g, device=DEV).mul_(0.6 / math.sqrt(dim))
-        x += centers[torch.randint(0, k, (n,), generator=g, device=DEV)]
-        x /= x.norm(dim=1, keepdim=True)
-        start = centers + 0.2 / math.sqrt(dim) * torch.randn((k, dim), generator=g, device=DEV)      # an iteration on the way
-        return dict(case=case, points=x, centroids=start.contiguous(), labels=torch.empty(n, dtype=torch.int32, device=DEV),
+        return dict(case=case, points=x, centroids=centroids, labels=torch.empty(n, dtype=torch.int32, device=DEV),
                     out=torch.empty((k, dim), device=DEV), counts=torch.empty(k, dtype=torch.int64, device=DEV),
                     inertia=torch.empty(1, dtype=torch.float64, device=DEV))
     with torch.cuda.stream(_stream()):
         ctx, V = _context(case, seed, g)
         n, gamma = case["batch"], case.get("gamma", 0)
-        prompts = [torch.randint(0, V, (m,), generator=g, device=DEV, dtype=torch.int32).cpu().numpy() for m in _lengths(case)]
-        s = dict(case=case, ctx=ctx, seqs=list(range(n)), prompts=prompts, tasks=[_task(case, i) for i in range(n)],
+        s = dict(case=case, ctx=ctx, seqs=list(range(n)), prompts=_prompts(case, V, g), tasks=[_task(case, i) for i in range(n)],
                  logits=torch.empty((n, gamma + 1, V), device=DEV))
         if case["kind"] != "decode":
             s.update(x=torch.empty((n, gamma), dtype=torch.int32, device=DEV), q=torch.empty((n, gamma, V), device=DEV),
@@ -276,7 +301,7 @@ def work(case):
         D, Di, N, R = 128, 256, 16, 8
         T = case["prompts"] * (case["len_lo"] + case["len_hi"]) / 2
         per_token = 2 * (2 * Di * D + 4 * Di + (R + 2 * N) * Di + Di * R) + 6 * Di * N
-        return dict(bytes=4.0 * (T + min(T, 21128) * D + 2 * Di * D + (R + 2 * N) * Di + 2 * Di * (N + R) + Di * D), flops=T * per_token)
+        return dict(bytes=4.0 * (T + min(T, MAMBA_VOCAB) * D + 2 * Di * D + (R + 2 * N) * Di + 2 * Di * (N + R) + Di * D), flops=T * per_token)
     dtype, target, drafts, _ = _models(case)
     esz = 2 if dtype == "bf16" else 4
     lens, n, gamma, V = _lengths(case), case["batch"], case.get("gamma", 0), target["vocab"]
@@ -316,3 +341,154 @@ def tolerance(case):
     if case["kind"] == "classify":
         return dict(rel=2e-5)
     return dict(rel=2e-5) if case["model"] == "tiny" else dict(rel=2e-2)
+
+
+# ------------------------------------------------------------------------------------------- the same in 64 bits
+class _Weights:
+    """Takes the tensors that a context would, and keeps them."""
+
+    def __init__(self):
+        self.tensors, self.lora = {}, {}
+
+    def sd_load_tensor(self, model, kind, layer, tensor):
+        self.tensors[model, kind, layer] = tensor
+
+    def sd_load_lora(self, adapter, layer, mat, a, b):
+        self.lora[adapter, layer, mat] = (a, b)
+
+
+def _norm(h):                                            # all norm gains are 1
+    return h * torch.rsqrt((h * h).mean(-1, keepdim=True) + 1e-5)
+
+
+class _Model64:
+    """One sequence's view of a model: weights as given, arithmetic and cache in 64 bits."""
+
+    def __init__(self, w, model, dims, adapter=None):
+        self.w, self.model, self.d, self.adapter, self.n = w, model, dims, adapter, 0
+        self.k, self.v = ([None] * dims["n_layers"] for _ in range(2))
+
+    def _mats(self, layer, names, mat):
+        m = torch.cat([self.w.tensors[self.model, binding.TENSOR_KIND[name], layer].double() for name in names])
+        if self.adapter is not None:
+            a, b = self.w.lora[self.adapter, layer, mat]
+            m += LORA["scale"] * (b.double() @ a.double())
+        return m
+
+    def __call__(self, tokens, lm_head=True):
+        """Logits of the rows (or None) after `tokens` are appended to the first self.n positions."""
+        d, n0, rows = self.d, self.n, len(tokens)
+        H, Hkv, hd, F = d["n_heads"], d["n_kv_heads"], d["head_dim"], d["d_ffn"]
+        h = self.w.tensors[self.model, binding.T_EMBED, 0][torch.as_tensor(tokens, device=DEV).long()].double()
+        pos = torch.arange(n0, n0 + rows, device=DEV, dtype=torch.float64)
+        ang = pos[:, None] * 10000.0 ** (-torch.arange(0, hd, 2, device=DEV, dtype=torch.float64) / hd)
+        cos, sin = ang.cos()[:, None], ang.sin()[:, None]
+
+        def rope(x):
+            a, b = x[..., : hd // 2], x[..., hd // 2:]
+            return torch.cat([a * cos - b * sin, a * sin + b * cos], -1)
+
+        mask = torch.arange(n0 + rows, device=DEV)[None] > torch.arange(n0, n0 + rows, device=DEV)[:, None]
+        for l in range(d["n_layers"]):
+            qkv = (_norm(h) @ self._mats(l, ("wq", "wk", "wv"), 0).T).view(rows, H + 2 * Hkv, hd)
+            q, k, v = rope(qkv[:, :H]), rope(qkv[:, H: H + Hkv]), qkv[:, H + Hkv:]
+            if self.k[l] is not None:
+                k, v = torch.cat([self.k[l][:n0], k]), torch.cat([self.v[l][:n0], v])
+            self.k[l], self.v[l] = k, v
+            att = torch.empty_like(q)
+            for j in range(Hkv):
+                mine = slice(j * (H // Hkv), (j + 1) * (H // Hkv))
+                s = (q[:, mine].transpose(0, 1) @ k[:, j].T / math.sqrt(hd)).masked_fill(mask, -math.inf)
+                att[:, mine] = (s.softmax(-1) @ v[:, j]).transpose(0, 1)
+            h = h + att.reshape(rows, H * hd) @ self._mats(l, ("wo",), 1).T
+            gu = _norm(h) @ self._mats(l, ("wg", "wu"), 2).T
+            h = h + (torch.nn.functional.silu(gu[:, :F]) * gu[:, F:]) @ self._mats(l, ("wd",), 3).T
+        self.n = n0 + rows
+        return _norm(h) @ self.w.tensors[self.model, binding.T_LM_HEAD, 0].double().T if lm_head else None
+
+
+def _exact_cluster(case, g):
+    x, c = (t.double() for t in _corpus(case, g))
+    d2 = torch.stack([((x - ck) ** 2).sum(1) for ck in c], 1)
+    near, labels = d2.min(1)
+    counts = torch.bincount(labels, minlength=len(c))
+    out = torch.stack([x[labels == k].mean(0) if counts[k] else c[k] for k in range(len(c))])
+    return labels.int(), out, counts, near.sum()[None]
+
+
+def _exact_classify(case, seed, g):
+    tokens, starts, lens = _queue(case, seed, g)
+    w = {k: torch.from_numpy(a).to(DEV).double() for k, a in
+         synth.make_mamba_classifier(MAMBA_VOCAB, n_classes=case["classes"], seed=seed).items()}
+    n, top, (Di, R), N, taps = len(lens), int(lens.max()), w["w_dt"].shape, w["a_log"].shape[1], w["w_conv"].shape[1]
+    ids = torch.zeros((n, top), dtype=torch.long, device=DEV)
+    for i, (a, m) in enumerate(zip(starts, lens)):
+        ids[i, :m] = tokens[a: a + m]
+    last = torch.from_numpy(lens).to(DEV)
+    before = torch.zeros((n, taps, Di), dtype=torch.float64, device=DEV)
+    state, total = torch.zeros((n, Di, N), dtype=torch.float64, device=DEV), torch.zeros((n, Di), dtype=torch.float64, device=DEV)
+    A, silu = -w["a_log"].exp(), torch.nn.functional.silu
+    for t in range(top):
+        u, z = (w["embed"][ids[:, t]] @ w["w_in"].T).split(Di, 1)
+        before = torch.cat([before[:, 1:], u[:, None]], 1)
+        v = silu(w["b_conv"] + (before * w["w_conv"].T).sum(1))
+        r, B, C = (v @ w["w_x"].T).split([R, N, N], 1)
+        dt = torch.nn.functional.softplus(r @ w["w_dt"].T + w["b_dt"])
+        state = (dt[:, :, None] * A).exp() * state + (dt * v)[:, :, None] * B[:, None]
+        total += (((state * C[:, None]).sum(2) + w["d_skip"] * v) * silu(z)) * (t < last)[:, None]
+    scores = (total @ w["w_out"].T / last[:, None]) @ w["w_fc"].T + w["b_fc"]
+    return scores, scores.argmax(1).int()
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits.  One token stands out at every position, so every draw is the most probable one."""
+    g = _generator(seed)
+    if case["kind"] == "cluster":
+        return _exact_cluster(case, g)
+    if case["kind"] == "classify":
+        return _exact_classify(case, seed, g)
+    _, target, drafts, clf = _models(case)
+    lens, n, T = _lengths(case), case["batch"], case["temperature"]
+    if 2.0 * _params(target, False) * sum(lens) > 1.5e14:                 # too long at the rate of 64-bit sums
+        return None
+    w = _Weights()
+    with torch.cuda.stream(_stream()):
+        V = _fill(w, case, g)
+        texts = [list(map(int, p)) for p in _prompts(case, V, g)]
+    torch.cuda.synchronize()
+    classifier = {k: torch.from_numpy(a).to(DEV).double() for k, a in synth.make_classifier(*clf, seed=seed).items()}
+    gamma = case.get("gamma", 0)
+    logits = torch.empty((n, gamma + 1, V), dtype=torch.float64, device=DEV)
+    q = torch.empty((n, gamma, V), dtype=torch.float64, device=DEV)
+    x = torch.empty((n, gamma), dtype=torch.int32)
+    n_acc, out_tok = torch.empty(n, dtype=torch.int32), torch.full((n, gamma + 1), -1, dtype=torch.int32)
+    for i, text in enumerate(texts):
+        task = _task(case, i)
+        if case.get("classifier"):
+            mean = w.tensors[0, binding.T_EMBED, 0][torch.tensor(text, device=DEV)].double().mean(0)
+            task = int((classifier["w2"] @ torch.relu(classifier["w1"] @ mean + classifier["b1"]) + classifier["b2"]).argmax())
+        model = _Model64(w, 0, target)
+        model(text[:-1], lm_head=False)
+        if case["kind"] == "decode":
+            logits[i] = model(text[-1:])
+            continue
+        draft = _Model64(w, 1, drafts[0], task) if case.get("adapters") else _Model64(w, 1 + task, drafts[task])
+        wanted, have = case.get("new_tokens", 1), 0
+        while have < wanted:
+            drawn = []
+            for s in range(gamma):
+                row = draft((text + drawn)[draft.n:])[-1]
+                drawn.append(int(row.argmax()))
+                q[i, s] = (row / T).softmax(0) if T > 0 else torch.nn.functional.one_hot(row.argmax(), V)
+            logits[i] = model(text[-1:] + drawn)
+            says = logits[i].argmax(1).tolist()
+            kept = next((s for s in range(gamma) if drawn[s] != says[s]), gamma)
+            x[i], n_acc[i] = torch.tensor(drawn), kept
+            out_tok[i] = torch.tensor(drawn[:kept] + [says[kept]] + [-1] * (gamma - kept))
+            text += drawn[:kept] + [says[kept]]
+            have += kept + 1
+            model.n, draft.n = len(text) - 1, min(len(text) - 1, draft.n)
+    if case["kind"] == "decode":
+        return logits
+    out = (x.to(DEV), q, logits, n_acc.to(DEV), out_tok.to(DEV))
+    return (np.array(texts[0][: case["ctx_hi"] + case["new_tokens"]], dtype=np.int32), *out) if case["kind"] == "request" else out
