@@ -10,6 +10,7 @@
 #include "gemm_tc.h"
 #include "kernels.h"
 #include "pass_stream.h"
+#include "prefill.h"
 
 using namespace sd;
 
@@ -68,6 +69,7 @@ constexpr int PASS_ROWS_CAP = 32;               // most query rows of a pass on 
 constexpr size_t PASS_REGION_BYTES = (size_t)64 << 20;      // each of the two workspace regions of that kernel
 constexpr size_t PASS_PROG_BYTES = (size_t)768 << 10;       // one cached program
 constexpr int PASS_PROG_SLOTS = 8;
+constexpr int PF_MIN_ROWS = 17;                 // fewest rows of a prefill pass (prefill.cu); below, and sequence by sequence: forward().  One prompt of 20 rows: 1B 0.93 against 0.99 ms, 7B 3.57 against 3.69
 
 struct sd_ctx {
     sd_config cfg;
@@ -99,6 +101,10 @@ struct sd_ctx {
     std::vector<cudaEvent_t> ev_join;
     cudaEvent_t ev_fork;
     bool groups_concurrent;
+    // prefill passes (prefill.cu): scratch of pf_rows rows, shared by all models; 0 rows: no model takes that path
+    int pf_rows;
+    float* pf_h; bf16* pf_xn; bf16* pf_q; bf16* pf_attn; bf16* pf_act; float* pf_part; float* pf_scale;
+    int32_t* pf_slot; int32_t* pf_pos; int32_t* pf_task; float* pf_t;
     // persistent streaming kernel (pass_stream.cu): packed input rows, workspace, programs
     // (everything CTAs of that kernel hand to one another is tagged 64-bit words; the whole block is cleared when tags are about to repeat)
     tagged_t* tg_h; tagged_t* tg_xn; tagged_t* tg_attn; tagged_t* tg_act; tagged_t* tg_q; tagged_t* tg_newkv; tagged_t* tg_ssq;
@@ -148,6 +154,12 @@ struct sd_ctx {
 namespace {
 
 size_t esize(int dtype) { return dtype == SD_BF16 ? 2 : 4; }
+
+// Whether a model's passes run on the tensor-core kernels.
+bool tensor_path(const sd_model_desc& m) {
+    return m.dtype == SD_BF16 && (m.head_dim == 64 || m.head_dim == 128) && m.d_model <= 128 * SSQ_STRIDE && m.d_ffn % 64 == 0 &&
+           attention_split_supported(m.dtype, m.n_heads, m.n_kv_heads, m.head_dim);
+}
 
 int sm_count() {                               // of the current device
     int dev = 0, v = 0;
@@ -318,6 +330,21 @@ void layout(sd_ctx* c, const sd_model_desc* ms, Bump& B) {
             s.rope_row_sin = (float*)B.take(sizeof(float) * SD_MAX_ROWS * dhalf);
             c->sets.push_back(s);
         }
+    }
+    {   // prefill passes: sized for the largest tensor-core model
+        size_t d = 0, dq = 0, f = 0;
+        for (int i = 0; i < nm; ++i)
+            if (tensor_path(ms[i])) {
+                d = std::max(d, (size_t)ms[i].d_model); dq = std::max(dq, (size_t)ms[i].n_heads * ms[i].head_dim); f = std::max(f, (size_t)ms[i].d_ffn);
+            }
+        c->pf_rows = d ? (int)std::min<long long>(PF_MAX_ROWS, (long long)S * cfg.max_ctx) : 0;
+        const size_t n = c->pf_rows;
+        c->pf_h = (float*)B.take(sizeof(float) * n * d); c->pf_part = (float*)B.take(sizeof(float) * n * d);
+        c->pf_xn = (bf16*)B.take(sizeof(bf16) * n * d); c->pf_q = (bf16*)B.take(sizeof(bf16) * n * dq);
+        c->pf_attn = (bf16*)B.take(sizeof(bf16) * n * dq); c->pf_act = (bf16*)B.take(sizeof(bf16) * n * f);
+        c->pf_scale = (float*)B.take(sizeof(float) * (n + 256));
+        c->pf_slot = (int32_t*)B.take(sizeof(int32_t) * n); c->pf_pos = (int32_t*)B.take(sizeof(int32_t) * n); c->pf_task = (int32_t*)B.take(sizeof(int32_t) * n);
+        c->pf_t = (float*)B.take(cfg.lora_adapters > 0 ? sizeof(float) * n * 128 : 0);
     }
     {   // persistent streaming kernel: tagged 64-bit words for up to PASS_ROWS_CAP rows (padded to a multiple of 16)
         const size_t rows_pad = (PASS_ROWS_CAP + 15) & ~15;
@@ -678,6 +705,108 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     return SD_OK;
 }
 
+// One prefill pass over the packed rows of `segs` (prefill.cu): leaves the rows' keys and values in the model's cache.
+sd_status forward_prefill(sd_ctx* c, Model& M, const PrefillSegs& segs) {
+    const sd_model_desc& m = M.d;
+    const int d = m.d_model, H = m.n_heads, Hkv = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, n = segs.rows, sm = sm_count();
+    cudaStream_t st = c->st;
+    auto gemm = [&](const TensorMap& tw, const bf16* x, PrefillGemm& g) -> sd_status {
+        TensorMap tx;
+        if (!make_tensor_map_bf16(&tx, x, n, g.K, g.bn / 2)) return SD_ERR_CUDA;
+        LAUNCH(CAT_LINEAR, launch_prefill_gemm(tw, tx, g, sm, c->S.status, st));
+        return SD_OK;
+    };
+    // the matrix's adapters: x A^T of all of them first, then the matrix itself, which adds B times the row's own
+    auto with_lora = [&](const TensorMap& tw, const bf16* x, PrefillGemm& g, const Layer& L, int mat) -> sd_status {
+        if (!M.lora) return SD_OK;
+        PrefillGemm t = prefill_geometry(PF_PARTIAL, n, g.n_out + 128, g.K, sm, 0, g.n_out / 256);
+        t.part = c->pf_t; t.part_ld = 128; t.f_lo = g.n_out;
+        SD_TRY(gemm(tw, x, t));
+        g.lora_b = L.lora_b[mat]; g.lora_t = c->pf_t; g.lora_task = c->pf_task;
+        g.lora_r = c->cfg.lora_rank; g.lora_n = c->cfg.lora_adapters; g.lora_scale = c->cfg.lora_scale;
+        return SD_OK;
+    };
+    auto residual = [&](const TensorMap& tw, const bf16* x, int K, const float* gain, const Layer& L, int mat) -> sd_status {
+        PrefillGemm g = prefill_geometry(PF_PARTIAL, n, d, K, sm, c->pf_rows);
+        g.part = c->pf_part;
+        SD_TRY(with_lora(tw, x, g, L, mat));
+        SD_TRY(gemm(tw, x, g));
+        LAUNCH(CAT_FUSED_STEP, launch_prefill_norm(c->pf_h, c->pf_part, g.split, n, d, gain, m.rms_eps, c->pf_xn, c->pf_scale, st));
+        return SD_OK;
+    };
+    LAUNCH(CAT_ELEMENTWISE, launch_prefill_embed(c->S, segs, (const bf16*)M.embed, d, m.vocab, M.layers[0].norm1, m.rms_eps, c->pf_h, c->pf_xn,
+                                                 c->pf_scale, c->pf_slot, c->pf_pos, c->pf_task, st));
+    for (int l = 0; l < m.n_layers; ++l) {
+        const Layer& L = M.layers[l];
+        const bool last = l + 1 == m.n_layers;              // only its keys and values are ever read
+        bf16* kc = (bf16*)(M.kcache + M.kv_layer_bytes * l);
+        bf16* vc = (bf16*)(M.vcache + M.kv_layer_bytes * l);
+        PrefillGemm g = prefill_geometry(PF_QKV, n, M.n_qkv(), d, sm, 0, last ? H * hd / 256 : 0);
+        g.scale = c->pf_scale; g.q_out = c->pf_q; g.kc = kc; g.vc = vc; g.row_slot = c->pf_slot; g.row_pos = c->pf_pos;
+        g.H = H; g.Hkv = Hkv; g.hd = hd; g.max_ctx = c->cfg.max_ctx; g.rcos = M.rope_cos; g.rsin = M.rope_sin;
+        SD_TRY(with_lora(L.tm_qkv, c->pf_xn, g, L, SD_LORA_QKV));
+        SD_TRY(gemm(L.tm_qkv, c->pf_xn, g));
+        if (last) break;
+        LAUNCH(CAT_ATTENTION, launch_prefill_attention(c->pf_q, kc, vc, c->pf_attn, segs, H, Hkv, hd, c->cfg.max_ctx, st));
+        SD_TRY(residual(L.tm_wo, c->pf_attn, H * hd, L.norm2, L, SD_LORA_WO));
+        g = prefill_geometry(PF_SWIGLU, n, 2 * F, d, sm, 0);
+        g.scale = c->pf_scale; g.act = c->pf_act; g.F = F;
+        SD_TRY(with_lora(L.tm_gu, c->pf_xn, g, L, SD_LORA_GU));
+        SD_TRY(gemm(L.tm_gu, c->pf_xn, g));
+        SD_TRY(residual(L.tm_wd, c->pf_act, F, M.layers[l + 1].norm1, L, SD_LORA_WD));
+    }
+    CUDA_TRY(prof_mark(c, CAT_NONE));
+    return SD_OK;
+}
+
+// Prompts of the listed sequences, all but their last token, through one model.
+sd_status prefill_model(sd_ctx* c, Model& M, const SeqList& list) {
+    int done[SD_MAX_BATCH] = {};                            // rows of each sequence that have been through
+    if (c->pf_rows > 0 && M.tc && !c->force_plain) {
+        // All sequences' rows packed into as few passes as the scratch allows, of about equal size.  What a sequence has
+        // beyond a multiple of 256 rows stays out when it is 3...16 rows: passes of that size carry their activations in two
+        // bf16 parts (forward_tc), and so they do below.
+        int take[SD_MAX_BATCH], total = 0;
+        for (int i = 0; i < list.n; ++i) {
+            const int n = c->n_prompt[list.ids[i]] - 1, rest = n % SD_MAX_ROWS;
+            take[i] = c->two_part && rest >= 3 && rest <= 16 ? n - rest : n;
+            total += take[i];
+        }
+        if (total >= PF_MIN_ROWS) {
+            const int passes = (total + c->pf_rows - 1) / c->pf_rows, per = (total + passes - 1) / passes;
+            int i = 0;
+            while (total > 0) {
+                PrefillSegs segs;
+                segs.n = 0; segs.rows = 0; segs.row0[0] = 0; segs.blk0[0] = 0;
+                for (; i < list.n && segs.rows < per; ++i) {
+                    const int n = std::min(take[i] - done[i], per - segs.rows);
+                    if (n > 0) {
+                        segs.slot[segs.n] = list.ids[i]; segs.pos0[segs.n] = done[i];
+                        done[i] += n; segs.rows += n;
+                        segs.row0[segs.n + 1] = segs.rows;
+                        segs.blk0[segs.n + 1] = segs.blk0[segs.n] + (n + PF_QBLOCK - 1) / PF_QBLOCK;
+                        ++segs.n;
+                    }
+                    if (done[i] < take[i]) break;           // the rest of this sequence opens the next pass
+                }
+                total -= segs.rows;
+                SD_TRY(forward_prefill(c, M, segs));
+            }
+        }
+    }
+    for (int i = 0; i < list.n; ++i) {
+        const int s = list.ids[i], n = c->n_prompt[s] - 1;
+        SeqList one = list;
+        one.n = 1; one.ids[0] = s; one.out[0] = 0;
+        for (int p0 = done[i]; p0 < n; p0 += SD_MAX_ROWS) {
+            const int rows = std::min(SD_MAX_ROWS, n - p0);
+            RowPlan plan{PLAN_PREFILL, rows, p0, 0, 0, nullptr, p0 + rows};
+            SD_TRY(forward(c, M, one, plan, rows, LOGITS_NONE, nullptr));
+        }
+    }
+    return SD_OK;
+}
+
 // The same pass as one launch of the persistent streaming kernel (few query rows): the embedding kernel writes the first
 // input rows in the packed layout, then every layer and the lm_head run inside k_pass_stream.
 sd_status forward_pass(sd_ctx* c, Model& M, const sd_ctx::CachedProgram& cp, const SeqList& list, const RowPlan& plan, int n_rows, int mode,
@@ -935,8 +1064,7 @@ sd_status sd_create(const sd_config* cfg, const sd_model_desc* models, void* cud
     for (Model& M : c->models) {
         const sd_model_desc& m = M.d;
         M.pass_ok = false;
-        M.tc = m.dtype == SD_BF16 && (m.head_dim == 64 || m.head_dim == 128) && m.d_model <= 128 * SSQ_STRIDE && m.d_ffn % 64 == 0 &&
-               attention_split_supported(m.dtype, m.n_heads, m.n_kv_heads, m.head_dim);
+        M.tc = tensor_path(m);
         if (!M.tc && M.lora) return fail(SD_ERR_UNSUPPORTED);
         if (!M.tc) continue;
         const int dq = m.n_heads * m.head_dim;
@@ -1140,19 +1268,16 @@ sd_status sd_route_prompt_mamba(sd_ctx* c, const sd_mamba_desc* desc, const sd_m
 sd_status sd_prefill(sd_ctx* c, const int32_t* seqs, int n_seq) {
     SeqList all;
     SD_TRY(make_list(c, seqs, n_seq, c->cfg.n_drafts > 0 ? PH_ROUTED : PH_BEGUN, all));
+    SD_TRY(prefill_model(c, c->models[0], all));
+    for (size_t k = 1; k < c->models.size(); ++k) {            // every draft over the sequences routed to it
+        SeqList g = all;
+        g.n = 0;
+        for (int i = 0; i < n_seq; ++i)
+            if (draft_model_index(c->cfg, c->draft_id[seqs[i]]) == (int)k) g.ids[g.n++] = seqs[i];
+        if (g.n) SD_TRY(prefill_model(c, c->models[k], g));
+    }
     for (int i = 0; i < n_seq; ++i) {
         const int s = seqs[i], n = c->n_prompt[s] - 1;
-        SeqList one = all;
-        one.n = 1; one.ids[0] = s; one.out[0] = 0;
-        for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 1 && c->cfg.n_drafts < 1) break;
-            Model& M = c->models[pass == 0 ? 0 : draft_model_index(c->cfg, c->draft_id[s])];
-            for (int p0 = 0; p0 < n; p0 += SD_MAX_ROWS) {
-                const int rows = std::min(SD_MAX_ROWS, n - p0);
-                RowPlan plan{PLAN_PREFILL, rows, p0, 0, 0, nullptr, p0 + rows};
-                SD_TRY(forward(c, M, one, plan, rows, LOGITS_NONE, nullptr));
-            }
-        }
         LAUNCH(CAT_STATE, launch_set_state(c->S, s, n + 1, n, n, 0u, 0u, 0, c->st));
         c->phase[s] = PH_READY;
     }
