@@ -19,7 +19,10 @@
 //     once; the first part of its weight stream does not wait for the predecessor (the token rows
 //     and the workspace do), so most of the ring is full when the consumers are released.
 // Roles: warp 0 streams weights, warp 1 allocates TMEM and issues MMAs, warps 2..5 drain TMEM
-// into the workspace, warp 6 loads the token rows.  Every mbarrier wait is bounded; on expiry
+// into the workspace, warp 6 loads the token rows.  Warps 0, 1 and 6 walk their loops whole, one elected lane issues (see
+// elect_one): what a boundary between two GEMMs costs is the time the MMA warp takes to catch up with a full ring, 0.3 us a stage
+// as a one-lane loop (7B verify step with its drafts 4.81 -> 4.57 ms, 7B decoding step 3.08 -> 2.85 ms, 1B 1.29 -> 1.22 ms).
+// Every mbarrier wait is bounded; on expiry
 // the kernel flags SD_DEV_WAIT_EXPIRED and winds down.
 #include <cuda.h>
 
@@ -62,7 +65,7 @@ struct RingPos {
     int stage; uint32_t use; int filled;
     __device__ __forceinline__ RingPos() : stage(0), use(0u), filled(0) {}
     __device__ __forceinline__ void next(int stages, int steady) {         // position of the following load (no divisions: the MMA
-        ++stage;                                                           // thread's loop is bound by its own instruction latencies)
+        ++stage;                                                           // warp's loop is bound by its own instruction latencies)
         if (!filled) { if (stage == stages) { stage = 0; use = 1u; filled = 1; } }
         else if (stage == steady) { stage = 0; ++use; }
     }
@@ -163,33 +166,34 @@ k_gemm_streamk(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
         // ------------------------------------------------------------------ weight producer
         // The first tiles do not wait for the previous kernel (weights do not depend on it): the stream
         // starts as soon as the CTA is resident, while the consumers wait on the previous kernel.
-        if (lane == 0) {
-            uint64_t pol_stream;
-            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
-            RingPos rp;
-            bool dep_ok = false;
-            uint64_t t_last = 0;
-            volatile int* dep_seen = &sh.dep_seen;
-            int tile = u0 / g.kb_per_tile, kb = u0 % g.kb_per_tile;
-            for (uint32_t it = 0; it < n_units; ++it, rp.next(g.stages, g.steady)) {
-                const int s = rp.stage;
-                // A full ring of requests at this point slowed the step down: they compete with the small,
-                // latency-critical reads of the kernel that reduces the previous GEMM.  So the run-ahead stops
-                // short of the ring's depth until that kernel has finished.
-                if (it >= (uint32_t)g.prefill && !dep_ok) {
-                    if (g.pace_ns <= 0) { pdl_wait(); dep_ok = true; }
-                    else {          // paced: one more stage every pace_ns, so that requests stay in flight until the kernel before is done
-                        const uint64_t t_next = t_last + (uint64_t)g.pace_ns;
-                        while (!(dep_ok = *dep_seen != 0) && global_ns() < t_next) {}
-                    }
+        const bool leader = elect_one();
+        uint64_t pol_stream;
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol_stream));
+        RingPos rp;
+        bool dep_ok = false;
+        uint64_t t_last = 0;
+        volatile int* dep_seen = &sh.dep_seen;
+        int tile = u0 / g.kb_per_tile, kb = u0 % g.kb_per_tile;
+        for (uint32_t it = 0; it < n_units; ++it, rp.next(g.stages, g.steady)) {
+            const int s = rp.stage;
+            // A full ring of requests at this point slowed the step down: they compete with the small,
+            // latency-critical reads of the kernel that reduces the previous GEMM.  So the run-ahead stops
+            // short of the ring's depth until that kernel has finished.
+            if (it >= (uint32_t)g.prefill && !dep_ok) {
+                if (g.pace_ns <= 0) { pdl_wait(); dep_ok = true; }
+                else {              // paced: one more stage every pace_ns, so that requests stay in flight until the kernel before is done
+                    const uint64_t t_next = t_last + (uint64_t)g.pace_ns;
+                    while (!(dep_ok = __all_sync(0xffffffffu, *dep_seen != 0)) && !__all_sync(0xffffffffu, global_ns() >= t_next)) {}
                 }
-                if (rp.use > 0u && !mbar_wait(smem_u32(&sh.empty[s]), (rp.use & 1u) ^ 1u, abort_flag)) break;
-                const uint32_t bar = smem_u32(&sh.full[s]);
+            }
+            if (rp.use > 0u && !mbar_wait_warp(smem_u32(&sh.empty[s]), (rp.use & 1u) ^ 1u, abort_flag)) break;
+            const uint32_t bar = smem_u32(&sh.full[s]);
+            if (leader) {
                 mbar_expect_tx(bar, A_BYTES);
                 tma_load_2d(tiles0 + s * stage_bytes, &tm_w, kb * TILE_K, tile * TILE_N, bar, pol_stream);
-                if (g.pace_ns > 0 && !dep_ok) t_last = global_ns();
-                if (++kb == g.kb_per_tile) { kb = 0; ++tile; }
             }
+            if (g.pace_ns > 0 && !dep_ok) t_last = global_ns();
+            if (++kb == g.kb_per_tile) { kb = 0; ++tile; }
         }
     } else if (warp == 6) {
         // ------------------------------------------------------------------ token-row producer
@@ -244,52 +248,55 @@ k_gemm_streamk(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__
                 stop = __shfl_sync(0xffffffffu, (int)stop, 0) != 0;
                 if (++kb == g.kb_per_tile) kb = 0;
             }
-        } else if (lane == 0) {
+        } else {
+            const bool leader = elect_one();
             uint64_t pol_keep;
             asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol_keep));
             pdl_wait();                                           // the token rows are the previous kernel's output
-            *(volatile int*)&sh.dep_seen = 1;
-            stamp_pair(g.stamp, ST_DEP_FIRST);
+            if (leader) { *(volatile int*)&sh.dep_seen = 1; stamp_pair(g.stamp, ST_DEP_FIRST); }
             RingPos rp;
             int kb = u0 % g.kb_per_tile;
             for (uint32_t it = 0; it < n_units; ++it, rp.next(g.stages, g.steady)) {
                 const int s = rp.stage;
-                if (rp.use > 0u && !mbar_wait(smem_u32(&sh.empty[s]), (rp.use & 1u) ^ 1u, abort_flag)) break;
+                if (rp.use > 0u && !mbar_wait_warp(smem_u32(&sh.empty[s]), (rp.use & 1u) ^ 1u, abort_flag)) break;
                 const uint32_t bar = smem_u32(&sh.full[s]);
-                mbar_expect_tx(bar, x_bytes);
-                tma_load_2d(tiles0 + s * stage_bytes + A_BYTES, &tm_x, kb * TILE_K, 0, bar, pol_keep);
+                if (leader) {
+                    mbar_expect_tx(bar, x_bytes);
+                    tma_load_2d(tiles0 + s * stage_bytes + A_BYTES, &tm_x, kb * TILE_K, 0, bar, pol_keep);
+                }
                 if (++kb == g.kb_per_tile) kb = 0;
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.m_pad >> 3) << 17) | ((uint32_t)(TILE_N >> 4) << 24);
-            uint32_t seg = 0;
-            bool ok = true;
-            RingPos rp;
-            const uint64_t desc0 = umma_desc(tiles0);
-            uint32_t kb0 = u0 % g.kb_per_tile;
-            for (uint32_t u = u0; u < u1 && ok; ++seg, kb0 = 0) {
-                const uint32_t n_kb = min((uint32_t)g.kb_per_tile - kb0, u1 - u);
-                const uint32_t buf = seg & 1u;
-                if (!mbar_wait(smem_u32(&sh.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag)) break;
+        const bool leader = elect_one();
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.m_pad >> 3) << 17) | ((uint32_t)(TILE_N >> 4) << 24);
+        uint32_t seg = 0;
+        bool ok = true;
+        RingPos rp;
+        const uint64_t desc0 = umma_desc(tiles0);
+        uint32_t kb0 = u0 % g.kb_per_tile;
+        for (uint32_t u = u0; u < u1 && ok; ++seg, kb0 = 0) {
+            const uint32_t n_kb = min((uint32_t)g.kb_per_tile - kb0, u1 - u);
+            const uint32_t buf = seg & 1u;
+            if (!mbar_wait_warp(smem_u32(&sh.tmem_empty[buf]), ((seg >> 1) & 1u) ^ 1u, abort_flag)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t d_tmem = tmem_base + buf * (uint32_t)g.m_pad;
+            for (uint32_t j = 0; j < n_kb; ++j, rp.next(g.stages, g.steady)) {
+                const int s = rp.stage;
+                if (!mbar_wait_warp(smem_u32(&sh.full[s]), rp.use & 1u, abort_flag)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d_tmem = tmem_base + buf * (uint32_t)g.m_pad;
-                for (uint32_t j = 0; j < n_kb; ++j, rp.next(g.stages, g.steady)) {
-                    const int s = rp.stage;
-                    if (!mbar_wait(smem_u32(&sh.full[s]), rp.use & 1u, abort_flag)) { ok = false; break; }
+                const uint64_t da = desc0 + (uint64_t)((uint32_t)s * (stage_bytes >> 4)), db = da + (A_BYTES >> 4);   // start-address field counts 16 bytes
+                if (leader) {
                     if (u == u0 && j == 0) stamp_pair(g.stamp, ST_DATA_FIRST);
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint64_t da = desc0 + (uint64_t)((uint32_t)s * (stage_bytes >> 4)), db = da + (A_BYTES >> 4);   // start-address field counts 16 bytes
 #pragma unroll
                     for (uint32_t k = 0; k < TILE_K / 16; ++k)     // 16 elements = 32 bytes further along the swizzled row
                         umma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (j | k) != 0u);
                     umma_commit(smem_u32(&sh.empty[s]));           // frees the stage once these MMAs have read it
                 }
-                if (ok) umma_commit(smem_u32(&sh.tmem_full[buf]));
-                u += n_kb;
             }
+            if (ok && leader) umma_commit(smem_u32(&sh.tmem_full[buf]));
+            u += n_kb;
         }
     } else {
         // ------------------------------------------------------------------ epilogue: TMEM -> workspace
