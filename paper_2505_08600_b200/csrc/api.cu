@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "gemm_tc.h"
+#include "gemv.h"
 #include "kernels.h"
 #include "pass_stream.h"
 #include "prefill.h"
@@ -88,6 +89,7 @@ struct sd_ctx {
     uint32_t* xready; size_t xready_used; bool xready_on;
     struct XReady { uint32_t* words; int n_tiles; int shift; uint32_t need; };
     XReady x_from;                              // what the most recent step kernel counts into (words == nullptr: nothing)
+    float* lora_t;                              // [row][128]: x A^T of a matrix's adapters (few-rows passes)
     float* rope_row_cos; float* rope_row_sin;   // [row][head_dim/2] rotary factors of the pass's rows (their positions applied)
     // Draft groups side by side: sequences routed to different draft models run their draft passes on streams of their own,
     // each with a scratch set of its own (set 0 is the fields above; sets 1... are sized for the draft models only).
@@ -293,6 +295,7 @@ void layout(sd_ctx* c, const sd_model_desc* ms, Bump& B) {
     c->rope_row_sin = (float*)B.take(sizeof(float) * SD_MAX_ROWS * half_max);
     c->xready = (uint32_t*)B.take(sizeof(uint32_t) * XREADY_WORDS);
     c->xready_used = 0;
+    c->lora_t = (float*)B.take(cfg.lora_adapters > 0 ? sizeof(float) * GEMV_MAX_ROWS * 128 : 0);
     c->sets.clear();
     c->sets.push_back(sd_ctx::ScratchSet{c->h, c->xn, c->q, c->attn, c->act, c->lin, c->draft_logits, c->row_slot, c->row_pos, c->attn_ws,
                                          c->attn_ws_bytes, c->partials, c->partials_bytes, c->ssq, c->gemm_arrive, c->xready, c->rope_row_cos,
@@ -622,6 +625,37 @@ sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n
     return SD_OK;
 }
 
+// Whether a pass takes the few-rows kernels (gemv.cu): the draft models, whose matrices a pass is through with in less time
+// than the weight-streaming GEMM and its step kernel need to hand over.
+bool few_rows_pass(sd_ctx* c, const Model& M, int n_rows) {
+    const sd_model_desc& m = M.d;
+    if (&M == &c->models[0] || n_rows > GEMV_MAX_ROWS || m.d_model % 16 || m.d_model > 16 * GEMV_SSQ_STRIDE) return false;
+    Gemv g;
+    memset(&g, 0, sizeof(g));
+    g.rows = n_rows;
+    auto ok = [&](int mode, int n_out, int K) { g.ep.mode = mode; g.ep.hd = m.head_dim; g.ep.F = m.d_ffn; g.n_out = n_out; g.K = K; return gemv_supported(g); };
+    return ok(EPI_QKV_ROPE, M.n_qkv(), m.d_model) && ok(EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) && ok(EPI_SWIGLU, 2 * m.d_ffn, m.d_model) &&
+           ok(EPI_RESIDUAL, m.d_model, m.d_ffn) && ok(EPI_PLAIN, m.vocab, m.d_model);
+}
+
+// One matrix and the step that follows it, on those kernels.
+sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out, int K, const Epilogue& ep, int ssq_stride) {
+    Gemv g;
+    memset(&g, 0, sizeof(g));
+    g.w = (const bf16*)w; g.x = (const bf16*)x; g.rows = rows; g.n_out = n_out; g.K = K; g.ep = ep;
+    g.ssq_stride = ssq_stride; g.ssq_out_stride = GEMV_SSQ_STRIDE;
+    if (ep.lora_b) {                            // x A^T of all adapters first (the rows behind the matrix's own)
+        Gemv t = g;
+        memset(&t.ep, 0, sizeof(t.ep));
+        t.ep.mode = EPI_PLAIN; t.ep.lo_off = ep.lo_off; t.ep.m_real = rows; t.ep.y = c->lora_t; t.ep.n_out_rows = rows; t.ep.row_stride = 1;
+        t.w = g.w + (size_t)n_out * K; t.n_out = 128;
+        LAUNCH(CAT_LINEAR, launch_gemv(t, c->st));
+        g.lora_t = c->lora_t;
+    }
+    LAUNCH(CAT_LINEAR, launch_gemv(g, c->st));
+    return SD_OK;
+}
+
 // The same pass on the tensor-core path (bf16 models): per layer the QKV GEMM, attention, the Wo,
 // gate/up and down GEMMs, each GEMM followed by a small kernel that sums its split accumulators
 // and applies the step after it; every kernel is a programmatic dependent of the one before.
@@ -640,7 +674,8 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     // With 3..16 rows (the verify rows of one sequence) the 16 (or 32) columns of the MMA hold every activation twice over:
     // as bf16(x) and as bf16(x - bf16(x)), 8 (or 16) rows apart.  The weights stream once all the same, and the GEMMs'
     // inputs are no longer rounded to 8 bits of mantissa.
-    const int lo = !c->two_part ? 0 : (n_rows >= 3 && n_rows <= 8) ? 8 : (n_rows >= 9 && n_rows <= 16) ? 16 : 0;
+    const bool few = few_rows_pass(c, M, n_rows);            // (there the second parts cost nothing, for one or two rows either)
+    const int lo = !c->two_part ? 0 : (n_rows >= (few ? 1 : 3) && n_rows <= 8) ? 8 : (n_rows >= 9 && n_rows <= 16) ? 16 : 0;
     if (c->stamps_on) {                                                     // the stamps of this pass replace the previous pass's
         c->stamp_kinds.clear();
         CUDA_TRY(cudaMemsetAsync(c->stamp_buf, 0xFF, sizeof(unsigned long long) * ST_WORDS * STAMP_CAP, st));
@@ -653,7 +688,10 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     int len_hint[SD_MAX_BATCH];                                             // context bounds of the pass's sequences, for attention's launch order
     for (int i = 0; i < list.n && i < SD_MAX_BATCH; ++i) len_hint[i] = c->len_ub[list.ids[i]];
     const RowScale first{c->ssq, 1, 1.f / d, m.rms_eps};                    // sum of squares in one piece (after the embedding)
-    const RowScale tiled{c->ssq, (d + 127) / 128, 1.f / d, m.rms_eps};      // ... in one piece per 128-wide tile of h
+    const RowScale tiled{c->ssq, few ? d / 16 : (d + 127) / 128, 1.f / d, m.rms_eps};      // ... in one piece per tile of h of the kernel before
+    auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e, int ssq_stride) {
+        return few ? gemv_step(c, w, x, n_rows, n_out, K, e, ssq_stride) : gemm_tc(c, tm, x, n_rows, n_out, K, e);
+    };
     LAUNCH(CAT_ELEMENTWISE, launch_embed(c->S, list, plan, n_rows, M.embed, dt, d, m.vocab, c->h, c->row_slot, c->row_pos,
                                          M.layers[0].norm1, c->xn, c->ssq, M.rope_cos, M.rope_sin, hd / 2, c->rope_row_cos, c->rope_row_sin, 0, nullptr, st, lo));
     for (int l = 0; l < m.n_layers; ++l) {
@@ -667,7 +705,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         e.q_out = (bf16*)c->q; e.kc = (bf16*)kc; e.vc = (bf16*)vc; e.row_slot = c->row_slot; e.row_pos = c->row_pos;
         e.H = H; e.Hkv = Hkv; e.hd = hd; e.max_ctx = c->cfg.max_ctx; e.rcos = c->rope_row_cos; e.rsin = c->rope_row_sin;
         with_lora(e, L, SD_LORA_QKV);
-        SD_TRY(gemm_tc(c, L.tm_qkv, c->xn, n_rows, M.n_qkv(), d, e));
+        SD_TRY(step(L.tm_qkv, L.wqkv, c->xn, M.n_qkv(), d, e, l == 0 ? SSQ_STRIDE : GEMV_SSQ_STRIDE));
         LAUNCH(CAT_ATTENTION, launch_attention_split(c->q, kc, vc, c->attn, c->row_slot, c->row_pos, n_rows, plan.rows_per_seq, H, Hkv,
                                                      hd, c->cfg.max_ctx, plan.ctx_bound, c->attn_ws, c->attn_ws_bytes, 1, st, lo,
                                                      next_stamp(c, SD_STAMP_ATTENTION), c->tune[SD_TUNE_ATTN_WARPS], c->tune[SD_TUNE_ATTN_CLUSTER],
@@ -677,18 +715,18 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         e.ring_stages = c->tune[SD_TUNE_WO_STAGES]; e.prefill_all = c->tune[SD_TUNE_WO_PREFILL_ALL];
         e.mode = EPI_RESIDUAL; e.h = c->h; e.gain_next = L.norm2; e.xn = (bf16*)c->xn; e.ssq_out = c->ssq;
         with_lora(e, L, SD_LORA_WO);
-        SD_TRY(gemm_tc(c, L.tm_wo, c->attn, n_rows, d, H * hd, e));
+        SD_TRY(step(L.tm_wo, L.wo, c->attn, d, H * hd, e, 0));
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
         e.mode = EPI_SWIGLU; e.rs = tiled; e.act = (bf16*)c->act; e.F = F;
         with_lora(e, L, SD_LORA_GU);
-        SD_TRY(gemm_tc(c, L.tm_gu, c->xn, n_rows, 2 * F, d, e));
+        SD_TRY(step(L.tm_gu, L.wgu, c->xn, 2 * F, d, e, GEMV_SSQ_STRIDE));
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
         e.mode = EPI_RESIDUAL; e.h = c->h; e.xn = (bf16*)c->xn; e.ssq_out = c->ssq;
         e.gain_next = l + 1 < m.n_layers ? M.layers[l + 1].norm1 : (mode != LOGITS_NONE ? M.final_norm : nullptr);
         with_lora(e, L, SD_LORA_WD);
-        SD_TRY(gemm_tc(c, L.tm_wd, c->act, n_rows, d, F, e));
+        SD_TRY(step(L.tm_wd, L.wd, c->act, d, F, e, 0));
     }
     if (mode != LOGITS_NONE) {
         // the lm_head GEMM runs over all rows (they share the one pass over the weights); only the wanted rows are written
@@ -699,7 +737,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         e.mode = EPI_PLAIN; e.rs = tiled; e.y = logits_out;
         if (mode == LOGITS_ALL) { e.n_out_rows = n_rows; e.row_stride = 1; e.row_offset = 0; }
         else { e.n_out_rows = list.n; e.row_stride = R; e.row_offset = R - 1; }
-        SD_TRY(gemm_tc(c, M.tm_lm, c->xn, n_rows, m.vocab, d, e));
+        SD_TRY(step(M.tm_lm, M.lm_head, c->xn, m.vocab, d, e, GEMV_SSQ_STRIDE));
     }
     CUDA_TRY(prof_mark(c, CAT_NONE));
     return SD_OK;

@@ -1,0 +1,52 @@
+"""The few-rows kernels of the draft passes against the CPU oracle: reductions that do not fill the kernel's form, a vocabulary
+that does not fill its tiles, heads of 64 and 128, 1...16 rows in one and two groups of eight, and one call beyond them."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2505_08600_b200 import synth
+from gpu_util import DEV
+
+pytestmark = pytest.mark.gpu
+
+# log q = logit - log sum exp: two numbers that are each within the logits' 5e-2 of the oracle's
+LOG_TOL = 1e-1
+
+
+def _m(L, d, H, hd, F, V):
+    return dict(n_layers=L, d_model=d, n_heads=H, n_kv_heads=H, head_dim=hd, d_ffn=F, vocab=V)
+
+
+DRAFTS = {
+    "d288": _m(2, 288, 3, 64, 320, 509),           # 9 k blocks of 32, F = 10; odd vocabulary
+    "hd128_f2112": _m(2, 256, 2, 128, 2112, 509),   # the form for up to 3072
+    "d1056": _m(1, 1056, 4, 64, 4096, 509),         # the forms for up to 2048 and 4096
+}
+
+
+@pytest.mark.parametrize("n_seq", [1, 3, 4, 5, 8, 9])    # first pass of an iteration: 2 n rows, later ones n
+@pytest.mark.parametrize("name", sorted(DRAFTS))
+def test_draft_passes_follow_the_oracle(name, n_seq):
+    from paper_2505_08600_b200 import binding
+    draft, target, gamma = DRAFTS[name], _m(1, 64, 1, 64, 64, 509), 3
+    wt, wd = synth.make_weights(target, seed=3, model_index=0, dtype="bf16"), synth.make_weights(draft, seed=3, model_index=1, dtype="bf16")
+    ctx = binding.Context(target, [draft], "bf16", n_seq, 96, gamma, 1.0, 7)
+    ctx.load_weights(0, wt); ctx.load_weights(1, wd)
+    toks = [synth.make_prompt(509, 7 + 9 * i, seed=9, seq=i) for i in range(n_seq)]
+    seqs = list(range(n_seq))
+    for s in seqs:
+        ctx.sd_seq_begin(s, toks[s], s)
+    ctx.sd_route_prompt(seqs, forced_task=[0] * n_seq)
+    ctx.sd_prefill(seqs)
+    x, q = torch.zeros((n_seq, gamma), dtype=torch.int32, device=DEV), torch.zeros((n_seq, gamma, 509), dtype=torch.float32, device=DEV)
+    ctx.sd_draft_steps(seqs, gamma, x, q)
+    xg, qg = x.cpu().numpy(), q.cpu().numpy().astype(np.float64)
+    assert ctx.sd_device_status() == 0
+    ctx.close()
+    om = oracle.OracleModel(draft, wd)
+    for s in seqs:
+        logits = om.new_cache(128).forward(np.concatenate([toks[s], xg[s, :-1]]), 0)[-gamma:]
+        top = logits.max(axis=1, keepdims=True)
+        want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
+        assert np.abs(np.log(qg[s]) - want).max() <= LOG_TOL, s
