@@ -625,25 +625,36 @@ sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n
     return SD_OK;
 }
 
-// Whether a pass takes the few-rows kernels (gemv.cu): the draft models, whose matrices a pass is through with in less time
-// than the weight-streaming GEMM and its step kernel need to hand over.
+// Whether a matrix and its step can take the few-rows kernels (gemv.cu).
+bool gemv_fits(const Model& M, int n_rows, int mode, int n_out, int K) {
+    Gemv g;
+    memset(&g, 0, sizeof(g));
+    g.rows = n_rows; g.ep.mode = mode; g.ep.hd = M.d.head_dim; g.ep.F = M.d.d_ffn; g.n_out = n_out; g.K = K;
+    return gemv_supported(g);
+}
+// Whether all of a pass does: the draft models, whose matrices are through in less time than the weight-streaming GEMM and its
+// step kernel need to hand over.
 bool few_rows_pass(sd_ctx* c, const Model& M, int n_rows) {
     const sd_model_desc& m = M.d;
     if (&M == &c->models[0] || n_rows > GEMV_MAX_ROWS || m.d_model % 16 || m.d_model > 16 * GEMV_SSQ_STRIDE) return false;
-    Gemv g;
-    memset(&g, 0, sizeof(g));
-    g.rows = n_rows;
-    auto ok = [&](int mode, int n_out, int K) { g.ep.mode = mode; g.ep.hd = m.head_dim; g.ep.F = m.d_ffn; g.n_out = n_out; g.K = K; return gemv_supported(g); };
-    return ok(EPI_QKV_ROPE, M.n_qkv(), m.d_model) && ok(EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) && ok(EPI_SWIGLU, 2 * m.d_ffn, m.d_model) &&
-           ok(EPI_RESIDUAL, m.d_model, m.d_ffn) && ok(EPI_PLAIN, m.vocab, m.d_model);
+    return gemv_fits(M, n_rows, EPI_QKV_ROPE, M.n_qkv(), m.d_model) && gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) &&
+           gemv_fits(M, n_rows, EPI_SWIGLU, 2 * m.d_ffn, m.d_model) && gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.d_ffn) &&
+           gemv_fits(M, n_rows, EPI_PLAIN, m.vocab, m.d_model);
+}
+// ... or a single matrix of a pass that streams the others: up to 16 MB.  1B target, six rows: with QKV (12.6 MB) and Wo (8.4 MB) on
+// these kernels an iteration takes 1.100 ms instead of 1.142; with gate/up (67 MB) as well 1.31, with the lm_head (131 MB) 1.19:
+// a CTA that holds its whole share in registers cannot keep HBM busy across CTAs.
+constexpr size_t GEMV_LARGEST = (size_t)16 << 20;
+bool few_rows_matrix(const Model& M, int n_rows, int mode, int n_out, int K) {
+    return n_rows <= GEMV_MAX_ROWS && !M.lora && (size_t)n_out * K * sizeof(bf16) <= GEMV_LARGEST && gemv_fits(M, n_rows, mode, n_out, K) &&
+           (mode != EPI_RESIDUAL || n_out <= 16 * SSQ_MAX_PARTS);
 }
 
 // One matrix and the step that follows it, on those kernels.
-sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out, int K, const Epilogue& ep, int ssq_stride) {
+sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out, int K, const Epilogue& ep) {
     Gemv g;
     memset(&g, 0, sizeof(g));
     g.w = (const bf16*)w; g.x = (const bf16*)x; g.rows = rows; g.n_out = n_out; g.K = K; g.ep = ep;
-    g.ssq_stride = ssq_stride; g.ssq_out_stride = GEMV_SSQ_STRIDE;
     if (ep.lora_b) {                            // x A^T of all adapters first (the rows behind the matrix's own)
         Gemv t = g;
         memset(&t.ep, 0, sizeof(t.ep));
@@ -652,6 +663,7 @@ sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out
         LAUNCH(CAT_LINEAR, launch_gemv(t, c->st));
         g.lora_t = c->lora_t;
     }
+    c->x_from.words = nullptr;                  // (no tile-by-tile hand-off from this kernel)
     LAUNCH(CAT_LINEAR, launch_gemv(g, c->st));
     return SD_OK;
 }
@@ -687,10 +699,14 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     };
     int len_hint[SD_MAX_BATCH];                                             // context bounds of the pass's sequences, for attention's launch order
     for (int i = 0; i < list.n && i < SD_MAX_BATCH; ++i) len_hint[i] = c->len_ub[list.ids[i]];
-    const RowScale first{c->ssq, 1, 1.f / d, m.rms_eps};                    // sum of squares in one piece (after the embedding)
-    const RowScale tiled{c->ssq, few ? d / 16 : (d + 127) / 128, 1.f / d, m.rms_eps};      // ... in one piece per tile of h of the kernel before
-    auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e, int ssq_stride) {
-        return few ? gemv_step(c, w, x, n_rows, n_out, K, e, ssq_stride) : gemm_tc(c, tm, x, n_rows, n_out, K, e);
+    RowScale scale{c->ssq, 1, 1.f / d, m.rms_eps, SSQ_STRIDE};              // sum of squares in one piece (after the embedding),
+    auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e) {
+        const bool gv = few || few_rows_matrix(M, n_rows, e.mode, n_out, K);
+        if (e.mode == EPI_RESIDUAL) {                                       // ... then in one piece per tile of the kernel that wrote h
+            scale.n_parts = gv ? d / 16 : (d + 127) / 128;
+            scale.stride = gv ? GEMV_SSQ_STRIDE : SSQ_STRIDE;
+        }
+        return gv ? gemv_step(c, w, x, n_rows, n_out, K, e) : gemm_tc(c, tm, x, n_rows, n_out, K, e);
     };
     LAUNCH(CAT_ELEMENTWISE, launch_embed(c->S, list, plan, n_rows, M.embed, dt, d, m.vocab, c->h, c->row_slot, c->row_pos,
                                          M.layers[0].norm1, c->xn, c->ssq, M.rope_cos, M.rope_sin, hd / 2, c->rope_row_cos, c->rope_row_sin, 0, nullptr, st, lo));
@@ -701,11 +717,11 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         Epilogue e;
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
-        e.mode = EPI_QKV_ROPE; e.rs = l == 0 ? first : tiled;
+        e.mode = EPI_QKV_ROPE; e.rs = scale;
         e.q_out = (bf16*)c->q; e.kc = (bf16*)kc; e.vc = (bf16*)vc; e.row_slot = c->row_slot; e.row_pos = c->row_pos;
         e.H = H; e.Hkv = Hkv; e.hd = hd; e.max_ctx = c->cfg.max_ctx; e.rcos = c->rope_row_cos; e.rsin = c->rope_row_sin;
         with_lora(e, L, SD_LORA_QKV);
-        SD_TRY(step(L.tm_qkv, L.wqkv, c->xn, M.n_qkv(), d, e, l == 0 ? SSQ_STRIDE : GEMV_SSQ_STRIDE));
+        SD_TRY(step(L.tm_qkv, L.wqkv, c->xn, M.n_qkv(), d, e));
         LAUNCH(CAT_ATTENTION, launch_attention_split(c->q, kc, vc, c->attn, c->row_slot, c->row_pos, n_rows, plan.rows_per_seq, H, Hkv,
                                                      hd, c->cfg.max_ctx, plan.ctx_bound, c->attn_ws, c->attn_ws_bytes, 1, st, lo,
                                                      next_stamp(c, SD_STAMP_ATTENTION), c->tune[SD_TUNE_ATTN_WARPS], c->tune[SD_TUNE_ATTN_CLUSTER],
@@ -715,18 +731,18 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         e.ring_stages = c->tune[SD_TUNE_WO_STAGES]; e.prefill_all = c->tune[SD_TUNE_WO_PREFILL_ALL];
         e.mode = EPI_RESIDUAL; e.h = c->h; e.gain_next = L.norm2; e.xn = (bf16*)c->xn; e.ssq_out = c->ssq;
         with_lora(e, L, SD_LORA_WO);
-        SD_TRY(step(L.tm_wo, L.wo, c->attn, d, H * hd, e, 0));
+        SD_TRY(step(L.tm_wo, L.wo, c->attn, d, H * hd, e));
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
-        e.mode = EPI_SWIGLU; e.rs = tiled; e.act = (bf16*)c->act; e.F = F;
+        e.mode = EPI_SWIGLU; e.rs = scale; e.act = (bf16*)c->act; e.F = F;
         with_lora(e, L, SD_LORA_GU);
-        SD_TRY(step(L.tm_gu, L.wgu, c->xn, 2 * F, d, e, GEMV_SSQ_STRIDE));
+        SD_TRY(step(L.tm_gu, L.wgu, c->xn, 2 * F, d, e));
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
         e.mode = EPI_RESIDUAL; e.h = c->h; e.xn = (bf16*)c->xn; e.ssq_out = c->ssq;
         e.gain_next = l + 1 < m.n_layers ? M.layers[l + 1].norm1 : (mode != LOGITS_NONE ? M.final_norm : nullptr);
         with_lora(e, L, SD_LORA_WD);
-        SD_TRY(step(L.tm_wd, L.wd, c->act, d, F, e, 0));
+        SD_TRY(step(L.tm_wd, L.wd, c->act, d, F, e));
     }
     if (mode != LOGITS_NONE) {
         // the lm_head GEMM runs over all rows (they share the one pass over the weights); only the wanted rows are written
@@ -734,10 +750,10 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         Epilogue e;
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
-        e.mode = EPI_PLAIN; e.rs = tiled; e.y = logits_out;
+        e.mode = EPI_PLAIN; e.rs = scale; e.y = logits_out;
         if (mode == LOGITS_ALL) { e.n_out_rows = n_rows; e.row_stride = 1; e.row_offset = 0; }
         else { e.n_out_rows = list.n; e.row_stride = R; e.row_offset = R - 1; }
-        SD_TRY(step(M.tm_lm, M.lm_head, c->xn, m.vocab, d, e, GEMV_SSQ_STRIDE));
+        SD_TRY(step(M.tm_lm, M.lm_head, c->xn, m.vocab, d, e));
     }
     CUDA_TRY(prof_mark(c, CAT_NONE));
     return SD_OK;
@@ -1297,7 +1313,7 @@ sd_status sd_route_prompt_mamba(sd_ctx* c, const sd_mamba_desc* desc, const sd_m
     }
     // labels land in the scratch words the accept path uses for its counts (n_seq <= max_seqs of them)
     SD_TRY(sd_mamba_classify(desc, w, c->S.tokens, starts.data(), lens.data(), n_seq, nullptr, c->st_nacc, ws, ws_bytes, c->st));
-    c->launches += 6;
+    c->launches += 4;
     CUDA_TRY(cudaMemcpyAsync(labels.data(), c->st_nacc, sizeof(int32_t) * n_seq, cudaMemcpyDeviceToHost, c->st));
     CUDA_TRY(cudaStreamSynchronize(c->st));
     return sd_route_prompt(c, seqs, n_seq, labels.data(), draft_out);

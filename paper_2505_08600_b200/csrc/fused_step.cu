@@ -147,15 +147,22 @@ __global__ void __launch_bounds__(128) k_fused_step(GemmGeom g, Epilogue ep, con
             }
         }
     }
-    float ssa[(MB + 3) / 4], ssb[(MB + 3) / 4];
+    // (more than 64 pieces: the rows were written by the few-rows kernels, in passes of at most 16 rows)
+    constexpr bool WIDE = MB <= 8 || HL;
+    float ssa[(MB + 3) / 4], ssb[(MB + 3) / 4], ssc[WIDE ? (MB + 3) / 4 : 1], ssd[WIDE ? (MB + 3) / 4 : 1];
     if (ep.rs.ssq) {                              // one warp per token row, one lane per piece of its sum of squares
 #pragma unroll
         for (int ii = 0; ii < (MB + 3) / 4; ++ii) {
             const int i = warp + 4 * ii, r = m0 + i;
             const bool ok = i < MB && r < n_rows;
-            const float* ps = ep.rs.ssq + (size_t)(ok ? (mode == EPI_PLAIN ? r * ep.row_stride + ep.row_offset : r) : 0) * SSQ_STRIDE;
+            const float* ps = ep.rs.ssq + (size_t)(ok ? (mode == EPI_PLAIN ? r * ep.row_stride + ep.row_offset : r) : 0) * ep.rs.stride;
             ssa[ii] = (ok && lane < ep.rs.n_parts) ? __ldcg(ps + lane) : 0.f;
             ssb[ii] = (ok && lane + 32 < ep.rs.n_parts) ? __ldcg(ps + lane + 32) : 0.f;
+            if (WIDE) ssc[WIDE ? ii : 0] = ssd[WIDE ? ii : 0] = 0.f;
+            if (WIDE && ep.rs.n_parts > 64) {
+                ssc[WIDE ? ii : 0] = (ok && lane + 64 < ep.rs.n_parts) ? __ldcg(ps + lane + 64) : 0.f;
+                ssd[WIDE ? ii : 0] = (ok && lane + 96 < ep.rs.n_parts) ? __ldcg(ps + lane + 96) : 0.f;
+            }
         }
     }
     float hv[MB];
@@ -247,7 +254,7 @@ __global__ void __launch_bounds__(128) k_fused_step(GemmGeom g, Epilogue ep, con
 #pragma unroll
         for (int ii = 0; ii < (MB + 3) / 4; ++ii) {
             const int i = warp + 4 * ii;
-            const float ss = warp_sum(ssa[ii] + ssb[ii]);
+            const float ss = warp_sum(WIDE ? (ssa[ii] + ssb[ii]) + (ssc[WIDE ? ii : 0] + ssd[WIDE ? ii : 0]) : ssa[ii] + ssb[ii]);
             if (lane == 0 && i < MB) sh.scale[i] = rsqrtf(ss * ep.rs.inv_d + ep.rs.eps);
         }
         __syncthreads();
@@ -417,7 +424,7 @@ cudaError_t launch_fused_step(const GemmGeom& g, const Epilogue& ep, const float
     if (ep.mode == EPI_QKV_ROPE && (128 % ep.hd)) return cudaErrorInvalidValue;            // a head must not straddle two tiles
     if (ep.mode == EPI_RESIDUAL && g.n_tiles > SSQ_STRIDE) return cudaErrorInvalidValue;
     if (ep.mode == EPI_SWIGLU && (ep.F % 64)) return cudaErrorInvalidValue;
-    if (ep.rs.ssq && ep.rs.n_parts > 64) return cudaErrorInvalidValue;
+    if (ep.rs.ssq && (ep.rs.n_parts > (g.m_tok <= 32 ? SSQ_MAX_PARTS : 64) || ep.rs.stride < ep.rs.n_parts)) return cudaErrorInvalidValue;
     if (ep.lora_b) {                                   // the adapter's tile is complete only when the GEMM's grid is
         if (ep.lora_r < 8 || ep.lora_r > 32 || (ep.lora_r & 7) || ep.lora_n * ep.lora_r > TILE_N || !ep.lora_task ||
             ep.mode == EPI_PLAIN || g.n_out % TILE_N || g.n_tiles != g.n_out / TILE_N + 1)

@@ -31,13 +31,16 @@ struct GemmGeom {
 
 // RMSNorm folded around a GEMM: the GEMM's input rows are h * gain (no 1/rms factor), the
 // factor rsqrt(mean(h^2) + eps) of each row multiplies the GEMM's output instead.  The sum of
-// squares of a row arrives in n_parts pieces (one per 128-wide tile of the kernel that wrote h).
+// squares of a row arrives in n_parts pieces (one per tile of the kernel that wrote h: 128 features wide, or 16 where that was
+// launch_gemv).
 struct RowScale {
-    const float* ssq;       // [row][SSQ_STRIDE]; nullptr: no scaling
+    const float* ssq;       // [row][stride]; nullptr: no scaling
     int n_parts;
     float inv_d, eps;
+    int stride;
 };
 constexpr int SSQ_STRIDE = 64;
+constexpr int SSQ_MAX_PARTS = 128;      // most pieces that launch_fused_step adds up (64 in passes of more than 16 rows)
 
 // What happens to a 128-row output tile once its pieces are summed (the step that follows the
 // GEMM in the decoder layer), so that no fp32 intermediate matrix goes through memory.

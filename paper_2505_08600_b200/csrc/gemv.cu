@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
             const int m = warp + W * i;
             ss[i] = 0.f;
             if (m < g.rows)
-                for (int p = lane; p < ep.rs.n_parts; p += 32) ss[i] += __ldcg(ep.rs.ssq + (size_t)m * g.ssq_stride + p);
+                for (int p = lane; p < ep.rs.n_parts; p += 32) ss[i] += __ldcg(ep.rs.ssq + (size_t)m * ep.rs.stride + p);
         }
     }
     float acc[NT][4];
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
             float s = mine ? h0 * h0 + h1 * h1 : 0.f;
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (mine && ui == 0) ep.ssq_out[(size_t)um * g.ssq_out_stride + tile] = s;
+            if (mine && ui == 0) ep.ssq_out[(size_t)um * GEMV_SSQ_STRIDE + tile] = s;
         }
         break;
     }

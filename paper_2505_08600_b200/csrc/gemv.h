@@ -11,7 +11,6 @@ struct Gemv {
     const bf16* w;                      // [n_out][K]
     const bf16* x;                      // [rows][K], second parts ep.lo_off rows further down
     int rows, n_out, K;
-    int ssq_stride, ssq_out_stride;     // of ep.rs.ssq and ep.ssq_out
     const float* lora_t;                // [row][128]: x A^T of all adapters (with ep.lora_b)
     Epilogue ep;                        // as for launch_fused_step; rs.n_parts counts this kernel's 16-feature tiles where it wrote them
 };
