@@ -130,6 +130,7 @@ __device__ __forceinline__ void stage_row(const float* __restrict__ src, float* 
     }
     __syncthreads();
 }
+constexpr int SLICED_FROM = 4096;                // vocabularies from here on are worth a cluster (below, its barriers cost more than they save)
 constexpr int STAGE_MAX_BYTES = 200 * 1024;      // a row of up to 51200 fp32 values fits beside the static shared memory
 
 // Dynamic shared memory for one staged row, or 0 when the vocabulary is too large to stage.
@@ -198,9 +199,170 @@ __global__ void __launch_bounds__(1024) k_draft_sample(const float* __restrict__
     int k = softmax_sample_row(logits + (size_t)i * V, V, T, u, q_out + ((size_t)b * gamma + step) * V, sh, staged ? rowbuf : nullptr);
     if (threadIdx.x == 0) x_out[(size_t)b * gamma + step] = k;
 }
+// The same over a cluster of eight CTAs per row, each with an eighth of the vocabulary in shared memory: a row of 32000 is 32
+// exponentials per thread for one CTA of 1024, four for eight CTAs of 1024.  What the slices have to know of one another (maximum,
+// sum, integer total) goes to every CTA of the cluster through distributed shared memory.  The token is the one of the integer
+// inverse CDF over the written fp32 values, whatever the split.  32000 values: 16 -> 11 us.
+constexpr int SLICES = 8;
+struct SliceScratch {
+    BlockScratch b;
+    float f[2][SLICES];
+    int idx[SLICES];
+    unsigned long long total[SLICES];
+};
+__host__ __device__ __forceinline__ int slice_len(int V) { return (V + 4 * SLICES - 1) / (4 * SLICES) * 4; }
+
+// block_icdf over this CTA's slice of n weights, `base` being the weight of everything in front of it, `thr` the running sum to be
+// reached: the index inside the slice in the CTA whose slice holds it, -1 in the others.  local: the slice's weight of this thread.
+template <class F>
+__device__ __forceinline__ int slice_pick(F w, int n, unsigned long long base, unsigned long long thr, unsigned long long local, BlockScratch& sh) {
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    const int chunk = (n + blockDim.x - 1) / blockDim.x, k0 = min(n, t * chunk), k1 = min(n, k0 + chunk);
+    unsigned long long incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    __syncthreads();
+    if (lane == 31) sh.scan[wid] = incl;
+    if (t == 0) sh.tok = -1;
+    __syncthreads();
+    unsigned long long before = base;
+    for (int i = 0; i < wid && i < nw; ++i) before += sh.scan[i];
+    incl += before;
+    const unsigned long long excl = incl - local;
+    if (excl < thr && thr <= incl) {
+        unsigned long long run = excl;
+        for (int k = k0; k < k1; ++k) {
+            run += __float2ull_rz(w(k) * 4294967296.0f);
+            if (run >= thr) { sh.tok = k; break; }
+        }
+    }
+    __syncthreads();
+    return sh.tok;
+}
+// The integer weight of this thread's chunk of a slice, and the slice's total (valid in every thread).
+template <class F>
+__device__ __forceinline__ unsigned long long slice_weight(F w, int n, unsigned long long* total, BlockScratch& sh) {
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nw = blockDim.x >> 5;
+    const int chunk = (n + blockDim.x - 1) / blockDim.x, k0 = min(n, t * chunk), k1 = min(n, k0 + chunk);
+    unsigned long long local = 0;
+    for (int k = k0; k < k1; ++k) local += __float2ull_rz(w(k) * 4294967296.0f);
+    unsigned long long s = local;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __syncthreads();
+    if (lane == 0) sh.scan[wid] = s;
+    __syncthreads();
+    s = 0;
+    for (int i = 0; i < nw; ++i) s += sh.scan[i];
+    *total = s;
+    return local;
+}
+
+// Which slice holds the draw with uniform u_int / 2^24 and where in the running sum that is (the same answer in every CTA).
+struct SliceDraw { int owner; unsigned long long before, thr; };
+__device__ __forceinline__ SliceDraw slice_draw(const unsigned long long (&total)[SLICES], uint32_t u_int) {
+    unsigned long long tot = 0, run = 0;
+#pragma unroll
+    for (int r = 0; r < SLICES; ++r) tot += total[r];
+    SliceDraw d{-1, 0ull, ((unsigned long long)u_int * tot + 16777215ull) >> 24};
+#pragma unroll
+    for (int r = 0; r < SLICES; ++r) {
+        if (d.owner < 0 && run < d.thr && d.thr <= run + total[r]) { d.owner = r; d.before = run; }
+        run += total[r];
+    }
+    return d;                                                   // owner < 0: every weight is zero (or not a number)
+}
+
+__global__ void __cluster_dims__(SLICES, 1, 1) __launch_bounds__(1024)
+k_draft_sample_sliced(const float* __restrict__ logits, SeqState S, SeqList list, int V, float T, uint64_t seed, int step, int gamma,
+                      float* __restrict__ q_out, int32_t* __restrict__ x_out) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) float buf[];
+    __shared__ SliceScratch sh;
+    pdl_launch_dependents();
+    const int i = blockIdx.x / SLICES, rank = blockIdx.x % SLICES, slot = list.ids[i], b = list.out[i];
+    const int len = slice_len(V), base = min(V, rank * len), n = min(V, base + len) - base;
+    float* probs = q_out + ((size_t)b * gamma + step) * V + base;
+    auto share = [&](auto* mine, auto v) {                     // to every CTA of the cluster; visible after cluster.sync()
+        if (threadIdx.x < SLICES) cluster.map_shared_rank(mine, threadIdx.x)[rank] = v;
+    };
+    pdl_wait();
+    const float* l = logits + (size_t)i * V + base;
+    float m = -INFINITY;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) { const float v = __ldcg(l + k); buf[k] = v; m = fmaxf(m, v); }
+    m = block_max(m, sh.b.red);
+    cluster.sync();                                             // every CTA is there before the others write into it
+    share(sh.f[0], m);
+    cluster.sync();
+#pragma unroll
+    for (int r = 0; r < SLICES; ++r) m = fmaxf(m, sh.f[0][r]);
+    // lowest index that holds value v of the slices (all CTAs take part)
+    auto first_index = [&](float v) {
+        int best = 0x7fffffff;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) if (buf[k] == v) { best = base + k; break; }
+        best = block_min_int(best, sh.b);
+        share(sh.idx, best);
+        cluster.sync();
+#pragma unroll
+        for (int r = 0; r < SLICES; ++r) best = min(best, sh.idx[r]);
+        return best;
+    };
+    int tok;
+    if (T == 0.f) {
+        tok = first_index(m);
+        for (int k = threadIdx.x; k < n; k += blockDim.x) probs[k] = base + k == tok ? 1.f : 0.f;
+        if (rank == 0 && threadIdx.x == 0) x_out[(size_t)b * gamma + step] = tok;
+    } else {
+        const float inv_T = 1.f / T;                            // (multiplications by 1/T and 1/sum: see softmax_sample_row)
+        float s = 0.f;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) { const float e = expf((buf[k] - m) * inv_T); buf[k] = e; s += e; }
+        s = block_sum(s, sh.b.red);
+        share(sh.f[1], s);
+        cluster.sync();
+        s = 0.f;
+#pragma unroll
+        for (int r = 0; r < SLICES; ++r) s += sh.f[1][r];
+        const float inv_s = 1.f / s;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) { const float p = buf[k] * inv_s; buf[k] = p; probs[k] = p; }
+        __syncthreads();
+        unsigned long long mine;
+        const unsigned long long local = slice_weight([&](int k) { return buf[k]; }, n, &mine, sh.b);
+        share(sh.total, mine);
+        cluster.sync();
+        const SliceDraw d = slice_draw(sh.total, uniform24(seed, S.iter[slot], (uint32_t)step, S.seq_id[slot], DRAW_DRAFT));
+        if (d.owner >= 0) {
+            if (d.owner == rank) {
+                tok = max(slice_pick([&](int k) { return buf[k]; }, n, d.before, d.thr, local, sh.b), 0);
+                if (threadIdx.x == 0) x_out[(size_t)b * gamma + step] = base + tok;
+            }
+        } else {                                                // every weight rounds to zero: the largest probability
+            float pm = -INFINITY;
+            for (int k = threadIdx.x; k < n; k += blockDim.x) pm = fmaxf(pm, buf[k]);
+            pm = block_max(pm, sh.b.red);
+            share(sh.f[0], pm);
+            cluster.sync();
+#pragma unroll
+            for (int r = 0; r < SLICES; ++r) pm = fmaxf(pm, sh.f[0][r]);
+            tok = first_index(pm);
+            if (rank == 0 && threadIdx.x == 0) x_out[(size_t)b * gamma + step] = tok;
+        }
+    }
+    cluster.sync();                                             // no CTA leaves while the others may still write into it
+}
+
 cudaError_t launch_draft_sample(const float* logits, const SeqState& S, const SeqList& list, int V, float T,
                                 uint64_t seed, int step, int gamma, float* q_out, int32_t* x_out, cudaStream_t st) {
     if (list.n <= 0) return cudaSuccess;
+    const size_t slice = (size_t)slice_len(V) * sizeof(float);
+    if (V >= SLICED_FROM && slice <= (size_t)STAGE_MAX_BYTES) {
+        cudaError_t e = cudaFuncSetAttribute(k_draft_sample_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k_draft_sample_sliced, dim3(list.n * SLICES), dim3(1024), slice, st, 1, logits, S, list, V, T, seed, step, gamma, q_out, x_out);
+    }
     const size_t smem = row_stage_bytes(V);
     cudaError_t e = cudaFuncSetAttribute(k_draft_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
     if (e != cudaSuccess) return e;
@@ -349,8 +511,170 @@ __global__ void __launch_bounds__(1024) k_accept(AcceptParams P, int csize, int 
     cluster.sync();                                             // no CTA leaves while its flags may still be read
 }
 
+// The same rule with the vocabulary cut over the cluster instead of the rows: every CTA holds an eighth of all gamma + 1 rows in
+// shared memory, so that each exponential is computed once and by eight times as many threads, and the draw from row n is
+// spread as well.  Taken when the slices fit (gamma + 1 rows of V / 8).  One sequence, gamma = 5, V = 32000: 33 -> 21 us
+// (1B iteration, five draws and one accept: 1.100 -> 1.058 ms).
+constexpr int ACC_MAX_ROWS = SD_MAX_GAMMA + 1;
+struct AcceptSliceScratch {
+    BlockScratch b;
+    float warp_f[ACC_MAX_ROWS][32];                            // per row and warp
+    float mx[ACC_MAX_ROWS][SLICES], sum[ACC_MAX_ROWS][SLICES], alpha[ACC_MAX_ROWS][SLICES];
+    int arg[ACC_MAX_ROWS][SLICES], ok[ACC_MAX_ROWS];
+    unsigned long long total[2][SLICES];
+};
+__global__ void __cluster_dims__(SLICES, 1, 1) __launch_bounds__(1024) k_accept_sliced(AcceptParams P) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) float buf[];               // [row][slice]: logits, then exponentials (or the probabilities as given)
+    __shared__ AcceptSliceScratch sh;
+    pdl_launch_dependents();
+    const int i = blockIdx.x / SLICES, rank = blockIdx.x % SLICES, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int idx = P.use_list ? P.list.ids[i] : i, b = P.use_list ? P.list.out[i] : i;
+    const int V = P.V, gamma = P.gamma, rows = gamma + 1;
+    const int len = slice_len(V), base = min(V, rank * len), n = min(V, base + len) - base;
+    const float T = P.T, inv_T = T > 0.f ? 1.f / T : 0.f;
+    const float* tgt = P.target + (size_t)b * rows * V + base;
+    const float* q = P.q + (size_t)b * gamma * V + base;
+    const int32_t* x = P.x + (size_t)b * gamma;
+    const bool logits = P.target_is_logits != 0, soft = logits && T > 0.f;
+    if (tid < rows) sh.ok[tid] = 0;
+    pdl_wait();                                                // target rows, drafts and per-sequence state come from earlier kernels
+    // a per-row reduction over the CTA, then to every CTA of the cluster
+    auto reduce_rows = [&](int n_rows, bool is_max, float (*out)[SLICES]) {      // of warp_f
+        __syncthreads();
+        for (int j = warp; j < n_rows; j += 32) {
+            float v = sh.warp_f[j][lane];
+            v = is_max ? warp_max(v) : warp_sum(v);
+            if (lane < SLICES) cluster.map_shared_rank(&out[j][0], lane)[rank] = v;
+        }
+        cluster.sync();
+    };
+    for (int j = 0; j < rows; ++j) {
+        float m = -INFINITY;
+        for (int k = tid; k < n; k += 1024) { const float v = __ldcg(tgt + (size_t)j * V + k); buf[j * len + k] = v; m = fmaxf(m, v); }
+        if (logits) { m = warp_max(m); if (lane == 0) sh.warp_f[j][warp] = m; }
+    }
+    cluster.sync();                                            // every CTA is there before the others write into it
+    float inv_s = 1.f;                                          // (of row `lane` in every warp, below)
+    if (logits) reduce_rows(rows, true, sh.mx);
+    auto row_max = [&](int j) {
+        float m = sh.mx[j][0];
+#pragma unroll
+        for (int r = 1; r < SLICES; ++r) m = fmaxf(m, sh.mx[j][r]);
+        return m;
+    };
+    if (soft) {
+        for (int j = 0; j < rows; ++j) {
+            const float m = row_max(j);
+            float s = 0.f;
+            for (int k = tid; k < n; k += 1024) { const float e = expf((buf[j * len + k] - m) * inv_T); buf[j * len + k] = e; s += e; }      // (1/T: see softmax_sample_row)
+            s = warp_sum(s);
+            if (lane == 0) sh.warp_f[j][warp] = s;
+        }
+        reduce_rows(rows, false, sh.sum);
+        if (lane < rows) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < SLICES; ++r) s += sh.sum[lane][r];
+            inv_s = 1.f / s;
+        }
+    } else if (logits) {                                       // one-hot: lowest index of the maximum
+        for (int j = 0; j < rows; ++j) {
+            const float m = row_max(j);
+            int best = 0x7fffffff;
+            for (int k = tid; k < n; k += 1024) if (buf[j * len + k] == m) { best = base + k; break; }
+            best = block_min_int(best, sh.b);
+            if (tid < SLICES) cluster.map_shared_rank(&sh.arg[j][0], tid)[rank] = best;
+        }
+        cluster.sync();
+        for (int j = 0; j < rows; ++j) {
+            int a = sh.arg[j][0];
+#pragma unroll
+            for (int r = 1; r < SLICES; ++r) a = min(a, sh.arg[j][r]);
+            for (int k = tid; k < n; k += 1024) buf[j * len + k] = base + k == a ? 1.f : 0.f;
+        }
+    }
+    // probability of the row's k-th value of this slice: what is in the buffer times the row's factor
+    auto factor = [&](int j) { return soft ? __shfl_sync(0xffffffffu, inv_s, j) : 1.f; };
+    __syncthreads();
+    for (int j = 0; j < gamma; ++j) {
+        const float f = factor(j);
+        if (P.alpha_terms) {                                   // Eq. 1's alpha for this slot: the draft is kept with probability sum_k min(p, q)
+            const float* qj = q + (size_t)j * V;
+            float a = 0.f;
+#pragma unroll 4
+            for (int k = tid; k < n; k += 1024) a += fminf(buf[j * len + k] * f, __ldg(qj + k));
+            a = warp_sum(a);
+            if (lane == 0) sh.warp_f[j][warp] = a;
+        }
+        if (tid == 0) {
+            const int xs = x[j] - base;
+            if (xs >= 0 && xs < n) {                           // the CTA whose slice holds the token (an impossible token stays rejected)
+                const uint32_t ui = uniform24(P.seed, P.iter[idx], (uint32_t)j, P.seq_id[idx], DRAW_ACCEPT);
+                const float u = (float)ui * (1.0f / 16777216.0f);
+                const int ok = __fmul_rn(u, q[(size_t)j * V + xs]) <= buf[j * len + xs] * f;
+                for (int r = 0; r < SLICES; ++r) cluster.map_shared_rank(sh.ok, r)[j] = ok;
+            }
+        }
+    }
+    if (P.alpha_terms && gamma > 0) reduce_rows(gamma, false, sh.alpha); else cluster.sync();
+    if (P.alpha_terms && rank == 0 && tid < gamma) {
+        float a = 0.f;
+#pragma unroll
+        for (int r = 0; r < SLICES; ++r) a += sh.alpha[tid][r];
+        P.alpha_terms[(size_t)b * gamma + tid] = a;
+    }
+    int nacc = 0;
+    while (nacc < gamma && sh.ok[nacc]) ++nacc;
+    // the draw: residual max(0, p_n - q_n), or p_gamma itself; all of it zero -> the target distribution -> its largest value
+    float* w = buf + nacc * len;
+    const float fn = factor(nacc);
+    const float* qn = q + (size_t)(nacc < gamma ? nacc : 0) * V;
+    const uint32_t ui = uniform24(P.seed, P.iter[idx], (uint32_t)nacc, P.seq_id[idx], DRAW_RESAMPLE);
+    int y = 0, owner = -1;                                     // the CTA that writes the result, and (there) the token
+    for (int attempt = nacc < gamma ? 0 : 1; attempt < 2 && owner < 0; ++attempt) {
+        auto weight = [&](int k) { const float p = w[k] * fn; return attempt == 0 ? fmaxf(__fsub_rn(p, __ldg(qn + k)), 0.f) : p; };
+        unsigned long long mine;
+        const unsigned long long local = slice_weight(weight, n, &mine, sh.b);
+        if (tid < SLICES) cluster.map_shared_rank(&sh.total[attempt][0], tid)[rank] = mine;
+        cluster.sync();
+        const SliceDraw d = slice_draw(sh.total[attempt], ui);
+        owner = d.owner;
+        if (owner == rank) y = base + max(slice_pick(weight, n, d.before, d.thr, local, sh.b), 0);
+    }
+    if (owner < 0) {                                           // the largest probability, lowest index on ties
+        float pm = -INFINITY;
+        for (int k = tid; k < n; k += 1024) pm = fmaxf(pm, w[k] * fn);
+        pm = block_max(pm, sh.b.red);
+        if (tid < SLICES) cluster.map_shared_rank(&sh.mx[0][0], tid)[rank] = pm;
+        cluster.sync();
+        pm = row_max(0);
+        int best = 0x7fffffff;
+        for (int k = tid; k < n; k += 1024) if (w[k] * fn == pm) { best = base + k; break; }
+        best = block_min_int(best, sh.b);
+        if (tid < SLICES) cluster.map_shared_rank(&sh.arg[0][0], tid)[rank] = best;
+        cluster.sync();
+        y = sh.arg[0][0];
+#pragma unroll
+        for (int r = 1; r < SLICES; ++r) y = min(y, sh.arg[0][r]);
+        owner = 0;
+    }
+    if (owner == rank) {
+        if (tid == 0) P.n_acc[b] = nacc;
+        if (tid <= gamma) P.out_tok[(size_t)b * rows + tid] = tid < nacc ? x[tid] : (tid == nacc ? y : -1);
+    }
+    cluster.sync();                                            // no CTA leaves while the others may still write into it
+}
+
 cudaError_t launch_accept(const AcceptParams& p, int dependent, cudaStream_t st) {
     if (p.B <= 0) return cudaSuccess;
+    const size_t slices = (size_t)slice_len(p.V) * (p.gamma + 1) * sizeof(float);
+    if (p.V >= SLICED_FROM && slices <= (size_t)STAGE_MAX_BYTES && p.gamma <= SD_MAX_GAMMA) {
+        cudaError_t e = cudaFuncSetAttribute(k_accept_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k_accept_sliced, dim3(p.B * SLICES), dim3(1024), slices, st, dependent, p);
+    }
     int csize = 1;
     while (csize < p.gamma + 1 && csize < 8) csize <<= 1;      // portable cluster sizes only
     if (csize * ACC_ROWS_PER_CTA < p.gamma + 1) return cudaErrorInvalidValue;
