@@ -1,15 +1,17 @@
 // The Mamba-based prompt classifier (Section 2.4, Section 3.3.3): embedding -> one selective state-space layer ->
 // average pooling over the prompt -> fully connected layer -> argmax.  Everything is fp32.
 //
-// The layer's recurrence h_t = a_t * h_{t-1} + b_t is linear in h, so a prompt is cut into chunks of MB_CHUNK tokens
-// that are scanned side by side: (A) every chunk is scanned from a zero state and leaves its end state and the product
-// of its decays, (B) a short serial pass over a prompt's chunks turns those into the state each chunk starts from,
-// (C) every chunk is scanned again from that state and emits the gated outputs.  Prompts of one chunk skip (A) and (B).
+// The layer's recurrence h_t = a_t * h_{t-1} + b_t is linear in h, so a prompt is cut into chunks of MB_CHUNK tokens that are
+// scanned side by side, once, from a zero state: with P_t the product of a chunk's decays up to token t and s the state the
+// chunk starts from, h_t = h_t(zero) + P_t s, so what a chunk adds to the pooled sum of g_t = (C_t h_t + D v_t) silu(z_t) is
+//   sum_t (C_t h_t(zero) + D v_t) silu(z_t)  +  s . sum_t silu(z_t) C_t P_t,
+// both sums of the one scan.  The states s follow from the chunks' end states and decays in a short serial pass per prompt.
 // The pooled vector is the mean over tokens of W_out g_t, which is W_out applied to the mean of g_t: the kernels sum
 // g_t per channel (chunks in order) and apply W_out and the classification layer once per prompt.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <vector>
 
@@ -19,7 +21,6 @@ namespace sd {
 namespace {
 
 constexpr int MB_CHUNK = 64;         // tokens per chunk of the scan
-constexpr int MB_TOK_TILE = 16;      // tokens per CTA of the input projection
 constexpr int MB_MAX_N = 16;         // state size kept in registers
 constexpr int MB_MAX_CONV = 8;
 
@@ -30,210 +31,308 @@ struct ChunkRec { int32_t prompt, tok0, n_tok, pos0; };      // tok0: index into
 __device__ __forceinline__ float silu_f(float x) { return x / (1.f + expf(-x)); }
 __device__ __forceinline__ float softplus_f(float x) { return x > 20.f ? x : log1pf(expf(x)); }
 
-// Where every flattened token comes from and its position in its prompt, from the chunk records (one CTA per chunk).
-__global__ void k_mamba_tables(const ChunkRec* __restrict__ chunks, const int64_t* __restrict__ starts, int64_t* __restrict__ tok_src,
-                               int32_t* __restrict__ tok_pos) {
+// Where every flattened token's projected row is: its own, or its token's when whole vocabulary was projected (one CTA per chunk).
+__global__ void k_mamba_tables(const ChunkRec* __restrict__ chunks, const int64_t* __restrict__ starts, const int32_t* __restrict__ tokens, int V, int by_token,
+                               int32_t* __restrict__ tok_id, int32_t* __restrict__ tok_row) {
     const ChunkRec ch = chunks[blockIdx.x];
     for (int i = threadIdx.x; i < ch.n_tok; i += blockDim.x) {
-        tok_src[ch.tok0 + i] = starts[ch.prompt] + ch.pos0 + i;
-        tok_pos[ch.tok0 + i] = ch.pos0 + i;
+        const int tok = min(max(tokens[starts[ch.prompt] + ch.pos0 + i], 0), V - 1);
+        tok_id[ch.tok0 + i] = tok;
+        tok_row[ch.tok0 + i] = by_token ? tok : ch.tok0 + i;
     }
 }
 
-// u, z = split(W_in E[token]) for a tile of tokens.  One thread per output feature; the tile's embedding rows sit in
-// shared memory, and W_in passes through shared memory in blocks of 256 rows x 32 columns so that global loads are
-// coalesced (a warp reads 128 contiguous bytes of one row) and every thread then walks its own row without bank
-// conflicts (rows padded to 33 words).
-__global__ void __launch_bounds__(256)
-k_mamba_in(MambaDims m, const int32_t* __restrict__ tokens, const int64_t* __restrict__ tok_src, int T, const float* __restrict__ embed,
+// Two fp32 values in one register pair and the packed multiply-add of sm_100 on them (two independent IEEE operations).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ float2 f2_unpack(f32x2 v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+
+// u, z = split(W_in E[row]) for every row: token by token, or, when the prompts hold more tokens than the vocabulary has, once per
+// token of the vocabulary (the projection depends on nothing else).  Bound: fp32 multiply-adds (21,128 rows: 69 us; 109,096 token
+// by token, a thread per feature, 757).  128 x 128 tiles of 256
+// threads, 8 x 8 sums each in register pairs, 16-deep slices of both operands through two buffers.
+constexpr int MI_TILE = 128, MI_K = 16, MI_PITCH = MI_TILE + 4;
+__global__ void __launch_bounds__(256, 2)
+k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = token*/, int rows, const float* __restrict__ embed,
            const float* __restrict__ w_in, float* __restrict__ u, float* __restrict__ z) {
-    extern __shared__ __align__(16) float in_smem[];
-    float* e_s = in_smem;                                // [MB_TOK_TILE][D]
-    float* w_s = in_smem + MB_TOK_TILE * m.D;            // [256][36]: rows padded to 36 words (16-byte aligned, conflict-free float4 reads)
-    const int t0 = blockIdx.x * MB_TOK_TILE, nt = min(MB_TOK_TILE, T - t0);
-    for (int i = threadIdx.x; i < MB_TOK_TILE * m.D; i += blockDim.x) {
-        const int tt = i / m.D, d = i % m.D;
-        float e = 0.f;                                   // rows past the end of the token list are zero
-        if (tt < nt) {
-            int tok = tokens[tok_src[t0 + tt]];
-            tok = min(max(tok, 0), m.V - 1);
-            e = embed[(size_t)tok * m.D + d];
-        }
-        e_s[tt * m.D + d] = e;
+    __shared__ __align__(16) float as[2][MI_K][MI_PITCH], bs[2][MI_K][MI_PITCH];
+    const int tid = threadIdx.x, r0 = blockIdx.x * MI_TILE, j0 = blockIdx.y * MI_TILE;
+    const int lr = tid >> 2, lk = (tid & 3) * 4;                        // this thread loads rows lr and lr + 64, columns lk ... lk + 3
+    const float* a_src[2]; const float* b_src[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int r = r0 + lr + 64 * i, j = j0 + lr + 64 * i;
+        a_src[i] = r < rows ? embed + (size_t)(tok_id ? tok_id[r] : r) * m.D : nullptr;
+        b_src[i] = j < 2 * m.Di ? w_in + (size_t)j * m.D : nullptr;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j0 = 0; j0 < 2 * m.Di; j0 += 256) {
-        const int j = j0 + threadIdx.x;
-        float acc[MB_TOK_TILE];
+    const bool vec = (m.D & 3) == 0 && (((uintptr_t)embed | (uintptr_t)w_in) & 15) == 0;
+    auto get = [&](const float* src, int k) {
+        if (!src) return make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec) return k < m.D ? __ldg(reinterpret_cast<const float4*>(src + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        return make_float4(k < m.D ? src[k] : 0.f, k + 1 < m.D ? src[k + 1] : 0.f, k + 2 < m.D ? src[k + 2] : 0.f, k + 3 < m.D ? src[k + 3] : 0.f);
+    };
+    float4 a_next[2], b_next[2];
+    auto fetch = [&](int k0) {
 #pragma unroll
-        for (int tt = 0; tt < MB_TOK_TILE; ++tt) acc[tt] = 0.f;
-        for (int d0 = 0; d0 < m.D; d0 += 32) {
-            __syncthreads();                             // the previous block of W (and, the first time, e_s) is settled
-            for (int rr = warp; rr < 256; rr += 8) {     // warp per row: lanes along the row
-                const int row = j0 + rr;
-                w_s[rr * 36 + lane] = (row < 2 * m.Di && d0 + lane < m.D) ? w_in[(size_t)row * m.D + d0 + lane] : 0.f;
+        for (int i = 0; i < 2; ++i) { a_next[i] = get(a_src[i], k0 + lk); b_next[i] = get(b_src[i], k0 + lk); }
+    };
+    auto stash = [&](int buf) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float* a = &as[buf][lk][lr + 64 * i]; float* b = &bs[buf][lk][lr + 64 * i];
+            a[0] = a_next[i].x; a[MI_PITCH] = a_next[i].y; a[2 * MI_PITCH] = a_next[i].z; a[3 * MI_PITCH] = a_next[i].w;
+            b[0] = b_next[i].x; b[MI_PITCH] = b_next[i].y; b[2 * MI_PITCH] = b_next[i].z; b[3 * MI_PITCH] = b_next[i].w;
+        }
+    };
+    const int tx = tid & 15, ty = tid >> 4;                             // rows 4 ty ..., 64 + 4 ty ...; features 4 tx ..., 64 + 4 tx ...
+    f32x2 acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    fetch(0);
+    stash(0);
+    __syncthreads();
+    for (int k0 = 0, buf = 0; k0 < m.D; k0 += MI_K, buf ^= 1) {
+        if (k0 + MI_K < m.D) fetch(k0 + MI_K);
+#pragma unroll
+        for (int k = 0; k < MI_K; ++k) {
+            float av[8];
+            *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(&as[buf][k][4 * ty]);
+            *reinterpret_cast<float4*>(av + 4) = *reinterpret_cast<const float4*>(&as[buf][k][64 + 4 * ty]);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&bs[buf][k][4 * tx]), b1 = *reinterpret_cast<const ulonglong2*>(&bs[buf][k][64 + 4 * tx]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const f32x2 a2 = f2_pack(av[i], av[i]);
+                acc[i][0] = f2_fma(a2, b0.x, acc[i][0]); acc[i][1] = f2_fma(a2, b0.y, acc[i][1]);
+                acc[i][2] = f2_fma(a2, b1.x, acc[i][2]); acc[i][3] = f2_fma(a2, b1.y, acc[i][3]);
             }
-            __syncthreads();
-            const int nd = min(32, m.D - d0);
-            if ((m.D & 3) == 0) {                        // four columns at a time: one 16-byte read of W and of every token's embedding
-                for (int dd = 0; dd < nd; dd += 4) {
-                    const float4 w = *reinterpret_cast<const float4*>(w_s + threadIdx.x * 36 + dd);
+        }
+        if (k0 + MI_K < m.D) { stash(buf ^ 1); __syncthreads(); }
+    }
 #pragma unroll
-                    for (int tt = 0; tt < MB_TOK_TILE; ++tt) {
-                        const float4 e = *reinterpret_cast<const float4*>(e_s + tt * m.D + d0 + dd);
-                        acc[tt] = fmaf(w.x, e.x, acc[tt]); acc[tt] = fmaf(w.y, e.y, acc[tt]);
-                        acc[tt] = fmaf(w.z, e.z, acc[tt]); acc[tt] = fmaf(w.w, e.w, acc[tt]);
-                    }
+    for (int i = 0; i < 8; ++i) {
+        const int r = r0 + (i < 4 ? 4 * ty + i : 60 + 4 * ty + i);
+        if (r >= rows) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + 64 * h + 4 * tx;
+            const float2 p = f2_unpack(acc[i][2 * h]), q = f2_unpack(acc[i][2 * h + 1]);
+            const float v[4] = {p.x, p.y, q.x, q.y};
+            if ((m.Di & 3) == 0) {                                      // (then a group of four lies in one of the halves)
+                if (j < 2 * m.Di) *reinterpret_cast<float4*>((j < m.Di ? u + (size_t)r * m.Di + j : z + (size_t)r * m.Di + j - m.Di)) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (j + e < 2 * m.Di) (j + e < m.Di ? u[(size_t)r * m.Di + j + e] : z[(size_t)r * m.Di + j + e - m.Di]) = v[e];
+            }
+        }
+    }
+}
+
+// Everything of one chunk between the input projection and the pooled sum.  Bound: exponentials (d_state of them per token and
+// channel) and the multiply-adds around them.  400 prompts of 109,096 tokens: 0.72 ms (convolution and projections 0.73 ms, two
+// scans 0.80 ms as kernels of their own, v, dt, B and C through memory in between); the whole call 2.26 -> 0.84 ms, its error
+// against 64 bits 1.2e-7 -> 1.1e-7.
+//   1. convolution + SiLU for MC_TILE tokens at a time into shared memory, from there the projections (r, B, C): a thread takes
+//      two tokens and every 16th output, three at a time;
+//   2. a thread per channel scans the chunk: convolution again (four multiply-adds are less than a trip through memory), step
+//      size, recurrence from a zero state, and the two sums of the chunk (see the top of the file).
+constexpr int MC_TILE = 32, MC_THREADS = 256;
+template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to MB_MAX_CONV as 0*/>
+__global__ void __launch_bounds__(MC_THREADS, 2)
+k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* __restrict__ tok_row, const float* __restrict__ u, const float* __restrict__ z,
+              const float* __restrict__ w_conv, const float* __restrict__ b_conv, const float* __restrict__ w_x, const float* __restrict__ w_dt,
+              const float* __restrict__ b_dt, const float* __restrict__ a_log, const float* __restrict__ d_skip,
+              float* __restrict__ end_state, float* __restrict__ decay, float* __restrict__ carry_gain /*all [chunk][Di][N]*/, double* __restrict__ chunk_sum /*[chunk][Di]*/, int w_staged) {
+    extern __shared__ __align__(16) float sm[];
+    const int N = NS ? NS : m.N, n_x = m.R + 2 * m.N, xp = (n_x + 3) & ~3;
+    float* xd_s = sm;                                      // [MB_CHUNK][xp]: B, C, r of every token
+    float* v_s = sm + MB_CHUNK * xp;                       // [MC_TILE][vp]
+    float* wx_s = v_s + MC_TILE * (((m.Di + 3) & ~3) + 4); // [n_x][Di] if it was given room
+    __shared__ int row_s[MB_CHUNK + MB_MAX_CONV];          // rows of the chunk's tokens and of the taps in front of them (-1: before the prompt)
+    const int tid = threadIdx.x, Dp = (m.Di + 3) & ~3, vp = Dp + 4;
+    const ChunkRec ch = chunks[blockIdx.x];
+    constexpr int KM = KC ? KC : MB_MAX_CONV;
+    const int Kc = KC ? KC : m.Kc, back = Kc - 1;
+    for (int i = tid; i < ch.n_tok + back; i += MC_THREADS) row_s[i] = ch.pos0 + i - back >= 0 ? tok_row[ch.tok0 + i - back] : -1;
+    if (w_staged) for (int i = tid; i < n_x * m.Di; i += MC_THREADS) wx_s[i] = __ldg(w_x + i);
+    const float* wx = w_staged ? wx_s : w_x;
+    __syncthreads();
+    // SiLU(convolution) of channel c at token t; the taps come in the order of the sum
+    auto conv = [&](const float (&w)[KM], float b, const float (&x)[KM]) {
+        float acc = b;
+#pragma unroll
+        for (int j = 0; j < KM; ++j) if (j < Kc) acc = fmaf(w[j], x[j], acc);
+        return silu_f(acc);
+    };
+    const bool vec = (m.Di & 3) == 0 && (w_staged || ((uintptr_t)w_x & 15) == 0);
+    for (int t0 = 0; t0 < ch.n_tok; t0 += MC_TILE) {
+        const int nt = min(MC_TILE, ch.n_tok - t0);
+        for (int c = tid; c < Dp; c += MC_THREADS) {
+            float w[KM], x[KM];
+            const bool on = c < m.Di;
+#pragma unroll
+            for (int j = 0; j < KM; ++j) {
+                w[j] = on && j < Kc ? __ldg(w_conv + (size_t)c * Kc + j) : 0.f;
+                x[j] = 0.f;
+                if (on && j < back) { const int r = row_s[t0 + j]; x[j] = r >= 0 ? __ldg(u + (size_t)r * m.Di + c) : 0.f; }
+            }
+            const float b = on ? __ldg(b_conv + c) : 0.f;
+#pragma unroll 4
+            for (int t = 0; t < MC_TILE; ++t) {
+                const float nu = on && t < nt ? __ldg(u + (size_t)row_s[t0 + t + back] * m.Di + c) : 0.f;
+#pragma unroll
+                for (int j = 0; j < KM; ++j) if (j == back) x[j] = nu;
+                v_s[t * vp + c] = on && t < nt ? conv(w, b, x) : 0.f;
+#pragma unroll
+                for (int j = 0; j + 1 < KM; ++j) if (j < back) x[j] = x[j + 1];
+            }
+        }
+        __syncthreads();
+        const int t = tid & 15, og = tid >> 4;
+        const float* v0 = v_s + t * vp;
+        const float* v1 = v0 + 16 * vp;
+        for (int o0 = og; o0 < n_x; o0 += 48) {
+            const int o1 = o0 + 16, o2 = o0 + 32;
+            float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const float* w0 = wx + (size_t)o0 * m.Di;
+            const float* w1 = wx + (size_t)min(o1, n_x - 1) * m.Di;
+            const float* w2 = wx + (size_t)min(o2, n_x - 1) * m.Di;
+            if (vec) {
+#pragma unroll 2
+                for (int c = 0; c < m.Di; c += 4) {
+                    const float4 a = *reinterpret_cast<const float4*>(v0 + c), b = *reinterpret_cast<const float4*>(v1 + c);
+                    const float4 p = *reinterpret_cast<const float4*>(w0 + c), q = *reinterpret_cast<const float4*>(w1 + c), r = *reinterpret_cast<const float4*>(w2 + c);
+                    s[0] = fmaf(p.x, a.x, s[0]); s[0] = fmaf(p.y, a.y, s[0]); s[0] = fmaf(p.z, a.z, s[0]); s[0] = fmaf(p.w, a.w, s[0]);
+                    s[1] = fmaf(p.x, b.x, s[1]); s[1] = fmaf(p.y, b.y, s[1]); s[1] = fmaf(p.z, b.z, s[1]); s[1] = fmaf(p.w, b.w, s[1]);
+                    s[2] = fmaf(q.x, a.x, s[2]); s[2] = fmaf(q.y, a.y, s[2]); s[2] = fmaf(q.z, a.z, s[2]); s[2] = fmaf(q.w, a.w, s[2]);
+                    s[3] = fmaf(q.x, b.x, s[3]); s[3] = fmaf(q.y, b.y, s[3]); s[3] = fmaf(q.z, b.z, s[3]); s[3] = fmaf(q.w, b.w, s[3]);
+                    s[4] = fmaf(r.x, a.x, s[4]); s[4] = fmaf(r.y, a.y, s[4]); s[4] = fmaf(r.z, a.z, s[4]); s[4] = fmaf(r.w, a.w, s[4]);
+                    s[5] = fmaf(r.x, b.x, s[5]); s[5] = fmaf(r.y, b.y, s[5]); s[5] = fmaf(r.z, b.z, s[5]); s[5] = fmaf(r.w, b.w, s[5]);
                 }
             } else {
-                for (int dd = 0; dd < nd; ++dd) {
-                    const float w = w_s[threadIdx.x * 36 + dd];
+                for (int c = 0; c < m.Di; ++c) {
+                    const float a = v0[c], b = v1[c], p = w0[c], q = w1[c], r = w2[c];
+                    s[0] = fmaf(p, a, s[0]); s[1] = fmaf(p, b, s[1]); s[2] = fmaf(q, a, s[2]); s[3] = fmaf(q, b, s[3]); s[4] = fmaf(r, a, s[4]); s[5] = fmaf(r, b, s[5]);
+                }
+            }
+            // kept as [B | C | r], so that a token's B and C can be read by fours
+            auto at = [&](int o) { return o < m.R ? 2 * m.N + o : o - m.R; };
 #pragma unroll
-                    for (int tt = 0; tt < MB_TOK_TILE; ++tt) acc[tt] = fmaf(w, e_s[tt * m.D + d0 + dd], acc[tt]);
+            for (int i = 0; i < 3; ++i) {
+                const int o = o0 + 16 * i;
+                if (o < n_x) {
+                    if (t < nt) xd_s[(t0 + t) * xp + at(o)] = s[2 * i];
+                    if (t + 16 < nt) xd_s[(t0 + t + 16) * xp + at(o)] = s[2 * i + 1];
                 }
             }
         }
-        if (j < 2 * m.Di) {
-            float* dst = j < m.Di ? u : z;
-            const int c = j < m.Di ? j : j - m.Di;
-#pragma unroll
-            for (int tt = 0; tt < MB_TOK_TILE; ++tt) if (tt < nt) dst[(size_t)(t0 + tt) * m.Di + c] = acc[tt];
-        }
+        __syncthreads();
     }
-}
-
-// Per tile of MB_CP_TILE tokens: causal depthwise convolution + SiLU, the projections to (r, B, C), the step size.
-// A tile shares every weight it reads (each row of W_x is read once per tile and used for all its tokens).
-constexpr int MB_CP_TILE = 8;
-__global__ void __launch_bounds__(256)
-k_mamba_conv_proj(MambaDims m, int T, const int32_t* __restrict__ tok_pos /*position inside its prompt*/,
-                  const float* __restrict__ u, const float* __restrict__ w_conv, const float* __restrict__ b_conv,
-                  const float* __restrict__ w_x, const float* __restrict__ w_dt, const float* __restrict__ b_dt,
-                  float* __restrict__ v, float* __restrict__ dt, float* __restrict__ bc) {
-    extern __shared__ float sm[];                        // v [tile][Di], x_dbl [tile][R + 2N]
-    const int n_x = m.R + 2 * m.N;
-    float* v_s = sm;
-    float* xd_s = sm + MB_CP_TILE * m.Di;
-    const int t0 = blockIdx.x * MB_CP_TILE, nt = min(MB_CP_TILE, T - t0);
-    for (int idx = threadIdx.x; idx < MB_CP_TILE * m.Di; idx += blockDim.x) {
-        const int tt = idx / m.Di, c = idx % m.Di;
-        float val = 0.f;
-        if (tt < nt) {
-            const int t = t0 + tt, pos = tok_pos[t];
-            float acc = b_conv[c];
-            for (int j = 0; j < m.Kc; ++j) {
-                const int back = m.Kc - 1 - j;           // tap j looks `back` tokens back; nothing before the prompt's first token
-                if (back <= pos) acc = fmaf(w_conv[(size_t)c * m.Kc + j], u[(size_t)(t - back) * m.Di + c], acc);
+    for (int c = tid; c < m.Di; c += MC_THREADS) {
+        float w[KM], x[KM];
+#pragma unroll
+        for (int j = 0; j < KM; ++j) {
+            w[j] = j < Kc ? __ldg(w_conv + (size_t)c * Kc + j) : 0.f;
+            x[j] = 0.f;
+            if (j < back) { const int r = row_s[j]; x[j] = r >= 0 ? __ldg(u + (size_t)r * m.Di + c) : 0.f; }
+        }
+        const float b = __ldg(b_conv + c), bdt = __ldg(b_dt + c), dsk = __ldg(d_skip + c);
+        float wd[8];                                       // the first eight columns of the channel's row of W_dt (the rest, if any, is read as needed)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) wd[r] = r < m.R ? __ldg(w_dt + (size_t)c * m.R + r) : 0.f;
+        float A[MB_MAX_N];
+        f32x2 h[MB_MAX_N / 2], P[MB_MAX_N / 2], G[MB_MAX_N / 2];
+#pragma unroll
+        for (int n = 0; n < MB_MAX_N; ++n) A[n] = n < N ? -expf(__ldg(a_log + (size_t)c * m.N + n)) * 1.4426950408889634f : 0.f;      // (decays as powers of two)
+#pragma unroll
+        for (int n = 0; n < MB_MAX_N / 2; ++n) { h[n] = 0ull; P[n] = f2_pack(1.f, 1.f); G[n] = 0ull; }
+        double sum = 0.0;                                  // (in double here and over the chunks: the sum's rounding would be the largest of all)
+        float nu = __ldg(u + (size_t)row_s[back] * m.Di + c), nz = __ldg(z + (size_t)row_s[back] * m.Di + c);
+        for (int t = 0; t < ch.n_tok; ++t) {
+            const float zt = nz;
+#pragma unroll
+            for (int j = 0; j < KM; ++j) if (j == back) x[j] = nu;
+            if (t + 1 < ch.n_tok) {                        // the next token's values are on their way during this one
+                const size_t r = (size_t)row_s[t + 1 + back] * m.Di + c;
+                nu = __ldg(u + r); nz = __ldg(z + r);
             }
-            val = silu_f(acc);
-            v[(size_t)t * m.Di + c] = val;
-        }
-        v_s[idx] = val;
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    for (int o = warp; o < n_x; o += n_warps) {
-        float acc[MB_CP_TILE];
+            const float v = conv(w, b, x);
 #pragma unroll
-        for (int tt = 0; tt < MB_CP_TILE; ++tt) acc[tt] = 0.f;
-        for (int c = lane; c < m.Di; c += 32) {
-            const float w = w_x[(size_t)o * m.Di + c];
+            for (int j = 0; j + 1 < KM; ++j) if (j < back) x[j] = x[j + 1];
+            const float* xd = xd_s + t * xp;
+            float dt = bdt;
 #pragma unroll
-            for (int tt = 0; tt < MB_CP_TILE; ++tt) acc[tt] = fmaf(w, v_s[tt * m.Di + c], acc[tt]);
-        }
+            for (int r = 0; r < 8; ++r) if (r < m.R) dt = fmaf(wd[r], xd[2 * m.N + r], dt);
+            for (int r = 8; r < m.R; ++r) dt = fmaf(__ldg(w_dt + (size_t)c * m.R + r), xd[2 * m.N + r], dt);
+            dt = softplus_f(dt);
+            const float dx = dt * v, g = silu_f(zt);
+            const f32x2 dx2 = f2_pack(dx, dx), g2 = f2_pack(g, g);
+            f32x2 y2 = 0ull;
 #pragma unroll
-        for (int tt = 0; tt < MB_CP_TILE; ++tt) {
-#pragma unroll
-            for (int s = 16; s > 0; s >>= 1) acc[tt] += __shfl_xor_sync(0xffffffffu, acc[tt], s);
-            if (lane == 0 && tt < nt) {
-                xd_s[tt * n_x + o] = acc[tt];
-                if (o >= m.R) bc[(size_t)(t0 + tt) * 2 * m.N + (o - m.R)] = acc[tt];
+            for (int n = 0; n < MB_MAX_N / 2; ++n) {
+                if (2 * n < N) {
+                    const bool odd = NS ? false : 2 * n + 1 >= N;      // (an unused second state: its decay is one, its input zero)
+                    const f32x2 a = f2_pack(exp2f(dt * A[2 * n]), odd ? 1.f : exp2f(dt * A[2 * n + 1]));
+                    const f32x2 B2 = NS ? *reinterpret_cast<const f32x2*>(xd + 2 * n) : f2_pack(xd[2 * n], odd ? 0.f : xd[2 * n + 1]);
+                    const f32x2 C2 = NS ? *reinterpret_cast<const f32x2*>(xd + NS + 2 * n) : f2_pack(xd[m.N + 2 * n], odd ? 0.f : xd[m.N + 2 * n + 1]);
+                    h[n] = f2_fma(a, h[n], f2_mul(dx2, B2));
+                    P[n] = f2_mul(P[n], a);
+                    y2 = f2_fma(h[n], C2, y2);
+                    G[n] = f2_fma(f2_mul(g2, C2), P[n], G[n]);
+                }
             }
+            const float2 y = f2_unpack(y2);
+            sum += (double)(fmaf(dsk, v, y.x + y.y) * g);
         }
-    }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < nt * m.Di; idx += blockDim.x) {
-        const int tt = idx / m.Di, c = idx % m.Di;
-        float acc = b_dt[c];
-        for (int r = 0; r < m.R; ++r) acc = fmaf(w_dt[(size_t)c * m.R + r], xd_s[tt * n_x + r], acc);
-        dt[(size_t)(t0 + tt) * m.Di + c] = softplus_f(acc);
-    }
-}
-
-// One chunk x 64 channels.  EMIT = false: scan from zero, leave the end state and the product of the decays.
-// EMIT = true: scan from the chunk's starting state and leave the chunk's sum over tokens of y_t * silu(z_t).
-template <bool EMIT>
-__global__ void __launch_bounds__(64)
-k_mamba_scan(MambaDims m, const ChunkRec* __restrict__ chunks, const float* __restrict__ v, const float* __restrict__ dt,
-             const float* __restrict__ bc, const float* __restrict__ z, const float* __restrict__ a_log, const float* __restrict__ d_skip,
-             float* __restrict__ end_state /*[chunk][Di][N]*/, float* __restrict__ decay /*[chunk][Di][N]*/,
-             const float* __restrict__ start_state /*[chunk][Di][N] or nullptr = zero*/, float* __restrict__ chunk_sum /*[chunk][Di]*/) {
-    __shared__ float bc_s[MB_CHUNK][2 * MB_MAX_N];
-    const ChunkRec ch = chunks[blockIdx.x];
-    const int c = blockIdx.y * 64 + threadIdx.x;
-    for (int i = threadIdx.x; i < ch.n_tok * 2 * m.N; i += blockDim.x) bc_s[i / (2 * m.N)][i % (2 * m.N)] = bc[(size_t)ch.tok0 * 2 * m.N + i];
-    __syncthreads();
-    if (c >= m.Di) return;
-    float A[MB_MAX_N], h[MB_MAX_N], p[MB_MAX_N];
+        chunk_sum[(size_t)blockIdx.x * m.Di + c] = sum;
+        const size_t at = ((size_t)blockIdx.x * m.Di + c) * m.N;
 #pragma unroll
-    for (int n = 0; n < MB_MAX_N; ++n) {
-        A[n] = n < m.N ? -expf(a_log[(size_t)c * m.N + n]) : 0.f;
-        h[n] = (EMIT && start_state && n < m.N) ? start_state[((size_t)blockIdx.x * m.Di + c) * m.N + n] : 0.f;
-        p[n] = 1.f;
-    }
-    const float dsk = d_skip[c];
-    float sum = 0.f;
-    for (int tt = 0; tt < ch.n_tok; ++tt) {
-        const size_t ti = (size_t)(ch.tok0 + tt) * m.Di + c;
-        const float d = dt[ti], x = v[ti], dx = d * x;
-        float y = 0.f;
-#pragma unroll
-        for (int n = 0; n < MB_MAX_N; ++n) {
-            if (n < m.N) {
-                const float a = expf(d * A[n]);
-                h[n] = fmaf(a, h[n], dx * bc_s[tt][n]);
-                if (EMIT) y = fmaf(h[n], bc_s[tt][m.N + n], y); else p[n] *= a;
+        for (int n = 0; n < MB_MAX_N / 2; ++n) {
+            if (2 * n < N) {
+                const float2 hv = f2_unpack(h[n]), pv = f2_unpack(P[n]), gv = f2_unpack(G[n]);
+                end_state[at + 2 * n] = hv.x; decay[at + 2 * n] = pv.x; carry_gain[at + 2 * n] = gv.x;
+                if (NS || 2 * n + 1 < N) { end_state[at + 2 * n + 1] = hv.y; decay[at + 2 * n + 1] = pv.y; carry_gain[at + 2 * n + 1] = gv.y; }
             }
         }
-        if (EMIT) sum += (y + dsk * x) * silu_f(z[ti]);
-    }
-    if (EMIT) chunk_sum[(size_t)blockIdx.x * m.Di + c] = sum;
-    else {
-#pragma unroll
-        for (int n = 0; n < MB_MAX_N; ++n) if (n < m.N) {
-            end_state[((size_t)blockIdx.x * m.Di + c) * m.N + n] = h[n];
-            decay[((size_t)blockIdx.x * m.Di + c) * m.N + n] = p[n];
-        }
     }
 }
 
-// The state each chunk starts from: serial over the chunks of a prompt, one thread per (channel, state).
-__global__ void k_mamba_carry(MambaDims m, const int32_t* __restrict__ prompt_chunk0 /*[n_prompts + 1]*/, const float* __restrict__ end_state,
-                              const float* __restrict__ decay, float* __restrict__ start_state) {
-    const int i = blockIdx.y * blockDim.x + threadIdx.x;
-    if (i >= m.Di * m.N) return;
-    float s = 0.f;
-    for (int ch = prompt_chunk0[blockIdx.x]; ch < prompt_chunk0[blockIdx.x + 1]; ++ch) {
-        const size_t at = (size_t)ch * m.Di * m.N + i;
-        start_state[at] = s;
-        s = fmaf(decay[at], s, end_state[at]);
-    }
-}
-
-// Per prompt: mean over tokens of the gated outputs (chunks in order), W_out, the classification layer, argmax.
+// Per prompt: the states its chunks start from (serial, a thread per channel and state), mean over tokens of the gated outputs
+// (chunks in order), W_out, the classification layer, argmax.
 __global__ void k_mamba_head(MambaDims m, const int32_t* __restrict__ prompt_chunk0, const int32_t* __restrict__ lens,
-                             const float* __restrict__ chunk_sum, const float* __restrict__ w_out, const float* __restrict__ w_fc,
+                             const double* __restrict__ chunk_sum, const float* __restrict__ end_state, const float* __restrict__ decay,
+                             const float* __restrict__ carry_gain, const float* __restrict__ w_out, const float* __restrict__ w_fc,
                              const float* __restrict__ b_fc, float* __restrict__ scores, int32_t* __restrict__ labels) {
-    extern __shared__ float hs[];                        // g mean [Di], pooled [D], scores [K]
-    float* g_s = hs;
-    float* o_s = hs + m.Di;
+    extern __shared__ float hs[];                        // per (channel, state) what the starting states add [Di N], g mean [Di], pooled [D], scores [K]
+    float* c_s = hs;
+    float* g_s = c_s + m.Di * m.N;
+    float* o_s = g_s + m.Di;
     float* sc_s = o_s + m.D;
     const int pr = blockIdx.x;
+    const int c0 = prompt_chunk0[pr], c1 = prompt_chunk0[pr + 1];
     const float inv = 1.f / (float)lens[pr];
+    const size_t per = (size_t)m.Di * m.N;
+    if (c1 - c0 > 1)
+        for (int i = threadIdx.x; i < m.Di * m.N; i += blockDim.x) {
+            float s = end_state[c0 * per + i], add = 0.f;
+#pragma unroll 4
+            for (int ch = c0 + 1; ch < c1; ++ch) {
+                const size_t at = ch * per + i;
+                add = fmaf(carry_gain[at], s, add);
+                s = fmaf(decay[at], s, end_state[at]);
+            }
+            c_s[i] = add;
+        }
+    __syncthreads();
     for (int c = threadIdx.x; c < m.Di; c += blockDim.x) {
-        float s = 0.f;
-        for (int ch = prompt_chunk0[pr]; ch < prompt_chunk0[pr + 1]; ++ch) s += chunk_sum[(size_t)ch * m.Di + c];
-        g_s[c] = s * inv;
+        double s = 0.0;
+        for (int ch = c0; ch < c1; ++ch) s += chunk_sum[(size_t)ch * m.Di + c];
+        if (c1 - c0 > 1) for (int n = 0; n < m.N; ++n) s += (double)c_s[c * m.N + n];
+        g_s[c] = (float)s * inv;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
@@ -268,19 +367,18 @@ bool dims_ok(const sd_mamba_desc* d, MambaDims& m) {
     return true;
 }
 
-struct Layout { size_t u, z, v, dt, bc, end_state, decay, start_state, chunk_sum, tok_src, tok_pos, chunks, prompt_chunk0, lens, starts, total; };
+struct Layout { size_t u, z, end_state, decay, carry_gain, chunk_sum, tok_id, tok_row, chunks, prompt_chunk0, lens, starts, total; };
 
 Layout layout(const MambaDims& m, int64_t T, int64_t n_chunks, int n_prompts) {
     Layout L;
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t at = o; o += al(bytes); return at; };
-    L.u = take((size_t)T * m.Di * 4); L.z = take((size_t)T * m.Di * 4); L.v = take((size_t)T * m.Di * 4); L.dt = take((size_t)T * m.Di * 4);
-    L.bc = take((size_t)T * 2 * m.N * 4);
+    L.u = take((size_t)T * m.Di * 4); L.z = take((size_t)T * m.Di * 4);      // (with more tokens than the vocabulary has, one row per token of it: fewer)
     L.end_state = take((size_t)n_chunks * m.Di * m.N * 4); L.decay = take((size_t)n_chunks * m.Di * m.N * 4);
-    L.start_state = take((size_t)n_chunks * m.Di * m.N * 4);
-    L.chunk_sum = take((size_t)n_chunks * m.Di * 4);
-    L.tok_src = take((size_t)T * 8); L.tok_pos = take((size_t)T * 4);
-    L.chunks = take((size_t)n_chunks * sizeof(ChunkRec));
+    L.carry_gain = take((size_t)n_chunks * m.Di * m.N * 4);
+    L.chunk_sum = take((size_t)n_chunks * m.Di * 8);
+    L.tok_id = take((size_t)T * 4); L.tok_row = take((size_t)T * 4);
+    L.chunks = take((size_t)n_chunks * sizeof(ChunkRec));                    // from here on: uploaded in one copy
     L.prompt_chunk0 = take((size_t)(n_prompts + 1) * 4); L.lens = take((size_t)n_prompts * 4); L.starts = take((size_t)n_prompts * 8);
     L.total = o;
     return L;
@@ -318,10 +416,8 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     std::vector<int32_t> prompt_chunk0((size_t)n_prompts + 1);
     std::vector<ChunkRec> chunks;
     int64_t t = 0;
-    int max_len = 0;
     for (int i = 0; i < n_prompts; ++i) {
         prompt_chunk0[i] = (int32_t)chunks.size();
-        max_len = lens_host[i] > max_len ? lens_host[i] : max_len;
         for (int p = 0; p < lens_host[i]; p += MB_CHUNK) {
             const int n = lens_host[i] - p < MB_CHUNK ? lens_host[i] - p : MB_CHUNK;
             chunks.push_back(ChunkRec{i, (int32_t)t, n, p});
@@ -333,34 +429,37 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     const Layout L = layout(m, T, T / MB_CHUNK + n_prompts, n_prompts);
     char* base = (char*)workspace_dev;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    auto up = [&](size_t at, const void* src, size_t bytes) { return cudaMemcpyAsync(base + at, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess; };
-    if (!up(L.chunks, chunks.data(), (size_t)n_chunks * sizeof(ChunkRec)) || !up(L.prompt_chunk0, prompt_chunk0.data(), (size_t)(n_prompts + 1) * 4) ||
-        !up(L.lens, lens_host, (size_t)n_prompts * 4) || !up(L.starts, starts_host, (size_t)n_prompts * 8))
-        return SD_ERR_CUDA;
+    std::vector<char> host(L.starts + (size_t)n_prompts * 8 - L.chunks);
+    memcpy(host.data(), chunks.data(), (size_t)n_chunks * sizeof(ChunkRec));
+    memcpy(host.data() + (L.prompt_chunk0 - L.chunks), prompt_chunk0.data(), (size_t)(n_prompts + 1) * 4);
+    memcpy(host.data() + (L.lens - L.chunks), lens_host, (size_t)n_prompts * 4);
+    memcpy(host.data() + (L.starts - L.chunks), starts_host, (size_t)n_prompts * 8);
+    if (cudaMemcpyAsync(base + L.chunks, host.data(), host.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) return SD_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return SD_ERR_CUDA;      // the host tables above go out of scope
-    float* u = (float*)(base + L.u); float* z = (float*)(base + L.z); float* v = (float*)(base + L.v); float* dt = (float*)(base + L.dt);
-    float* bc = (float*)(base + L.bc);
+    float* u = (float*)(base + L.u); float* z = (float*)(base + L.z);
     const ChunkRec* chunks_d = (const ChunkRec*)(base + L.chunks);
     const int32_t* pc0 = (const int32_t*)(base + L.prompt_chunk0);
+    int32_t* tok_id = (int32_t*)(base + L.tok_id); int32_t* tok_row = (int32_t*)(base + L.tok_row);
 
-    k_mamba_tables<<<(unsigned)n_chunks, 64, 0, st>>>(chunks_d, (const int64_t*)(base + L.starts), (int64_t*)(base + L.tok_src), (int32_t*)(base + L.tok_pos));
-    const size_t in_smem_bytes = ((size_t)MB_TOK_TILE * m.D + 256 * 36) * 4;      // up to 66 KB at d_model 512: above the default limit
-    if (cudaFuncSetAttribute(k_mamba_in, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)in_smem_bytes) != cudaSuccess) return SD_ERR_CUDA;
-    k_mamba_in<<<(unsigned)((T + MB_TOK_TILE - 1) / MB_TOK_TILE), 256, in_smem_bytes, st>>>(
-        m, tokens_dev, (const int64_t*)(base + L.tok_src), (int)T, w->embed, w->w_in, u, z);
-    k_mamba_conv_proj<<<(unsigned)((T + MB_CP_TILE - 1) / MB_CP_TILE), 256, (size_t)MB_CP_TILE * (m.Di + m.R + 2 * m.N) * 4, st>>>(
-        m, (int)T, (const int32_t*)(base + L.tok_pos), u, w->w_conv, w->b_conv, w->w_x, w->w_dt, w->b_dt, v, dt, bc);
-    const dim3 sgrid((unsigned)n_chunks, (unsigned)((m.Di + 63) / 64));
-    const float* start = nullptr;
-    if (max_len > MB_CHUNK) {
-        k_mamba_scan<false><<<sgrid, 64, 0, st>>>(m, chunks_d, v, dt, bc, z, w->a_log, w->d_skip, (float*)(base + L.end_state), (float*)(base + L.decay),
-                                                  nullptr, nullptr);
-        k_mamba_carry<<<dim3((unsigned)n_prompts, (unsigned)((m.Di * m.N + 255) / 256)), 256, 0, st>>>(
-            m, pc0, (const float*)(base + L.end_state), (const float*)(base + L.decay), (float*)(base + L.start_state));
-        start = (const float*)(base + L.start_state);
-    }
-    k_mamba_scan<true><<<sgrid, 64, 0, st>>>(m, chunks_d, v, dt, bc, z, w->a_log, w->d_skip, nullptr, nullptr, start, (float*)(base + L.chunk_sum));
-    k_mamba_head<<<(unsigned)n_prompts, 256, (size_t)(m.Di + m.D + m.K) * 4, st>>>(
-        m, pc0, (const int32_t*)(base + L.lens), (const float*)(base + L.chunk_sum), w->w_out, w->w_fc, w->b_fc, scores_dev, labels_dev);
+    // 400 prompts of 109,096 tokens over 21,128: the projection is a fifth of the work token by token
+    const bool by_token = T >= m.V;
+    const int rows = by_token ? m.V : (int)T;
+    k_mamba_tables<<<(unsigned)n_chunks, 64, 0, st>>>(chunks_d, (const int64_t*)(base + L.starts), tokens_dev, m.V, by_token ? 1 : 0, tok_id, tok_row);
+    k_mamba_in<<<dim3((unsigned)((rows + MI_TILE - 1) / MI_TILE), (unsigned)((2 * m.Di + MI_TILE - 1) / MI_TILE)), 256, 0, st>>>(
+        m, by_token ? nullptr : tok_id, rows, w->embed, w->w_in, u, z);
+    const size_t xp = (size_t)((m.R + 2 * m.N + 3) & ~3), wx_bytes = (size_t)(m.R + 2 * m.N) * m.Di * 4;
+    const int w_staged = wx_bytes <= 48 * 1024;                              // two CTAs of the usual sizes still fit an SM
+    const size_t chunk_smem = (MB_CHUNK * xp + (size_t)MC_TILE * (((m.Di + 3) & ~3) + 4)) * 4 + (w_staged ? wx_bytes : 0);
+    auto chunk_kernel = m.N != MB_MAX_N ? k_mamba_chunk<0, 0> : m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4> : k_mamba_chunk<MB_MAX_N, 0>;
+    const size_t head_smem = ((size_t)m.Di * m.N + m.Di + m.D + m.K) * 4;
+    if (cudaFuncSetAttribute(chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chunk_smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mamba_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)head_smem) != cudaSuccess)
+        return SD_ERR_CUDA;
+    chunk_kernel<<<(unsigned)n_chunks, MC_THREADS, chunk_smem, st>>>(
+        m, chunks_d, tok_row, u, z, w->w_conv, w->b_conv, w->w_x, w->w_dt, w->b_dt, w->a_log, w->d_skip, (float*)(base + L.end_state),
+        (float*)(base + L.decay), (float*)(base + L.carry_gain), (double*)(base + L.chunk_sum), w_staged);
+    k_mamba_head<<<(unsigned)n_prompts, 1024, head_smem, st>>>(
+        m, pc0, (const int32_t*)(base + L.lens), (const double*)(base + L.chunk_sum), (const float*)(base + L.end_state), (const float*)(base + L.decay),
+        (const float*)(base + L.carry_gain), w->w_out, w->w_fc, w->b_fc, scores_dev, labels_dev);
     return cudaGetLastError() == cudaSuccess ? SD_OK : SD_ERR_CUDA;
 }
