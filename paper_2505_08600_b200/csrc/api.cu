@@ -11,6 +11,7 @@
 #include "gemv.h"
 #include "kernels.h"
 #include "pass_stream.h"
+#include "plain_steps.h"
 #include "prefill.h"
 
 using namespace sd;
@@ -527,6 +528,40 @@ sd_status prepare_pass(sd_ctx* c, int model, const RowPlan& plan, int n_rows, in
 sd_status forward_pass(sd_ctx* c, Model& M, const sd_ctx::CachedProgram& cp, const SeqList& list, const RowPlan& plan, int n_rows, int mode,
                        float* logits_out);
 
+// The pass of an fp32 model over a few rows (plain_steps.cu).
+sd_status forward_plain_few(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan, int n_rows, int mode, float* logits_out) {
+    const sd_model_desc& m = M.d;
+    const int d = m.d_model, H = m.n_heads, Hkv = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn;
+    cudaStream_t st = c->st;
+    LAUNCH(CAT_ELEMENTWISE, launch_embed(c->S, list, plan, n_rows, M.embed, m.dtype, d, m.vocab, c->h, c->row_slot, c->row_pos,
+                                         nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr, 0, nullptr, st));
+    PlainStep p;
+    memset(&p, 0, sizeof(p));
+    p.eps = m.rms_eps; p.F = F; p.q = (float*)c->q; p.row_slot = c->row_slot; p.row_pos = c->row_pos;
+    p.H = H; p.Hkv = Hkv; p.hd = hd; p.max_ctx = c->cfg.max_ctx; p.rcos = M.rope_cos; p.rsin = M.rope_sin;
+    auto step = [&](int kind, const void* w, const float* x, int rows, int n_out, int K, const float* gain, float* y) {
+        p.mode = kind; p.w = (const float*)w; p.x = x; p.rows = rows; p.n_out = n_out; p.K = K; p.gain = gain; p.y = y;
+        LAUNCH(CAT_LINEAR, launch_plain_step(p, st));
+        return SD_OK;
+    };
+    for (int l = 0; l < m.n_layers; ++l) {
+        const Layer& L = M.layers[l];
+        p.kc = (float*)(M.kcache + M.kv_layer_bytes * l); p.vc = (float*)(M.vcache + M.kv_layer_bytes * l);
+        SD_TRY(step(PS_QKV, L.wqkv, c->h, n_rows, M.n_qkv(), d, L.norm1, nullptr));
+        LAUNCH(CAT_ATTENTION, launch_plain_attention(p.q, p.kc, p.vc, (float*)c->attn, c->row_slot, c->row_pos, n_rows, H, Hkv, hd, c->cfg.max_ctx, st));
+        SD_TRY(step(PS_RESIDUAL, L.wo, (float*)c->attn, n_rows, d, H * hd, nullptr, c->h));
+        SD_TRY(step(PS_GU, L.wgu, c->h, n_rows, 2 * F, d, L.norm2, (float*)c->act));
+        SD_TRY(step(PS_RESIDUAL, L.wd, (float*)c->act, n_rows, d, F, nullptr, c->h));
+    }
+    if (mode != LOGITS_NONE) {
+        const int R = plan.rows_per_seq;
+        p.row_stride = mode == LOGITS_LAST ? R : 1; p.row_offset = mode == LOGITS_LAST ? R - 1 : 0;
+        SD_TRY(step(PS_LM, M.lm_head, c->h, mode == LOGITS_LAST ? list.n : n_rows, m.vocab, d, M.final_norm, logits_out));
+    }
+    CUDA_TRY(prof_mark(c, CAT_NONE));
+    return SD_OK;
+}
+
 sd_status forward(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan, int n_rows, int mode, float* logits_out) {
     if (pass_wanted(c, M, plan, n_rows)) {
         const int model = (int)(&M - &c->models[0]);
@@ -535,6 +570,7 @@ sd_status forward(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan,
         if (cp && cp->slot >= 0) return forward_pass(c, M, *cp, list, plan, n_rows, mode, logits_out);
     }
     if (M.tc && !c->force_plain) return forward_tc(c, M, list, plan, n_rows, mode, logits_out);
+    if (!c->force_plain && plain_steps_fit(M.d, n_rows, c->cfg.max_ctx)) return forward_plain_few(c, M, list, plan, n_rows, mode, logits_out);
     const sd_model_desc& m = M.d;
     const int d = m.d_model, H = m.n_heads, Hkv = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, dt = m.dtype;
     cudaStream_t st = c->st;

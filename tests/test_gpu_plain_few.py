@@ -1,0 +1,43 @@
+"""fp32 models over a few rows (norm, matrix and step in one kernel) against the CPU oracle: reductions of more than one round of
+weights, odd vocabularies, grouped heads, heads of 16 and 256, 1...8 rows and one call beyond them."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2505_08600_b200 import synth
+from gpu_util import DEV
+
+pytestmark = pytest.mark.gpu
+
+MODELS = {
+    "gqa16": dict(n_layers=2, d_model=104, n_heads=6, n_kv_heads=2, head_dim=16, d_ffn=72, vocab=333),
+    "hd256": dict(n_layers=1, d_model=256, n_heads=2, n_kv_heads=1, head_dim=256, d_ffn=1544, vocab=1001),     # three rounds of weights
+}
+
+
+@pytest.mark.parametrize("name", sorted(MODELS))
+@pytest.mark.parametrize("n_seq,gamma", [(1, 0), (1, 1), (1, 4), (2, 3), (3, 2)])      # 1, 2, 5, 8 and 9 verify rows
+def test_verify_rows_follow_the_oracle(name, n_seq, gamma):
+    from paper_2505_08600_b200 import binding
+    dims = MODELS[name]
+    V = dims["vocab"]
+    w = synth.make_weights(dims, seed=3, model_index=0, dtype="f32")
+    ctx = binding.Context(dims, [dims], "f32", n_seq, 96, max(gamma, 1), 1.0, 7)
+    ctx.load_weights(0, w); ctx.load_weights(1, w)
+    toks = [synth.make_prompt(V, (3, 70, 33)[s], seed=9, seq=s) for s in range(n_seq)]
+    seqs = list(range(n_seq))
+    for s in seqs:
+        ctx.sd_seq_begin(s, toks[s], s)
+    ctx.sd_route_prompt(seqs, forced_task=[0] * n_seq)
+    ctx.sd_prefill(seqs)
+    x = np.stack([synth.make_prompt(V, gamma, seed=5, seq=s) for s in seqs]) if gamma else np.zeros((n_seq, 0), np.int32)
+    logits = torch.zeros((n_seq, gamma + 1, V), dtype=torch.float32, device=DEV)
+    ctx.sd_verify(seqs, gamma, torch.from_numpy(x).to(DEV), logits)
+    got = logits.cpu().numpy().astype(np.float64)
+    assert ctx.sd_device_status() == 0
+    ctx.close()
+    om = oracle.OracleModel(dims, w)
+    for s in seqs:
+        want = om.new_cache(128).forward(np.concatenate([toks[s], x[s]]), 0)[-(gamma + 1):]
+        assert np.abs(got[s] - want).max() <= 1e-4, s          # logits of magnitude 1 over a few hundred fp32 terms per matrix
