@@ -619,8 +619,8 @@ def run_mamba_bench(args):
 
 
 def run_prefill_bench(args):
-    """Prefill of one 512-token prompt of the configuration's target model (the contraction-bound regime): forward over the
-    prompt in batches of at most 256 rows through the same weight GEMM as the verify step, no logits.  The draft's prefill
+    """Prefill of one 512-token prompt of the configuration's target model (the contraction-bound regime): the prompt's
+    rows packed into passes of up to 2048 on the two-CTA GEMM, no logits.  The draft's prefill
     runs in the same call and is timed with it; flops counted are the target's weight GEMMs only."""
     env = setup(args, 1, 8)
     torch, ctx, dev, cfg, seqs = (env[k] for k in ("torch", "ctx", "dev", "cfg", "seqs"))

@@ -248,7 +248,8 @@ int sd_best_gamma(double alpha, double c, int gamma_max, double* speedup_out);
  *   [5],[6] first / last CTA finished      [7] 0.            A word is 0 when nothing reported it.
  * kinds_host[i] = SD_STAMP_GEMM / _STEP / _ATTENTION | (step after the GEMM: 0 plain, 1 QKV+rotary, 2 residual,
  * 3 SwiGLU) << 8; *n_out = records of the pass (may exceed cap).  Enabling changes the captured graphs' keys: the
- * first call afterwards captures anew.  A few atomics per CTA: for measurement, off by default. */
+ * first call afterwards captures anew.  Matrix and step in one kernel (passes of few rows) and prompt passes leave no
+ * records.  A few atomics per CTA: for measurement, off by default. */
 /* Sequences routed to different draft models run their draft passes side by side (default, when the context has two or
  * more separate draft models): every group after the first is enqueued on a stream of its own, forked from and joined
  * back to the context's stream, with its own scratch memory from the arena.  on = 0: group after group on the

@@ -183,6 +183,9 @@ cudaError_t launch_mode(const PlainStep& p, cudaStream_t st) {
 
 }  // namespace
 
+// Up to eight rows, each with two accumulators per unit in registers; the largest matrix at most 16 MB, so that L2 holds the model and
+// launches, not bytes, are the bound (the tiny pair: 154 us here, 204 through the plain kernels; larger fp32 models keep those).
+// Rows and scores have to fit in shared memory; head_dim % 16 == 0 for the float4 reads of a quarter of a key.
 bool plain_steps_fit(const sd_model_desc& m, int rows, int max_ctx) {
     const size_t d = m.d_model, dq = (size_t)m.n_heads * m.head_dim, n_qkv = dq + 2 * (size_t)m.n_kv_heads * m.head_dim, F = m.d_ffn, V = m.vocab;
     const size_t largest = std::max(std::max(n_qkv * d, d * dq), std::max(2 * F * d, V * d)) * sizeof(float);
