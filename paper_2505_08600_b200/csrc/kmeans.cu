@@ -16,8 +16,11 @@ namespace sd {
 namespace {
 
 constexpr int KM_MAX_K = 8;
-constexpr int KM_WARPS = 8;
-constexpr int KM_DEPTH = 6;            // points of a warp in flight
+// Points of a warp that its ring holds, warps of a CTA and CTAs of an SM.  Two points at a time at 384 components take 160 registers:
+// one CTA of twelve warps; 512: eight warps; fewer components: two CTAs of eight.
+constexpr __host__ __device__ int km_depth(int km) { return km == 4 ? 8 : 6; }
+constexpr __host__ __device__ int km_warps(int nv, int km) { return km == 4 && nv == 3 ? 12 : 8; }
+constexpr __host__ __device__ int km_per_sm(int nv, int km) { return km == 4 && nv >= 3 ? 1 : 2; }
 
 // Two fp32 values in one 64-bit register and the packed arithmetic of sm_100 on them: each instruction is two
 // independent IEEE operations (same results as the scalar forms), which halves the instructions per loaded byte.
@@ -28,10 +31,10 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; as
 __device__ __forceinline__ float f2_hsum(f32x2 v) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); return a + b; }
 
 template <int NV, int KM>          // KM: compiled cluster bound (4 or 8); with 4 the centroids are kept in registers
-__global__ void __launch_bounds__(32 * KM_WARPS, (KM == 4 && NV <= 3) ? 2 : 1)
+__global__ void __launch_bounds__(32 * km_warps(NV, KM), (KM == 4 && NV <= 2) ? 2 : 1)
 k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* __restrict__ cent, int32_t* __restrict__ labels,
                 float* __restrict__ part_sums, long long* __restrict__ part_counts, double* __restrict__ part_inertia) {
-    constexpr int DIM = 128 * NV;
+    constexpr int DIM = 128 * NV, KM_WARPS = km_warps(NV, KM), KM_DEPTH = km_depth(KM);
     extern __shared__ __align__(16) float km_smem[];
     float* cs = km_smem;                       // [k][DIM] centroids
     float* acc_s = km_smem + KM * DIM;         // [k][DIM] the block's sums
@@ -57,9 +60,7 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
     for (int kk = 0; kk < KM; ++kk)
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[kk][v] = make_ulonglong2(0ull, 0ull);
-    int cnt[KM];                                // points of this warp per cluster (a warp sees n / (8 * blocks) points)
-#pragma unroll
-    for (int kk = 0; kk < KM; ++kk) cnt[kk] = 0;
+    int cnt = 0;                                // lane kk: points of this warp in cluster kk (a warp sees n / (8 * blocks) points)
     double inertia = 0.0;
 
     // Every lane copies its own columns of the next KM_DEPTH - 1 points of its warp into shared memory with
@@ -83,68 +84,114 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
         idx_next += total_warps; src_next += src_step;
         slot_next = slot_next + 1 == KM_DEPTH ? 0 : slot_next + 1;
     };
-    for (int t = 0; t < KM_DEPTH - 1; ++t) stage();
     int slot = 0;
-    for (long long i = i0; i < n; i += total_warps) {
-        stage();
-        asm volatile("cp.async.wait_group %0;" ::"n"(KM_DEPTH - 1) : "memory");    // this point has landed
-        ulonglong2 x[NV];
+    auto ring_at = [&](int sl, int v) { return *reinterpret_cast<const ulonglong2*>(ring + sl * DIM + v * 128); };
+    auto partial = [&](const ulonglong2 (&x)[NV], int kk) {                       // this lane's share of a squared distance
+        f32x2 d2 = 0ull;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) x[v] = *reinterpret_cast<const ulonglong2*>(ring + slot * DIM + v * 128);
-        slot = slot + 1 == KM_DEPTH ? 0 : slot + 1;
-        float dk[KM];                                                             // this lane's share of every squared distance
+        for (int v = 0; v < NV; ++v) {
+            const ulonglong2 c = creg[CREG ? kk : 0][CREG ? v : 0];
+            const f32x2 a = f2_sub(x[v].x, c.x), b = f2_sub(x[v].y, c.y);
+            d2 = f2_fma(a, a, d2); d2 = f2_fma(b, b, d2);
+        }
+        return f2_hsum(d2);
+    };
+    auto count = [&](const ulonglong2 (&x)[NV], int label) {                      // label: uniform
+        cnt += label == lane ? 1 : 0;
 #pragma unroll
         for (int kk = 0; kk < KM; ++kk) {
-            dk[kk] = 0.f;
-            if (kk < k) {                                                         // uniform
-                f32x2 d2 = 0ull;
+            if (kk == label) {
 #pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const ulonglong2 c = CREG ? creg[CREG ? kk : 0][CREG ? v : 0] : *reinterpret_cast<const ulonglong2*>(cs + kk * DIM + (v * 32 + lane) * 4);
-                    const f32x2 a = f2_sub(x[v].x, c.x), b = f2_sub(x[v].y, c.y);
-                    d2 = f2_fma(a, a, d2); d2 = f2_fma(b, b, d2);
-                }
-                dk[kk] = f2_hsum(d2);
+                for (int v = 0; v < NV; ++v) { acc[kk][v].x = f2_add(acc[kk][v].x, x[v].x); acc[kk][v].y = f2_add(acc[kk][v].y, x[v].y); }
             }
         }
-        if (KM == 4) {
-            // Four sums over the warp with ten shuffles instead of twenty: halves of the warp trade two of the four
-            // values, quarters one of the two, three more steps finish one value per lane group, and the four totals
-            // are read back from lanes 0, 8, 16 and 24 (every lane ends with the same four numbers).
-            const bool hi16 = lane & 16, hi8 = lane & 8;
-            float a = hi16 ? dk[KM == 4 ? 2 : 0] : dk[0], sa = hi16 ? dk[0] : dk[KM == 4 ? 2 : 0];
-            float b = hi16 ? dk[KM == 4 ? 3 : 0] : dk[KM == 4 ? 1 : 0], sb = hi16 ? dk[KM == 4 ? 1 : 0] : dk[KM == 4 ? 3 : 0];
-            a += __shfl_xor_sync(0xffffffffu, sa, 16);
-            b += __shfl_xor_sync(0xffffffffu, sb, 16);
-            float e = hi8 ? b : a;
-            const float se = hi8 ? a : b;
-            e += __shfl_xor_sync(0xffffffffu, se, 8);
-            e += __shfl_xor_sync(0xffffffffu, e, 4);
+    };
+    if (KM == 4) {
+        // Two points at a time: their eight sums over the warp cost nine shuffles (halves of the warp trade one point for the other,
+        // then clusters), the smallest of four per half four more, and the two chains of latencies run side by side; the distances are
+        // added in the same order as one by one.  2,000,003 x 384, 4 clusters: 636 us one point at a time (16 warps per SM of 128
+        // registers), 579 with two points, twelve warps of 168 registers (at 128 registers they spill: 1,100); 4,000,000 x 128:
+        // 691 and 564; 1,000,000 x 512: 429 and 408.  A ring of ten points is no faster than one of eight.
+        constexpr int AHEAD = KM_DEPTH - 2;
+        for (int t = 0; t < AHEAD; ++t) stage();
+        for (long long i = i0; i < n; i += 2 * total_warps) {
+            stage(); stage();
+            asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD) : "memory");       // these two points have landed
+            const int slot1 = slot + 1 == KM_DEPTH ? 0 : slot + 1;
+            const bool both = i + total_warps < n;                                // uniform
+            float d[2][4];
+            ulonglong2 x0[NV], x1[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) { x0[v] = ring_at(slot, v); x1[v] = ring_at(slot1, v); }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {                                      // (centroids past k are zeros and drop out below)
+                d[0][kk] = partial(x0, KM == 4 ? kk : 0);
+                d[1][kk] = partial(x1, KM == 4 ? kk : 0);
+            }
+            const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
+            float a[4];
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) a[kk] = (hi16 ? d[1][kk] : d[0][kk]) + __shfl_xor_sync(0xffffffffu, hi16 ? d[0][kk] : d[1][kk], 16);
+            float b0 = (hi8 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[2], 8);
+            float b1 = (hi8 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[1] : a[3], 8);
+            float e = (hi4 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, hi4 ? b0 : b1, 4);
             e += __shfl_xor_sync(0xffffffffu, e, 2);
             e += __shfl_xor_sync(0xffffffffu, e, 1);
-            // lane group (bit 4, bit 3) holds cluster 2 * bit4 + bit3
-            dk[0] = __shfl_sync(0xffffffffu, e, 0);
-            if (KM == 4) { dk[KM == 4 ? 1 : 0] = __shfl_sync(0xffffffffu, e, 8); dk[KM == 4 ? 2 : 0] = __shfl_sync(0xffffffffu, e, 16); dk[KM == 4 ? 3 : 0] = __shfl_sync(0xffffffffu, e, 24); }
-        } else {
+            // lane group (bit 4 | bit 3, bit 2) holds point bit 4, cluster 2 * bit 3 + bit 2; the smallest wins, the lowest index on ties
+            int label = (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
+            if (label >= k || !(e == e)) e = INFINITY;
+#pragma unroll
+            for (int o = 4; o <= 8; o <<= 1) {
+                const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
+                const int l2 = __shfl_xor_sync(0xffffffffu, label, o);
+                if (e2 < e || (e2 == e && l2 < label)) { e = e2; label = l2; }
+            }
+            if (!hi16 || both) {
+                inertia += (double)e;                                             // (the lower half sums the first points, the upper half the second ones)
+                if ((lane & 15) == 0) labels[hi16 ? i + total_warps : i] = label;
+            }
+            const int label0 = __shfl_sync(0xffffffffu, label, 0), label1 = __shfl_sync(0xffffffffu, label, 16);
+            count(x0, label0);
+            if (both) count(x1, label1);
+            slot = slot1 + 1 == KM_DEPTH ? 0 : slot1 + 1;
+        }
+        inertia += __shfl_sync(0xffffffffu, inertia, 16);                         // (what lane 0 writes)
+    } else {
+        for (int t = 0; t < KM_DEPTH - 1; ++t) stage();
+        for (long long i = i0; i < n; i += total_warps) {
+            stage();
+            asm volatile("cp.async.wait_group %0;" ::"n"(KM_DEPTH - 1) : "memory");    // this point has landed
+            ulonglong2 x[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) x[v] = ring_at(slot, v);
+            float dk[KM];                                                         // this lane's share of every squared distance
+#pragma unroll
+            for (int kk = 0; kk < KM; ++kk) {
+                dk[kk] = 0.f;
+                if (kk < k) {                                                     // uniform
+                    f32x2 d2 = 0ull;
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(cs + kk * DIM + (v * 32 + lane) * 4);
+                        const f32x2 a = f2_sub(x[v].x, c.x), b = f2_sub(x[v].y, c.y);
+                        d2 = f2_fma(a, a, d2); d2 = f2_fma(b, b, d2);
+                    }
+                    dk[kk] = f2_hsum(d2);
+                }
+            }
 #pragma unroll
             for (int kk = 0; kk < KM; ++kk)
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) dk[kk] += __shfl_xor_sync(0xffffffffu, dk[kk], o);      // every lane ends with the same sums
-        }
-        float best = INFINITY;
-        int label = 0;
+            float best = INFINITY;
+            int label = 0;
 #pragma unroll
-        for (int kk = 0; kk < KM; ++kk)
-            if (kk < k && dk[kk] < best) { best = dk[kk]; label = kk; }            // a later centroid must be strictly closer
-        if (lane == 0) labels[i] = label;
-        inertia += (double)best;
-#pragma unroll
-        for (int kk = 0; kk < KM; ++kk) {
-            if (kk == label) {                                                    // uniform
-                cnt[kk] += 1;
-#pragma unroll
-                for (int v = 0; v < NV; ++v) { acc[kk][v].x = f2_add(acc[kk][v].x, x[v].x); acc[kk][v].y = f2_add(acc[kk][v].y, x[v].y); }
-            }
+            for (int kk = 0; kk < KM; ++kk)
+                if (kk < k && dk[kk] < best) { best = dk[kk]; label = kk; }        // a later centroid must be strictly closer
+            if (lane == 0) labels[i] = label;
+            inertia += (double)best;
+            count(x, label);
+            slot = slot + 1 == KM_DEPTH ? 0 : slot + 1;
         }
     }
 
@@ -161,7 +208,7 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
                         s.x = f2_add(s.x, acc[kk][v].x); s.y = f2_add(s.y, acc[kk][v].y);
                         *dst = s;
                     }
-                    if (lane == 0) cnt_s[kk] = (w == 0 ? 0 : cnt_s[kk]) + (long long)cnt[kk];
+                    if (lane == kk) cnt_s[kk] = (w == 0 ? 0 : cnt_s[kk]) + (long long)cnt;
                 }
             }
             if (lane == 0) inertia_s = (w == 0 ? 0.0 : inertia_s) + inertia;
@@ -238,18 +285,18 @@ extern "C" sd_status sd_kmeans_step(const float* points, int64_t n, int dim, con
     if (((uintptr_t)points & 15) || ((uintptr_t)centroids & 15)) return SD_ERR_INVALID_ARG;
     if (!workspace || workspace_bytes < sd_kmeans_workspace(dim, k)) return SD_ERR_CAPACITY;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int blocks = km_blocks();
+    const int km = k <= 4 ? 4 : KM_MAX_K;
+    const int blocks = km_blocks() / (2 / km_per_sm(dim / 128, km));
     char* w = (char*)workspace;
     float* part_sums = (float*)w;              w += km_align((size_t)blocks * k * dim * sizeof(float));
     long long* part_counts = (long long*)w;    w += km_align((size_t)blocks * k * sizeof(long long));
     double* part_inertia = (double*)w;
-    const int km = k <= 4 ? 4 : KM_MAX_K;
-    const size_t smem = ((size_t)2 * km + (size_t)KM_WARPS * KM_DEPTH) * dim * sizeof(float);
+    const size_t smem = ((size_t)2 * km + (size_t)km_warps(dim / 128, km) * km_depth(km)) * dim * sizeof(float);
     cudaError_t e = cudaSuccess;
 #define KM_LAUNCH(NV, KM)                                                                                                        \
     do {                                                                                                                     \
         e = cudaFuncSetAttribute(k_kmeans_assign<NV, KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);           \
-        if (e == cudaSuccess) k_kmeans_assign<NV, KM><<<blocks, 32 * KM_WARPS, smem, st>>>(points, n, k, centroids, labels, part_sums, part_counts, part_inertia); \
+        if (e == cudaSuccess) k_kmeans_assign<NV, KM><<<blocks, 32 * km_warps(NV, KM), smem, st>>>(points, n, k, centroids, labels, part_sums, part_counts, part_inertia); \
     } while (0)
     switch (dim / 128) {
     case 1: if (km == 4) KM_LAUNCH(1, 4); else KM_LAUNCH(1, 8); break;
