@@ -382,9 +382,9 @@ k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUte
     }
 }
 
-// A row is spread over d / 16 threads of one CTA, four float4 each.
+// A row is spread over whole warps of one CTA, four float4 per thread: the last warp may hold as few as eight columns.
 constexpr int NORM_VECS = 4;
-int norm_threads(int d) { return (d / (4 * NORM_VECS) + 31) / 32 * 32; }
+int norm_threads(int d) { return (d + 4 * NORM_VECS * 32 - 1) / (4 * NORM_VECS * 32) * 32; }
 
 // xn = bf16(v * gain) and 1/rms(v) for a row held in registers.
 __device__ __forceinline__ void norm_row(const float4 (&v)[NORM_VECS], int d, const float* __restrict__ gain, float eps, bf16* __restrict__ xn,

@@ -17,11 +17,15 @@ def _m(L, d, H, Hkv, hd, F, V):
     return dict(n_layers=L, d_model=d, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=F, vocab=V)
 
 
-# matrices that do not fill a 256-feature tile, grouped heads of 64, heads of 128, one layer (keys and values only)
+# matrices that do not fill a 256-feature tile, grouped heads of 64, heads of 128, one layer (keys and values only); widths of
+# eight columns, and of eight columns beyond a multiple of the 512 that a warp of the row kernels covers
 MODELS = {
     "gqa64": _m(3, 320, 6, 2, 64, 448, 512),
     "mha128": _m(2, 384, 3, 3, 128, 1024, 512),
     "one_layer": _m(1, 128, 2, 1, 64, 192, 512),
+    "d8": _m(2, 8, 1, 1, 64, 64, 512),
+    "d520": _m(2, 520, 8, 8, 64, 576, 512),
+    "d1032": _m(2, 1032, 4, 2, 128, 576, 512),
 }
 # prompt lengths (rows = length - 1): around attention blocks of 64 and around 256, remainders of 3...16 rows (two-part
 # activations), fewer rows than a pass takes, more rows than a pass takes
@@ -34,7 +38,7 @@ PROMPTS = {
 }
 
 
-@pytest.mark.parametrize("model,prompts", [("gqa64", k) for k in PROMPTS] + [("mha128", "block_edges"), ("mha128", "two_part_rests"), ("one_layer", "row_256_edges")])
+@pytest.mark.parametrize("model,prompts", [("gqa64", k) for k in PROMPTS] + [("mha128", "block_edges"), ("mha128", "two_part_rests"), ("one_layer", "row_256_edges"), ("d8", "fewest"), ("d520", "block_edges"), ("d1032", "fewest")])
 def test_prefill_leaves_the_oracles_caches(model, prompts):
     from paper_2505_08600_b200 import binding
     dims, lens = MODELS[model], PROMPTS[prompts]
