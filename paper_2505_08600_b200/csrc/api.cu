@@ -681,9 +681,12 @@ bool few_rows_pass(sd_ctx* c, const Model& M, int n_rows) {
 // these kernels an iteration takes 1.100 ms instead of 1.142; with gate/up (67 MB) as well 1.31, with the lm_head (131 MB) 1.19:
 // a CTA that holds its whole share in registers cannot keep HBM busy across CTAs.
 constexpr size_t GEMV_LARGEST = (size_t)16 << 20;
-bool few_rows_matrix(const Model& M, int n_rows, int mode, int n_out, int K) {
+// A residual step on them leaves a piece of the rows' sums of squares per 16 features to a step kernel, which has to be able to add
+// them all: 128, or 64 with 9...16 rows in one part.
+bool few_rows_matrix(const Model& M, int n_rows, int lo, int mode, int n_out, int K) {
+    const int parts = lo || n_rows <= 8 ? SSQ_MAX_PARTS : SSQ_STRIDE;
     return n_rows <= GEMV_MAX_ROWS && !M.lora && (size_t)n_out * K * sizeof(bf16) <= GEMV_LARGEST && gemv_fits(M, n_rows, mode, n_out, K) &&
-           (mode != EPI_RESIDUAL || n_out <= 16 * SSQ_MAX_PARTS);
+           (mode != EPI_RESIDUAL || n_out <= 16 * parts);
 }
 
 // One matrix and the step that follows it, on those kernels.
@@ -737,7 +740,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     for (int i = 0; i < list.n && i < SD_MAX_BATCH; ++i) len_hint[i] = c->len_ub[list.ids[i]];
     RowScale scale{c->ssq, 1, 1.f / d, m.rms_eps, SSQ_STRIDE};              // sum of squares in one piece (after the embedding),
     auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e) {
-        const bool gv = few || few_rows_matrix(M, n_rows, e.mode, n_out, K);
+        const bool gv = few || few_rows_matrix(M, n_rows, lo, e.mode, n_out, K);
         if (e.mode == EPI_RESIDUAL) {                                       // ... then in one piece per tile of the kernel that wrote h
             scale.n_parts = gv ? d / 16 : (d + 127) / 128;
             scale.stride = gv ? GEMV_SSQ_STRIDE : SSQ_STRIDE;

@@ -28,6 +28,11 @@ struct StepShared {
     float lora_t[MB][32];           // x A^T of the CTA's token rows for their own adapters
 };
 
+// Whether the form with mb token rows per CTA (hl: rows in two bf16 parts) adds up more than 64 pieces of a row's sum of squares.
+// The sixteen-row forms in one part, which serve passes of hundreds of rows as well, do not: the registers of two more loads per
+// row would cost them resident CTAs, and whoever feeds them keeps to 64 pieces.
+__host__ __device__ constexpr bool wide_ssq(int mb, bool hl) { return mb <= 8 || hl; }
+
 // MB token rows x CB pieces are in flight together: (8, 8) for the verify rows, (2, 32) for one or
 // two rows (draft steps), where a tile of a small matrix is cut into many pieces, (16, 4) or (16, 2)
 // for many rows on few pieces.  MODE < 0: the step is read from ep.mode; with many row batches one
@@ -147,8 +152,8 @@ __global__ void __launch_bounds__(128) k_fused_step(GemmGeom g, Epilogue ep, con
             }
         }
     }
-    // (more than 64 pieces: the rows were written by the few-rows kernels, in passes of at most 16 rows)
-    constexpr bool WIDE = MB <= 8 || HL;
+    // (more than 64 pieces: the rows were written by the few-rows kernels; the forms for many rows in one part never see them)
+    constexpr bool WIDE = wide_ssq(MB, HL);
     float ssa[(MB + 3) / 4], ssb[(MB + 3) / 4], ssc[WIDE ? (MB + 3) / 4 : 1], ssd[WIDE ? (MB + 3) / 4 : 1];
     if (ep.rs.ssq) {                              // one warp per token row, one lane per piece of its sum of squares
 #pragma unroll
@@ -424,15 +429,16 @@ cudaError_t launch_fused_step(const GemmGeom& g, const Epilogue& ep, const float
     if (ep.mode == EPI_QKV_ROPE && (128 % ep.hd)) return cudaErrorInvalidValue;            // a head must not straddle two tiles
     if (ep.mode == EPI_RESIDUAL && g.n_tiles > SSQ_STRIDE) return cudaErrorInvalidValue;
     if (ep.mode == EPI_SWIGLU && (ep.F % 64)) return cudaErrorInvalidValue;
-    if (ep.rs.ssq && (ep.rs.n_parts > (g.m_tok <= 32 ? SSQ_MAX_PARTS : 64) || ep.rs.stride < ep.rs.n_parts)) return cudaErrorInvalidValue;
+    const int n_rows = ep.mode == EPI_PLAIN ? ep.n_out_rows : (ep.lo_off ? ep.m_real : g.m_tok);
+    const int pieces = pieces_bound(g);
+    if (ep.rs.ssq && (ep.rs.n_parts > (wide_ssq(rows_per_cta(n_rows, pieces), ep.lo_off > 0) ? SSQ_MAX_PARTS : 64) || ep.rs.stride < ep.rs.n_parts))
+        return cudaErrorInvalidValue;
     if (ep.lora_b) {                                   // the adapter's tile is complete only when the GEMM's grid is
         if (ep.lora_r < 8 || ep.lora_r > 32 || (ep.lora_r & 7) || ep.lora_n * ep.lora_r > TILE_N || !ep.lora_task ||
             ep.mode == EPI_PLAIN || g.n_out % TILE_N || g.n_tiles != g.n_out / TILE_N + 1)
             return cudaErrorInvalidValue;
         arrive = nullptr;
     }
-    const int n_rows = ep.mode == EPI_PLAIN ? ep.n_out_rows : (ep.lo_off ? ep.m_real : g.m_tok);
-    const int pieces = pieces_bound(g);
     if (ep.lo_off) {                                   // two-part activations: accumulator rows r and r + lo_off belong together
         // (the GEMM's epilogue has already added the two columns of a row: the pieces hold m_real merged rows)
         if (ep.m_real < 1 || ep.m_real > ep.lo_off || ep.m_real + ep.lo_off != g.m_tok || g.lo_off != ep.lo_off || g.m_real != ep.m_real) return cudaErrorInvalidValue;

@@ -40,7 +40,7 @@ struct RowScale {
     int stride;
 };
 constexpr int SSQ_STRIDE = 64;
-constexpr int SSQ_MAX_PARTS = 128;      // most pieces that launch_fused_step adds up (64 in passes of more than 16 rows)
+constexpr int SSQ_MAX_PARTS = 128;      // most pieces that launch_fused_step adds up (SSQ_STRIDE with more than 8 rows in one part)
 
 // What happens to a 128-row output tile once its pieces are summed (the step that follows the
 // GEMM in the decoder layer), so that no fp32 intermediate matrix goes through memory.

@@ -50,3 +50,32 @@ def test_draft_passes_follow_the_oracle(name, n_seq):
         top = logits.max(axis=1, keepdims=True)
         want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
         assert np.abs(np.log(qg[s]) - want).max() <= LOG_TOL, s
+
+
+@pytest.mark.parametrize("two_part", [0, 1])
+@pytest.mark.parametrize("n_seq,gamma", [(1, 7), (1, 8), (1, 15), (3, 3)])     # 8, 9, 16 and 12 rows
+@pytest.mark.parametrize("d", [1024, 1152, 2048])                              # Wo leaves 64, 72 and 128 pieces of a row's sum of squares
+def test_mixed_passes_add_all_pieces_of_the_sum_of_squares(d, n_seq, gamma, two_part):
+    """A target whose Wo takes the few-rows kernel while gate/up and the lm_head stream, with the rows in one and in two bf16 parts."""
+    from paper_2505_08600_b200 import binding
+    target, draft = _m(1, d, 4, 64, 4608, 4096), _m(1, 64, 1, 64, 64, 4096)
+    wt, wd = synth.make_weights(target, seed=3, model_index=0, dtype="bf16"), synth.make_weights(draft, seed=3, model_index=1, dtype="bf16")
+    ctx = binding.Context(target, [draft], "bf16", n_seq, 96, gamma, 1.0, 7)
+    ctx.load_weights(0, wt); ctx.load_weights(1, wd)
+    ctx.sd_use_two_part_activations(two_part)
+    toks = [synth.make_prompt(4096, 20 + 9 * i, seed=9, seq=i) for i in range(n_seq)]
+    seqs = list(range(n_seq))
+    for s in seqs:
+        ctx.sd_seq_begin(s, toks[s], s)
+    ctx.sd_route_prompt(seqs, forced_task=[0] * n_seq)
+    ctx.sd_prefill(seqs)
+    x = np.stack([synth.make_prompt(4096, gamma, seed=5, seq=s) for s in seqs])
+    logits = torch.zeros((n_seq, gamma + 1, 4096), dtype=torch.float32, device=DEV)
+    ctx.sd_verify(seqs, gamma, torch.from_numpy(x).to(DEV), logits)
+    got = logits.cpu().numpy().astype(np.float64)
+    assert ctx.sd_device_status() == 0
+    ctx.close()
+    om = oracle.OracleModel(target, wt)
+    for s in seqs:
+        want = om.new_cache(128).forward(np.concatenate([toks[s], x[s]]), 0)[-(gamma + 1):]
+        assert np.abs(got[s] - want).max() <= 5e-2, s          # bf16 against the fp64 oracle, as for the verify rows elsewhere
