@@ -622,8 +622,8 @@ unsigned long long* next_stamp(sd_ctx* c, int kind) {
     return c->stamp_buf + (size_t)ST_WORDS * (c->stamp_kinds.size() - 1);
 }
 
-// One weight GEMM and the step that follows it.
-sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n_out, int K, const Epilogue& ep) {
+// One weight GEMM and the step that follows it.  dependent = 0: launched in full stream order (see forward_tc).
+sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n_out, int K, const Epilogue& ep, int dependent) {
     if (ep.lo_off) rows += ep.lo_off;           // the input rows come in two bf16 parts: [x_hi rows][x_lo rows at + lo_off]
     GemmGeom g = gemm_geometry(rows, n_out, K, sm_count(), ep.ring_stages, ep.prefill_all != 0, ep.lora_b ? 1 : 0);
     if (ep.lo_off) { g.lo_off = ep.lo_off; g.m_real = ep.m_real; }
@@ -656,7 +656,7 @@ sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n
         arrive = c->gemm_arrive + c->arrive_used;
         c->arrive_used += (size_t)g.n_tiles;
     }
-    LAUNCH(CAT_LINEAR, launch_gemm_streamk(tw, tx, g, c->partials, arrive, c->S.status, 1, c->st));
+    LAUNCH(CAT_LINEAR, launch_gemm_streamk(tw, tx, g, c->partials, arrive, c->S.status, dependent, c->st));
     LAUNCH(CAT_FUSED_STEP, launch_fused_step(g, eps, c->partials, arrive, c->S.status, 1, c->st));
     return SD_OK;
 }
@@ -690,7 +690,7 @@ bool few_rows_matrix(const Model& M, int n_rows, int lo, int mode, int n_out, in
 }
 
 // One matrix and the step that follows it, on those kernels.
-sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out, int K, const Epilogue& ep) {
+sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out, int K, const Epilogue& ep, int dependent) {
     Gemv g;
     memset(&g, 0, sizeof(g));
     g.w = (const bf16*)w; g.x = (const bf16*)x; g.rows = rows; g.n_out = n_out; g.K = K; g.ep = ep;
@@ -699,11 +699,12 @@ sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out
         memset(&t.ep, 0, sizeof(t.ep));
         t.ep.mode = EPI_PLAIN; t.ep.lo_off = ep.lo_off; t.ep.m_real = rows; t.ep.y = c->lora_t; t.ep.n_out_rows = rows; t.ep.row_stride = 1;
         t.w = g.w + (size_t)n_out * K; t.n_out = 128;
-        LAUNCH(CAT_LINEAR, launch_gemv(t, c->st));
+        LAUNCH(CAT_LINEAR, launch_gemv(t, dependent, c->st));
+        dependent = 1;
         g.lora_t = c->lora_t;
     }
     c->x_from.words = nullptr;                  // (no tile-by-tile hand-off from this kernel)
-    LAUNCH(CAT_LINEAR, launch_gemv(g, c->st));
+    LAUNCH(CAT_LINEAR, launch_gemv(g, dependent, c->st));
     return SD_OK;
 }
 
@@ -738,6 +739,12 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     };
     int len_hint[SD_MAX_BATCH];                                             // context bounds of the pass's sequences, for attention's launch order
     for (int i = 0; i < list.n && i < SD_MAX_BATCH; ++i) len_hint[i] = c->len_ub[list.ids[i]];
+    // The pass's first matrix kernel is launched in full stream order: it begins when the embedding kernel's stores are visible.
+    // Every later kernel of the pass begins after it did, which is why they may read the row plan (slots, positions, rotary
+    // factors, adapters) before they wait for the kernel before them; as the embedding kernel's programmatic dependent it could
+    // not, since that kernel's stores are promised to a dependent only behind its wait.  (The embedding kernel lets nothing start early, so this
+    // costs no overlap.)
+    int dependent = 0;
     RowScale scale{c->ssq, 1, 1.f / d, m.rms_eps, SSQ_STRIDE};              // sum of squares in one piece (after the embedding),
     auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e) {
         const bool gv = few || few_rows_matrix(M, n_rows, lo, e.mode, n_out, K);
@@ -745,7 +752,9 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
             scale.n_parts = gv ? d / 16 : (d + 127) / 128;
             scale.stride = gv ? GEMV_SSQ_STRIDE : SSQ_STRIDE;
         }
-        return gv ? gemv_step(c, w, x, n_rows, n_out, K, e) : gemm_tc(c, tm, x, n_rows, n_out, K, e);
+        const int dep = dependent;
+        dependent = 1;
+        return gv ? gemv_step(c, w, x, n_rows, n_out, K, e, dep) : gemm_tc(c, tm, x, n_rows, n_out, K, e, dep);
     };
     LAUNCH(CAT_ELEMENTWISE, launch_embed(c->S, list, plan, n_rows, M.embed, dt, d, m.vocab, c->h, c->row_slot, c->row_pos,
                                          M.layers[0].norm1, c->xn, c->ssq, M.rope_cos, M.rope_sin, hd / 2, c->rope_row_cos, c->rope_row_sin, 0, nullptr, st, lo));

@@ -97,9 +97,9 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(sm_raw);
     __shared__ int last_sm;
 
-    // The row plan (positions, slots) was written by the pass's first kernel, an ordinary launch that every later
-    // kernel of the pass started after: it may be read before the wait below, and so may the cache positions in
-    // front of the pass's first new one, which earlier passes wrote.
+    // The row plan (positions, slots) was written by the pass's first kernel, whose stores the second one, launched in full
+    // stream order, began behind; every later kernel of the pass began after that one: the plan may be read before the wait
+    // below, and so may the cache positions in front of the pass's first new one, which earlier passes wrote.
     // longest context among the block's rows (every warp works it out for itself), and the sequence slot
     int mp = lane < nr ? __ldcg(P.row_pos + r0 + lane) : -1;
     const int slot = __ldcg(P.row_slot + r0);

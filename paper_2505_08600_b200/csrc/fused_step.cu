@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(128) k_fused_step(GemmGeom g, Epilogue ep, con
         rows[i] = r < n_rows ? (mode == EPI_PLAIN ? r * ep.row_stride + ep.row_offset : r) : -1;
     }
     const float gain = (mode == EPI_RESIDUAL && ep.gain_next && live) ? ep.gain_next[n] : 0.f;   // a weight: needs no wait
-    // The row plan and the rows' rotary factors were written by the pass's first kernel, an ordinary launch that every
-    // later kernel of the pass started after: they need no wait either.
+    // The row plan and the rows' rotary factors were written by the pass's first kernel, whose stores the second one, launched
+    // in full stream order, began behind; every later kernel of the pass began after that one: they need no wait either.
     float cs[MB], sn[MB];
     int pos[MB], slot[MB];
     if (mode == EPI_QKV_ROPE) {

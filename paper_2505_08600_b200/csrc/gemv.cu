@@ -61,8 +61,8 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
             a1[b] = kb < KB && r1 < g.n_out ? ldg_stream(w1 + 32 * kb) : make_uint4(0, 0, 0, 0);
         }
     }
-    // what the finishing threads need besides: their unit's features, gains, the rows' plan and rotary factors (written by
-    // the pass's first kernel, an ordinary launch that every later kernel of the pass started after)
+    // what the finishing threads need besides: their unit's features, gains, the rows' plan and rotary factors (written by the
+    // pass's first kernel; the second one is launched in full stream order after it, every later one begins after that)
     const int ui = tid & 7, um = tid >> 3;                              // unit and token row this thread finishes
     const bool mine = um < g.rows && tid < 8 * M;
     const int f0 = first_row(ui), f1 = f0 + apart;
@@ -237,11 +237,11 @@ bool gemv_supported(const Gemv& g) {
     }
 }
 
-cudaError_t launch_gemv(const Gemv& g, cudaStream_t st) {
+cudaError_t launch_gemv(const Gemv& g, int dependent, cudaStream_t st) {
     if (!gemv_supported(g) || g.ep.lo_off < 0 || (g.ep.lo_off && g.ep.lo_off < g.rows)) return cudaErrorInvalidValue;
     if (g.ep.lora_b && (g.ep.lora_r < 8 || g.ep.lora_r > 32 || (g.ep.lora_r & 7) || g.ep.lora_n * g.ep.lora_r > 128 || !g.lora_t)) return cudaErrorInvalidValue;
     const Form* f = form_of(g.K);
-    return launch_pdl(g.rows <= 8 ? f->one : f->two, dim3((g.n_out + 15) / 16), dim3(32 * f->warps), 0, st, 1, g);
+    return launch_pdl(g.rows <= 8 ? f->one : f->two, dim3((g.n_out + 15) / 16), dim3(32 * f->warps), 0, st, dependent, g);
 }
 
 }  // namespace sd

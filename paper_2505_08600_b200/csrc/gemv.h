@@ -15,6 +15,7 @@ struct Gemv {
     Epilogue ep;                        // as for launch_fused_step; rs.n_parts counts this kernel's 16-feature tiles where it wrote them
 };
 bool gemv_supported(const Gemv& g);
-cudaError_t launch_gemv(const Gemv& g, cudaStream_t st);
+// dependent = 0 for the kernel that follows the one that wrote the row plan (which is read ahead of the wait).
+cudaError_t launch_gemv(const Gemv& g, int dependent, cudaStream_t st);
 
 }  // namespace sd

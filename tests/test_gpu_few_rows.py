@@ -79,3 +79,31 @@ def test_mixed_passes_add_all_pieces_of_the_sum_of_squares(d, n_seq, gamma, two_
     for s in seqs:
         want = om.new_cache(128).forward(np.concatenate([toks[s], x[s]]), 0)[-(gamma + 1):]
         assert np.abs(got[s] - want).max() <= 5e-2, s          # bf16 against the fp64 oracle, as for the verify rows elsewhere
+
+
+def test_passes_use_their_own_row_plan():
+    """Draft passes of sequences with other slots and positions in turn, each first matrix kernel right behind the kernel that writes
+    the row plan: what a call returns does not depend on the call before it."""
+    from paper_2505_08600_b200 import binding
+    draft, target, gamma = DRAFTS["d288"], _m(1, 64, 1, 64, 64, 509), 3
+    ctx = binding.Context(target, [draft], "bf16", 3, 160, gamma, 1.0, 7)
+    ctx.load_weights(0, synth.make_weights(target, seed=3, model_index=0, dtype="bf16"))
+    ctx.load_weights(1, synth.make_weights(draft, seed=3, model_index=1, dtype="bf16"))
+    for s, m in enumerate((9, 70, 150)):
+        ctx.sd_seq_begin(s, synth.make_prompt(509, m, seed=9, seq=s), s)
+    ctx.sd_route_prompt([0, 1, 2], forced_task=[0, 0, 0])
+    ctx.sd_prefill([0, 1, 2])
+    calls, first = [[0], [1], [2], [2, 0], [1, 2, 0]], {}
+    x, q = torch.zeros((3, gamma), dtype=torch.int32, device=DEV), torch.zeros((3, gamma, 509), dtype=torch.float32, device=DEV)
+    for graphs in (1, 0):
+        ctx.sd_use_graphs(graphs)
+        for i in range(40):
+            seqs = calls[i * 3 % len(calls)]
+            n = len(seqs)
+            ctx.sd_draft_steps(seqs, gamma, x[:n], q[:n])
+            for j, s in enumerate(seqs):
+                got = (x[j].cpu().numpy(), q[j].cpu().numpy())
+                want = first.setdefault((s, n), got)               # (with another number of rows other forms may be taken)
+                assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1]), (i, seqs, s)
+    assert ctx.sd_device_status() == 0
+    ctx.close()
