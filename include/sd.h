@@ -464,8 +464,8 @@ size_t sd_op_attention_workspace(int rows, int n_heads, int head_dim, int max_ct
  * sd_mamba_classify scores n_prompts prompts in one go: prompt i is tokens_dev[starts_host[i] .. + lens_host[i]) (device
  * tokens, host offsets and lengths >= 1; token ids are clamped to the vocabulary); scores_dev [n_prompts][n_classes]
  * fp32 and labels_dev [n_prompts] int32 (argmax, lowest index on ties) are device buffers, either may be NULL.
- * workspace_dev: sd_mamba_workspace(desc, sum of lengths, n_prompts) bytes of device memory.  Long prompts are scanned
- * in chunks side by side.  Limits: d_state <= 16, d_conv <= 8, d_model <= 512, Di <= 1024 (else SD_ERR_UNSUPPORTED).
+ * workspace_dev: sd_mamba_workspace(desc, sum of lengths, n_prompts) bytes of device memory at a multiple of 8 bytes
+ * (at a multiple of 16 it is written by fours).  Long prompts are scanned in chunks side by side.  Limits: d_state <= 16, d_conv <= 8, d_model <= 512, Di <= 1024 (else SD_ERR_UNSUPPORTED).
  * Copies small host tables to the device and synchronises the stream once before launching; the launches are
  * asynchronous on cuda_stream. */
 typedef struct { int32_t vocab, d_model, d_state, d_conv, expand, n_classes, dt_rank; } sd_mamba_desc;

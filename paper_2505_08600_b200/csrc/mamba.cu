@@ -68,6 +68,7 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
         b_src[i] = j < 2 * m.Di ? w_in + (size_t)j * m.D : nullptr;
     }
     const bool vec = (m.D & 3) == 0 && (((uintptr_t)embed | (uintptr_t)w_in) & 15) == 0;
+    const bool vec_out = (m.Di & 3) == 0 && (((uintptr_t)u | (uintptr_t)z) & 15) == 0;      // (the workspace may begin at any multiple of 8)
     auto get = [&](const float* src, int k) {
         if (!src) return make_float4(0.f, 0.f, 0.f, 0.f);
         if (vec) return k < m.D ? __ldg(reinterpret_cast<const float4*>(src + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -121,7 +122,7 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
             const int j = j0 + 64 * h + 4 * tx;
             const float2 p = f2_unpack(acc[i][2 * h]), q = f2_unpack(acc[i][2 * h + 1]);
             const float v[4] = {p.x, p.y, q.x, q.y};
-            if ((m.Di & 3) == 0) {                                      // (then a group of four lies in one of the halves)
+            if (vec_out) {                                              // (a group of four lies in one of the halves)
                 if (j < 2 * m.Di) *reinterpret_cast<float4*>((j < m.Di ? u + (size_t)r * m.Di + j : z + (size_t)r * m.Di + j - m.Di)) = make_float4(v[0], v[1], v[2], v[3]);
             } else {
 #pragma unroll

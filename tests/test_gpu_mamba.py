@@ -88,3 +88,20 @@ def test_routing_through_the_context_and_unsupported_sizes(sd):
     big = synth.make_mamba_classifier(100, d_model=64, d_state=32, d_conv=4, expand=2, n_classes=2, seed=1)      # 32 states: not supported
     with pytest.raises(RuntimeError):
         sd.MambaClassifier(big).classify(torch.zeros(8, dtype=torch.int32, device=DEV), [0], [8])
+
+
+def test_workspace_at_a_multiple_of_eight_bytes(sd):
+    """The workspace needs the alignment of its 64-bit words and no more: the same scores, bit for bit, from one eight bytes further on."""
+    import ctypes
+    vocab, lens = 500, np.array([70, 9, 300], dtype=np.int32)
+    clf = sd.MambaClassifier(synth.make_mamba_classifier(vocab, d_model=64, d_state=16, d_conv=4, expand=2, n_classes=4, seed=5))
+    tokens = torch.from_numpy(np.concatenate([synth.make_prompt(vocab, int(n), seed=6, seq=i) for i, n in enumerate(lens)])).to(DEV)
+    starts = np.array([0, 70, 79], dtype=np.int64)
+    want, _ = clf.classify(tokens, starts, lens)
+    need = sd.lib().sd_mamba_workspace(ctypes.byref(clf.desc), int(lens.sum()), 3)
+    buf, scores = torch.empty(need + 16, dtype=torch.uint8, device=DEV), torch.zeros((3, 4), dtype=torch.float32, device=DEV)
+    assert buf.data_ptr() % 16 == 0
+    status = sd.lib().sd_mamba_classify(ctypes.byref(clf.desc), ctypes.byref(clf.w), tokens.data_ptr(), starts.ctypes.data_as(ctypes.c_void_p),
+                                        lens.ctypes.data_as(ctypes.c_void_p), 3, scores.data_ptr(), None, buf.data_ptr() + 8, need, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert status == 0 and torch.equal(scores, want)
