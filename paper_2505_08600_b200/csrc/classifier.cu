@@ -7,6 +7,7 @@
 namespace sd {
 
 constexpr int CLF_CTAS = 8, CLF_WARPS = 16;
+constexpr int CLF_PART_BYTES = CLF_WARPS * 256 * 4, CLF_MAX_SMEM = 227 * 1024 - CLF_PART_BYTES;      // static, and the dynamic shared memory left
 
 // Eight consecutive columns of an embedding row, added to acc.
 __device__ __forceinline__ void add_cols(const bf16* p, float (&acc)[8]) {
@@ -103,8 +104,10 @@ cudaError_t launch_classifier(const SeqState& S, const SeqList& list, const SeqL
                               int n_classes, cudaStream_t st) {
     if (list.n <= 0) return cudaSuccess;
     size_t smem = sizeof(float) * (size_t)(d + d_hidden + n_classes);
-    const cudaError_t err = dtype == SD_BF16 ? cudaFuncSetAttribute(k_classifier<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                                             : cudaFuncSetAttribute(k_classifier<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > (size_t)CLF_MAX_SMEM) return cudaErrorInvalidValue;
+    // (always the largest, not this call's: another context's call on another thread must not lower it before the launch)
+    const cudaError_t err = dtype == SD_BF16 ? cudaFuncSetAttribute(k_classifier<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, CLF_MAX_SMEM)
+                                             : cudaFuncSetAttribute(k_classifier<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CLF_MAX_SMEM);
     if (err != cudaSuccess) return err;
     if (dtype == SD_BF16) k_classifier<bf16><<<list.n * CLF_CTAS, 32 * CLF_WARPS, smem, st>>>(S, list, forced, (const bf16*)embed, d, vocab, w1, b1, d_hidden, w2, b2, n_classes);
     else k_classifier<float><<<list.n * CLF_CTAS, 32 * CLF_WARPS, smem, st>>>(S, list, forced, (const float*)embed, d, vocab, w1, b1, d_hidden, w2, b2, n_classes);
