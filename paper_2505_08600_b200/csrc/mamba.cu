@@ -23,6 +23,7 @@ namespace {
 constexpr int MB_CHUNK = 64;         // tokens per chunk of the scan
 constexpr int MB_MAX_N = 16;         // state size kept in registers
 constexpr int MB_MAX_CONV = 8;
+constexpr int MB_MAX_DI = 1024, MB_MAX_D = 512, MB_MAX_X = 256, MB_MAX_K = 64;      // largest d_inner, d_model, r + B + C, classes
 
 struct MambaDims { int V, D, Di, N, R, Kc, K; };
 
@@ -141,7 +142,11 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
 //      two tokens and every 16th output, three at a time;
 //   2. a thread per channel scans the chunk: convolution again (four multiply-adds are less than a trip through memory), step
 //      size, recurrence from a zero state, and the two sums of the chunk (see the top of the file).
-constexpr int MC_TILE = 32, MC_THREADS = 256;
+constexpr int MC_TILE = 32, MC_THREADS = 256, MC_STAGED = 48 * 1024;      // W_x is staged up to this size: two CTAs of the usual sizes still fit an SM
+// Most dynamic shared memory a launch takes: B, C, r of a chunk and a tile of v at their largest (W_x is beyond its limit then; where
+// it is staged, n_x Di <= MC_STAGED / 4 and the rest is smaller by more than MC_STAGED).
+constexpr int MC_MAX_SMEM = (MB_CHUNK * MB_MAX_X + MC_TILE * (MB_MAX_DI + 4)) * 4;
+constexpr int MH_MAX_SMEM = (MB_MAX_DI * MB_MAX_N + MB_MAX_DI + MB_MAX_D + MB_MAX_K) * 4;
 template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to MB_MAX_CONV as 0*/>
 __global__ void __launch_bounds__(MC_THREADS, 2)
 k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* __restrict__ tok_row, const float* __restrict__ u, const float* __restrict__ z,
@@ -404,7 +409,7 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     if (!dims_ok(desc, m) || !w || !tokens_dev || !starts_host || !lens_host || n_prompts < 0 || (!scores_dev && !labels_dev)) return SD_ERR_INVALID_ARG;
     if (!w->embed || !w->w_in || !w->w_conv || !w->b_conv || !w->w_x || !w->w_dt || !w->b_dt || !w->a_log || !w->d_skip || !w->w_out || !w->w_fc || !w->b_fc)
         return SD_ERR_INVALID_ARG;
-    if (m.N > MB_MAX_N || m.Kc > MB_MAX_CONV || m.Di > 1024 || m.D > 512 || m.R + 2 * m.N > 256 || m.K > 64) return SD_ERR_UNSUPPORTED;
+    if (m.N > MB_MAX_N || m.Kc > MB_MAX_CONV || m.Di > MB_MAX_DI || m.D > MB_MAX_D || m.R + 2 * m.N > MB_MAX_X || m.K > MB_MAX_K) return SD_ERR_UNSUPPORTED;
     if (n_prompts == 0) return SD_OK;
     int64_t T = 0;
     for (int i = 0; i < n_prompts; ++i) {
@@ -449,12 +454,14 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     k_mamba_in<<<dim3((unsigned)((rows + MI_TILE - 1) / MI_TILE), (unsigned)((2 * m.Di + MI_TILE - 1) / MI_TILE)), 256, 0, st>>>(
         m, by_token ? nullptr : tok_id, rows, w->embed, w->w_in, u, z);
     const size_t xp = (size_t)((m.R + 2 * m.N + 3) & ~3), wx_bytes = (size_t)(m.R + 2 * m.N) * m.Di * 4;
-    const int w_staged = wx_bytes <= 48 * 1024;                              // two CTAs of the usual sizes still fit an SM
+    const int w_staged = wx_bytes <= MC_STAGED;
     const size_t chunk_smem = (MB_CHUNK * xp + (size_t)MC_TILE * (((m.Di + 3) & ~3) + 4)) * 4 + (w_staged ? wx_bytes : 0);
     auto chunk_kernel = m.N != MB_MAX_N ? k_mamba_chunk<0, 0> : m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4> : k_mamba_chunk<MB_MAX_N, 0>;
     const size_t head_smem = ((size_t)m.Di * m.N + m.Di + m.D + m.K) * 4;
-    if (cudaFuncSetAttribute(chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chunk_smem) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mamba_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)head_smem) != cudaSuccess)
+    // Always the bound over all sizes that are accepted: the attribute belongs to the kernel, and a smaller classifier's call on
+    // another thread must not lower it between here and the launch.
+    if (cudaFuncSetAttribute(chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MC_MAX_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mamba_head, cudaFuncAttributeMaxDynamicSharedMemorySize, MH_MAX_SMEM) != cudaSuccess)
         return SD_ERR_CUDA;
     chunk_kernel<<<(unsigned)n_chunks, MC_THREADS, chunk_smem, st>>>(
         m, chunks_d, tok_row, u, z, w->w_conv, w->b_conv, w->w_x, w->w_dt, w->b_dt, w->a_log, w->d_skip, (float*)(base + L.end_state),

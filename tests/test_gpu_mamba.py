@@ -105,3 +105,33 @@ def test_workspace_at_a_multiple_of_eight_bytes(sd):
                                         lens.ctypes.data_as(ctypes.c_void_p), 3, scores.data_ptr(), None, buf.data_ptr() + 8, need, torch.cuda.current_stream().cuda_stream)
     torch.cuda.synchronize()
     assert status == 0 and torch.equal(scores, want)
+
+
+def test_classifiers_of_other_sizes_on_several_threads(sd):
+    """A large and a small classifier called from two threads on streams of their own: neither call changes what the other may launch."""
+    import threading
+    calls = []
+    for d_model, seed in ((512, 3), (16, 4)):
+        clf = sd.MambaClassifier(synth.make_mamba_classifier(100, d_model=d_model, d_state=16, d_conv=4, expand=2, n_classes=4, seed=seed))
+        tokens = torch.from_numpy(synth.make_prompt(100, 90, seed=6)).to(DEV)
+        calls.append((clf, tokens, clf.classify(tokens, [0], [90])[0], torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    wrong = []
+
+    def loop(clf, tokens, want, stream):
+        try:
+            with torch.cuda.stream(stream):
+                for _ in range(1500):
+                    scores, _ = clf.classify(tokens, [0], [90])
+                stream.synchronize()
+                if not torch.equal(scores, want):
+                    wrong.append("scores")
+        except RuntimeError as e:
+            wrong.append(str(e))
+
+    threads = [threading.Thread(target=loop, args=c) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
