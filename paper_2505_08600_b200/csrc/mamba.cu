@@ -8,11 +8,13 @@
 // both sums of the one scan.  The states s follow from the chunks' end states and decays in a short serial pass per prompt.
 // The pooled vector is the mean over tokens of W_out g_t, which is W_out applied to the mean of g_t: the kernels sum
 // g_t per channel (chunks in order) and apply W_out and the classification layer once per prompt.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "../../include/sd.h"
@@ -142,30 +144,36 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
 //      two tokens and every 16th output, three at a time;
 //   2. a thread per channel scans the chunk: convolution again (four multiply-adds are less than a trip through memory), step
 //      size, recurrence from a zero state, and the two sums of the chunk (see the top of the file).
-constexpr int MC_TILE = 32, MC_THREADS = 256, MC_STAGED = 48 * 1024;      // W_x is staged up to this size: two CTAs of the usual sizes still fit an SM
-// Most dynamic shared memory a launch takes: B, C, r of a chunk and a tile of v at their largest (W_x is beyond its limit then; where
-// it is staged, n_x Di <= MC_STAGED / 4 and the rest is smaller by more than MC_STAGED).
-constexpr int MC_MAX_SMEM = (MB_CHUNK * MB_MAX_X + MC_TILE * (MB_MAX_DI + 4)) * 4;
+//   More than MC_CHANNELS channels: a cluster of up to four CTAs per chunk with as many channels each.  A CTA projects its own channels;
+//   the parts of r, B, C meet through distributed shared memory (each CTA adds a share of them, parts in the CTAs' order).  1,024
+//   channels, whole call: one prompt of 64 tokens 425 us (1,329 with one CTA for all channels, 904 as kernels of their own), four of
+//   100...300 462 (1,378, 999), 400 of 32...512 15.3 ms (17.0, 32.2); 512 channels, one prompt of 64: 172 us (256, 303).
+constexpr int MC_TILE = 32, MC_THREADS = 256, MC_CHANNELS = 256, MC_STAGED = 48 * 1024;      // W_x is staged up to this size: two CTAs of the usual sizes still fit an SM
+// Most dynamic shared memory a launch takes: B, C, r of a chunk, a tile of v and the staged W_x at their largest.
+constexpr int MC_MAX_SMEM = (MB_CHUNK * MB_MAX_X + MC_TILE * (MC_CHANNELS + 4)) * 4 + MC_STAGED;
 constexpr int MH_MAX_SMEM = (MB_MAX_DI * MB_MAX_N + MB_MAX_DI + MB_MAX_D + MB_MAX_K) * 4;
-template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to MB_MAX_CONV as 0*/>
+template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to MB_MAX_CONV as 0*/, bool CL /*several CTAs per chunk*/>
 __global__ void __launch_bounds__(MC_THREADS, 2)
 k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* __restrict__ tok_row, const float* __restrict__ u, const float* __restrict__ z,
               const float* __restrict__ w_conv, const float* __restrict__ b_conv, const float* __restrict__ w_x, const float* __restrict__ w_dt,
               const float* __restrict__ b_dt, const float* __restrict__ a_log, const float* __restrict__ d_skip,
-              float* __restrict__ end_state, float* __restrict__ decay, float* __restrict__ carry_gain /*all [chunk][Di][N]*/, double* __restrict__ chunk_sum /*[chunk][Di]*/, int w_staged) {
+              float* __restrict__ end_state, float* __restrict__ decay, float* __restrict__ carry_gain /*all [chunk][Di][N]*/, double* __restrict__ chunk_sum /*[chunk][Di]*/, int w_staged, int n_cta, int per_cta) {
     extern __shared__ __align__(16) float sm[];
+    const int Dp = (m.Di + 3) & ~3, per = CL ? per_cta : Dp;                             // channels of a CTA, padded to a multiple of 4
     const int N = NS ? NS : m.N, n_x = m.R + 2 * m.N, xp = (n_x + 3) & ~3;
     float* xd_s = sm;                                      // [MB_CHUNK][xp]: B, C, r of every token
     float* v_s = sm + MB_CHUNK * xp;                       // [MC_TILE][vp]
-    float* wx_s = v_s + MC_TILE * (((m.Di + 3) & ~3) + 4); // [n_x][Di] if it was given room
+    float* wx_s = v_s + MC_TILE * (per + 4);               // this CTA's columns of W_x, [n_x][n_c], if they were given room
     __shared__ int row_s[MB_CHUNK + MB_MAX_CONV];          // rows of the chunk's tokens and of the taps in front of them (-1: before the prompt)
-    const int tid = threadIdx.x, Dp = (m.Di + 3) & ~3, vp = Dp + 4;
-    const ChunkRec ch = chunks[blockIdx.x];
+    const int tid = threadIdx.x, vp = per + 4;
+    const int chunk = CL ? blockIdx.x / n_cta : blockIdx.x, c_lo = CL ? (int)(blockIdx.x % n_cta) * per : 0, n_c = CL ? min(m.Di - c_lo, per) : m.Di;
+    const ChunkRec ch = chunks[chunk];
     constexpr int KM = KC ? KC : MB_MAX_CONV;
     const int Kc = KC ? KC : m.Kc, back = Kc - 1;
     for (int i = tid; i < ch.n_tok + back; i += MC_THREADS) row_s[i] = ch.pos0 + i - back >= 0 ? tok_row[ch.tok0 + i - back] : -1;
-    if (w_staged) for (int i = tid; i < n_x * m.Di; i += MC_THREADS) wx_s[i] = __ldg(w_x + i);
-    const float* wx = w_staged ? wx_s : w_x;
+    if (w_staged) for (int i = tid; i < n_x * n_c; i += MC_THREADS) wx_s[i] = __ldg(CL ? w_x + (size_t)(i / n_c) * m.Di + c_lo + i % n_c : w_x + i);
+    const float* wx = w_staged ? wx_s : w_x + c_lo;
+    const int w_ld = CL && w_staged ? n_c : m.Di;
     __syncthreads();
     // SiLU(convolution) of channel c at token t; the taps come in the order of the sum
     auto conv = [&](const float (&w)[KM], float b, const float (&x)[KM]) {
@@ -174,12 +182,13 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
         for (int j = 0; j < KM; ++j) if (j < Kc) acc = fmaf(w[j], x[j], acc);
         return silu_f(acc);
     };
-    const bool vec = (m.Di & 3) == 0 && (w_staged || ((uintptr_t)w_x & 15) == 0);
+    const bool vec = (m.Di & 3) == 0 && (w_staged || ((uintptr_t)w_x & 15) == 0);      // (then n_c is a multiple of 4 as well)
     for (int t0 = 0; t0 < ch.n_tok; t0 += MC_TILE) {
         const int nt = min(MC_TILE, ch.n_tok - t0);
-        for (int c = tid; c < Dp; c += MC_THREADS) {
+        for (int i = tid; i < per; i += MC_THREADS) {
             float w[KM], x[KM];
-            const bool on = c < m.Di;
+            const int c = c_lo + i;
+            const bool on = i < n_c;
 #pragma unroll
             for (int j = 0; j < KM; ++j) {
                 w[j] = on && j < Kc ? __ldg(w_conv + (size_t)c * Kc + j) : 0.f;
@@ -192,7 +201,7 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
                 const float nu = on && t < nt ? __ldg(u + (size_t)row_s[t0 + t + back] * m.Di + c) : 0.f;
 #pragma unroll
                 for (int j = 0; j < KM; ++j) if (j == back) x[j] = nu;
-                v_s[t * vp + c] = on && t < nt ? conv(w, b, x) : 0.f;
+                v_s[t * vp + i] = on && t < nt ? conv(w, b, x) : 0.f;
 #pragma unroll
                 for (int j = 0; j + 1 < KM; ++j) if (j < back) x[j] = x[j + 1];
             }
@@ -204,12 +213,12 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
         for (int o0 = og; o0 < n_x; o0 += 48) {
             const int o1 = o0 + 16, o2 = o0 + 32;
             float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            const float* w0 = wx + (size_t)o0 * m.Di;
-            const float* w1 = wx + (size_t)min(o1, n_x - 1) * m.Di;
-            const float* w2 = wx + (size_t)min(o2, n_x - 1) * m.Di;
+            const float* w0 = wx + (size_t)o0 * w_ld;
+            const float* w1 = wx + (size_t)min(o1, n_x - 1) * w_ld;
+            const float* w2 = wx + (size_t)min(o2, n_x - 1) * w_ld;
             if (vec) {
 #pragma unroll 2
-                for (int c = 0; c < m.Di; c += 4) {
+                for (int c = 0; c < n_c; c += 4) {
                     const float4 a = *reinterpret_cast<const float4*>(v0 + c), b = *reinterpret_cast<const float4*>(v1 + c);
                     const float4 p = *reinterpret_cast<const float4*>(w0 + c), q = *reinterpret_cast<const float4*>(w1 + c), r = *reinterpret_cast<const float4*>(w2 + c);
                     s[0] = fmaf(p.x, a.x, s[0]); s[0] = fmaf(p.y, a.y, s[0]); s[0] = fmaf(p.z, a.z, s[0]); s[0] = fmaf(p.w, a.w, s[0]);
@@ -220,7 +229,7 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
                     s[5] = fmaf(r.x, b.x, s[5]); s[5] = fmaf(r.y, b.y, s[5]); s[5] = fmaf(r.z, b.z, s[5]); s[5] = fmaf(r.w, b.w, s[5]);
                 }
             } else {
-                for (int c = 0; c < m.Di; ++c) {
+                for (int c = 0; c < n_c; ++c) {
                     const float a = v0[c], b = v1[c], p = w0[c], q = w1[c], r = w2[c];
                     s[0] = fmaf(p, a, s[0]); s[1] = fmaf(p, b, s[1]); s[2] = fmaf(q, a, s[2]); s[3] = fmaf(q, b, s[3]); s[4] = fmaf(r, a, s[4]); s[5] = fmaf(r, b, s[5]);
                 }
@@ -238,7 +247,22 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
         }
         __syncthreads();
     }
-    for (int c = tid; c < m.Di; c += MC_THREADS) {
+    if (CL) {                                              // the other CTAs' channels: every value is added by one CTA, which hands the sum to all
+        namespace cg = cooperative_groups;
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        const int n = ch.n_tok * xp, share = (n + n_cta - 1) / n_cta, i0 = (int)(blockIdx.x % n_cta) * share;
+        for (int i = i0 + tid; i < min(n, i0 + share); i += MC_THREADS) {
+            float v[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) v[r] = r < n_cta ? cluster.map_shared_rank(xd_s, r)[i] : 0.f;
+            const float sum = ((v[0] + v[1]) + v[2]) + v[3];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) if (r < n_cta) cluster.map_shared_rank(xd_s, r)[i] = sum;
+        }
+        cluster.sync();                                    // (no CTA touches another's shared memory from here on)
+    }
+    for (int c = c_lo + tid; c < c_lo + n_c; c += MC_THREADS) {
         float w[KM], x[KM];
 #pragma unroll
         for (int j = 0; j < KM; ++j) {
@@ -294,8 +318,8 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
             const float2 y = f2_unpack(y2);
             sum += (double)(fmaf(dsk, v, y.x + y.y) * g);
         }
-        chunk_sum[(size_t)blockIdx.x * m.Di + c] = sum;
-        const size_t at = ((size_t)blockIdx.x * m.Di + c) * m.N;
+        chunk_sum[(size_t)chunk * m.Di + c] = sum;
+        const size_t at = ((size_t)chunk * m.Di + c) * m.N;
 #pragma unroll
         for (int n = 0; n < MB_MAX_N / 2; ++n) {
             if (2 * n < N) {
@@ -453,19 +477,31 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     k_mamba_tables<<<(unsigned)n_chunks, 64, 0, st>>>(chunks_d, (const int64_t*)(base + L.starts), tokens_dev, m.V, by_token ? 1 : 0, tok_id, tok_row);
     k_mamba_in<<<dim3((unsigned)((rows + MI_TILE - 1) / MI_TILE), (unsigned)((2 * m.Di + MI_TILE - 1) / MI_TILE)), 256, 0, st>>>(
         m, by_token ? nullptr : tok_id, rows, w->embed, w->w_in, u, z);
-    const size_t xp = (size_t)((m.R + 2 * m.N + 3) & ~3), wx_bytes = (size_t)(m.R + 2 * m.N) * m.Di * 4;
+    const int n_cta = (m.Di + MC_CHANNELS - 1) / MC_CHANNELS, per = ((m.Di + n_cta - 1) / n_cta + 3) & ~3;      // (the last CTA has at least one channel)
+    const size_t xp = (size_t)((m.R + 2 * m.N + 3) & ~3), wx_bytes = (size_t)(m.R + 2 * m.N) * per * 4;
     const int w_staged = wx_bytes <= MC_STAGED;
-    const size_t chunk_smem = (MB_CHUNK * xp + (size_t)MC_TILE * (((m.Di + 3) & ~3) + 4)) * 4 + (w_staged ? wx_bytes : 0);
-    auto chunk_kernel = m.N != MB_MAX_N ? k_mamba_chunk<0, 0> : m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4> : k_mamba_chunk<MB_MAX_N, 0>;
+    const size_t chunk_smem = (MB_CHUNK * xp + (size_t)MC_TILE * (per + 4)) * 4 + (w_staged ? wx_bytes : 0);
+    auto pick = [&](auto cl) {
+        constexpr bool CL = decltype(cl)::value;
+        return m.N != MB_MAX_N ? k_mamba_chunk<0, 0, CL> : m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4, CL> : k_mamba_chunk<MB_MAX_N, 0, CL>;
+    };
+    auto chunk_kernel = n_cta > 1 ? pick(std::true_type()) : pick(std::false_type());
     const size_t head_smem = ((size_t)m.Di * m.N + m.Di + m.D + m.K) * 4;
     // Always the bound over all sizes that are accepted: the attribute belongs to the kernel, and a smaller classifier's call on
     // another thread must not lower it between here and the launch.
     if (cudaFuncSetAttribute(chunk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MC_MAX_SMEM) != cudaSuccess ||
         cudaFuncSetAttribute(k_mamba_head, cudaFuncAttributeMaxDynamicSharedMemorySize, MH_MAX_SMEM) != cudaSuccess)
         return SD_ERR_CUDA;
-    chunk_kernel<<<(unsigned)n_chunks, MC_THREADS, chunk_smem, st>>>(
-        m, chunks_d, tok_row, u, z, w->w_conv, w->b_conv, w->w_x, w->w_dt, w->b_dt, w->a_log, w->d_skip, (float*)(base + L.end_state),
-        (float*)(base + L.decay), (float*)(base + L.carry_gain), (double*)(base + L.chunk_sum), w_staged);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n_chunks * n_cta)); cfg.blockDim = dim3(MC_THREADS); cfg.dynamicSmemBytes = chunk_smem; cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)n_cta; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr; cfg.numAttrs = n_cta > 1 ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, chunk_kernel, m, chunks_d, (const int32_t*)tok_row, (const float*)u, (const float*)z, w->w_conv, w->b_conv, w->w_x, w->w_dt, w->b_dt,
+                           w->a_log, w->d_skip, (float*)(base + L.end_state), (float*)(base + L.decay), (float*)(base + L.carry_gain),
+                           (double*)(base + L.chunk_sum), w_staged, n_cta, per) != cudaSuccess)
+        return SD_ERR_CUDA;
     k_mamba_head<<<(unsigned)n_prompts, 1024, head_smem, st>>>(
         m, pc0, (const int32_t*)(base + L.lens), (const double*)(base + L.chunk_sum), (const float*)(base + L.end_state), (const float*)(base + L.decay),
         (const float*)(base + L.carry_gain), w->w_out, w->w_fc, w->b_fc, scores_dev, labels_dev);

@@ -135,3 +135,11 @@ def test_classifiers_of_other_sizes_on_several_threads(sd):
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("d_model,expand,d_state,d_conv", [(512, 2, 16, 4), (150, 2, 16, 3), (257, 1, 5, 4), (129, 6, 8, 6)])
+def test_channels_of_several_ctas(sd, d_model, expand, d_state, d_conv):
+    """More than 256 channels: two to four CTAs per chunk, the last with fewer channels, channels that are no multiple of four (257, 774)."""
+    vocab = 200
+    w = synth.make_mamba_classifier(vocab, d_model=d_model, d_state=d_state, d_conv=d_conv, expand=expand, n_classes=3, seed=12)
+    _compare(sd, w, [1, 31, 33, 64, 150], vocab, seed=8)
