@@ -152,7 +152,7 @@ constexpr int MC_TILE = 32, MC_THREADS = 256, MC_CHANNELS = 256, MC_STAGED = 48 
 // Most dynamic shared memory a launch takes: B, C, r of a chunk, a tile of v and the staged W_x at their largest.
 constexpr int MC_MAX_SMEM = (MB_CHUNK * MB_MAX_X + MC_TILE * (MC_CHANNELS + 4)) * 4 + MC_STAGED;
 constexpr int MH_MAX_SMEM = (MB_MAX_DI * MB_MAX_N + MB_MAX_DI + MB_MAX_D + MB_MAX_K) * 4;
-template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to MB_MAX_CONV as 0*/, bool CL /*several CTAs per chunk*/>
+template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to four as -4, or up to MB_MAX_CONV as 0*/, bool CL /*several CTAs per chunk*/>
 __global__ void __launch_bounds__(MC_THREADS, 2)
 k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* __restrict__ tok_row, const float* __restrict__ u, const float* __restrict__ z,
               const float* __restrict__ w_conv, const float* __restrict__ b_conv, const float* __restrict__ w_x, const float* __restrict__ w_dt,
@@ -168,8 +168,8 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
     const int tid = threadIdx.x, vp = per + 4;
     const int chunk = CL ? blockIdx.x / n_cta : blockIdx.x, c_lo = CL ? (int)(blockIdx.x % n_cta) * per : 0, n_c = CL ? min(m.Di - c_lo, per) : m.Di;
     const ChunkRec ch = chunks[chunk];
-    constexpr int KM = KC ? KC : MB_MAX_CONV;
-    const int Kc = KC ? KC : m.Kc, back = Kc - 1;
+    constexpr int KM = KC > 0 ? KC : KC < 0 ? -KC : MB_MAX_CONV;
+    const int Kc = KC > 0 ? KC : m.Kc, back = Kc - 1;
     for (int i = tid; i < ch.n_tok + back; i += MC_THREADS) row_s[i] = ch.pos0 + i - back >= 0 ? tok_row[ch.tok0 + i - back] : -1;
     if (w_staged) for (int i = tid; i < n_x * n_c; i += MC_THREADS) wx_s[i] = __ldg(CL ? w_x + (size_t)(i / n_c) * m.Di + c_lo + i % n_c : w_x + i);
     const float* wx = w_staged ? wx_s : w_x + c_lo;
@@ -483,7 +483,8 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
     const size_t chunk_smem = (MB_CHUNK * xp + (size_t)MC_TILE * (per + 4)) * 4 + (w_staged ? wx_bytes : 0);
     auto pick = [&](auto cl) {
         constexpr bool CL = decltype(cl)::value;
-        return m.N != MB_MAX_N ? k_mamba_chunk<0, 0, CL> : m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4, CL> : k_mamba_chunk<MB_MAX_N, 0, CL>;
+        if (m.N == MB_MAX_N) return m.Kc == 4 ? k_mamba_chunk<MB_MAX_N, 4, CL> : k_mamba_chunk<MB_MAX_N, 0, CL>;
+        return m.Kc <= 4 ? k_mamba_chunk<0, -4, CL> : k_mamba_chunk<0, 0, CL>;
     };
     auto chunk_kernel = n_cta > 1 ? pick(std::true_type()) : pick(std::false_type());
     const size_t head_smem = ((size_t)m.Di * m.N + m.Di + m.D + m.K) * 4;
