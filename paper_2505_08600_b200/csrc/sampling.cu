@@ -2,6 +2,8 @@
 // draft's per-step sampler and the fused accept / reject / resample kernel.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "gemm_tc.h"
 #include "kernels.h"
 
@@ -130,7 +132,6 @@ __device__ __forceinline__ void stage_row(const float* __restrict__ src, float* 
     }
     __syncthreads();
 }
-constexpr int SLICED_FROM = 4096;                // vocabularies from here on are worth a cluster (below, its barriers cost more than they save)
 constexpr int STAGE_MAX_BYTES = 200 * 1024;      // a row of up to 51200 fp32 values fits beside the static shared memory
 
 // Dynamic shared memory for one staged row, or 0 when the vocabulary is too large to stage.
@@ -204,13 +205,24 @@ __global__ void __launch_bounds__(1024) k_draft_sample(const float* __restrict__
 // sum, integer total) goes to every CTA of the cluster through distributed shared memory.  The token is the one of the integer
 // inverse CDF over the written fp32 values, whatever the split.  32000 values: 16 -> 11 us.
 constexpr int SLICES = 8;
+__host__ __device__ __forceinline__ int slice_len(int V) { return (V + 4 * SLICES - 1) / (4 * SLICES) * 4; }
+// Rows whose clusters run side by side (a CTA of 1024 threads per SM, a cluster inside one GPC): 12 rows take one wave, 16 and 24 two, 32
+// three, 64 five.
+constexpr int SLICED_WAVE = 14;
+static double sliced_waves(int n) { return (n + SLICED_WAVE - 1) / SLICED_WAVE; }
+// Where the slices are the faster form.  Against a CTA per row (which has all rows in one wave) they save 0.3 us per thousand values above
+// 8192 (32000: 7.3 us a draw, 16384: 2.4, 4096: -1.4 for one to twelve rows) and cost 6.5 us and a little more per further wave (32000 values,
+// 16 rows: -1.1, 32 rows: -9.7; 50000: +4.2 and -5.8).  A row that cannot be staged (64000 values) takes a CTA three times as long.
+static bool draft_sliced(int V, int n) {
+    if ((size_t)slice_len(V) * sizeof(float) > (size_t)STAGE_MAX_BYTES) return false;
+    return !row_stage_bytes(V) || 3e-4 * (V - 8192) > (sliced_waves(n) - 1) * (6.5 + 6e-5 * V);
+}
 struct SliceScratch {
     BlockScratch b;
     float f[2][SLICES];
     int idx[SLICES];
     unsigned long long total[SLICES];
 };
-__host__ __device__ __forceinline__ int slice_len(int V) { return (V + 4 * SLICES - 1) / (4 * SLICES) * 4; }
 
 // block_icdf over this CTA's slice of n weights, `base` being the weight of everything in front of it, `thr` the running sum to be
 // reached: the index inside the slice in the CTA whose slice holds it, -1 in the others.  local: the slice's weight of this thread.
@@ -358,7 +370,7 @@ cudaError_t launch_draft_sample(const float* logits, const SeqState& S, const Se
                                 uint64_t seed, int step, int gamma, float* q_out, int32_t* x_out, cudaStream_t st) {
     if (list.n <= 0) return cudaSuccess;
     const size_t slice = (size_t)slice_len(V) * sizeof(float);
-    if (V >= SLICED_FROM && slice <= (size_t)STAGE_MAX_BYTES) {
+    if (draft_sliced(V, list.n)) {
         cudaError_t e = cudaFuncSetAttribute(k_draft_sample_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_draft_sample_sliced, dim3(list.n * SLICES), dim3(1024), slice, st, 1, logits, S, list, V, T, seed, step, gamma, q_out, x_out);
@@ -667,10 +679,23 @@ __global__ void __cluster_dims__(SLICES, 1, 1) __launch_bounds__(1024) k_accept_
     cluster.sync();                                            // no CTA leaves while the others may still write into it
 }
 
+// Where that is the faster form, by what both take (us, measured at 1,000...50,000 values, 1...16 rows, 1...64 sequences; one wave of
+// clusters, 12288 / 32000 values: 2 rows 11.8 / 12.6 sliced, 17.6 / 33.3 a CTA per row; 6 rows 18.6 / 19.0 and 17.1 / 32.8; 9 rows 23.4 / 24.0
+// and 22.4 / 41.9; 16 rows 34.5 / 37 (24000) and 26.7 / 41): the slices pay a barrier or two per row, a CTA per row its row's length, twice
+// from nine rows on.  Equal at 4,000 values for 2 rows, 8,200 for 4, 13,000 for 6, 18,000 for 8, 13,000 for 9, 14,000 for 12, 20,500 for 16.
+static bool accept_sliced(int V, int rows, int n) {
+    if ((size_t)slice_len(V) * rows * sizeof(float) > (size_t)STAGE_MAX_BYTES || rows > ACC_MAX_ROWS) return false;
+    if (!row_stage_bytes(V)) return true;                      // (64000 values, 3 rows: 18 against 120)
+    const int two = std::min(std::max(rows - 9, 0), 3);
+    const double row = rows == 1 ? 7.0 + 3.9e-4 * V : rows <= 8 ? 8.2 + 7.7e-4 * V : 10.7 + 0.33 * two + (9.8e-4 + 0.7e-4 * two) * V;
+    const int side_by_side = rows > 4 ? SLICED_WAVE : rows > 2 ? 36 : 148;       // clusters of eight, four, and fewer CTAs
+    return sliced_waves(n) * (8.5 + rows * (1.32 + 2.1e-5 * V)) < (n + side_by_side - 1) / side_by_side * row;
+}
+
 cudaError_t launch_accept(const AcceptParams& p, int dependent, cudaStream_t st) {
     if (p.B <= 0) return cudaSuccess;
     const size_t slices = (size_t)slice_len(p.V) * (p.gamma + 1) * sizeof(float);
-    if (p.V >= SLICED_FROM && slices <= (size_t)STAGE_MAX_BYTES && p.gamma <= SD_MAX_GAMMA) {
+    if (accept_sliced(p.V, p.gamma + 1, p.B)) {
         cudaError_t e = cudaFuncSetAttribute(k_accept_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_accept_sliced, dim3(p.B * SLICES), dim3(1024), slices, st, dependent, p);
