@@ -183,13 +183,16 @@ cudaError_t launch_mode(const PlainStep& p, cudaStream_t st) {
 
 }  // namespace
 
-// Up to eight rows, each with two accumulators per unit in registers; the largest matrix at most 16 MB, so that L2 holds the model and
-// launches, not bytes, are the bound (the tiny pair: 154 us here, 204 through the plain kernels; larger fp32 models keep those).
+// Up to five rows, each with two accumulators per unit in registers, up to eight where the largest matrix has 8 MB or more; that matrix at
+// most 16 MB, so that L2 holds the model and launches, not bytes, are the bound (larger fp32 models keep the plain kernels).  A pass,
+// plain / here, us: largest matrix 1.4 MB 1 row 55 / 39, 5 rows 66 / 61, 6 rows 67.6 / 71.6; 5.6 MB 127 / 80, 150 / 143, 163 / 165; 12.6 MB
+// 210 / 146, 231 / 208, 248 / 242, 8 rows 273 / 259; 16.8 MB 229 / 165, 263 / 235, 284 / 278, 315 / 295; beyond the line, 32.8 MB: 249 / 182, 285 / 274,
+// 304 / 317.
 // Rows and scores have to fit in shared memory; head_dim % 16 == 0 for the float4 reads of a quarter of a key.
 bool plain_steps_fit(const sd_model_desc& m, int rows, int max_ctx) {
     const size_t d = m.d_model, dq = (size_t)m.n_heads * m.head_dim, n_qkv = dq + 2 * (size_t)m.n_kv_heads * m.head_dim, F = m.d_ffn, V = m.vocab;
     const size_t largest = std::max(std::max(n_qkv * d, d * dq), std::max(2 * F * d, V * d)) * sizeof(float);
-    return m.dtype == SD_F32 && rows >= 1 && rows <= PS_MAX_ROWS && m.head_dim % 16 == 0 && m.d_model % 4 == 0 && m.d_ffn % 4 == 0 &&
+    return m.dtype == SD_F32 && rows >= 1 && rows <= (largest >= ((size_t)8 << 20) ? PS_MAX_ROWS : 5) && m.head_dim % 16 == 0 && m.d_model % 4 == 0 && m.d_ffn % 4 == 0 &&
            largest <= ((size_t)16 << 20) && (size_t)rows * std::max(std::max(d, dq), F) * sizeof(float) <= (size_t)PS_ROW_BYTES && (size_t)(m.head_dim + max_ctx) * sizeof(float) <= 40 * 1024;
 }
 

@@ -13,11 +13,12 @@ pytestmark = pytest.mark.gpu
 MODELS = {
     "gqa16": dict(n_layers=2, d_model=104, n_heads=6, n_kv_heads=2, head_dim=16, d_ffn=72, vocab=333),
     "hd256": dict(n_layers=1, d_model=256, n_heads=2, n_kv_heads=1, head_dim=256, d_ffn=1544, vocab=1001),     # three rounds of weights
+    "mb8": dict(n_layers=2, d_model=512, n_heads=4, n_kv_heads=2, head_dim=64, d_ffn=2048, vocab=333),         # gate/up of 8 MB: 6...8 rows as well
 }
 
 
 @pytest.mark.parametrize("name", sorted(MODELS))
-@pytest.mark.parametrize("n_seq,gamma", [(1, 0), (1, 1), (1, 4), (2, 3), (3, 2)])      # 1, 2, 5, 8 and 9 verify rows
+@pytest.mark.parametrize("n_seq,gamma", [(1, 0), (1, 1), (1, 4), (1, 5), (2, 3), (3, 2)])      # 1, 2, 5, 6, 8 and 9 verify rows
 def test_verify_rows_follow_the_oracle(name, n_seq, gamma):
     from paper_2505_08600_b200 import binding
     dims = MODELS[name]
