@@ -668,25 +668,41 @@ bool gemv_fits(const Model& M, int n_rows, int mode, int n_out, int K) {
     g.rows = n_rows; g.ep.mode = mode; g.ep.hd = M.d.head_dim; g.ep.F = M.d.d_ffn; g.n_out = n_out; g.K = K;
     return gemv_supported(g);
 }
-// Whether all of a pass does: the draft models, whose matrices are through in less time than the weight-streaming GEMM and its
-// step kernel need to hand over.
-bool few_rows_pass(sd_ctx* c, const Model& M, int n_rows) {
-    const sd_model_desc& m = M.d;
-    if (&M == &c->models[0] || n_rows > GEMV_MAX_ROWS || m.d_model % 16 || m.d_model > 16 * GEMV_SSQ_STRIDE) return false;
-    return gemv_fits(M, n_rows, EPI_QKV_ROPE, M.n_qkv(), m.d_model) && gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) &&
-           gemv_fits(M, n_rows, EPI_SWIGLU, 2 * m.d_ffn, m.d_model) && gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.d_ffn) &&
-           gemv_fits(M, n_rows, EPI_PLAIN, m.vocab, m.d_model);
-}
-// ... or a single matrix of a pass that streams the others: up to 16 MB.  1B target, six rows: with QKV (12.6 MB) and Wo (8.4 MB) on
-// these kernels an iteration takes 1.100 ms instead of 1.142; with gate/up (67 MB) as well 1.31, with the lm_head (131 MB) 1.19:
-// a CTA that holds its whole share in registers cannot keep HBM busy across CTAs.
-constexpr size_t GEMV_LARGEST = (size_t)16 << 20;
+// ... and whether it should.  The weight-streaming GEMM and its step kernel are two launches that share a matrix out over all SMs; these
+// kernels are one, in which a CTA's 16 features arrive at one SM's rate.  Three lines (five draft steps, or one step of a target, us):
+//   - at most 16 MB: a CTA that holds its whole share in registers cannot keep HBM busy across CTAs.  768-wide draft with its 9.4 MB
+//     gate/up on these kernels 1,122, without 1,447; 1536-wide target with its 25 MB gate/up 329, without 317; 2048-wide target with
+//     25 MB QKV 395, without 381; 3072-wide draft (19...57 MB) 1,545, without 1,131; 1B target with gate/up (67 MB) 1,310, without 1,100;
+//     A draft's lm_head, behind layers on these kernels: at most 64 MB.  The streaming GEMM is the faster one alone (768 wide, 49 MB, one to eight
+//     rows: 1,122 against 1,133, 1,331 against 1,369), but it takes every SM and its shared memory from draft models that run beside this one
+//     (13B with two, 65 MB: iteration 13,393 against 13,000; 7B with four: 7,207 against 7,122); 98 MB, alone: 1,504 against 1,630;
+//   - more than eight rows (two groups of MMA columns, one CTA per SM): at most two CTAs' worth per SM.  1024-wide draft, 16 sequences,
+//     with gate/up (512 CTAs) 3,474, without 3,063; 1536-wide target, 12 rows, with QKV (288 CTAs) 338, without 355;
+//   - one or two rows, where the pair of kernels is at its cheapest: reductions of up to 1024, unless the whole layer is on these kernels.
+//     Longer ones take CTAs of sixteen warps, beside which the next GEMM's CTAs find no registers to begin loading in.  2048-wide draft with
+//     Wo and down 1,845, without 1,623; 1B target's decoding step 360, without 345; 1024-wide draft with QKV and Wo 2,282, without 2,491.
 // A residual step on them leaves a piece of the rows' sums of squares per 16 features to a step kernel, which has to be able to add
 // them all: 128, or 64 with 9...16 rows in one part.
-bool few_rows_matrix(const Model& M, int n_rows, int lo, int mode, int n_out, int K) {
+constexpr size_t GEMV_LARGEST = (size_t)16 << 20, GEMV_LARGEST_HEAD = (size_t)64 << 20;
+constexpr int GEMV_SHORT_K = 1024;
+bool few_rows_matrix(const Model& M, bool draft, int n_rows, int lo, bool whole_layer, int mode, int n_out, int K) {
     const int parts = lo || n_rows <= 8 ? SSQ_MAX_PARTS : SSQ_STRIDE;
-    return n_rows <= GEMV_MAX_ROWS && !M.lora && (size_t)n_out * K * sizeof(bf16) <= GEMV_LARGEST && gemv_fits(M, n_rows, mode, n_out, K) &&
-           (mode != EPI_RESIDUAL || n_out <= 16 * parts);
+    const size_t largest = draft && whole_layer && mode == EPI_PLAIN ? GEMV_LARGEST_HEAD : GEMV_LARGEST;
+    return n_rows <= GEMV_MAX_ROWS && (size_t)n_out * K * sizeof(bf16) <= largest && gemv_fits(M, n_rows, mode, n_out, K) &&
+           (mode != EPI_RESIDUAL || n_out <= 16 * parts) && (n_rows <= 8 || n_out <= 16 * 2 * sm_count()) &&
+           (n_rows > 2 || K <= GEMV_SHORT_K || whole_layer);
+}
+// Whether these kernels could hold all of a pass: its activations come in two parts from one row on then, whichever kernel a matrix takes.
+bool few_rows_pass(const Model& M, int n_rows) {
+    const sd_model_desc& m = M.d;
+    return n_rows <= GEMV_MAX_ROWS && m.d_model % 16 == 0 && gemv_fits(M, n_rows, EPI_QKV_ROPE, M.n_qkv(), m.d_model) &&
+           gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) && gemv_fits(M, n_rows, EPI_SWIGLU, 2 * m.d_ffn, m.d_model) &&
+           gemv_fits(M, n_rows, EPI_RESIDUAL, m.d_model, m.d_ffn) && gemv_fits(M, n_rows, EPI_PLAIN, m.vocab, m.d_model);
+}
+bool few_rows_layer(const Model& M, int n_rows, int lo) {
+    const sd_model_desc& m = M.d;
+    return few_rows_matrix(M, false, n_rows, lo, true, EPI_QKV_ROPE, M.n_qkv(), m.d_model) && few_rows_matrix(M, false, n_rows, lo, true, EPI_RESIDUAL, m.d_model, m.n_heads * m.head_dim) &&
+           few_rows_matrix(M, false, n_rows, lo, true, EPI_SWIGLU, 2 * m.d_ffn, m.d_model) && few_rows_matrix(M, false, n_rows, lo, true, EPI_RESIDUAL, m.d_model, m.d_ffn);
 }
 
 // One matrix and the step that follows it, on those kernels.
@@ -726,8 +742,10 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     // With 3..16 rows (the verify rows of one sequence) the 16 (or 32) columns of the MMA hold every activation twice over:
     // as bf16(x) and as bf16(x - bf16(x)), 8 (or 16) rows apart.  The weights stream once all the same, and the GEMMs'
     // inputs are no longer rounded to 8 bits of mantissa.
-    const bool few = few_rows_pass(c, M, n_rows);            // (there the second parts cost nothing, for one or two rows either)
-    const int lo = !c->two_part ? 0 : (n_rows >= (few ? 1 : 3) && n_rows <= 8) ? 8 : (n_rows >= 9 && n_rows <= 16) ? 16 : 0;
+    // (Draft passes that the few-rows kernels can hold: from one row on.  There the second part costs nothing.)
+    const bool draft = &M != &c->models[0];
+    const int lo = !c->two_part ? 0 : (n_rows >= (draft && few_rows_pass(M, n_rows) ? 1 : 3) && n_rows <= 8) ? 8 : (n_rows >= 9 && n_rows <= 16) ? 16 : 0;
+    const bool few = few_rows_layer(M, n_rows, lo);
     if (c->stamps_on) {                                                     // the stamps of this pass replace the previous pass's
         c->stamp_kinds.clear();
         CUDA_TRY(cudaMemsetAsync(c->stamp_buf, 0xFF, sizeof(unsigned long long) * ST_WORDS * STAMP_CAP, st));
@@ -747,7 +765,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     int dependent = 0;
     RowScale scale{c->ssq, 1, 1.f / d, m.rms_eps, SSQ_STRIDE};              // sum of squares in one piece (after the embedding),
     auto step = [&](const TensorMap& tm, const void* w, const void* x, int n_out, int K, const Epilogue& e) {
-        const bool gv = few || few_rows_matrix(M, n_rows, lo, e.mode, n_out, K);
+        const bool gv = few_rows_matrix(M, draft, n_rows, lo, few, e.mode, n_out, K);
         if (e.mode == EPI_RESIDUAL) {                                       // ... then in one piece per tile of the kernel that wrote h
             scale.n_parts = gv ? d / 16 : (d + 127) / 128;
             scale.stride = gv ? GEMV_SSQ_STRIDE : SSQ_STRIDE;

@@ -22,6 +22,8 @@ DRAFTS = {
     "d288": _m(2, 288, 3, 64, 320, 509),           # 9 k blocks of 32, F = 10; odd vocabulary
     "hd128_f2112": _m(2, 256, 2, 128, 2112, 509),   # the form for up to 3072
     "d1056": _m(1, 1056, 4, 64, 4096, 509),         # the forms for up to 2048 and 4096
+    "mixed": _m(1, 1152, 4, 64, 7680, 509),         # gate/up and down stream; QKV as well with one or two rows
+    "two_waves": _m(1, 512, 4, 64, 2432, 509),      # gate/up is 304 CTAs: it streams from nine rows on
 }
 
 
@@ -47,6 +49,39 @@ def test_draft_passes_follow_the_oracle(name, n_seq):
     om = oracle.OracleModel(draft, wd)
     for s in seqs:
         logits = om.new_cache(128).forward(np.concatenate([toks[s], xg[s, :-1]]), 0)[-gamma:]
+        top = logits.max(axis=1, keepdims=True)
+        want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
+        assert np.abs(np.log(qg[s]) - want).max() <= LOG_TOL, s
+
+
+@pytest.mark.parametrize("n_seq", [1, 5])                           # 2, then 1 row; 10, then 5
+def test_mixed_passes_with_adapters_follow_the_merged_models(n_seq):
+    from oracle import lora
+    from paper_2505_08600_b200 import binding
+    draft, target, gamma, rank = _m(1, 1152, 4, 64, 7680, 512), _m(1, 64, 1, 64, 64, 512), 2, 8
+    wt, wd = synth.make_weights(target, seed=3, model_index=0, dtype="bf16"), synth.make_weights(draft, seed=3, model_index=1, dtype="bf16")
+    ctx = binding.Context(target, [draft], "bf16", n_seq, 96, gamma, 1.0, 7, lora_adapters=2, lora_rank=rank, lora_scale=1.0)
+    ctx.load_weights(0, wt); ctx.load_weights(1, wd)
+    merged = []
+    for task in range(2):
+        ad = synth.make_lora(draft, rank, task, seed=0)
+        for mat, name in enumerate(("qkv", "wo", "gu", "wd")):
+            for l, (a, b) in enumerate(ad[name]):
+                ctx.sd_load_lora(task, l, mat, a, b)
+        merged.append(oracle.OracleModel(draft, lora.merged_weights(draft, wd, ad, 1.0)))
+    toks = [synth.make_prompt(512, 7 + 9 * i, seed=9, seq=i) for i in range(n_seq)]
+    seqs = list(range(n_seq))
+    for s in seqs:
+        ctx.sd_seq_begin(s, toks[s], s)
+    ctx.sd_route_prompt(seqs, forced_task=[s % 2 for s in seqs])
+    ctx.sd_prefill(seqs)
+    x, q = torch.zeros((n_seq, gamma), dtype=torch.int32, device=DEV), torch.zeros((n_seq, gamma, 512), dtype=torch.float32, device=DEV)
+    ctx.sd_draft_steps(seqs, gamma, x, q)
+    xg, qg = x.cpu().numpy(), q.cpu().numpy().astype(np.float64)
+    assert ctx.sd_device_status() == 0
+    ctx.close()
+    for s in seqs:
+        logits = merged[s % 2].new_cache(128).forward(np.concatenate([toks[s], xg[s, :-1]]), 0)[-gamma:]
         top = logits.max(axis=1, keepdims=True)
         want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
         assert np.abs(np.log(qg[s]) - want).max() <= LOG_TOL, s
