@@ -21,6 +21,7 @@ constexpr int KM_MAX_K = 8;
 constexpr __host__ __device__ int km_depth(int km) { return km == 4 ? 8 : 6; }
 constexpr __host__ __device__ int km_warps(int nv, int km) { return km == 4 && nv == 3 ? 12 : 8; }
 constexpr __host__ __device__ int km_per_sm(int nv, int km) { return km == 4 && nv >= 3 ? 1 : 2; }
+constexpr int KM_RUN = 128;            // points in one run of fp32 sums, where a warp keeps runs
 
 // Two fp32 values in one 64-bit register and the packed arithmetic of sm_100 on them: each instruction is two
 // independent IEEE operations (same results as the scalar forms), which halves the instructions per loaded byte.
@@ -60,11 +61,11 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
     for (int kk = 0; kk < KM; ++kk)
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[kk][v] = make_ulonglong2(0ull, 0ull);
-    int cnt = 0;                                // lane kk: points of this warp in cluster kk (a warp sees n / (8 * blocks) points)
+    int cnt = 0;                                // lane kk: points of this warp in cluster kk (a warp sees n / (KM_WARPS * blocks) points)
     double inertia = 0.0;
 
-    // Every lane copies its own columns of the next KM_DEPTH - 1 points of its warp into shared memory with
-    // asynchronous 16-byte copies and reads back only what it copied itself: no barrier, and enough bytes in flight per SM
+    // Every lane copies its own columns of its warp's next points (KM_DEPTH - 1 of them, KM_DEPTH - 2 two at a time) into shared memory
+    // with asynchronous 16-byte copies and reads back only what it copied itself: no barrier, and enough bytes in flight per SM
     // (warps x depth x row) to cover the memory latency at full bandwidth.
     const long long total_warps = (long long)gridDim.x * KM_WARPS;
     const long long i0 = (long long)blockIdx.x * KM_WARPS + warp;
@@ -83,6 +84,26 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
         asm volatile("cp.async.commit_group;" ::: "memory");                      // (an empty group past the end keeps the count uniform)
         idx_next += total_warps; src_next += src_step;
         slot_next = slot_next + 1 == KM_DEPTH ? 0 : slot_next + 1;
+    };
+    // One CTA per SM has fewer warps than two, and so more points in each warp's fp32 sums: there a lane moves its sums to shared memory
+    // every KM_RUN points and begins anew (no other lane reads them: no barrier).  Error against 64 bits of the centroid of a million copies
+    // of one 512-component point: 0.9e-6; 6.1e-6 without; two CTAs per SM: 3.0e-6.  2,000,003 x 384, 4 clusters: 616 -> 622 us
+    // (every 256 points: 621).
+    constexpr bool RUNS = km_per_sm(NV, KM) == 1 && KM == 4;
+    // [KM][DIM] of this warp, this lane's first column: behind the rings; the first warp's where the block's sums will be, which it writes first
+    float* runs = (warp == 0 ? acc_s : acc_s + KM * DIM + KM_WARPS * KM_DEPTH * DIM + (warp - 1) * KM * DIM) + lane * 4;
+    bool moved = false;
+    auto move_sums = [&]() {
+#pragma unroll
+        for (int kk = 0; kk < KM; ++kk)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                ulonglong2* dst = reinterpret_cast<ulonglong2*>(runs + kk * DIM + v * 128);
+                if (moved) { const ulonglong2 s = *dst; acc[kk][v].x = f2_add(s.x, acc[kk][v].x); acc[kk][v].y = f2_add(s.y, acc[kk][v].y); }
+                *dst = acc[kk][v];
+                acc[kk][v] = make_ulonglong2(0ull, 0ull);
+            }
+        moved = true;
     };
     int slot = 0;
     auto ring_at = [&](int sl, int v) { return *reinterpret_cast<const ulonglong2*>(ring + sl * DIM + v * 128); };
@@ -114,46 +135,50 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
         // 691 and 564; 1,000,000 x 512: 429 and 408.  A ring of ten points is no faster than one of eight.
         constexpr int AHEAD = KM_DEPTH - 2;
         for (int t = 0; t < AHEAD; ++t) stage();
-        for (long long i = i0; i < n; i += 2 * total_warps) {
-            stage(); stage();
-            asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD) : "memory");       // these two points have landed
-            const int slot1 = slot + 1 == KM_DEPTH ? 0 : slot + 1;
-            const bool both = i + total_warps < n;                                // uniform
-            float d[2][4];
-            ulonglong2 x0[NV], x1[NV];
+        for (long long i = i0; i < n;) {
+            const long long i_end = RUNS ? min(n, i + KM_RUN * total_warps) : n;
+            for (; i < i_end; i += 2 * total_warps) {
+                stage(); stage();
+                asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD) : "memory");       // these two points have landed
+                const int slot1 = slot + 1 == KM_DEPTH ? 0 : slot + 1;
+                const bool both = i + total_warps < n;                                // uniform
+                float d[2][4];
+                ulonglong2 x0[NV], x1[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) { x0[v] = ring_at(slot, v); x1[v] = ring_at(slot1, v); }
+                for (int v = 0; v < NV; ++v) { x0[v] = ring_at(slot, v); x1[v] = ring_at(slot1, v); }
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {                                      // (centroids past k are zeros and drop out below)
-                d[0][kk] = partial(x0, KM == 4 ? kk : 0);
-                d[1][kk] = partial(x1, KM == 4 ? kk : 0);
+                for (int kk = 0; kk < 4; ++kk) {                                      // (centroids past k are zeros and drop out below)
+                    d[0][kk] = partial(x0, KM == 4 ? kk : 0);
+                    d[1][kk] = partial(x1, KM == 4 ? kk : 0);
+                }
+                const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
+                float a[4];
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) a[kk] = (hi16 ? d[1][kk] : d[0][kk]) + __shfl_xor_sync(0xffffffffu, hi16 ? d[0][kk] : d[1][kk], 16);
+                float b0 = (hi8 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[2], 8);
+                float b1 = (hi8 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[1] : a[3], 8);
+                float e = (hi4 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, hi4 ? b0 : b1, 4);
+                e += __shfl_xor_sync(0xffffffffu, e, 2);
+                e += __shfl_xor_sync(0xffffffffu, e, 1);
+                // lane group (bit 4 | bit 3, bit 2) holds point bit 4, cluster 2 * bit 3 + bit 2; the smallest wins, the lowest index on ties
+                int label = (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
+                if (label >= k || !(e == e)) e = INFINITY;
+#pragma unroll
+                for (int o = 4; o <= 8; o <<= 1) {
+                    const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
+                    const int l2 = __shfl_xor_sync(0xffffffffu, label, o);
+                    if (e2 < e || (e2 == e && l2 < label)) { e = e2; label = l2; }
+                }
+                if (!hi16 || both) {
+                    inertia += (double)e;                                             // (the lower half sums the first points, the upper half the second ones)
+                    if ((lane & 15) == 0) labels[hi16 ? i + total_warps : i] = label;
+                }
+                const int label0 = __shfl_sync(0xffffffffu, label, 0), label1 = __shfl_sync(0xffffffffu, label, 16);
+                count(x0, label0);
+                if (both) count(x1, label1);
+                slot = slot1 + 1 == KM_DEPTH ? 0 : slot1 + 1;
             }
-            const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
-            float a[4];
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) a[kk] = (hi16 ? d[1][kk] : d[0][kk]) + __shfl_xor_sync(0xffffffffu, hi16 ? d[0][kk] : d[1][kk], 16);
-            float b0 = (hi8 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[2], 8);
-            float b1 = (hi8 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[1] : a[3], 8);
-            float e = (hi4 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, hi4 ? b0 : b1, 4);
-            e += __shfl_xor_sync(0xffffffffu, e, 2);
-            e += __shfl_xor_sync(0xffffffffu, e, 1);
-            // lane group (bit 4 | bit 3, bit 2) holds point bit 4, cluster 2 * bit 3 + bit 2; the smallest wins, the lowest index on ties
-            int label = (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
-            if (label >= k || !(e == e)) e = INFINITY;
-#pragma unroll
-            for (int o = 4; o <= 8; o <<= 1) {
-                const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
-                const int l2 = __shfl_xor_sync(0xffffffffu, label, o);
-                if (e2 < e || (e2 == e && l2 < label)) { e = e2; label = l2; }
-            }
-            if (!hi16 || both) {
-                inertia += (double)e;                                             // (the lower half sums the first points, the upper half the second ones)
-                if ((lane & 15) == 0) labels[hi16 ? i + total_warps : i] = label;
-            }
-            const int label0 = __shfl_sync(0xffffffffu, label, 0), label1 = __shfl_sync(0xffffffffu, label, 16);
-            count(x0, label0);
-            if (both) count(x1, label1);
-            slot = slot1 + 1 == KM_DEPTH ? 0 : slot1 + 1;
+            if (RUNS && i < n) move_sums();
         }
         inertia += __shfl_sync(0xffffffffu, inertia, 16);                         // (what lane 0 writes)
     } else {
@@ -193,6 +218,16 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
             count(x, label);
             slot = slot + 1 == KM_DEPTH ? 0 : slot + 1;
         }
+    }
+
+    if (RUNS && moved) {
+#pragma unroll
+        for (int kk = 0; kk < KM; ++kk)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const ulonglong2 s = *reinterpret_cast<const ulonglong2*>(runs + kk * DIM + v * 128);
+                acc[kk][v].x = f2_add(s.x, acc[kk][v].x); acc[kk][v].y = f2_add(s.y, acc[kk][v].y);
+            }
     }
 
     // the block's sums: its warps in warp order
@@ -291,7 +326,8 @@ extern "C" sd_status sd_kmeans_step(const float* points, int64_t n, int dim, con
     float* part_sums = (float*)w;              w += km_align((size_t)blocks * k * dim * sizeof(float));
     long long* part_counts = (long long*)w;    w += km_align((size_t)blocks * k * sizeof(long long));
     double* part_inertia = (double*)w;
-    const size_t smem = ((size_t)2 * km + (size_t)km_warps(dim / 128, km) * km_depth(km)) * dim * sizeof(float);
+    const int warps = km_warps(dim / 128, km), runs = km == 4 && km_per_sm(dim / 128, km) == 1 ? (warps - 1) * km : 0;
+    const size_t smem = ((size_t)2 * km + (size_t)warps * km_depth(km) + runs) * dim * sizeof(float);
     cudaError_t e = cudaSuccess;
 #define KM_LAUNCH(NV, KM)                                                                                                        \
     do {                                                                                                                     \

@@ -41,3 +41,47 @@ def test_pairs_are_exact_on_small_integers(n, dim, k):
     want[[n - 1, n // 2]] = 0
     labels, _, cnt, _ = run(x)
     assert np.array_equal(labels, want) and np.array_equal(cnt, np.bincount(want, minlength=k))
+
+
+@pytest.mark.parametrize("dim,k,warps", [(384, 4, 1776), (512, 3, 1184)])
+@pytest.mark.parametrize("per_warp,extra", [(128, 0), (128, 1), (129, 0), (130, -1), (256, 0), (257, 3)])
+def test_runs_of_sums_hold_every_point_once(dim, k, warps, per_warp, extra):
+    """A warp's sums are moved away every 128 points: numbers of points just at and beyond that, in all and in some warps; small integers,
+    as above."""
+    from paper_2505_08600_b200 import binding as sd
+    n = per_warp * warps + extra
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n + dim)
+    x = torch.zeros((n, dim), device=DEV)
+    x[:, :8] = torch.randint(-2, 3, (n, 8), generator=g, device=DEV).float()
+    c = torch.zeros((k, dim), device=DEV)
+    c[:, :8] = torch.randint(-2, 3, (k, 8), generator=g, device=DEV).float()
+    labels = torch.full((n,), -1, dtype=torch.int32, device=DEV)
+    out, cnt, inertia = torch.zeros((k, dim), device=DEV), torch.zeros(k, dtype=torch.int64, device=DEV), torch.zeros(1, dtype=torch.float64, device=DEV)
+    sd.sd_kmeans_step(x, c, labels, out, cnt, inertia)
+    d = ((x[:, None, :8].double() - c[None, :, :8].double()) ** 2).sum(2)
+    near = d.min(1).values
+    want = torch.stack([torch.where(d[:, j] == near, j, k) for j in range(k)], 1).min(1).values
+    assert torch.equal(labels.long(), want) and torch.equal(cnt, torch.bincount(want, minlength=k)) and inertia.item() == near.sum().item()
+    for j in range(k):
+        assert torch.equal(out[j], (x[want == j].double().sum(0) / max(1, int(cnt[j]))).float() if cnt[j] else c[j])
+
+
+@pytest.mark.parametrize("dim", [384, 512])
+def test_sums_are_as_precise_as_those_of_two_blocks_per_sm(dim):
+    """A million copies of one point: every addition of a warp's running fp32 sum rounds the same way, so that the centroid is off in
+    proportion to the points in one sum.  No more than with 2,368 warps of n / 2368 points each, added by eights."""
+    from paper_2505_08600_b200 import binding as sd
+    n = 1_000_000
+    v = np.random.default_rng(1).uniform(1, 2, dim).astype(np.float32)
+    run = np.zeros_like(v)
+    for _ in range(n // 2368):
+        run += v
+    block = np.zeros_like(v)
+    for _ in range(8):
+        block += run
+    bound = np.linalg.norm(block.astype(np.float64) / (n // 2368 * 8) - v) / np.linalg.norm(v)
+    x = torch.from_numpy(v).to(DEV).repeat(n, 1)
+    labels, out = torch.empty(n, dtype=torch.int32, device=DEV), torch.zeros((4, dim), device=DEV)
+    sd.sd_kmeans_step(x, torch.stack([x[0]] * 4), labels, out)
+    assert np.linalg.norm(out[0].cpu().numpy().astype(np.float64) - v) / np.linalg.norm(v) <= 1.05 * bound      # (a few more points in some sums)
