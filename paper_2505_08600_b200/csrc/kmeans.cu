@@ -16,9 +16,10 @@ namespace sd {
 namespace {
 
 constexpr int KM_MAX_K = 8;
-// Points of a warp that its ring holds, warps of a CTA and CTAs of an SM.  Two points at a time at 384 components take 160 registers:
-// one CTA of twelve warps; 512: eight warps; fewer components: two CTAs of eight.
-constexpr __host__ __device__ int km_depth(int km) { return km == 4 ? 8 : 6; }
+// Points of a warp that its ring holds, warps of a CTA and CTAs of an SM, for 128 nv components and up to km clusters.  Two points at a
+// time with four centroids in registers take 160 registers at 384 components: one CTA of twelve warps; 512: eight warps; fewer
+// components, or two centroids: two CTAs of eight (rings of six points at 512, so that two fit the shared memory).
+constexpr __host__ __device__ int km_depth(int nv, int km) { return km == 8 || (km == 2 && nv == 4) ? 6 : 8; }
 constexpr __host__ __device__ int km_warps(int nv, int km) { return km == 4 && nv == 3 ? 12 : 8; }
 constexpr __host__ __device__ int km_per_sm(int nv, int km) { return km == 4 && nv >= 3 ? 1 : 2; }
 constexpr int KM_RUN = 128;            // points in one run of fp32 sums, where a warp keeps runs
@@ -31,11 +32,11 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn
 __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ float f2_hsum(f32x2 v) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); return a + b; }
 
-template <int NV, int KM>          // KM: compiled cluster bound (4 or 8); with 4 the centroids are kept in registers
-__global__ void __launch_bounds__(32 * km_warps(NV, KM), (KM == 4 && NV <= 2) ? 2 : 1)
+template <int NV, int KM>          // KM: compiled cluster bound (2, 4 or 8); up to 4 the centroids are kept in registers
+__global__ void __launch_bounds__(32 * km_warps(NV, KM), KM == 8 ? 1 : km_per_sm(NV, KM))
 k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* __restrict__ cent, int32_t* __restrict__ labels,
                 float* __restrict__ part_sums, long long* __restrict__ part_counts, double* __restrict__ part_inertia) {
-    constexpr int DIM = 128 * NV, KM_WARPS = km_warps(NV, KM), KM_DEPTH = km_depth(KM);
+    constexpr int DIM = 128 * NV, KM_WARPS = km_warps(NV, KM), KM_DEPTH = km_depth(NV, KM);
     extern __shared__ __align__(16) float km_smem[];
     float* cs = km_smem;                       // [k][DIM] centroids
     float* acc_s = km_smem + KM * DIM;         // [k][DIM] the block's sums
@@ -47,7 +48,7 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
 
     // Up to four centroids: every lane keeps its columns of them in registers (shared memory could not feed four
     // centroid reads per point at the rate the points arrive); more: read from shared memory.
-    constexpr bool CREG = KM == 4;
+    constexpr bool CREG = KM <= 4;
     ulonglong2 creg[CREG ? KM : 1][CREG ? NV : 1];
     if (CREG) {
 #pragma unroll
@@ -127,12 +128,14 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
             }
         }
     };
-    if (KM == 4) {
-        // Two points at a time: their eight sums over the warp cost nine shuffles (halves of the warp trade one point for the other,
+    if (KM <= 4) {
+        // Two points at a time (four clusters): their eight sums over the warp cost nine shuffles (halves of the warp trade one point for the other,
         // then clusters), the smallest of four per half four more, and the two chains of latencies run side by side; the distances are
         // added in the same order as one by one.  2,000,003 x 384, 4 clusters: 636 us one point at a time (16 warps per SM of 128
         // registers), 579 with two points, twelve warps of 168 registers (at 128 registers they spill: 1,100); 4,000,000 x 128:
         // 691 and 564; 1,000,000 x 512: 429 and 408.  A ring of ten points is no faster than one of eight.
+        // One or two clusters have a form of their own (1,000,003 x 256 and 512, two clusters: 223 and 429 us one point at a time, 234 and
+        // 449 with four sums for two, 192 and 354 with two).
         constexpr int AHEAD = KM_DEPTH - 2;
         for (int t = 0; t < AHEAD; ++t) stage();
         for (long long i = i0; i < n;) {
@@ -142,29 +145,36 @@ k_kmeans_assign(const float* __restrict__ pts, long long n, int k, const float* 
                 asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD) : "memory");       // these two points have landed
                 const int slot1 = slot + 1 == KM_DEPTH ? 0 : slot + 1;
                 const bool both = i + total_warps < n;                                // uniform
-                float d[2][4];
+                float d[2][KM];
                 ulonglong2 x0[NV], x1[NV];
 #pragma unroll
                 for (int v = 0; v < NV; ++v) { x0[v] = ring_at(slot, v); x1[v] = ring_at(slot1, v); }
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {                                      // (centroids past k are zeros and drop out below)
-                    d[0][kk] = partial(x0, KM == 4 ? kk : 0);
-                    d[1][kk] = partial(x1, KM == 4 ? kk : 0);
+                for (int kk = 0; kk < KM; ++kk) {                                     // (centroids past k are zeros and drop out below)
+                    d[0][kk] = partial(x0, CREG ? kk : 0);
+                    d[1][kk] = partial(x1, CREG ? kk : 0);
                 }
                 const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
-                float a[4];
+                float a[KM];
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) a[kk] = (hi16 ? d[1][kk] : d[0][kk]) + __shfl_xor_sync(0xffffffffu, hi16 ? d[0][kk] : d[1][kk], 16);
-                float b0 = (hi8 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[2], 8);
-                float b1 = (hi8 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[1] : a[3], 8);
-                float e = (hi4 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, hi4 ? b0 : b1, 4);
+                for (int kk = 0; kk < KM; ++kk) a[kk] = (hi16 ? d[1][kk] : d[0][kk]) + __shfl_xor_sync(0xffffffffu, hi16 ? d[0][kk] : d[1][kk], 16);
+                float e;
+                if (KM == 2) {
+                    e = (hi8 ? a[1] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[1], 8);
+                    e += __shfl_xor_sync(0xffffffffu, e, 4);
+                } else {
+                    constexpr int K2 = KM > 2 ? 2 : 0, K3 = KM > 2 ? 3 : 0;
+                    const float b0 = (hi8 ? a[K2] : a[0]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[0] : a[K2], 8);
+                    const float b1 = (hi8 ? a[K3] : a[1]) + __shfl_xor_sync(0xffffffffu, hi8 ? a[1] : a[K3], 8);
+                    e = (hi4 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, hi4 ? b0 : b1, 4);
+                }
                 e += __shfl_xor_sync(0xffffffffu, e, 2);
                 e += __shfl_xor_sync(0xffffffffu, e, 1);
-                // lane group (bit 4 | bit 3, bit 2) holds point bit 4, cluster 2 * bit 3 + bit 2; the smallest wins, the lowest index on ties
-                int label = (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
+                // a lane's bit 4 is the point, bits 3 and 2 are the cluster (two clusters: bit 3); the smallest wins, the lowest index on ties
+                int label = KM == 2 ? (hi8 ? 1 : 0) : (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
                 if (label >= k || !(e == e)) e = INFINITY;
 #pragma unroll
-                for (int o = 4; o <= 8; o <<= 1) {
+                for (int o = KM == 2 ? 8 : 4; o <= 8; o <<= 1) {
                     const float e2 = __shfl_xor_sync(0xffffffffu, e, o);
                     const int l2 = __shfl_xor_sync(0xffffffffu, label, o);
                     if (e2 < e || (e2 == e && l2 < label)) { e = e2; label = l2; }
@@ -320,14 +330,17 @@ extern "C" sd_status sd_kmeans_step(const float* points, int64_t n, int dim, con
     if (((uintptr_t)points & 15) || ((uintptr_t)centroids & 15)) return SD_ERR_INVALID_ARG;
     if (!workspace || workspace_bytes < sd_kmeans_workspace(dim, k)) return SD_ERR_CAPACITY;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int km = k <= 4 ? 4 : KM_MAX_K;
-    const int blocks = km_blocks() / (2 / km_per_sm(dim / 128, km));
+    const int km = k <= 2 ? 2 : k <= 4 ? 4 : KM_MAX_K;
+    // (two clusters of few long vectors: one CTA per SM as well, whose set-up and partial sums are half as many.  3,000 x 384: 18.5 us, with
+    // two 22.6; 512: 18.5 and 23.4)
+    const bool few = km == 2 && dim >= 384 && n < 16 * km_warps(dim / 128, km) * (km_blocks() / 2);
+    const int blocks = km_blocks() / (few ? 2 : 2 / km_per_sm(dim / 128, km));
     char* w = (char*)workspace;
     float* part_sums = (float*)w;              w += km_align((size_t)blocks * k * dim * sizeof(float));
     long long* part_counts = (long long*)w;    w += km_align((size_t)blocks * k * sizeof(long long));
     double* part_inertia = (double*)w;
     const int warps = km_warps(dim / 128, km), runs = km == 4 && km_per_sm(dim / 128, km) == 1 ? (warps - 1) * km : 0;
-    const size_t smem = ((size_t)2 * km + (size_t)warps * km_depth(km) + runs) * dim * sizeof(float);
+    const size_t smem = ((size_t)2 * km + (size_t)warps * km_depth(dim / 128, km) + runs) * dim * sizeof(float);
     cudaError_t e = cudaSuccess;
 #define KM_LAUNCH(NV, KM)                                                                                                        \
     do {                                                                                                                     \
@@ -335,10 +348,10 @@ extern "C" sd_status sd_kmeans_step(const float* points, int64_t n, int dim, con
         if (e == cudaSuccess) k_kmeans_assign<NV, KM><<<blocks, 32 * km_warps(NV, KM), smem, st>>>(points, n, k, centroids, labels, part_sums, part_counts, part_inertia); \
     } while (0)
     switch (dim / 128) {
-    case 1: if (km == 4) KM_LAUNCH(1, 4); else KM_LAUNCH(1, 8); break;
-    case 2: if (km == 4) KM_LAUNCH(2, 4); else KM_LAUNCH(2, 8); break;
-    case 3: if (km == 4) KM_LAUNCH(3, 4); else KM_LAUNCH(3, 8); break;
-    default: if (km == 4) KM_LAUNCH(4, 4); else KM_LAUNCH(4, 8); break;
+    case 1: if (km == 2) KM_LAUNCH(1, 2); else if (km == 4) KM_LAUNCH(1, 4); else KM_LAUNCH(1, 8); break;
+    case 2: if (km == 2) KM_LAUNCH(2, 2); else if (km == 4) KM_LAUNCH(2, 4); else KM_LAUNCH(2, 8); break;
+    case 3: if (km == 2) KM_LAUNCH(3, 2); else if (km == 4) KM_LAUNCH(3, 4); else KM_LAUNCH(3, 8); break;
+    default: if (km == 2) KM_LAUNCH(4, 2); else if (km == 4) KM_LAUNCH(4, 4); else KM_LAUNCH(4, 8); break;
     }
 #undef KM_LAUNCH
     if (e == cudaSuccess) e = cudaGetLastError();
