@@ -226,46 +226,67 @@ def setup(args, gamma_max, steps_per_phase):
                 routed=routed, rewind=rewind, max_ctx=max_ctx)
 
 
-STEP_AFTER = {0: "lm_head", 1: "qkv", 2: "residual", 3: "swiglu"}
-LAYER_LAUNCHES = ["gemm qkv", "step qkv", "attention", "gemm wo", "step wo", "gemm gate_up", "step gate_up", "gemm down", "step down"]
+LAUNCH_KIND = {0: "gemm", 1: "step", 2: "attention", 3: "matrix"}        # matrix: GEMM and step in one kernel
+
+
+def layer_launches(kinds, n_layers):
+    """Names of a layer's launches from the kinds of a pass's records, all layers being alike (None if they are not)."""
+    body = [int(k) for k in kinds]
+    n_tail = 1 if body and body[-1] & 0xff == 3 else 2                      # the lm_head's: one kernel, or GEMM and step
+    if (len(body) - n_tail) % n_layers:
+        return None
+    per = (len(body) - n_tail) // n_layers
+    if any(body[l * per:(l + 1) * per] != body[:per] for l in range(n_layers)):
+        return None
+    names, residual = [], 0
+    for k in body[:per]:
+        kind, after = LAUNCH_KIND[k & 0xff], k >> 8
+        if kind in ("gemm", "matrix") and after == 2:
+            residual += 1
+        names.append(kind if kind == "attention" else kind + " " + {1: "qkv", 2: "wo" if residual == 1 else "down", 3: "gate_up"}[after])
+    return names
 
 
 def in_graph_timeline(ctx, cfg, step_fn, esz):
     """Time stamps taken inside the kernels while the step runs as it always runs (captured graph, overlapping
     dependent launches): per launch of a layer, averaged over the inner layers, in microseconds after the layer's QKV
-    GEMM issued its first MMA.  A GEMM's in-graph duration is counted from the moment its token rows exist (the kernel
+    GEMM issued its first MMA (had its token rows, where QKV and its step are one kernel).  A GEMM's in-graph duration is counted from the moment its token rows exist (the kernel
     before it has finished) to its last CTA finishing; weights requested before that moment are part of the overlap."""
     t = cfg["target"]
-    nl, per = t["n_layers"], len(LAYER_LAUNCHES)
+    nl = t["n_layers"]
     ctx.sd_launch_stamps(1)
     for _ in range(3):
         step_fn()
     st, kinds = ctx.sd_launch_stamps_read()
     ctx.sd_launch_stamps(0)
-    if len(kinds) < nl * per + 2 or nl < 4:
+    launches = layer_launches(kinds, nl) if nl >= 4 else None
+    if not launches:
         return None
+    per = len(launches)
+    zero = 3 if launches[0].startswith("gemm") else 1
     st = st.astype(np.int64)
     cols = ["start", "dep_first", "dep_last", "data_first", "data_last", "done_first", "done_last"]
     inner = range(1, nl - 1)
-    rows = np.array([[[(st[l * per + j][k] - st[l * per][3]) / 1e3 if st[l * per + j][k] else np.nan for k in range(7)]
+    rows = np.array([[[(st[l * per + j][k] - st[l * per][zero]) / 1e3 if st[l * per + j][k] else np.nan for k in range(7)]
                       for j in range(per)] for l in inner])
     with np.errstate(all="ignore"):
         import warnings
         with warnings.catch_warnings():
             warnings.simplefilter("ignore", RuntimeWarning)
             avg = np.nanmean(rows, axis=0)           # (columns a kind of launch never reports stay NaN)
-    period = float(np.mean([(st[(l + 1) * per][3] - st[l * per][3]) / 1e3 for l in inner]))
-    table = {name: {c: (None if np.isnan(avg[j][k]) else round(float(avg[j][k]), 2)) for k, c in enumerate(cols)} for j, name in enumerate(LAYER_LAUNCHES)}
+    period = float(np.mean([(st[(l + 1) * per][zero] - st[l * per][zero]) / 1e3 for l in inner]))
+    table = {name: {c: (None if np.isnan(avg[j][k]) else round(float(avg[j][k]), 2)) for k, c in enumerate(cols)} for j, name in enumerate(launches)}
     gemm_us = 0.0
-    for j, name in enumerate(LAYER_LAUNCHES):
-        if name.startswith("gemm"):
+    for j, name in enumerate(launches):
+        if name.startswith(("gemm", "matrix")):
             gemm_us += float(avg[j][6] - avg[j][1])
-    # the lm_head GEMM: the last GEMM record of the pass
+    # the lm_head: the record behind the layers'
     lm = st[nl * per]
     lm_us = (lm[6] - lm[1]) / 1e3
     return {"layer_period_us": round(period, 2), "gemm_us_per_layer": round(gemm_us, 2), "lm_head_gemm_us": round(float(lm_us), 2),
-            "columns": "us after the layer's QKV GEMM had its first stage: first CTA start; first/last CTA saw its dependency; "
+            "columns": "us after the layer's QKV GEMM had its first stage (its token rows, where GEMM and step are one kernel): first CTA start; first/last CTA saw its dependency; "
                        "first/last CTA had its first stage (GEMM); first/last CTA done",
+            "one_kernel": sum(name.startswith("matrix") for name in launches) * nl + int(int(kinds[nl * per]) & 0xff == 3),      # matrices whose step is in their kernel
             "launches": table}
 
 
@@ -355,7 +376,9 @@ def run_gpu(args):
     gemm_share = split["linear"] / total_split
     in_step_ms = ms_step * gemm_share
     pair_ms = ms_step * (split["linear"] + split["fused_step"]) / total_split
-    roofline = {"bound": "hbm", "kernel": f"k_gemm_streamk ({n_gemm} launches per verify step, all weight matrices once)",
+    n_gemv = tl["one_kernel"] if tl else 0
+    kernel = "k_plain_step" if cfg["dtype"] != "bf16" else "k_gemm_streamk" if not n_gemv else f"k_gemm_streamk and k_gemv ({n_gemm - n_gemv} and {n_gemv} of them)"
+    roofline = {"bound": "hbm", "kernel": f"{kernel} ({n_gemm} launches per verify step, all weight matrices once)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
                 "avg_launch_us": gemm_ms * 1e3 / n_gemm, "timing": "CUDA events around each launch (launches serialised)",
                 # dram read+write per weight byte from the ncu capture summarised in profiles/gemm_streamk_1b_ncu_full.md

@@ -240,16 +240,18 @@ int sd_best_gamma(double alpha, double c, int gamma_max, double* speedup_out);
 
 /* Time stamps of the launches of a forward pass, taken inside the kernels (the device's nanosecond timer) while the
  * pass runs the way it always runs (captured graph, programmatic dependent launches): what a profiler's serialised
- * per-kernel times cannot show.  While enabled, every weight GEMM, the step kernel after it and every attention launch
- * of the most recent forward pass on the kernel-per-matrix path (bf16 models) fill one record of SD_STAMP_WORDS 64-bit
- * words; sd_launch_stamps_read synchronises and copies the first `cap` records (launch order) to the host:
+ * per-kernel times cannot show.  While enabled, every weight GEMM, the step kernel after it, every kernel that is both (a
+ * matrix of a pass of few rows; QKV and gate/up of a prompt pass) and every attention launch of the most recent forward
+ * pass on the kernel-per-matrix path (bf16 models) fill one record of SD_STAMP_WORDS 64-bit words;
+ * sd_launch_stamps_read synchronises and copies the first `cap` records (launch order) to the host:
  *   [0] first CTA began                    [1],[2] first / last CTA saw what it waits for (the kernel before it; its
- *   tile's pieces)                         [3],[4] GEMM only: first / last CTA had its first stage complete
+ *   tile's pieces)                         [3],[4] GEMM of a ring only: first / last CTA had its first stage complete
  *   [5],[6] first / last CTA finished      [7] 0.            A word is 0 when nothing reported it.
- * kinds_host[i] = SD_STAMP_GEMM / _STEP / _ATTENTION | (step after the GEMM: 0 plain, 1 QKV+rotary, 2 residual,
- * 3 SwiGLU) << 8; *n_out = records of the pass (may exceed cap).  Enabling changes the captured graphs' keys: the
- * first call afterwards captures anew.  Matrix and step in one kernel (passes of few rows) and prompt passes leave no
- * records.  A few atomics per CTA: for measurement, off by default. */
+ * kinds_host[i] = SD_STAMP_GEMM / _STEP / _ATTENTION / _MATRIX (GEMM and step in one kernel) | (step after the GEMM:
+ * 0 plain, 1 QKV+rotary, 2 residual, 3 SwiGLU) << 8; *n_out = records of the pass (may exceed cap).  Enabling changes
+ * the captured graphs' keys: the first call afterwards captures anew.  With adapters a matrix of a pass of few rows, or
+ * of a prompt pass, has a launch for x A^T in front, which has a record of its own (as SD_STAMP_MATRIX or SD_STAMP_GEMM
+ * with step 0).  A few atomics per CTA: for measurement, off by default. */
 /* Sequences routed to different draft models run their draft passes side by side (default, when the context has two or
  * more separate draft models): every group after the first is enqueued on a stream of its own, forked from and joined
  * back to the context's stream, with its own scratch memory from the arena.  on = 0: group after group on the
@@ -288,6 +290,7 @@ sd_status sd_tuning(sd_ctx* ctx, int knob, int value);
 #define SD_STAMP_GEMM 0
 #define SD_STAMP_STEP 1
 #define SD_STAMP_ATTENTION 2
+#define SD_STAMP_MATRIX 3
 sd_status sd_launch_stamps(sd_ctx* ctx, int enable);
 sd_status sd_launch_stamps_read(sd_ctx* ctx, uint64_t* stamps_host, int32_t* kinds_host, int cap, int32_t* n_out);
 

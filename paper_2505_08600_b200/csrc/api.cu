@@ -622,6 +622,14 @@ unsigned long long* next_stamp(sd_ctx* c, int kind) {
     return c->stamp_buf + (size_t)ST_WORDS * (c->stamp_kinds.size() - 1);
 }
 
+// The records of the pass being enqueued take the place of the one before's.
+sd_status begin_stamps(sd_ctx* c) {
+    if (!c->stamps_on) return SD_OK;
+    c->stamp_kinds.clear();
+    CUDA_TRY(cudaMemsetAsync(c->stamp_buf, 0xFF, sizeof(unsigned long long) * ST_WORDS * STAMP_CAP, c->st));
+    return SD_OK;
+}
+
 // One weight GEMM and the step that follows it.  dependent = 0: launched in full stream order (see forward_tc).
 sd_status gemm_tc(sd_ctx* c, const TensorMap& tw, const void* x, int rows, int n_out, int K, const Epilogue& ep, int dependent) {
     if (ep.lo_off) rows += ep.lo_off;           // the input rows come in two bf16 parts: [x_hi rows][x_lo rows at + lo_off]
@@ -715,11 +723,13 @@ sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out
         memset(&t.ep, 0, sizeof(t.ep));
         t.ep.mode = EPI_PLAIN; t.ep.lo_off = ep.lo_off; t.ep.m_real = rows; t.ep.y = c->lora_t; t.ep.n_out_rows = rows; t.ep.row_stride = 1;
         t.w = g.w + (size_t)n_out * K; t.n_out = 128;
+        t.ep.stamp = next_stamp(c, SD_STAMP_MATRIX | (EPI_PLAIN << 8));
         LAUNCH(CAT_LINEAR, launch_gemv(t, dependent, c->st));
         dependent = 1;
         g.lora_t = c->lora_t;
     }
     c->x_from.words = nullptr;                  // (no tile-by-tile hand-off from this kernel)
+    g.ep.stamp = next_stamp(c, SD_STAMP_MATRIX | (ep.mode << 8));
     LAUNCH(CAT_LINEAR, launch_gemv(g, dependent, c->st));
     return SD_OK;
 }
@@ -746,10 +756,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
     const bool draft = &M != &c->models[0];
     const int lo = !c->two_part ? 0 : (n_rows >= (draft && few_rows_pass(M, n_rows) ? 1 : 3) && n_rows <= 8) ? 8 : (n_rows >= 9 && n_rows <= 16) ? 16 : 0;
     const bool few = few_rows_layer(M, n_rows, lo);
-    if (c->stamps_on) {                                                     // the stamps of this pass replace the previous pass's
-        c->stamp_kinds.clear();
-        CUDA_TRY(cudaMemsetAsync(c->stamp_buf, 0xFF, sizeof(unsigned long long) * ST_WORDS * STAMP_CAP, st));
-    }
+    SD_TRY(begin_stamps(c));
     auto with_lora = [&](Epilogue& e, const Layer& L, int mat) {            // the adapters of this matrix, if the model has any
         if (!M.lora) return;
         e.lora_b = L.lora_b[mat]; e.lora_task = c->row_slot + SD_MAX_ROWS; e.lora_r = c->cfg.lora_rank; e.lora_n = c->cfg.lora_adapters;
@@ -830,8 +837,9 @@ sd_status forward_prefill(sd_ctx* c, Model& M, const PrefillSegs& segs) {
     const sd_model_desc& m = M.d;
     const int d = m.d_model, H = m.n_heads, Hkv = m.n_kv_heads, hd = m.head_dim, F = m.d_ffn, n = segs.rows, sm = sm_count();
     cudaStream_t st = c->st;
-    auto gemm = [&](const TensorMap& tw, const bf16* x, PrefillGemm& g) -> sd_status {
+    auto gemm = [&](const TensorMap& tw, const bf16* x, PrefillGemm& g, int kind) -> sd_status {
         TensorMap tx;
+        g.stamp = next_stamp(c, kind);
         if (!make_tensor_map_bf16(&tx, x, n, g.K, g.bn / 2)) return SD_ERR_CUDA;
         LAUNCH(CAT_LINEAR, launch_prefill_gemm(tw, tx, g, sm, c->S.status, st));
         return SD_OK;
@@ -841,7 +849,7 @@ sd_status forward_prefill(sd_ctx* c, Model& M, const PrefillSegs& segs) {
         if (!M.lora) return SD_OK;
         PrefillGemm t = prefill_geometry(PF_PARTIAL, n, g.n_out + 128, g.K, sm, 0, g.n_out / 256);
         t.part = c->pf_t; t.part_ld = 128; t.f_lo = g.n_out;
-        SD_TRY(gemm(tw, x, t));
+        SD_TRY(gemm(tw, x, t, SD_STAMP_GEMM | (EPI_PLAIN << 8)));
         g.lora_b = L.lora_b[mat]; g.lora_t = c->pf_t; g.lora_task = c->pf_task;
         g.lora_r = c->cfg.lora_rank; g.lora_n = c->cfg.lora_adapters; g.lora_scale = c->cfg.lora_scale;
         return SD_OK;
@@ -850,10 +858,12 @@ sd_status forward_prefill(sd_ctx* c, Model& M, const PrefillSegs& segs) {
         PrefillGemm g = prefill_geometry(PF_PARTIAL, n, d, K, sm, c->pf_rows);
         g.part = c->pf_part;
         SD_TRY(with_lora(tw, x, g, L, mat));
-        SD_TRY(gemm(tw, x, g));
-        LAUNCH(CAT_FUSED_STEP, launch_prefill_norm(c->pf_h, c->pf_part, g.split, n, d, gain, m.rms_eps, c->pf_xn, c->pf_scale, st));
+        SD_TRY(gemm(tw, x, g, SD_STAMP_GEMM | (EPI_RESIDUAL << 8)));
+        LAUNCH(CAT_FUSED_STEP, launch_prefill_norm(c->pf_h, c->pf_part, g.split, n, d, gain, m.rms_eps, c->pf_xn, c->pf_scale,
+                                                   next_stamp(c, SD_STAMP_STEP | (EPI_RESIDUAL << 8)), st));
         return SD_OK;
     };
+    SD_TRY(begin_stamps(c));
     LAUNCH(CAT_ELEMENTWISE, launch_prefill_embed(c->S, segs, (const bf16*)M.embed, d, m.vocab, M.layers[0].norm1, m.rms_eps, c->pf_h, c->pf_xn,
                                                  c->pf_scale, c->pf_slot, c->pf_pos, c->pf_task, st));
     for (int l = 0; l < m.n_layers; ++l) {
@@ -865,14 +875,14 @@ sd_status forward_prefill(sd_ctx* c, Model& M, const PrefillSegs& segs) {
         g.scale = c->pf_scale; g.q_out = c->pf_q; g.kc = kc; g.vc = vc; g.row_slot = c->pf_slot; g.row_pos = c->pf_pos;
         g.H = H; g.Hkv = Hkv; g.hd = hd; g.max_ctx = c->cfg.max_ctx; g.rcos = M.rope_cos; g.rsin = M.rope_sin;
         SD_TRY(with_lora(L.tm_qkv, c->pf_xn, g, L, SD_LORA_QKV));
-        SD_TRY(gemm(L.tm_qkv, c->pf_xn, g));
+        SD_TRY(gemm(L.tm_qkv, c->pf_xn, g, SD_STAMP_MATRIX | (EPI_QKV_ROPE << 8)));
         if (last) break;
-        LAUNCH(CAT_ATTENTION, launch_prefill_attention(c->pf_q, kc, vc, c->pf_attn, segs, H, Hkv, hd, c->cfg.max_ctx, st));
+        LAUNCH(CAT_ATTENTION, launch_prefill_attention(c->pf_q, kc, vc, c->pf_attn, segs, H, Hkv, hd, c->cfg.max_ctx, next_stamp(c, SD_STAMP_ATTENTION), st));
         SD_TRY(residual(L.tm_wo, c->pf_attn, H * hd, L.norm2, L, SD_LORA_WO));
         g = prefill_geometry(PF_SWIGLU, n, 2 * F, d, sm, 0);
         g.scale = c->pf_scale; g.act = c->pf_act; g.F = F;
         SD_TRY(with_lora(L.tm_gu, c->pf_xn, g, L, SD_LORA_GU));
-        SD_TRY(gemm(L.tm_gu, c->pf_xn, g));
+        SD_TRY(gemm(L.tm_gu, c->pf_xn, g, SD_STAMP_MATRIX | (EPI_SWIGLU << 8)));
         SD_TRY(residual(L.tm_wd, c->pf_act, F, M.layers[l + 1].norm1, L, SD_LORA_WD));
     }
     CUDA_TRY(prof_mark(c, CAT_NONE));

@@ -30,8 +30,9 @@ __device__ __forceinline__ uint4 ldg_stream(const bf16* p) {           // weight
     return v;
 }
 
-// W warps, NB 32-wide k blocks per warp, NT groups of eight token rows.
-template <int W, int NB, int NT>
+// W warps, NB 32-wide k blocks per warp, NT groups of eight token rows.  ST: with time stamps (as a test of the pointer they cost 0.1-0.2 us
+// per launch: 1B target's decoding step 367 -> 371 us).
+template <int W, int NB, int NT, bool ST>
 __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(const __grid_constant__ Gemv g) {
     constexpr int M = 8 * NT, PITCH = W + 4;                            // floats per (feature, row): the warps' sums, readable by fours
     __shared__ __align__(16) float red[16 * M * PITCH];
@@ -61,6 +62,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
             a1[b] = kb < KB && r1 < g.n_out ? ldg_stream(w1 + 32 * kb) : make_uint4(0, 0, 0, 0);
         }
     }
+    if (ST && tid == 0) stamp_first(ep.stamp, ST_START);                      // (behind the requests for the weights)
     // what the finishing threads need besides: their unit's features, gains, the rows' plan and rotary factors (written by the
     // pass's first kernel; the second one is launched in full stream order after it, every later one begins after that)
     const int ui = tid & 7, um = tid >> 3;                              // unit and token row this thread finishes
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
     if (mine && ep.lora_b) { task = __ldcg(ep.lora_task + um); if (task >= ep.lora_n) task = -1; }
 
     pdl_wait();                                                         // token rows, residual stream and sums of squares come from the kernels before
+    if (ST && tid == 0) stamp_pair(ep.stamp, ST_DEP_FIRST);
     float h0 = 0.f, h1 = 0.f;
     if (mine && ep.mode == EPI_RESIDUAL) { h0 = __ldcg(ep.h + (size_t)um * g.n_out + f0); h1 = __ldcg(ep.h + (size_t)um * g.n_out + f1); }
     float ss[(M + W - 1) / W];                                          // a warp per token row sums the row's pieces
@@ -213,12 +216,14 @@ __global__ void __launch_bounds__(32 * W, W == 8 && NT == 1 ? 3 : 1) k_gemv(cons
         break;
     }
     }
+    if (ST && tid == 0) stamp_pair(ep.stamp, ST_DONE_FIRST);
 }
 
 typedef void (*Kernel)(const Gemv);
-struct Form { int warps, blocks; Kernel one, two; };
-const Form FORMS[] = {{8, 3, k_gemv<8, 3, 1>, k_gemv<8, 3, 2>},   {8, 4, k_gemv<8, 4, 1>, k_gemv<8, 4, 2>},   {16, 4, k_gemv<16, 4, 1>, k_gemv<16, 4, 2>},
-                      {16, 6, k_gemv<16, 6, 1>, k_gemv<16, 6, 2>}, {16, 8, k_gemv<16, 8, 1>, k_gemv<16, 8, 2>}};
+struct Form { int warps, blocks; Kernel k[2][2]; };       // [two groups of rows][with time stamps]
+#define GEMV_FORM(W, NB) {W, NB, {{k_gemv<W, NB, 1, false>, k_gemv<W, NB, 1, true>}, {k_gemv<W, NB, 2, false>, k_gemv<W, NB, 2, true>}}}
+const Form FORMS[] = {GEMV_FORM(8, 3), GEMV_FORM(8, 4), GEMV_FORM(16, 4), GEMV_FORM(16, 6), GEMV_FORM(16, 8)};
+#undef GEMV_FORM
 
 const Form* form_of(int K) {
     for (const Form& f : FORMS) if (f.warps * f.blocks * 32 >= K) return &f;
@@ -241,7 +246,7 @@ cudaError_t launch_gemv(const Gemv& g, int dependent, cudaStream_t st) {
     if (!gemv_supported(g) || g.ep.lo_off < 0 || (g.ep.lo_off && g.ep.lo_off < g.rows)) return cudaErrorInvalidValue;
     if (g.ep.lora_b && (g.ep.lora_r < 8 || g.ep.lora_r > 32 || (g.ep.lora_r & 7) || g.ep.lora_n * g.ep.lora_r > 128 || !g.lora_t)) return cudaErrorInvalidValue;
     const Form* f = form_of(g.K);
-    return launch_pdl(g.rows <= 8 ? f->one : f->two, dim3((g.n_out + 15) / 16), dim3(32 * f->warps), 0, st, dependent, g);
+    return launch_pdl(f->k[g.rows > 8][g.ep.stamp != nullptr], dim3((g.n_out + 15) / 16), dim3(32 * f->warps), 0, st, dependent, g);
 }
 
 }  // namespace sd

@@ -119,8 +119,9 @@ __device__ __forceinline__ void add_lora(const PrefillGemm& g, int t0, int n, bo
     }
 }
 
-// Bound: tensor cores (hundreds of rows), or HBM when the rows are few.
-template <int MODE, bool LORA>
+// Bound: tensor cores (hundreds of rows), or HBM when the rows are few.  ST: with time stamps (as tests of the pointer they cost a prompt of
+// 17 rows 4 %: every kernel of a chain reads its parameters once more before its first load and after its last store).
+template <int MODE, bool LORA, bool ST>
 __global__ void __launch_bounds__(PF_THREADS, 1) __cluster_dims__(2, 1, 1)
 k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ PrefillGemm g, uint32_t* status) {
     extern __shared__ uint8_t dyn_smem[];
@@ -132,6 +133,7 @@ k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUte
     const uint32_t tiles0 = (smem_u32(dyn_smem) + 1023u) & ~1023u;
     const uint32_t x_bytes = (uint32_t)g.bn * 64u, stage_bytes = W_BYTES + x_bytes;      // half of the token rows x 128 bytes
     volatile int* abort_flag = &sh.abort_flag;
+    if (ST && threadIdx.x == 0) stamp_first(g.stamp, ST_START);
     uint32_t tmem_cols = 32;
     while (tmem_cols < 2u * (uint32_t)g.bn) tmem_cols <<= 1;
 
@@ -181,6 +183,7 @@ k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUte
                 const int ahead = min(g.stages, o.kb1 - o.kb0);
                 for (int j = 0; j < ahead; ++j) weights(o, kb + j, j);
                 pdl_wait();
+                if (ST && leader) stamp_pair(g.stamp, ST_DEP_FIRST);
                 waited = true;
                 for (int j = 0; j < ahead; ++j) rows(o, kb + j, j);
                 kb += ahead; s = ahead; done = ahead;
@@ -220,6 +223,7 @@ k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUte
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t da = desc0 + (uint64_t)((uint32_t)s * (stage_bytes >> 4)), db = da + (W_BYTES >> 4);
                     if (leader) {
+                        if (ST && it == pair && kb == o.kb0) stamp_pair(g.stamp, ST_DATA_FIRST);
 #pragma unroll
                         for (uint32_t k = 0; k < TILE_K / 16; ++k)
                             umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (uint32_t)(kb != o.kb0) | k);
@@ -369,6 +373,7 @@ k_pf_gemm(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUte
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (ST && threadIdx.x == 0) stamp_pair(g.stamp, ST_DONE_FIRST);
     if (sh.abort_flag) {
         if (threadIdx.x == 0 && status) atomicOr(status, SD_DEV_WAIT_EXPIRED);
         const uint64_t t0 = global_ns();                   // let copies in flight land before the CTA goes away
@@ -432,12 +437,16 @@ __global__ void __launch_bounds__(512) k_pf_embed(SeqState S, const __grid_const
 }
 
 // Bound: L2 (reads h and the pieces, writes h and half of that again).
+template <bool ST>
 __global__ void __launch_bounds__(512) k_pf_norm(float* __restrict__ h, const float* __restrict__ part, int split, int rows, int d,
-                                                 const float* __restrict__ gain, float eps, bf16* __restrict__ xn, float* __restrict__ scale) {
+                                                 const float* __restrict__ gain, float eps, bf16* __restrict__ xn, float* __restrict__ scale,
+                                                 unsigned long long* stamp) {
     __shared__ float red[32];
     pdl_launch_dependents();
     const int r = blockIdx.x;
+    if (ST && threadIdx.x == 0) stamp_first(stamp, ST_START);
     pdl_wait();
+    if (ST && threadIdx.x == 0) stamp_pair(stamp, ST_DEP_FIRST);
     float4 v[NORM_VECS];
 #pragma unroll
     for (int i = 0; i < NORM_VECS; ++i) {
@@ -455,6 +464,7 @@ __global__ void __launch_bounds__(512) k_pf_norm(float* __restrict__ h, const fl
         }
     }
     norm_row(v, d, gain, eps, xn + (size_t)r * d, scale + r, red);
+    if (ST && threadIdx.x == 0) stamp_pair(stamp, ST_DONE_FIRST);
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* gmem_src) {
@@ -478,13 +488,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // One CTA: 64 consecutive query rows of one run x one query head; a warp owns 16 rows.  The cache is walked in chunks of 64
 // positions up to the block's last row, double-buffered by 16-byte asynchronous copies into an XOR-swizzled layout.
 // Bound: latency of a block's chain of chunks (7B, 511 rows: eight chunks, 20 us).
-template <int HD>
+template <int HD, bool ST>
 __global__ void __launch_bounds__(128) k_pf_attention(const bf16* __restrict__ q, const bf16* __restrict__ kc, const bf16* __restrict__ vc, bf16* __restrict__ out,
-                                                      const __grid_constant__ PrefillSegs segs, int H, int Hkv, int max_ctx) {
+                                                      const __grid_constant__ PrefillSegs segs, int H, int Hkv, int max_ctx, unsigned long long* stamp) {
     constexpr int CK = 64, ROWB = HD * 2, CPR = HD / 8, KS = HD / 16, NV = HD / 8, BUF = CK * ROWB;
     extern __shared__ __align__(128) uint8_t sm_raw[];
     pdl_launch_dependents();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, gid = lane >> 2, tig = lane & 3;
+    if (ST && t == 0) stamp_first(stamp, ST_START);
     const uint32_t smem0 = smem_u32(sm_raw);
     const int blk = (int)gridDim.x - 1 - (int)blockIdx.x, head = blockIdx.y;      // a run's last rows see the most positions: they start first
     int s = 0;
@@ -512,6 +523,7 @@ __global__ void __launch_bounds__(128) k_pf_attention(const bf16* __restrict__ q
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     pdl_wait();
+    if (ST && t == 0) stamp_pair(stamp, ST_DEP_FIRST);
     issue(0);
     const int w0 = 16 * warp, i_lo = w0 + gid, i_hi = i_lo + 8;                   // this thread's two rows of the block
     const bool on_lo = i_lo < nr, on_hi = i_hi < nr;
@@ -614,6 +626,7 @@ __global__ void __launch_bounds__(128) k_pf_attention(const bf16* __restrict__ q
         if (on_lo) o_lo[4 * nv] = pack_bf16(O[nv][0] * inv_lo, O[nv][1] * inv_lo);
         if (on_hi) o_hi[4 * nv] = pack_bf16(O[nv][2] * inv_hi, O[nv][3] * inv_hi);
     }
+    if (ST && t == 0) stamp_pair(stamp, ST_DONE_FIRST);
 }
 
 }  // namespace
@@ -653,10 +666,12 @@ cudaError_t launch_prefill_gemm(const TensorMap& tm_w, const TensorMap& tm_x, co
     if (g.mode == PF_SWIGLU && (g.F % 64)) return cudaErrorInvalidValue;
     if (g.lora_b && (g.lora_r < 8 || g.lora_r > 32 || (g.lora_r & 7) || g.lora_n * g.lora_r > 128)) return cudaErrorInvalidValue;
     typedef void (*Kernel)(const CUtensorMap, const CUtensorMap, const PrefillGemm, uint32_t*);
-    static const Kernel kernels[2][3] = {{k_pf_gemm<PF_QKV, false>, k_pf_gemm<PF_SWIGLU, false>, k_pf_gemm<PF_PARTIAL, false>},
-                                         {k_pf_gemm<PF_QKV, true>, k_pf_gemm<PF_SWIGLU, true>, k_pf_gemm<PF_PARTIAL, true>}};
+    static const Kernel kernels[2][2][3] = {{{k_pf_gemm<PF_QKV, false, false>, k_pf_gemm<PF_SWIGLU, false, false>, k_pf_gemm<PF_PARTIAL, false, false>},
+                                             {k_pf_gemm<PF_QKV, true, false>, k_pf_gemm<PF_SWIGLU, true, false>, k_pf_gemm<PF_PARTIAL, true, false>}},
+                                            {{k_pf_gemm<PF_QKV, false, true>, k_pf_gemm<PF_SWIGLU, false, true>, k_pf_gemm<PF_PARTIAL, false, true>},
+                                             {k_pf_gemm<PF_QKV, true, true>, k_pf_gemm<PF_SWIGLU, true, true>, k_pf_gemm<PF_PARTIAL, true, true>}}};
     if (g.mode < 0 || g.mode > PF_PARTIAL) return cudaErrorInvalidValue;
-    const Kernel kern = kernels[g.lora_b ? 1 : 0][g.mode];
+    const Kernel kern = kernels[g.stamp ? 1 : 0][g.lora_b ? 1 : 0][g.mode];
     const size_t smem = (size_t)g.stages * (W_BYTES + g.bn * 64) + 1024;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_RING + 1024);
     if (e != cudaSuccess) return e;
@@ -671,19 +686,21 @@ cudaError_t launch_prefill_embed(const SeqState& S, const PrefillSegs& segs, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_prefill_norm(float* h, const float* part, int split, int rows, int d, const float* gain, float eps, bf16* xn, float* scale, cudaStream_t st) {
+cudaError_t launch_prefill_norm(float* h, const float* part, int split, int rows, int d, const float* gain, float eps, bf16* xn, float* scale,
+                                unsigned long long* stamp, cudaStream_t st) {
     if (norm_threads(d) > 512 || (d & 3)) return cudaErrorInvalidValue;
-    return launch_pdl(k_pf_norm, dim3(rows), dim3(norm_threads(d)), 0, st, 1, h, part, split, rows, d, gain, eps, xn, scale);
+    return launch_pdl(stamp ? k_pf_norm<true> : k_pf_norm<false>, dim3(rows), dim3(norm_threads(d)), 0, st, 1, h, part, split, rows, d, gain, eps, xn, scale, stamp);
 }
 
 cudaError_t launch_prefill_attention(const bf16* q, const bf16* kc, const bf16* vc, bf16* out, const PrefillSegs& segs, int H, int Hkv, int hd,
-                                     int max_ctx, cudaStream_t st) {
+                                     int max_ctx, unsigned long long* stamp, cudaStream_t st) {
     if (hd != 64 && hd != 128) return cudaErrorInvalidValue;
-    void (*kern)(const bf16*, const bf16*, const bf16*, bf16*, const PrefillSegs, int, int, int) = hd == 128 ? k_pf_attention<128> : k_pf_attention<64>;
+    void (*kern)(const bf16*, const bf16*, const bf16*, bf16*, const PrefillSegs, int, int, int, unsigned long long*) = hd == 128 ? (stamp ? k_pf_attention<128, true> : k_pf_attention<128, false>)
+                                                                              : (stamp ? k_pf_attention<64, true> : k_pf_attention<64, false>);
     const int smem = 4 * 64 * hd * 2;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, dim3(segs.blk0[segs.n], H), dim3(128), smem, st, 1, q, kc, vc, out, segs, H, Hkv, max_ctx);
+    return launch_pdl(kern, dim3(segs.blk0[segs.n], H), dim3(128), smem, st, 1, q, kc, vc, out, segs, H, Hkv, max_ctx, stamp);
 }
 
 }  // namespace sd

@@ -33,6 +33,7 @@ struct PrefillGemm {
     bf16* act; int F;
     // PF_PARTIAL: part[piece][row][part_ld], features from f_lo on
     float* part; int part_ld, f_lo;
+    unsigned long long* stamp;          // optional time stamps of the launch (see LaunchStamp)
     // Low-rank adapters (lora_b nullptr: none): lora_scale * sum_j t[row][task r + j] B[task][n][j] is added to output n (of the
     // first piece); t = X A^T comes from a launch of its own over the matrix's last 128 rows.
     const bf16* lora_b; const float* lora_t; const int32_t* lora_task; int lora_r, lora_n; float lora_scale;
@@ -45,9 +46,10 @@ cudaError_t launch_prefill_gemm(const TensorMap& tm_w, const TensorMap& tm_x, co
 cudaError_t launch_prefill_embed(const SeqState& S, const PrefillSegs& segs, const bf16* embed, int d, int vocab, const float* gain, float eps,
                                  float* h, bf16* xn, float* scale, int32_t* row_slot, int32_t* row_pos, int32_t* row_task, cudaStream_t st);
 // h += sum of the pieces (in their order); xn = bf16(h * gain), scale = 1/rms(h).
-cudaError_t launch_prefill_norm(float* h, const float* part, int split, int rows, int d, const float* gain, float eps, bf16* xn, float* scale, cudaStream_t st);
+cudaError_t launch_prefill_norm(float* h, const float* part, int split, int rows, int d, const float* gain, float eps, bf16* xn, float* scale,
+                                unsigned long long* stamp, cudaStream_t st);
 // Causal attention of the rows over their sequences' caches (the rows' own keys and values included).
 cudaError_t launch_prefill_attention(const bf16* q, const bf16* kc, const bf16* vc, bf16* out, const PrefillSegs& segs, int H, int Hkv, int hd,
-                                     int max_ctx, cudaStream_t st);
+                                     int max_ctx, unsigned long long* stamp, cudaStream_t st);
 
 }  // namespace sd
