@@ -16,14 +16,11 @@
 // One cooperative launch for the whole pass, with tagged words between CTAs, was no faster than the old path (24 us per layer:
 // a hand-over between 148 polling CTAs takes 1.5-2 us, a kernel boundary with the weights already in registers about 1.3).
 #include "gemv.h"
+#include "tc_ptx.cuh"
 
 namespace sd {
 namespace {
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 __device__ __forceinline__ uint4 ldg_stream(const bf16* p) {           // weights: read once
     uint4 v;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));

@@ -11,6 +11,7 @@
 #include <stdint.h>
 
 #include "../../include/sd.h"
+#include "f32x2.cuh"
 
 namespace sd {
 namespace {
@@ -23,14 +24,6 @@ constexpr __host__ __device__ int km_depth(int nv, int km) { return km == 8 || (
 constexpr __host__ __device__ int km_warps(int nv, int km) { return km == 4 && nv == 3 ? 12 : 8; }
 constexpr __host__ __device__ int km_per_sm(int nv, int km) { return km == 4 && nv >= 3 ? 1 : 2; }
 constexpr int KM_RUN = 128;            // points in one run of fp32 sums, where a warp keeps runs
-
-// Two fp32 values in one 64-bit register and the packed arithmetic of sm_100 on them: each instruction is two
-// independent IEEE operations (same results as the scalar forms), which halves the instructions per loaded byte.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) { f32x2 r; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-__device__ __forceinline__ float f2_hsum(f32x2 v) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); return a + b; }
 
 template <int NV, int KM>          // KM: compiled cluster bound (2, 4 or 8); up to 4 the centroids are kept in registers
 __global__ void __launch_bounds__(32 * km_warps(NV, KM), KM == 8 ? 1 : km_per_sm(NV, KM))

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "../../include/sd.h"
+#include "f32x2.cuh"
 
 namespace sd {
 namespace {
@@ -44,13 +45,6 @@ __global__ void k_mamba_tables(const ChunkRec* __restrict__ chunks, const int64_
         tok_row[ch.tok0 + i] = by_token ? tok : ch.tok0 + i;
     }
 }
-
-// Two fp32 values in one register pair and the packed multiply-add of sm_100 on them (two independent IEEE operations).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2_pack(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
-__device__ __forceinline__ float2 f2_unpack(f32x2 v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
 // u, z = split(W_in E[row]) for every row: token by token, or, when the prompts hold more tokens than the vocabulary has, once per
 // token of the vocabulary (the projection depends on nothing else).  Bound: fp32 multiply-adds (21,128 rows: 69 us; 109,096 token
