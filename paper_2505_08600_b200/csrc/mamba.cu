@@ -14,6 +14,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -325,11 +326,50 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
     }
 }
 
+// The pooled sums of long prompts: what the chunks' starting states add and the chunks' own sums, a thread per (channel, state) and a CTA
+// per eight channels instead of the head's one CTA per prompt, with the coefficients of eight chunks on their way at a time.  Bound: latency
+// of the chain over chunks.  One prompt of 4,000 / 30,000 / 200,000 tokens, whole call: 140 / 366 / 1,628 us,
+// in the head 203 / 869 / 6,758 (as kernels of their own, before: 275 / 802 / 4,757).  From eight chunks on a queue of shorter prompts is the slower
+// for the launch (100 prompts of 32...512 tokens: 323 against 319).
+constexpr int MB_LONG = 16;                              // chunks from which on a prompt is long
+constexpr int CARRY_CH = 8, CARRY_BATCH = 8;
+__global__ void __launch_bounds__(CARRY_CH * MB_MAX_N)
+k_mamba_carry(MambaDims m, const int32_t* __restrict__ prompt_chunk0, const double* __restrict__ chunk_sum, const float* __restrict__ end_state,
+              const float* __restrict__ decay, const float* __restrict__ carry_gain, double* __restrict__ g_sum /*[prompt][Di]*/) {
+    const int c0 = prompt_chunk0[blockIdx.x], c1 = prompt_chunk0[blockIdx.x + 1];
+    if (c1 - c0 < MB_LONG) return;
+    const int n = threadIdx.x % MB_MAX_N, c = blockIdx.y * CARRY_CH + threadIdx.x / MB_MAX_N;
+    const bool on = c < m.Di && n < m.N;
+    const size_t per = (size_t)m.Di * m.N, i = (size_t)min(c, m.Di - 1) * m.N + min(n, m.N - 1);
+    float s = on ? __ldg(end_state + c0 * per + i) : 0.f, add = 0.f;
+    for (int ch = c0 + 1; ch < c1; ch += CARRY_BATCH) {
+        float e[CARRY_BATCH], p[CARRY_BATCH], g[CARRY_BATCH];
+#pragma unroll
+        for (int b = 0; b < CARRY_BATCH; ++b) {
+            const bool in = on && ch + b < c1;
+            const size_t at = (size_t)(ch + b) * per + i;
+            e[b] = in ? __ldg(end_state + at) : 0.f; p[b] = in ? __ldg(decay + at) : 0.f; g[b] = in ? __ldg(carry_gain + at) : 0.f;
+        }
+#pragma unroll
+        for (int b = 0; b < CARRY_BATCH; ++b)
+            if (ch + b < c1) { add = fmaf(g[b], s, add); s = fmaf(p[b], s, e[b]); }
+    }
+    double sum = 0.0;
+    if (c < m.Di) {
+#pragma unroll 8
+        for (int ch = c0 + n; ch < c1; ch += MB_MAX_N) sum += __ldg(chunk_sum + (size_t)ch * m.Di + c);
+    }
+    sum += on ? (double)add : 0.0;
+#pragma unroll
+    for (int o = MB_MAX_N / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (n == 0 && c < m.Di) g_sum[(size_t)blockIdx.x * m.Di + c] = sum;
+}
+
 // Per prompt: the states its chunks start from (serial, a thread per channel and state), mean over tokens of the gated outputs
 // (chunks in order), W_out, the classification layer, argmax.
 __global__ void k_mamba_head(MambaDims m, const int32_t* __restrict__ prompt_chunk0, const int32_t* __restrict__ lens,
                              const double* __restrict__ chunk_sum, const float* __restrict__ end_state, const float* __restrict__ decay,
-                             const float* __restrict__ carry_gain, const float* __restrict__ w_out, const float* __restrict__ w_fc,
+                             const float* __restrict__ carry_gain, const double* __restrict__ g_sum /*of long prompts*/, const float* __restrict__ w_out, const float* __restrict__ w_fc,
                              const float* __restrict__ b_fc, float* __restrict__ scores, int32_t* __restrict__ labels) {
     extern __shared__ float hs[];                        // per (channel, state) what the starting states add [Di N], g mean [Di], pooled [D], scores [K]
     float* c_s = hs;
@@ -340,7 +380,8 @@ __global__ void k_mamba_head(MambaDims m, const int32_t* __restrict__ prompt_chu
     const int c0 = prompt_chunk0[pr], c1 = prompt_chunk0[pr + 1];
     const float inv = 1.f / (float)lens[pr];
     const size_t per = (size_t)m.Di * m.N;
-    if (c1 - c0 > 1)
+    const bool is_long = c1 - c0 >= MB_LONG;
+    if (c1 - c0 > 1 && !is_long)
         for (int i = threadIdx.x; i < m.Di * m.N; i += blockDim.x) {
             float s = end_state[c0 * per + i], add = 0.f;
 #pragma unroll 4
@@ -354,8 +395,9 @@ __global__ void k_mamba_head(MambaDims m, const int32_t* __restrict__ prompt_chu
     __syncthreads();
     for (int c = threadIdx.x; c < m.Di; c += blockDim.x) {
         double s = 0.0;
-        for (int ch = c0; ch < c1; ++ch) s += chunk_sum[(size_t)ch * m.Di + c];
-        if (c1 - c0 > 1) for (int n = 0; n < m.N; ++n) s += (double)c_s[c * m.N + n];
+        if (is_long) s = g_sum[(size_t)pr * m.Di + c];
+        else for (int ch = c0; ch < c1; ++ch) s += chunk_sum[(size_t)ch * m.Di + c];
+        if (c1 - c0 > 1 && !is_long) for (int n = 0; n < m.N; ++n) s += (double)c_s[c * m.N + n];
         g_s[c] = (float)s * inv;
     }
     __syncthreads();
@@ -449,6 +491,8 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
         }
     }
     prompt_chunk0[n_prompts] = (int32_t)chunks.size();
+    int longest = 0;                                         // chunks of a prompt
+    for (int i = 0; i < n_prompts; ++i) longest = std::max(longest, prompt_chunk0[i + 1] - prompt_chunk0[i]);
     const int64_t n_chunks = (int64_t)chunks.size();
     const Layout L = layout(m, T, T / MB_CHUNK + n_prompts, n_prompts);
     char* base = (char*)workspace_dev;
@@ -497,8 +541,14 @@ extern "C" sd_status sd_mamba_classify(const sd_mamba_desc* desc, const sd_mamba
                            w->a_log, w->d_skip, (float*)(base + L.end_state), (float*)(base + L.decay), (float*)(base + L.carry_gain),
                            (double*)(base + L.chunk_sum), w_staged, n_cta, per) != cudaSuccess)
         return SD_ERR_CUDA;
+    // (u and z are not read any more; their place, eight bytes per token and channel, holds eight per prompt and channel)
+    double* g_sum = (double*)(base + L.u);
+    if (longest >= MB_LONG)
+        k_mamba_carry<<<dim3((unsigned)n_prompts, (unsigned)((m.Di + CARRY_CH - 1) / CARRY_CH)), CARRY_CH * MB_MAX_N, 0, st>>>(
+            m, pc0, (const double*)(base + L.chunk_sum), (const float*)(base + L.end_state), (const float*)(base + L.decay),
+            (const float*)(base + L.carry_gain), g_sum);
     k_mamba_head<<<(unsigned)n_prompts, 1024, head_smem, st>>>(
         m, pc0, (const int32_t*)(base + L.lens), (const double*)(base + L.chunk_sum), (const float*)(base + L.end_state), (const float*)(base + L.decay),
-        (const float*)(base + L.carry_gain), w->w_out, w->w_fc, w->b_fc, scores_dev, labels_dev);
+        (const float*)(base + L.carry_gain), g_sum, w->w_out, w->w_fc, w->b_fc, scores_dev, labels_dev);
     return cudaGetLastError() == cudaSuccess ? SD_OK : SD_ERR_CUDA;
 }

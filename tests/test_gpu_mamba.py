@@ -143,3 +143,17 @@ def test_channels_of_several_ctas(sd, d_model, expand, d_state, d_conv):
     vocab = 200
     w = synth.make_mamba_classifier(vocab, d_model=d_model, d_state=d_state, d_conv=d_conv, expand=expand, n_classes=3, seed=12)
     _compare(sd, w, [1, 31, 33, 64, 150], vocab, seed=8)
+
+
+@pytest.mark.parametrize("d_model,expand,d_state,d_conv", [(64, 2, 16, 4), (37, 1, 5, 3), (300, 1, 8, 4)])
+def test_prompts_around_the_length_from_which_the_carry_has_a_kernel(sd, d_model, expand, d_state, d_conv):
+    """15, 16 and 17 chunks, and 40, beside short prompts; channels that do not fill a CTA's eight; a prompt's scores do not depend on its
+    neighbours' lengths."""
+    vocab = 300
+    w = synth.make_mamba_classifier(vocab, d_model=d_model, d_state=d_state, d_conv=d_conv, expand=expand, n_classes=4, seed=13)
+    lens = [960, 961, 1024, 1025, 2500, 30, 100]
+    scores, _ = _compare(sd, w, lens, vocab, seed=10)
+    clf = sd.MambaClassifier(w)
+    for i in (0, 1, 6):
+        alone, _ = clf.classify(torch.from_numpy(synth.make_prompt(vocab, lens[i], seed=10, seq=i)).to(DEV), [0], [lens[i]])
+        assert (alone.cpu().numpy()[0] == scores[i].astype(np.float32)).all()
