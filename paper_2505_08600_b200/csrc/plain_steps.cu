@@ -113,7 +113,11 @@ __global__ void __launch_bounds__(32 * PS_WARPS) k_plain_step(const __grid_const
 }
 
 // Attention of a few fp32 rows: a CTA per (row, query head), four lanes per key for the scores, as many groups of hd threads as
-// there are for the values.  The scores of the whole context sit in shared memory.
+// there are for the values.  The scores of the whole context sit in shared memory.  Bound: latency of the loads, so PA_KEYS keys per
+// lane and PA_VALUES values per thread are on their way at a time, and the four lanes of a key read whole sectors.  (Verify pass of a 2-layer, 256-
+// and 768-wide model, 5 rows, 8,000 positions: 614 and 928 us; one key and four values at a time, a quarter of a key per lane: 1,011 and 2,603;
+// the plain kernels 686 and 1,486.  64 positions, 256 wide: 57.6; 59.5; 61.5.)
+constexpr int PA_KEYS = 4, PA_VALUES = 16;
 __global__ void __launch_bounds__(256) k_plain_attention(const float* __restrict__ q, const float* __restrict__ kc, const float* __restrict__ vc, float* __restrict__ out,
                                                          const int32_t* __restrict__ row_slot, const int32_t* __restrict__ row_pos, int H, int Hkv, int hd, int max_ctx) {
     extern __shared__ __align__(16) float sm[];
@@ -135,22 +139,33 @@ __global__ void __launch_bounds__(256) k_plain_attention(const float* __restrict
     for (int i = t; i < hd; i += 256) qs[i] = __ldcg(q + ((size_t)r * H + h) * hd + i) * scale;
     __syncthreads();
     float mx = -INFINITY;
-    const int part = t & 3, dims = hd >> 2;               // hd is a multiple of 16
-    for (int p0 = 0; p0 < n; p0 += 64) {
-        const int p = p0 + (t >> 2);
-        float s = 0.f;
-        if (p < n) {
-            const float4* k4 = reinterpret_cast<const float4*>(K + (size_t)p * hd + part * dims);
-            const float4* q4 = reinterpret_cast<const float4*>(qs + part * dims);
-#pragma unroll 4
-            for (int i = 0; i < dims >> 2; ++i) {
-                const float4 a = __ldcg(k4 + i), b = q4[i];
-                s = fmaf(a.x, b.x, s); s = fmaf(a.y, b.y, s); s = fmaf(a.z, b.z, s); s = fmaf(a.w, b.w, s);
+    const int part = t & 3;
+    const float4* q4 = reinterpret_cast<const float4*>(qs);
+    for (int p0 = t >> 2; p0 < n; p0 += 64 * PA_KEYS) {   // (the four lanes of a key stay together)
+        float sk[PA_KEYS];
+#pragma unroll
+        for (int u = 0; u < PA_KEYS; ++u) sk[u] = 0.f;
+        for (int i = part; i < hd >> 2; i += 4) {         // hd is a multiple of 16
+            float4 k[PA_KEYS];
+#pragma unroll
+            for (int u = 0; u < PA_KEYS; ++u) {
+                const int p = p0 + 64 * u;
+                k[u] = p < n ? __ldcg(reinterpret_cast<const float4*>(K + (size_t)p * hd) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            const float4 b = q4[i];
+#pragma unroll
+            for (int u = 0; u < PA_KEYS; ++u) {
+                sk[u] = fmaf(k[u].x, b.x, sk[u]); sk[u] = fmaf(k[u].y, b.y, sk[u]); sk[u] = fmaf(k[u].z, b.z, sk[u]); sk[u] = fmaf(k[u].w, b.w, sk[u]);
             }
         }
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        s += __shfl_xor_sync(0xffffffffu, s, 2);
-        if (p < n) { if (part == 0) sc[p] = s; mx = fmaxf(mx, s); }
+        const unsigned four = 0xfu << (t & 28);
+#pragma unroll
+        for (int u = 0; u < PA_KEYS; ++u) {
+            sk[u] += __shfl_xor_sync(four, sk[u], 1);
+            sk[u] += __shfl_xor_sync(four, sk[u], 2);
+            const int p = p0 + 64 * u;
+            if (p < n) { if (part == 0) sc[p] = sk[u]; mx = fmaxf(mx, sk[u]); }
+        }
     }
     mx = block_max(mx, red);
     float den = 0.f;
@@ -159,8 +174,13 @@ __global__ void __launch_bounds__(256) k_plain_attention(const float* __restrict
     const int groups = 256 / hd, grp = t / hd, e = t % hd;
     float acc = 0.f;
     if (grp < groups) {
-#pragma unroll 4
-        for (int p = grp; p < n; p += groups) acc = fmaf(sc[p], __ldcg(V + (size_t)p * hd + e), acc);
+        for (int p0 = grp; p0 < n; p0 += groups * PA_VALUES) {
+            float v[PA_VALUES];
+#pragma unroll
+            for (int u = 0; u < PA_VALUES; ++u) { const int p = p0 + groups * u; v[u] = p < n ? __ldcg(V + (size_t)p * hd + e) : 0.f; }
+#pragma unroll
+            for (int u = 0; u < PA_VALUES; ++u) { const int p = p0 + groups * u; if (p < n) acc = fmaf(sc[p], v[u], acc); }
+        }
     }
     acc_s[t] = acc;
     __syncthreads();

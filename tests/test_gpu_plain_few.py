@@ -42,3 +42,26 @@ def test_verify_rows_follow_the_oracle(name, n_seq, gamma):
     for s in seqs:
         want = om.new_cache(128).forward(np.concatenate([toks[s], x[s]]), 0)[-(gamma + 1):]
         assert np.abs(got[s] - want).max() <= 1e-4, s          # logits of magnitude 1 over a few hundred fp32 terms per matrix
+
+
+@pytest.mark.parametrize("hd,H,Hkv", [(16, 4, 2), (64, 2, 2), (256, 1, 1)])
+def test_attention_over_long_contexts(hd, H, Hkv):
+    """Contexts around the keys (256) and values (16 per group of threads) that are on their way at a time, and several times that."""
+    from paper_2505_08600_b200 import binding
+    dims = dict(n_layers=1, d_model=64, n_heads=H, n_kv_heads=Hkv, head_dim=hd, d_ffn=64, vocab=211)
+    w = synth.make_weights(dims, seed=3, model_index=0, dtype="f32", std=0.2)
+    lens = [16, 65, 256, 257, 900]
+    om = oracle.OracleModel(dims, w)
+    ctx = binding.Context(dims, [dims], "f32", 1, 1000, 1, 1.0, 7)
+    ctx.load_weights(0, w); ctx.load_weights(1, w)
+    for m in lens:
+        toks, x = synth.make_prompt(211, m, seed=9, seq=m), np.array([[5]], dtype=np.int32)
+        ctx.sd_seq_begin(0, toks, 0)
+        ctx.sd_route_prompt([0], forced_task=[0])
+        ctx.sd_prefill([0])
+        logits = torch.zeros((1, 2, 211), dtype=torch.float32, device=DEV)
+        ctx.sd_verify([0], 1, torch.from_numpy(x).to(DEV), logits)
+        want = om.new_cache(1000).forward(np.concatenate([toks, x[0]]), 0)[-2:]
+        assert np.abs(logits.cpu().numpy()[0].astype(np.float64) - want).max() <= 1e-4 * max(1.0, np.abs(want).max()), m      # a few hundred fp32 terms
+    assert ctx.sd_device_status() == 0
+    ctx.close()
