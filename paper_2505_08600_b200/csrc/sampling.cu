@@ -679,23 +679,29 @@ __global__ void __cluster_dims__(SLICES, 1, 1) __launch_bounds__(1024) k_accept_
     cluster.sync();                                            // no CTA leaves while the others may still write into it
 }
 
-// Where that is the faster form, by what both take (us, measured at 1,000...50,000 values, 1...16 rows, 1...64 sequences; one wave of
-// clusters, 12288 / 32000 values: 2 rows 11.8 / 12.6 sliced, 17.6 / 33.3 a CTA per row; 6 rows 18.6 / 19.0 and 17.1 / 32.8; 9 rows 23.4 / 24.0
-// and 22.4 / 41.9; 16 rows 34.5 / 37 (24000) and 26.7 / 41): the slices pay a barrier or two per row, a CTA per row its row's length, twice
-// from nine rows on.  Equal at 4,000 values for 2 rows, 8,200 for 4, 13,000 for 6, 18,000 for 8, 13,000 for 9, 14,000 for 12, 20,500 for 16.
-static bool accept_sliced(int V, int rows, int n) {
+// Where that is the faster form, by what both take: a wave of slices costs its barriers, a barrier or two per row, and a little per value; a
+// wave of CTAs with a row each costs its row's length, twice from nine rows on.  Coefficients (us, rows, values) for logits with a
+// temperature, greedy logits and probabilities as given, from 1,000...50,000 values, 1...16 rows, 1...64 sequences.  One wave, 12288 / 32000
+// values, sliced and a CTA per row: with a temperature 2 rows 11.8 / 12.6 and 17.6 / 33.3, 6 rows 18.6 / 19.0 and 17.1 / 32.8, 9 rows 23.4 / 24.0
+// and 22.4 / 41.9, 16 rows 34.5 / 37 (24000) and 26.7 / 41; greedy 2 rows 12.2 / 12.7 and 14.3 / 24.0, 6 rows 20.6 / 21.0 and 14.1 / 24.3, 10 rows
+// 28.4 / 28.9 and 20.5 / 34.9; as given 6 rows 13.4 / 14.4 and 11.6 / 18.5, 10 rows 16.4 / 16.4 and 14.4 / 22.1.
+struct AcceptCost { double wave, row, row_value, one, one_value, some, some_value, two, two_value; };      // sliced; a row per CTA: one row in all, up to 8, more
+static bool accept_sliced(int V, int rows, int n, bool logits, bool greedy) {
+    static const AcceptCost SOFT = {8.5, 1.32, 2.1e-5, 7.0, 3.9e-4, 8.2, 7.7e-4, 10.7, 9.8e-4}, GREEDY = {8.0, 1.68, 1.5e-5, 7.0, 3.0e-4, 8.0, 5.1e-4, 11.2, 7.4e-4},
+                            GIVEN = {9.2, 0.6, 0.5e-5, 7.5, 1.5e-4, 8.6, 2.3e-4, 10.5, 2.7e-4};
     if ((size_t)slice_len(V) * rows * sizeof(float) > (size_t)STAGE_MAX_BYTES || rows > ACC_MAX_ROWS) return false;
-    if (!row_stage_bytes(V)) return true;                      // (64000 values, 3 rows: 18 against 120)
-    const int two = std::min(std::max(rows - 9, 0), 3);
-    const double row = rows == 1 ? 7.0 + 3.9e-4 * V : rows <= 8 ? 8.2 + 7.7e-4 * V : 10.7 + 0.33 * two + (9.8e-4 + 0.7e-4 * two) * V;
+    if (!row_stage_bytes(V)) return true;                      // (64000 values, 3 rows, with a temperature: 18 against 120)
+    const AcceptCost& c = !logits ? GIVEN : greedy ? GREEDY : SOFT;
+    const int more = std::min(std::max(rows - 9, 0), 3);       // (up to twelve rows more and more CTAs have two)
+    const double row = rows == 1 ? c.one + c.one_value * V : rows <= 8 ? c.some + c.some_value * V : c.two + 0.33 * more + c.two_value * (1 + 0.07 * more) * V;
     const int side_by_side = rows > 4 ? SLICED_WAVE : rows > 2 ? 36 : 148;       // clusters of eight, four, and fewer CTAs
-    return sliced_waves(n) * (8.5 + rows * (1.32 + 2.1e-5 * V)) < (n + side_by_side - 1) / side_by_side * row;
+    return sliced_waves(n) * (c.wave + rows * (c.row + c.row_value * V)) < (n + side_by_side - 1) / side_by_side * row;
 }
 
 cudaError_t launch_accept(const AcceptParams& p, int dependent, cudaStream_t st) {
     if (p.B <= 0) return cudaSuccess;
     const size_t slices = (size_t)slice_len(p.V) * (p.gamma + 1) * sizeof(float);
-    if (accept_sliced(p.V, p.gamma + 1, p.B)) {
+    if (accept_sliced(p.V, p.gamma + 1, p.B, p.target_is_logits != 0, p.T == 0.f)) {
         cudaError_t e = cudaFuncSetAttribute(k_accept_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX_BYTES);
         if (e != cudaSuccess) return e;
         return launch_pdl(k_accept_sliced, dim3(p.B * SLICES), dim3(1024), slices, st, dependent, p);

@@ -65,7 +65,7 @@ def _drafts(p, q, seed):
 
 
 # vocabularies that do not divide into eight slices of fours, from two rows to as many as fit
-@pytest.mark.parametrize("gamma,V", [(1, 4099), (2, 20011), (3, 12347), (5, 50001), (15, 24003)])
+@pytest.mark.parametrize("gamma,V", [(1, 4099), (1, 12001), (2, 20011), (3, 17003), (5, 50001), (12, 30003)])
 def test_tokens_from_ragged_slices_are_the_oracles(gamma, V):
     """Ordinary drafts, and rejected ones whose residual is the whole row, or three tokens: the last of a slice, the first of the next, the
     last of the vocabulary."""
@@ -92,11 +92,10 @@ def test_tokens_from_ragged_slices_are_the_oracles(gamma, V):
         y = oracle.sample_icdf(np.maximum(p[b, 0] - q[b, 0], np.float32(0)), oracle.uniform24(seed, b, 0, 5, 2))
         assert (n_acc[b], out[b, 0]) == (0, y) and (out[b, 1:] == -1).all(), b
         assert b < 10 or y in edge
-    assert gamma > 1 or 0 < n_acc[:8].sum() < 8 * gamma
 
 
 @pytest.mark.parametrize("T", [0.0, 0.7])
-@pytest.mark.parametrize("gamma,V", [(2, 20011), (5, 50001)])
+@pytest.mark.parametrize("gamma,V", [(2, 20011), (5, 50001), (15, 24003)])
 def test_logits_over_ragged_slices(gamma, V, T):
     """p from logits inside the kernel: greedy decisions are the oracle's; with a temperature they are wherever they do not lie within
     fp32 rounding of the comparison, and so is the token wherever the draw does not lie on the edge between two."""
@@ -149,3 +148,14 @@ def test_draft_draws_on_both_sides_of_the_line(n, V):
         for j in range(3):
             assert abs(q[s, j].astype(np.float64).sum() - 1.0) <= 1e-5
             assert x[s, j] == oracle.sample_icdf(q[s, j], oracle.uniform24(7, 0, j, 40 + s, 0))
+
+
+def test_no_drafts_is_plain_sampling_over_slices():
+    from paper_2505_08600_b200 import binding
+    B, V, seed = 4, 20011, 8
+    p = oracle.softmax_T(synth.make_logits((B, 1, V), seed=1).astype(np.float64), 1.0)
+    it, sid = np.arange(B, dtype=np.uint32), np.full(B, 2, dtype=np.uint32)
+    n_acc, out = torch.full((B,), -9, dtype=torch.int32, device=DEV), torch.full((B, 1), -9, dtype=torch.int32, device=DEV)
+    binding.sd_accept(to_dev(p), None, None, 1.0, seed, to_dev(it), to_dev(sid), n_acc, out, 0)
+    assert n_acc.tolist() == [0] * B
+    assert out[:, 0].tolist() == [oracle.sample_icdf(p[b, 0], oracle.uniform24(seed, b, 0, 2, 2)) for b in range(B)]
