@@ -10,6 +10,7 @@
 // fetched into shared memory once per CTA.)
 #include "gemm_tc.h"
 #include <algorithm>
+#include <type_traits>
 
 #include "plain_steps.h"
 
@@ -114,7 +115,8 @@ __global__ void __launch_bounds__(32 * PS_WARPS) k_plain_step(const __grid_const
 
 // Attention of a few fp32 rows: a CTA per (row, query head), four lanes per key for the scores, as many groups of hd threads as
 // there are for the values.  The scores of the whole context sit in shared memory.  Bound: latency of the loads, so PA_KEYS keys per
-// lane and PA_VALUES values per thread are on their way at a time, and the four lanes of a key read whole sectors.  (Verify pass of a 2-layer, 256-
+// lane (one up to 64 positions, with four parts of it) and PA_VALUES values per thread are on their way at a time, and the four lanes of a key
+// read whole sectors.  (Verify pass of a 2-layer, 256-
 // and 768-wide model, 5 rows, 8,000 positions: 614 and 928 us; one key and four values at a time, a quarter of a key per lane: 1,011 and 2,603;
 // the plain kernels 686 and 1,486.  64 positions, 256 wide: 57.6; 59.5; 61.5.)
 constexpr int PA_KEYS = 4, PA_VALUES = 16;
@@ -141,32 +143,38 @@ __global__ void __launch_bounds__(256) k_plain_attention(const float* __restrict
     float mx = -INFINITY;
     const int part = t & 3;
     const float4* q4 = reinterpret_cast<const float4*>(qs);
-    for (int p0 = t >> 2; p0 < n; p0 += 64 * PA_KEYS) {   // (the four lanes of a key stay together)
-        float sk[PA_KEYS];
+    auto scores = [&](auto keys) {
+        constexpr int KEYS = decltype(keys)::value;
+        for (int p0 = t >> 2; p0 < n; p0 += 64 * KEYS) {  // (the four lanes of a key stay together)
+            float sk[KEYS];
 #pragma unroll
-        for (int u = 0; u < PA_KEYS; ++u) sk[u] = 0.f;
-        for (int i = part; i < hd >> 2; i += 4) {         // hd is a multiple of 16
-            float4 k[PA_KEYS];
+            for (int u = 0; u < KEYS; ++u) sk[u] = 0.f;
+#pragma unroll 4
+            for (int i = part; i < hd >> 2; i += 4) {     // hd is a multiple of 16
+                float4 k[KEYS];
 #pragma unroll
-            for (int u = 0; u < PA_KEYS; ++u) {
+                for (int u = 0; u < KEYS; ++u) {
+                    const int p = p0 + 64 * u;
+                    k[u] = p < n ? __ldcg(reinterpret_cast<const float4*>(K + (size_t)p * hd) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                const float4 b = q4[i];
+#pragma unroll
+                for (int u = 0; u < KEYS; ++u) {
+                    sk[u] = fmaf(k[u].x, b.x, sk[u]); sk[u] = fmaf(k[u].y, b.y, sk[u]); sk[u] = fmaf(k[u].z, b.z, sk[u]); sk[u] = fmaf(k[u].w, b.w, sk[u]);
+                }
+            }
+            const unsigned four = 0xfu << (t & 28);
+#pragma unroll
+            for (int u = 0; u < KEYS; ++u) {
+                sk[u] += __shfl_xor_sync(four, sk[u], 1);
+                sk[u] += __shfl_xor_sync(four, sk[u], 2);
                 const int p = p0 + 64 * u;
-                k[u] = p < n ? __ldcg(reinterpret_cast<const float4*>(K + (size_t)p * hd) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            const float4 b = q4[i];
-#pragma unroll
-            for (int u = 0; u < PA_KEYS; ++u) {
-                sk[u] = fmaf(k[u].x, b.x, sk[u]); sk[u] = fmaf(k[u].y, b.y, sk[u]); sk[u] = fmaf(k[u].z, b.z, sk[u]); sk[u] = fmaf(k[u].w, b.w, sk[u]);
+                if (p < n) { if (part == 0) sc[p] = sk[u]; mx = fmaxf(mx, sk[u]); }
             }
         }
-        const unsigned four = 0xfu << (t & 28);
-#pragma unroll
-        for (int u = 0; u < PA_KEYS; ++u) {
-            sk[u] += __shfl_xor_sync(four, sk[u], 1);
-            sk[u] += __shfl_xor_sync(four, sk[u], 2);
-            const int p = p0 + 64 * u;
-            if (p < n) { if (part == 0) sc[p] = sk[u]; mx = fmaxf(mx, sk[u]); }
-        }
-    }
+    };
+    // (up to 64 positions a lane has one key: four would only wait for parts of it; iteration of the tiny pair at 33 positions 157 us with four, 151)
+    if (n <= 64) scores(std::integral_constant<int, 1>()); else scores(std::integral_constant<int, PA_KEYS>());
     mx = block_max(mx, red);
     float den = 0.f;
     for (int p = t; p < n; p += 256) { const float e = expf(sc[p] - mx); sc[p] = e; den += e; }
