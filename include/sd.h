@@ -363,10 +363,12 @@ sd_status sd_pass_schedule_check(const int32_t* shape12, const int32_t* waves, c
  * block, k blocks, matrix, flags, wait word, wait count, arrival word, workspace slot) and 20-byte task records. */
 size_t sd_pass_schedule_blob(const int32_t* shape12, const int32_t* waves, const int32_t* chunk_major, void* out, size_t cap);
 
-/* With 3..16 query rows (the verify rows of one sequence) the tensor-core path feeds every GEMM its input rows in two
- * bf16 parts, bf16(x) and bf16(x - bf16(x)), in the columns that the 16- or 32-wide MMA covers anyway: the weights stream
- * once all the same, and the activations enter the products with 16 bits of mantissa instead of 8.  on = 0 switches
- * that off (one bf16 part, as with other row counts); the tests measure both.  Synchronises, drops cached graphs. */
+/* With 3..16 query rows (the verify rows of one sequence; 1..16 in the passes of draft models whose matrices have at most
+ * 4096 inputs) the tensor-core path feeds every GEMM its input rows in two bf16 parts, bf16(x) and bf16(x - bf16(x)), in the
+ * columns that the MMA covers anyway: the weights stream once all the same, and the activations enter the products with 16
+ * bits of mantissa instead of 8.  Prompt rows are one part, except what a prompt has beyond a multiple of 256 rows when
+ * that is 3..16 rows.  on = 0 switches that off (one bf16 part, as with other row counts); the tests measure both.
+ * Synchronises, drops cached graphs. */
 sd_status sd_use_two_part_activations(sd_ctx* ctx, int on);
 
 /* Number of kernels this context has launched since sd_create. */

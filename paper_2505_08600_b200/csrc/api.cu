@@ -71,7 +71,10 @@ constexpr int PASS_ROWS_CAP = 32;               // most query rows of a pass on 
 constexpr size_t PASS_REGION_BYTES = (size_t)64 << 20;      // each of the two workspace regions of that kernel
 constexpr size_t PASS_PROG_BYTES = (size_t)768 << 10;       // one cached program
 constexpr int PASS_PROG_SLOTS = 8;
-constexpr int PF_MIN_ROWS = 17;                 // fewest rows of a prefill pass (prefill.cu); below, and sequence by sequence: forward().  One prompt of 20 rows: 1B 0.93 against 0.99 ms, 7B 3.57 against 3.69
+// Fewest rows of a prefill pass (prefill.cu); below, and sequence by sequence: forward().  Prompts of 17 / 32 / 64 rows, us: 1B 1,138 / 1,106 /
+// 1,151 against 1,182 / 1,200 / 1,307, eight layers of the 7B 1,217 / 1,182 / 1,250 against 1,347 / 1,368 / 1,494.  (One prompt of 3...16 rows does not
+// come here whatever the line: those rows go in two parts.)
+constexpr int PF_MIN_ROWS = 17;
 
 struct sd_ctx {
     sd_config cfg;

@@ -10,7 +10,7 @@
 //     both operands take them in the same order, so the order inside the MMA does not matter;
 //   - the warps split the reduction; their sums meet in shared memory, in warp order;
 //   - a tile is eight units of two features that the step needs together: a rotary pair, gate and up, or rows eight apart.
-// Measured (12-layer, 768-wide draft at 512 positions, one row): 27 -> 17.4 us per layer, of which attention takes 8-9; the 7B
+// Measured (12-layer, 768-wide draft at 512 positions, one row): 27 -> 17.4 us per layer, of which attention takes 5; the 7B
 // iteration 4.57 -> 4.05 ms, 16 sequences on four drafts 9.70 -> 7.22, one shared draft with adapters 5.39 -> 4.66.
 // Lines of the choice: at most 16 rows (two MMA column groups) and reductions of at most 4096 (the registers of 16 warps).
 // One cooperative launch for the whole pass, with tagged words between CTAs, was no faster than the old path (24 us per layer:

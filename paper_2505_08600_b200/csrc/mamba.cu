@@ -133,8 +133,8 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
 
 // Everything of one chunk between the input projection and the pooled sum.  Bound: exponentials (d_state of them per token and
 // channel) and the multiply-adds around them.  400 prompts of 109,096 tokens: 0.72 ms (convolution and projections 0.73 ms, two
-// scans 0.80 ms as kernels of their own, v, dt, B and C through memory in between); the whole call 2.26 -> 0.84 ms, its error
-// against 64 bits 1.2e-7 -> 1.1e-7.
+// scans 0.80 ms as kernels of their own, v, dt, B and C through memory in between); the whole call 2.28 -> 0.81 ms, the error of
+// its scores against 64 bits 1.8e-7 -> 1.7e-7.
 //   1. convolution + SiLU for MC_TILE tokens at a time into shared memory, from there the projections (r, B, C): a thread takes
 //      two tokens and every 16th output, three at a time;
 //   2. a thread per channel scans the chunk: convolution again (four multiply-adds are less than a trip through memory), step

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(1024) k_draft_sample(const float* __restrict__
 // The same over a cluster of eight CTAs per row, each with an eighth of the vocabulary in shared memory: a row of 32000 is 32
 // exponentials per thread for one CTA of 1024, four for eight CTAs of 1024.  What the slices have to know of one another (maximum,
 // sum, integer total) goes to every CTA of the cluster through distributed shared memory.  The token is the one of the integer
-// inverse CDF over the written fp32 values, whatever the split.  32000 values: 16 -> 11 us.
+// inverse CDF over the written fp32 values, whatever the split.  32000 values, five draft steps of a one-layer model: 210 -> 174 us.
 constexpr int SLICES = 8;
 __host__ __device__ __forceinline__ int slice_len(int V) { return (V + 4 * SLICES - 1) / (4 * SLICES) * 4; }
 // Rows whose clusters run side by side (a CTA of 1024 threads per SM, a cluster inside one GPC): 12 rows take one wave, 16 and 24 two, 32
@@ -525,7 +525,7 @@ __global__ void __launch_bounds__(1024) k_accept(AcceptParams P, int csize, int 
 
 // The same rule with the vocabulary cut over the cluster instead of the rows: every CTA holds an eighth of all gamma + 1 rows in
 // shared memory, so that each exponential is computed once and by eight times as many threads, and the draw from row n is
-// spread as well.  Taken when the slices fit (gamma + 1 rows of V / 8).  One sequence, gamma = 5, V = 32000: 33 -> 21 us
+// spread as well.  Taken when the slices fit (gamma + 1 rows of V / 8).  One sequence, gamma = 5, V = 32000: 33 -> 19 us
 // (1B iteration, five draws and one accept: 1.100 -> 1.058 ms).
 constexpr int ACC_MAX_ROWS = SD_MAX_GAMMA + 1;
 struct AcceptSliceScratch {
