@@ -251,7 +251,8 @@ int sd_best_gamma(double alpha, double c, int gamma_max, double* speedup_out);
  * 0 plain, 1 QKV+rotary, 2 residual, 3 SwiGLU) << 8; *n_out = records of the pass (may exceed cap).  Enabling changes
  * the captured graphs' keys: the first call afterwards captures anew.  With adapters a matrix of a pass of few rows, or
  * of a prompt pass, has a launch for x A^T in front, which has a record of its own (as SD_STAMP_MATRIX or SD_STAMP_GEMM
- * with step 0).  A few atomics per CTA: for measurement, off by default. */
+ * with step 0).  A draft layer that runs in two kernels fills two records: SD_STAMP_ATTENTION (with QKV and Wo) and
+ * SD_STAMP_MATRIX with step 3 (with the down matrix).  A few atomics per CTA: for measurement, off by default. */
 /* Sequences routed to different draft models run their draft passes side by side (default, when the context has two or
  * more separate draft models): every group after the first is enqueued on a stream of its own, forked from and joined
  * back to the context's stream, with its own scratch memory from the arena.  on = 0: group after group on the
