@@ -17,13 +17,16 @@ namespace sd {
 
 namespace {
 
-// Warps per CTA: eight when there are few CTAs (each finishes its slice sooner), four when there are several
-// per SM (three of them fit an SM, and one's set-up and merge overlap the others' streaming).
+// Warps per CTA: eight when there are few CTAs (each finishes its slice sooner), four when there are several per SM (three of them fit an
+// SM, and one's set-up and merge overlap the others' streaming); launch_attention_split has the rule between them.
 constexpr int WARPS_FEW = 8, WARPS_MANY = 4;
 constexpr int NQ = 16;              // query vectors per CTA (rows in the block x heads per KV head): one MMA row tile
 constexpr int SLICE_KEYS = 1024;    // a slice of the cache per CTA: up to this many positions
 constexpr int SLICE_KEYS_MANY = 2048; // ... when there are several CTAs per SM anyway (fewer set-ups and merges; 512...8192 swept)
 constexpr size_t ATTN_COUNTER_BYTES = 65536;     // one arrival counter per (query block, kv head)
+
+// 2^x, zero below the normal range (a weight that small is lost in its sum)
+__device__ __forceinline__ float exp2_ftz(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
 struct AttnParams {
     const bf16* q; const bf16* kc; const bf16* vc;
@@ -42,16 +45,20 @@ struct AttnParams {
 
 
 // One CTA = one slice of one KV head's cache x the query rows of one block (times the query
-// heads that share the KV head), as a 16-row tensor-core tile.  The slice is walked in chunks
-// of 64 keys, double-buffered in shared memory (16-byte asynchronous copies into an
-// XOR-swizzled layout that ldmatrix reads without bank conflicts); each warp owns 16 keys of a
-// chunk and keeps its own running max / sum / output (online softmax, exp2 domain), the warps
-// are merged at the end.  When there are few (head, row block, slice) items, two or four CTAs of
+// heads that share the KV head), as a 16-row tensor-core tile.  The slice is walked in chunks of
+// 16 keys per warp, double-buffered in shared memory (16-byte asynchronous copies into an
+// XOR-swizzled layout that ldmatrix reads without bank conflicts); each warp copies, reads and
+// scores its own 16 keys of a chunk and keeps its own running max / sum / output (online softmax,
+// exp2 domain), the warps are merged at the end.  When there are few (head, row block, slice) items, two or four CTAs of
 // a thread-block cluster share a slice and hand their results to the first one through
 // distributed shared memory.  A context of up to SLICE_KEYS positions is one slice, whose output
 // is written directly; longer contexts are cut into slices whose partial results are merged by
 // whichever slice arrives last.
-template <int HD, int NW>
+// Bound: HBM where the chip is full of CTAs (13B, contexts of 8,000), else a warp's chain through a chunk: scores, softmax, values.  So
+// the scores are two sums per tile, the output is scaled only when the largest score has grown, and EIGHT leaves out what belongs to
+// the tile's upper eight query vectors where there are none.  Iterations: 13B 13,050 -> 12,766 us, 7B of five sequences 4,602 -> 4,529,
+// decoding step of three 2,884 -> 2,815.  (Barriers between the warps at every chunk, or a third chunk on its way, make no difference.)
+template <int HD, int NW, bool EIGHT>
 __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     constexpr int NT = 32 * NW;              // threads; each warp takes 16 of the keys of a chunk
     constexpr int CK = 16 * NW;              // keys per chunk
@@ -61,6 +68,7 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     constexpr int KS = HD / 16;              // reduction steps of Q K^T
     constexpr int NV = HD / 8;               // 8-wide column tiles of the output
     constexpr int BUF = CK * ROWB;           // one chunk of keys (or values)
+    constexpr int E = EIGHT ? 2 : 4;         // values of a lane's score tile that are in use (EIGHT: at most eight query vectors, the tile's lower half)
     constexpr int OLD = HD + 8;              // padded row of the cross-warp merge buffer (floats)
     pdl_launch_dependents();
     if (threadIdx.x == 0) stamp_first(P.stamp, ST_START);
@@ -115,13 +123,14 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     }
     const bf16* K = P.kc + (((size_t)slot * P.Hkv + kvh) * P.max_ctx + max(p_begin, 0)) * HD;
     const bf16* V = P.vc + (((size_t)slot * P.Hkv + kvh) * P.max_ctx + max(p_begin, 0)) * HD;
-    // keys [k_lo, k_hi) of chunk c -> buffer c & 1: [K][V]; last: also clears the padding rows and closes the chunk
+    // This warp's share (its 16 keys) of keys [k_lo, k_hi) of chunk c -> buffer c & 1: [K][V]; last: also clears the padding rows and
+    // closes the chunk.  A warp reads what it copied itself, so that no warp waits for another until the merge.
     auto issue_part = [&](int c, int k_lo, int k_hi, bool last) {
             const int nk = min(CK, np - c * CK);
             const uint32_t kb = smem0 + (uint32_t)(c & 1) * 2u * BUF, vb = kb + BUF;
             const bf16* ks = K + (size_t)c * CK * HD;
             const bf16* vs = V + (size_t)c * CK * HD;
-            for (int i = k_lo * CPR + t; i < k_hi * CPR; i += NT) {
+            for (int i = max(k_lo, 16 * warp) * CPR + lane; i < min(k_hi, 16 * warp + 16) * CPR; i += 32) {
                 const int key = i / CPR, ch = i % CPR;
                 const uint32_t off = (uint32_t)key * ROWB + (uint32_t)((ch ^ (key & 7)) << 4);
                 cp_async16(kb + off, ks + (size_t)i * 8);
@@ -129,7 +138,7 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
             }
             // value rows past the end of the slice inside a warp's 16-key group must be finite (their weight is zero)
             const int nk16 = (nk + 15) & ~15;
-            for (int i = nk * CPR + t; last && i < nk16 * CPR; i += NT) {
+            for (int i = max(nk, 16 * warp) * CPR + lane; last && i < min(nk16, 16 * warp + 16) * CPR; i += 32) {
                 const int key = i / CPR, ch = i % CPR;
                 *reinterpret_cast<uint4*>(sm_raw + (size_t)(c & 1) * 2 * BUF + BUF + (size_t)key * ROWB + ((ch ^ (key & 7)) << 4)) = make_uint4(0, 0, 0, 0);
             }
@@ -149,9 +158,9 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
             a[ks][0] = j_lo < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_lo + 16 * ks + 2 * tig)) : 0u;
-            a[ks][1] = j_hi < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + 16 * ks + 2 * tig)) : 0u;
+            a[ks][1] = !EIGHT && j_hi < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + 16 * ks + 2 * tig)) : 0u;
             a[ks][2] = j_lo < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_lo + 16 * ks + 8 + 2 * tig)) : 0u;
-            a[ks][3] = j_hi < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + 16 * ks + 8 + 2 * tig)) : 0u;
+            a[ks][3] = !EIGHT && j_hi < nq ? __ldcg(reinterpret_cast<const uint32_t*>(q_hi + 16 * ks + 8 + 2 * tig)) : 0u;
         }
         const int pos_lo = j_lo < nq ? __ldcg(P.row_pos + r0 + j_lo / group) : -1;
         const int pos_hi = j_hi < nq ? __ldcg(P.row_pos + r0 + j_hi / group) : -1;
@@ -160,23 +169,26 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
         for (int c = 0; c < n_chunks; ++c) {
             if (c + 1 < n_chunks) { issue(c + 1); asm volatile("cp.async.wait_group 1;" ::: "memory"); }
             else asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncthreads();
+            __syncwarp();
             const int nk = min(CK, np - c * CK);
             if (16 * warp < nk) {
                 const uint32_t kb = smem0 + (uint32_t)(c & 1) * 2u * BUF, vb = kb + BUF;
-                float S[2][4];
+                float S[2][4], T[2][4];                      // (two sums, added below: the MMAs of one wait for one another)
 #pragma unroll
-                for (int i = 0; i < 2; ++i) { S[i][0] = S[i][1] = S[i][2] = S[i][3] = 0.f; }
+                for (int i = 0; i < 2; ++i) { S[i][0] = S[i][1] = S[i][2] = S[i][3] = 0.f; T[i][0] = T[i][1] = T[i][2] = T[i][3] = 0.f; }
                 {
                     const int mi = lane >> 3, r = lane & 7;
                     const int key = 16 * warp + 8 * (mi >> 1) + r;
                     const uint32_t rowaddr = kb + (uint32_t)key * ROWB;
 #pragma unroll
-                    for (int ks = 0; ks < KS; ++ks) {
-                        uint32_t b[4];
+                    for (int ks = 0; ks < KS; ks += 2) {
+                        uint32_t b[4], b2[4];
                         ldmatrix_x4(rowaddr + (uint32_t)(((2 * ks + (mi & 1)) ^ (key & 7)) << 4), b);
+                        ldmatrix_x4(rowaddr + (uint32_t)(((2 * ks + 2 + (mi & 1)) ^ (key & 7)) << 4), b2);
                         mma_bf16(S[0], a[ks], b[0], b[1]);
                         mma_bf16(S[1], a[ks], b[2], b[3]);
+                        mma_bf16(T[0], a[ks + 1], b2[0], b2[1]);
+                        mma_bf16(T[1], a[ks + 1], b2[2], b2[3]);
                     }
                 }
                 // scale, mask (past the slice, or after the row's own position), online softmax
@@ -185,41 +197,45 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
+                    for (int e = 0; e < E; ++e) {
                         const int p = pbase + 8 * nt + (e & 1);
                         const bool ok = (p - p_begin) < np && p <= ((e < 2) ? pos_lo : pos_hi);
-                        const float v = ok ? S[nt][e] * sl2 : -INFINITY;
+                        const float v = ok ? (S[nt][e] + T[nt][e]) * sl2 : -INFINITY;
                         S[nt][e] = v;
                         if (e < 2) mx_lo = fmaxf(mx_lo, v); else mx_hi = fmaxf(mx_hi, v);
                     }
                 mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1)); mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-                mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1)); mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
+                if (!EIGHT) { mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1)); mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2)); }
                 const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
-                const float c_lo = (mn_lo == -INFINITY) ? 1.f : exp2f(m_lo - mn_lo);
-                const float c_hi = (mn_hi == -INFINITY) ? 1.f : exp2f(m_hi - mn_hi);
-                m_lo = mn_lo; m_hi = mn_hi;
+                const bool grown = mn_lo > m_lo || (!EIGHT && mn_hi > m_hi);
+                // (nothing seen yet: any finite reference gives the weights zero that they have)
+                const float ref_lo = mn_lo == -INFINITY ? 0.f : mn_lo, ref_hi = mn_hi == -INFINITY ? 0.f : mn_hi;
                 float s_lo = 0.f, s_hi = 0.f;
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float mn = (e < 2) ? mn_lo : mn_hi;
-                        const float pr = (mn == -INFINITY) ? 0.f : exp2f(S[nt][e] - mn);
+                    for (int e = 0; e < E; ++e) {
+                        const float pr = exp2_ftz(S[nt][e] - (e < 2 ? ref_lo : ref_hi));
                         S[nt][e] = pr;
                         if (e < 2) s_lo += pr; else s_hi += pr;
                     }
-                l_lo = l_lo * c_lo + s_lo; l_hi = l_hi * c_hi + s_hi;
+                if (__any_sync(0xffffffffu, grown)) {        // (once the largest score has been seen, nothing is scaled any more)
+                    const float c_lo = exp2_ftz(m_lo - ref_lo), c_hi = EIGHT ? 1.f : exp2_ftz(m_hi - ref_hi);
+                    l_lo *= c_lo; l_hi *= c_hi;
+#pragma unroll
+                    for (int nv = 0; nv < NV; ++nv) { O[nv][0] *= c_lo; O[nv][1] *= c_lo; if (!EIGHT) { O[nv][2] *= c_hi; O[nv][3] *= c_hi; } }
+                }
+                m_lo = mn_lo; m_hi = mn_hi;
+                l_lo += s_lo; l_hi += s_hi;
                 uint32_t pa[4];
-                pa[0] = pack_bf16(S[0][0], S[0][1]); pa[1] = pack_bf16(S[0][2], S[0][3]);
-                pa[2] = pack_bf16(S[1][0], S[1][1]); pa[3] = pack_bf16(S[1][2], S[1][3]);
+                pa[0] = pack_bf16(S[0][0], S[0][1]); pa[1] = EIGHT ? 0u : pack_bf16(S[0][2], S[0][3]);
+                pa[2] = pack_bf16(S[1][0], S[1][1]); pa[3] = EIGHT ? 0u : pack_bf16(S[1][2], S[1][3]);
                 {
                     const int mi = lane >> 3, r = lane & 7;
                     const int key = 16 * warp + 8 * (mi & 1) + r;
                     const uint32_t rowaddr = vb + (uint32_t)key * ROWB;
 #pragma unroll
                     for (int nv = 0; nv < NV; nv += 2) {
-                        O[nv][0] *= c_lo; O[nv][1] *= c_lo; O[nv][2] *= c_hi; O[nv][3] *= c_hi;
-                        O[nv + 1][0] *= c_lo; O[nv + 1][1] *= c_lo; O[nv + 1][2] *= c_hi; O[nv + 1][3] *= c_hi;
                         uint32_t v[4];
                         ldmatrix_x4_trans(rowaddr + (uint32_t)(((nv + (mi >> 1)) ^ (key & 7)) << 4), v);
                         mma_bf16(O[nv], pa, v[0], v[1]);
@@ -227,7 +243,7 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
                     }
                 }
             }
-            __syncthreads();                     // the buffer may be refilled (or reused for the merge) from here on
+            __syncwarp();                        // the warp's part of the buffer may be refilled from here on
         }
         l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 1); l_lo += __shfl_xor_sync(0xffffffffu, l_lo, 2);
         l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 1); l_hi += __shfl_xor_sync(0xffffffffu, l_hi, 2);
@@ -237,6 +253,7 @@ __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     float* Ow = reinterpret_cast<float*>(sm_raw);                // [warps][16][OLD]
     float* mw = Ow + NW * NQ * OLD;                       // [warps][16]
     float* lw = mw + NW * NQ;                             // [warps][16]
+    __syncthreads();                                      // (in the place of the buffers)
     if (np > 0) {
 #pragma unroll
         for (int nv = 0; nv < NV; ++nv) {
@@ -481,8 +498,26 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
     // few (head, row block, slice) items: two or four CTAs of a cluster share each of them
     const int items = P.n_splits * Hkv * n_blocks;
     P.csize = items * 4 <= sm ? 4 : (items * 2 <= sm ? 2 : 1);
+    int nw = items > 2 * sm ? WARPS_MANY : WARPS_FEW;
+    if (P.csize == 1 && nw == WARPS_FEW) {
+        // A CTA of eight warps per SM, or three of four warps with up to four of them to an item?  By the longest chain of chunks, a CTA's
+        // set-up and merge counted as three of them and one of four warps' beside two others at 1.4; beyond one wave of the first form the
+        // second wave begins where the shortest items of the first end.  7B, one row, us per pass, eight warps / chosen: three contexts
+        // of 200...900 2,828 / 2,810, six of 300...500 2,964 / 2,888, eight of 128...256 2,896 / 2,828; where it stays with eight, four
+        // warps would take: five of 131...777 (four rows, drafts and target) 4,541 / 4,678.
+        const int n_seqs = n_rows / rows_per_seq, per_seq = items / n_seqs;
+        auto chunks = [&](int item, int keys, int parts) {           // of the item'th longest
+            const int len = P.use_order ? std::max(1, std::min(seq_len_hint[P.seq_order[std::min(item / per_seq, n_seqs - 1)]], ctx_bound)) : ctx_bound;
+            return ((len + P.n_splits * parts - 1) / (P.n_splits * parts) + keys - 1) / keys;
+        };
+        const double setup = 3.0;
+        double few = setup + chunks(0, 16 * WARPS_FEW, 1);
+        if (items > sm) few = std::max(few, 2 * setup + chunks(sm - 1, 16 * WARPS_FEW, 1) + chunks(sm, 16 * WARPS_FEW, 1));
+        const int c = items * 4 <= 3 * sm ? 4 : items * 2 <= 3 * sm ? 2 : 1;
+        if (setup + 1.4 * chunks(0, 16 * WARPS_MANY, c) < few) { nw = WARPS_MANY; P.csize = c; }
+    }
     if (max_cluster == 1 || max_cluster == 2) P.csize = std::min(P.csize, max_cluster);
-    const int nw = force_warps == WARPS_MANY || force_warps == WARPS_FEW ? force_warps : (items > 2 * sm ? WARPS_MANY : WARPS_FEW);
+    if (force_warps == WARPS_MANY || force_warps == WARPS_FEW) nw = force_warps;
     const size_t smem = std::max((size_t)4 * 16 * nw * hd * 2, sizeof(float) * ((size_t)nw * NQ * (hd + 8) + 2 * nw * NQ + (size_t)NQ * hd + 2 * NQ));
     dim3 grid(P.n_splits * P.csize, Hkv, n_blocks);
     cudaLaunchConfig_t cfg = {};
@@ -492,8 +527,10 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
     if (P.csize > 1) { attr[na].id = cudaLaunchAttributeClusterDimension; attr[na].val.clusterDim.x = P.csize; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1; ++na; }
     if (dependent) { attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization; attr[na].val.programmaticStreamSerializationAllowed = 1; ++na; }
     cfg.attrs = attr; cfg.numAttrs = na;
-    void (*kern)(AttnParams) = hd == 128 ? (nw == WARPS_MANY ? k_attn_mma<128, WARPS_MANY> : k_attn_mma<128, WARPS_FEW>)
-                                         : (nw == WARPS_MANY ? k_attn_mma<64, WARPS_MANY> : k_attn_mma<64, WARPS_FEW>);
+    typedef void (*Kernel)(AttnParams);
+    static const Kernel kernels[2][2][2] = {{{k_attn_mma<64, WARPS_FEW, false>, k_attn_mma<64, WARPS_FEW, true>}, {k_attn_mma<64, WARPS_MANY, false>, k_attn_mma<64, WARPS_MANY, true>}},
+                                            {{k_attn_mma<128, WARPS_FEW, false>, k_attn_mma<128, WARPS_FEW, true>}, {k_attn_mma<128, WARPS_MANY, false>, k_attn_mma<128, WARPS_MANY, true>}}};
+    const Kernel kern = kernels[hd == 128][nw == WARPS_MANY][P.rows_per_block * (H / Hkv) <= 8];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, kern, P);

@@ -1,0 +1,77 @@
+"""Attention over the cache in each form the launch picks (eight warps with clusters of four, two and one; four warps with clusters of four,
+two and one; at most eight query vectors per tile and more), against the CPU oracle: lengths that end a chunk, one more and one less,
+rows far from one another, an inactive row, a sequence of one position."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2505_08600_b200 import synth
+from gpu_util import DEV, quantize, to_dev, widen
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-2          # bf16 output rounding: 2^-9 relative on values up to ~3 (as in test_gpu_ops)
+
+
+# heads, kv heads, head dim, rows per sequence, last positions of the sequences
+FORMS = {
+    "8w_c4": (8, 8, 128, 6, [300]),
+    "8w_c2": (16, 16, 64, 6, [127, 128, 500, 6]),
+    "8w_c1": (40, 40, 128, 2, [60, 5, 127]),
+    "4w_c4": (32, 32, 128, 1, [899, 0, 255]),                       # 96 items, 384 CTAs
+    "4w_c4_gqa": (32, 8, 64, 4, [700, 63, 64, 65, 400, 33, 511, 512, 3, 640, 256, 90]),      # 96 items of 16 query vectors
+    "4w_c2": (32, 32, 128, 6, [400, 399, 401, 380, 350, 420]),       # 192 items
+    "4w_c1": (40, 40, 64, 8, [255, 254, 129, 128, 127, 200]),        # 240 items
+    "4w_many": (40, 40, 64, 9, [100, 64, 65, 63, 9, 120, 80, 127]),  # more than 2 per SM; nine query vectors
+    "slices": (16, 16, 128, 3, [2500, 1024, 2047]),                  # contexts cut into slices
+}
+
+
+@pytest.mark.parametrize("name", sorted(FORMS))
+def test_every_form_follows_the_oracle(name):
+    from paper_2505_08600_b200 import binding as sd
+    H, Hkv, hd, rps, last = FORMS[name]
+    max_ctx, n = max(last) + 1, len(last)
+    rng = np.random.default_rng(len(name))
+    q = quantize(synth.make_logits((n * rps, H, hd), seed=21, stream=hd), "bf16")
+    kc = quantize(synth.make_logits((n, Hkv, max_ctx, hd), seed=22, stream=hd), "bf16")
+    vc = quantize(synth.make_logits((n, Hkv, max_ctx, hd), seed=23, stream=hd), "bf16")
+    slots = np.repeat(np.arange(n, dtype=np.int32)[::-1], rps)
+    pos = np.concatenate([np.arange(p - rps + 1, p + 1) for p in last]).astype(np.int32)
+    pos[pos < 0] = -1                                               # (rows in front of a short sequence's first position are inactive)
+    out = torch.full((n * rps, H, hd), 7.0, dtype=torch.bfloat16, device=DEV)
+    args = (to_dev(q), to_dev(kc), to_dev(vc), out, to_dev(slots.copy()), to_dev(pos), H, Hkv, hd, max_ctx, sd.SD_BF16)
+    sd.sd_op_attention(*args, rows_per_seq=rps)
+    got = out.float().cpu().numpy().astype(np.float64)
+    qf, kf, vf = widen(q), widen(kc), widen(vc)
+    for r in range(n * rps):
+        for h in sorted({0, H - 1, *rng.integers(0, H, 2).tolist()}):
+            if pos[r] < 0:
+                assert (got[r, h] == 0).all()
+                continue
+            m = pos[r] + 1
+            ref = oracle.attention_head(qf[r, h], kf[slots[r], h // (H // Hkv), :m], vf[slots[r], h // (H // Hkv), :m])
+            np.testing.assert_allclose(got[r, h], ref, rtol=0, atol=TOL, err_msg=f"row {r} head {h}")
+    again = torch.zeros_like(out)
+    sd.sd_op_attention(*args[:3], again, *args[4:], rows_per_seq=rps)
+    assert torch.equal(out, again)
+
+
+def test_scores_that_grow_and_shrink_from_tile_to_tile():
+    """The running maximum moves in every tile, in none, and from far below: keys scaled up, down, and up at the very end."""
+    from paper_2505_08600_b200 import binding as sd
+    H, hd, m = 4, 128, 640
+    q = quantize(synth.make_logits((3, H, hd), seed=31, stream=1), "bf16")
+    base = synth.make_logits((3, H, m, hd), seed=32, stream=1)
+    for s, scale in enumerate([np.linspace(0.1, 6, m), np.linspace(6, 0.1, m), np.where(np.arange(m) < m - 1, 1e-3, 8.0)]):
+        base[s] *= scale[None, :, None]
+    kc, vc = quantize(base, "bf16"), quantize(synth.make_logits((3, H, m, hd), seed=33, stream=1), "bf16")
+    out = torch.zeros((3, H, hd), dtype=torch.bfloat16, device=DEV)
+    sd.sd_op_attention(to_dev(q), to_dev(kc), to_dev(vc), out, to_dev(np.arange(3, dtype=np.int32)), to_dev(np.full(3, m - 1, dtype=np.int32)), H, H, hd, m,
+                       sd.SD_BF16, rows_per_seq=1)
+    got = out.float().cpu().numpy().astype(np.float64)
+    qf, kf, vf = widen(q), widen(kc), widen(vc)
+    for s in range(3):
+        for h in range(H):
+            np.testing.assert_allclose(got[s, h], oracle.attention_head(qf[s, h], kf[s, h], vf[s, h]), rtol=0, atol=TOL)
