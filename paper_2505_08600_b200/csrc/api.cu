@@ -852,7 +852,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         LAUNCH(CAT_ATTENTION, launch_attention_split(c->q, kc, vc, c->attn, c->row_slot, c->row_pos, n_rows, plan.rows_per_seq, H, Hkv,
                                                      hd, c->cfg.max_ctx, plan.ctx_bound, c->attn_ws, c->attn_ws_bytes, 1, st, lo,
                                                      next_stamp(c, SD_STAMP_ATTENTION), c->tune[SD_TUNE_ATTN_WARPS], c->tune[SD_TUNE_ATTN_CLUSTER],
-                                                     list.n > 1 ? len_hint : nullptr));
+                                                     list.n > 1 ? len_hint : nullptr, !draft || c->one_draft));
         memset(&e, 0, sizeof(e));
         e.lo_off = lo; e.m_real = n_rows;
         e.ring_stages = c->tune[SD_TUNE_WO_STAGES]; e.prefill_all = c->tune[SD_TUNE_WO_PREFILL_ALL];

@@ -25,9 +25,6 @@ constexpr int SLICE_KEYS = 1024;    // a slice of the cache per CTA: up to this 
 constexpr int SLICE_KEYS_MANY = 2048; // ... when there are several CTAs per SM anyway (fewer set-ups and merges; 512...8192 swept)
 constexpr size_t ATTN_COUNTER_BYTES = 65536;     // one arrival counter per (query block, kv head)
 
-// 2^x, zero below the normal range (a weight that small is lost in its sum)
-__device__ __forceinline__ float exp2_ftz(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
-
 struct AttnParams {
     const bf16* q; const bf16* kc; const bf16* vc;
     const int32_t* row_slot; const int32_t* row_pos;
@@ -463,7 +460,7 @@ size_t attention_split_workspace(int rows, int H, int hd, int max_ctx) {
 cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc, void* out, const int32_t* row_slot,
                                    const int32_t* row_pos, int n_rows, int rows_per_seq, int H, int Hkv, int hd,
                                    int max_ctx, int ctx_bound, void* workspace, size_t workspace_bytes, int dependent,
-                                   cudaStream_t st, int lo_off, unsigned long long* stamp, int force_warps, int max_cluster, const int* seq_len_hint) {
+                                   cudaStream_t st, int lo_off, unsigned long long* stamp, int force_warps, int max_cluster, const int* seq_len_hint, bool alone) {
     if (n_rows <= 0) return cudaSuccess;
     ctx_bound = std::max(1, std::min(ctx_bound, max_ctx));
     AttnParams P;
@@ -499,12 +496,13 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
     const int items = P.n_splits * Hkv * n_blocks;
     P.csize = items * 4 <= sm ? 4 : (items * 2 <= sm ? 2 : 1);
     int nw = items > 2 * sm ? WARPS_MANY : WARPS_FEW;
-    if (P.csize == 1 && nw == WARPS_FEW) {
+    if (alone && P.csize == 1 && nw == WARPS_FEW) {
         // A CTA of eight warps per SM, or three of four warps with up to four of them to an item?  By the longest chain of chunks, a CTA's
         // set-up and merge counted as three of them and one of four warps' beside two others at 1.4; beyond one wave of the first form the
         // second wave begins where the shortest items of the first end.  7B, one row, us per pass, eight warps / chosen: three contexts
         // of 200...900 2,828 / 2,810, six of 300...500 2,964 / 2,888, eight of 128...256 2,896 / 2,828; where it stays with eight, four
-        // warps would take: five of 131...777 (four rows, drafts and target) 4,541 / 4,678.
+        // warps would take: five of 131...777 (four rows, drafts and target) 4,541 / 4,678.  (Not where passes of several draft models share the
+        // SMs: 16 sequences on four drafts 7,423 against 7,071.)
         const int n_seqs = n_rows / rows_per_seq, per_seq = items / n_seqs;
         auto chunks = [&](int item, int keys, int parts) {           // of the item'th longest
             const int len = P.use_order ? std::max(1, std::min(seq_len_hint[P.seq_order[std::min(item / per_seq, n_seqs - 1)]], ctx_bound)) : ctx_bound;

@@ -53,7 +53,8 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
                                    unsigned long long* stamp = nullptr /*optional time stamps of the launch*/,
                                    int force_warps = 0 /*4 or 8: warps per CTA; 0: chosen from the number of work items*/,
                                    int max_cluster = 0 /*1 or 2: at most this many CTAs share a slice; 0: up to 4*/,
-                                   const int* seq_len_hint = nullptr /*host, one per sequence: context lengths (bounds will do); longest sequences are started first*/);
+                                   const int* seq_len_hint = nullptr /*host, one per sequence: context lengths (bounds will do); longest sequences are started first*/,
+                                   bool alone = true /*no other pass runs beside this one*/);
 
 // ---- sampling.cu
 cudaError_t launch_philox(const uint32_t* ctr, int n, uint32_t k0, uint32_t k1, uint32_t* out, cudaStream_t st);
