@@ -9,6 +9,10 @@
 // Cache layout of one layer: [slot][kv_head][position][head_dim].
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <array>
+#include <functional>
+
 #include "gemm_tc.h"
 #include "kernels.h"
 #include "tc_ptx.cuh"
@@ -18,7 +22,7 @@ namespace sd {
 namespace {
 
 // Warps per CTA: eight when there are few CTAs (each finishes its slice sooner), four when there are several per SM (three of them fit an
-// SM, and one's set-up and merge overlap the others' streaming); launch_attention_split has the rule between them.
+// SM, and one's set-up and merge overlap the others' streaming); attention_split_form has the rule between them.
 constexpr int WARPS_FEW = 8, WARPS_MANY = 4;
 constexpr int NQ = 16;              // query vectors per CTA (rows in the block x heads per KV head): one MMA row tile
 constexpr int SLICE_KEYS = 1024;    // a slice of the cache per CTA: up to this many positions
@@ -453,6 +457,47 @@ size_t attention_split_workspace(int rows, int H, int hd, int max_ctx) {
     return ATTN_COUNTER_BYTES + sizeof(float) * (size_t)rows * H * n_splits * (hd + 2);
 }
 
+// How a launch shares out its work.  The results depend on it (keys are summed in another order), so whatever it is chosen by belongs into the
+// key of a captured graph: the number of rows, ctx_bound, and the sequences' lengths one by one, rounded up to multiples of LEN_STEP.
+constexpr int LEN_STEP = 256;
+AttnForm attention_split_form(int n_rows, int rows_per_seq, int H, int Hkv, int ctx_bound, const int* seq_len_hint, bool alone) {
+    const int n_seqs = n_rows / rows_per_seq, rows_per_block = std::max(1, std::min(rows_per_seq, NQ / (H / Hkv)));
+    const int blocks = n_seqs * ((rows_per_seq + rows_per_block - 1) / rows_per_block);
+    AttnForm f;
+    // one slice while the context is short (no cross-CTA merge at all), SLICE_KEYS positions per slice beyond
+    f.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS - 1) / SLICE_KEYS));
+    int sm = 148;
+    { int dev = 0; if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev); }
+    if (f.n_splits * Hkv * blocks > 2 * sm) f.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS_MANY - 1) / SLICE_KEYS_MANY));
+    // few (head, row block, slice) items: two or four CTAs of a cluster share each of them
+    const int items = f.n_splits * Hkv * blocks;
+    f.csize = items * 4 <= sm ? 4 : (items * 2 <= sm ? 2 : 1);
+    f.warps = items > 2 * sm ? WARPS_MANY : WARPS_FEW;
+    if (alone && f.csize == 1 && f.warps == WARPS_FEW) {
+        // A CTA of eight warps per SM, or three of four warps with up to four of them to an item?  By the longest chain of chunks, a CTA's
+        // set-up and merge counted as three of them and one of four warps' beside two others at 1.4; beyond one wave of the first form the
+        // second wave begins where the shortest items of the first end.  7B, one row, us per pass, eight warps / chosen: three contexts
+        // of 200...900 2,828 / 2,810, six of 300...500 2,964 / 2,888, eight of 128...256 2,896 / 2,828; where it stays with eight, four
+        // warps would take: five of 131...777 (four rows, drafts and target) 4,541 / 4,678.  (Not where passes of several draft models share the
+        // SMs: 16 sequences on four drafts 7,423 against 7,051.)
+        const int per_seq = items / n_seqs;
+        std::array<int, 64> len;                                     // longest first; without hints: all as long as the bound
+        const bool known = seq_len_hint && n_seqs <= 64;
+        for (int i = 0; known && i < n_seqs; ++i) len[i] = std::max(1, std::min((seq_len_hint[i] + LEN_STEP - 1) / LEN_STEP * LEN_STEP, ctx_bound));
+        if (known) std::sort(len.begin(), len.begin() + n_seqs, std::greater<int>());
+        auto chunks = [&](int item, int keys, int parts) {           // of the item'th longest
+            const int n = known ? len[std::min(item / per_seq, n_seqs - 1)] : ctx_bound;
+            return ((n + f.n_splits * parts - 1) / (f.n_splits * parts) + keys - 1) / keys;
+        };
+        const double setup = 3.0;
+        double few = setup + chunks(0, 16 * WARPS_FEW, 1);
+        if (items > sm) few = std::max(few, 2 * setup + chunks(sm - 1, 16 * WARPS_FEW, 1) + chunks(sm, 16 * WARPS_FEW, 1));
+        const int c = items * 4 <= 3 * sm ? 4 : items * 2 <= 3 * sm ? 2 : 1;
+        if (setup + 1.4 * chunks(0, 16 * WARPS_MANY, c) < few) { f.warps = WARPS_MANY; f.csize = c; }
+    }
+    return f;
+}
+
 // Rows come in runs of rows_per_seq consecutive rows of one sequence (n_rows is a multiple of it);
 // ctx_bound: no row sees a position >= ctx_bound (bounds the number of slices launched).
 // The first ATTN_COUNTER_BYTES of the workspace are arrival counters: zero before the first
@@ -480,42 +525,15 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
     P.rows_per_block = std::max(1, std::min(rows_per_seq, NQ / (H / Hkv)));
     const int bps = (rows_per_seq + P.rows_per_block - 1) / P.rows_per_block;
     const int n_blocks = (n_rows / rows_per_seq) * bps;
-    // one slice while the context is short (no cross-CTA merge at all), SLICE_KEYS positions per slice beyond
-    P.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS - 1) / SLICE_KEYS));
-    int sm = 148;
-    { int dev = 0; if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev); }
-    if (P.n_splits * Hkv * n_blocks > 2 * sm) {
-        P.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS_MANY - 1) / SLICE_KEYS_MANY));
-    }
+    const AttnForm form = attention_split_form(n_rows, rows_per_seq, H, Hkv, ctx_bound, seq_len_hint, alone);
+    P.n_splits = form.n_splits; P.csize = form.csize;
     const size_t need = ATTN_COUNTER_BYTES + sizeof(float) * (size_t)n_rows * H * P.n_splits * (hd + 2);
     if (need > workspace_bytes || (size_t)n_blocks * Hkv * sizeof(uint32_t) > ATTN_COUNTER_BYTES) return cudaErrorInvalidValue;
     P.counters = (uint32_t*)workspace;
     P.part_o = (float*)((char*)workspace + ATTN_COUNTER_BYTES);
     P.part_ml = P.part_o + (size_t)n_rows * H * P.n_splits * hd;
-    // few (head, row block, slice) items: two or four CTAs of a cluster share each of them
-    const int items = P.n_splits * Hkv * n_blocks;
-    P.csize = items * 4 <= sm ? 4 : (items * 2 <= sm ? 2 : 1);
-    int nw = items > 2 * sm ? WARPS_MANY : WARPS_FEW;
-    if (alone && P.csize == 1 && nw == WARPS_FEW) {
-        // A CTA of eight warps per SM, or three of four warps with up to four of them to an item?  By the longest chain of chunks, a CTA's
-        // set-up and merge counted as three of them and one of four warps' beside two others at 1.4; beyond one wave of the first form the
-        // second wave begins where the shortest items of the first end.  7B, one row, us per pass, eight warps / chosen: three contexts
-        // of 200...900 2,828 / 2,810, six of 300...500 2,964 / 2,888, eight of 128...256 2,896 / 2,828; where it stays with eight, four
-        // warps would take: five of 131...777 (four rows, drafts and target) 4,541 / 4,678.  (Not where passes of several draft models share the
-        // SMs: 16 sequences on four drafts 7,423 against 7,071.)
-        const int n_seqs = n_rows / rows_per_seq, per_seq = items / n_seqs;
-        auto chunks = [&](int item, int keys, int parts) {           // of the item'th longest
-            const int len = P.use_order ? std::max(1, std::min(seq_len_hint[P.seq_order[std::min(item / per_seq, n_seqs - 1)]], ctx_bound)) : ctx_bound;
-            return ((len + P.n_splits * parts - 1) / (P.n_splits * parts) + keys - 1) / keys;
-        };
-        const double setup = 3.0;
-        double few = setup + chunks(0, 16 * WARPS_FEW, 1);
-        if (items > sm) few = std::max(few, 2 * setup + chunks(sm - 1, 16 * WARPS_FEW, 1) + chunks(sm, 16 * WARPS_FEW, 1));
-        const int c = items * 4 <= 3 * sm ? 4 : items * 2 <= 3 * sm ? 2 : 1;
-        if (setup + 1.4 * chunks(0, 16 * WARPS_MANY, c) < few) { nw = WARPS_MANY; P.csize = c; }
-    }
     if (max_cluster == 1 || max_cluster == 2) P.csize = std::min(P.csize, max_cluster);
-    if (force_warps == WARPS_MANY || force_warps == WARPS_FEW) nw = force_warps;
+    const int nw = force_warps == WARPS_MANY || force_warps == WARPS_FEW ? force_warps : form.warps;
     const size_t smem = std::max((size_t)4 * 16 * nw * hd * 2, sizeof(float) * ((size_t)nw * NQ * (hd + 8) + 2 * nw * NQ + (size_t)NQ * hd + 2 * NQ));
     dim3 grid(P.n_splits * P.csize, Hkv, n_blocks);
     cudaLaunchConfig_t cfg = {};

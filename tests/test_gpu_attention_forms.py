@@ -75,3 +75,53 @@ def test_scores_that_grow_and_shrink_from_tile_to_tile():
     for s in range(3):
         for h in range(H):
             np.testing.assert_allclose(got[s, h], oracle.attention_head(qf[s, h], kf[s, h], vf[s, h]), rtol=0, atol=TOL)
+
+
+@pytest.mark.parametrize("call", ["draft", "verify", "step", "verify_accept"])
+def test_what_a_call_returns_does_not_depend_on_the_lengths_that_its_graph_was_captured_at(call):
+    """Attention's form follows the lengths of all sequences: the same five slots with one long context (eight warps), then with five (four warps in
+    clusters of two), the longest alike.  The second call returns bit for bit what it returns in a context that never saw the first, and without graphs."""
+    from paper_2505_08600_b200 import binding
+    V, gamma, seqs = 512, 3, list(range(5))
+    target = dict(n_layers=2, d_model=256, n_heads=32, n_kv_heads=32, head_dim=64, d_ffn=256, vocab=V)      # 160 (head, sequence) items
+    weights = [synth.make_weights(target, seed=3, model_index=k, dtype="bf16") for k in range(2)]
+
+    def results(ctx, lens):
+        for s in seqs:
+            ctx.sd_seq_begin(s, synth.make_prompt(V, lens[s], seed=9, seq=s), s)
+        ctx.sd_route_prompt(seqs, forced_task=[0] * 5)
+        ctx.sd_prefill(seqs)
+        if call == "draft":
+            ctx.sd_draft_steps(seqs, gamma, x, q)
+            return x.clone(), q.clone()
+        if call == "step":
+            ctx.sd_target_step(seqs, logits[:, 0])
+            return (logits.flatten()[: 5 * V].clone(),)
+        if call == "verify":
+            ctx.sd_verify(seqs, gamma, given, logits)
+        else:
+            ctx.sd_verify_accept(seqs, gamma, given, given_q, logits, n_acc, out_tok)
+        return logits.clone(), n_acc.clone(), out_tok.clone()
+
+    x, q = torch.zeros((5, gamma), dtype=torch.int32, device=DEV), torch.zeros((5, gamma, V), device=DEV)
+    given, given_q = torch.full((5, gamma), 7, dtype=torch.int32, device=DEV), torch.full((5, gamma, V), 1.0 / V, device=DEV)
+    logits, n_acc, out_tok = torch.zeros((5, gamma + 1, V), device=DEV), torch.zeros(5, dtype=torch.int32, device=DEV), torch.zeros((5, gamma + 1), dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    mixed, alike = [900, 40, 40, 40, 40], [900] * 5
+    got = []
+    for graphs, first in ((1, mixed), (1, None), (0, None)):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            ctx = binding.Context(target, [target], "bf16", 5, 1024, gamma, 1.0, 7, stream=stream)
+            for k in range(2):
+                ctx.load_weights(k, weights[k])
+            ctx.sd_use_graphs(graphs)
+            if first:
+                results(ctx, first)
+            got.append(results(ctx, alike))
+            assert ctx.sd_device_status() == 0
+            ctx.close()
+        torch.cuda.synchronize()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert torch.equal(a, b)
