@@ -106,3 +106,54 @@ def test_an_iteration_after_full_and_partial_acceptance():
         ctx.sd_kv_rollback([0, 1], gamma, torch.tensor(accepted, dtype=torch.int32, device=DEV), torch.from_numpy(out).to(DEV))
     assert ctx.sd_device_status() == 0
     ctx.close()
+
+
+# ---- what the tests above cannot see: their weights give nearly even attention and logits of a few hundredths, some of their shapes are beyond these
+#      kernels, and none asks which kernels ran
+
+CLUSTER_LAYER, FEW_ROWS_LAYER = [2, 3 | 3 << 8], [3 | 1 << 8, 2, 3 | 2 << 8, 3 | 3 << 8, 3 | 2 << 8]      # records of a layer: attention, matrix (QKV 1, residual 2, SwiGLU 3)
+DEEP = {
+    "d448": (_m(6, 448, 3, 384), True),             # 14 k blocks for 16 warps, 7 tiles, 128 features
+    "d512_f576": (_m(6, 512, 8, 576), True),        # clusters of 192 features, the form for up to 512 columns
+    "d768": (_m(3, 768, 12, 3072), True),           # ... 768
+    "d1024_f3072": (_m(3, 1024, 16, 3072), True),   # ... 1,024: as large as it goes
+    "d1024_f2048": (_m(3, 1024, 16, 2048), True),   # 128 features, 1,024 columns, 32 clusters
+    "d1024_f4096": (_m(3, 1024, 16, 4096), False),  # 48 clusters: one kernel per matrix
+}
+
+
+@pytest.mark.parametrize("n_seq", [1, 2, 4, 5, 6])
+@pytest.mark.parametrize("name", sorted(DEEP))
+def test_the_kernels_that_are_meant_run_and_follow_the_oracle(name, n_seq):
+    """Weights that keep every activation near one; which records a pass leaves tells the kernels apart (six layers: up to six sequences)."""
+    from paper_2505_08600_b200 import binding
+    (draft, fits), target, gamma = DEEP[name], _m(1, 64, 1, 64), 2
+    wt = synth.make_weights(target, seed=3, model_index=0, dtype="bf16")
+    wd = synth.make_weights(draft, seed=3, model_index=1, dtype="bf16", std=draft["d_model"] ** -0.5)
+    seqs = list(range(n_seq))
+    ctx = binding.Context(target, [draft], "bf16", n_seq, 96, gamma, 1.0, 7, stream=torch.cuda.Stream())
+    ctx.load_weights(0, wt); ctx.load_weights(1, wd)
+    toks = [synth.make_prompt(V, 7 + 9 * i, seed=9, seq=i) for i in seqs]
+    for s in seqs:
+        ctx.sd_seq_begin(s, toks[s], s)
+    ctx.sd_route_prompt(seqs, forced_task=[0] * n_seq)
+    ctx.sd_prefill(seqs)
+    x, q = torch.zeros((n_seq, gamma), dtype=torch.int32, device=DEV), torch.zeros((n_seq, gamma, V), device=DEV)
+    torch.cuda.synchronize()
+    ctx.sd_launch_stamps(1)
+    clusters = fits and (n_seq <= 4 or draft["n_layers"] >= 6)
+    for _ in range(2):                                                     # captured, replayed
+        ctx.sd_draft_steps(seqs, gamma, x, q)
+        stamps, kinds = ctx.sd_launch_stamps_read()
+        assert kinds.tolist() == draft["n_layers"] * (CLUSTER_LAYER if clusters else FEW_ROWS_LAYER) + [3]
+        t = stamps.astype(np.int64)
+        assert (t[:, [0, 1, 5]] > 0).all() and (t[:, 0] <= t[:, 1]).all() and (t[:, 1] <= t[:, 5]).all()
+    assert ctx.sd_device_status() == 0
+    xg, qg = x.cpu().numpy(), q.cpu().numpy().astype(np.float64)
+    ctx.close()
+    om = oracle.OracleModel(draft, wd)
+    for s in seqs:
+        logits = om.new_cache(128).forward(np.concatenate([toks[s], xg[s, :-1]]), 0)[-gamma:]
+        top = logits.max(axis=1, keepdims=True)
+        want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
+        assert np.abs(np.log(np.maximum(qg[s], 1e-30)) - want).max() <= LOG_TOL, s
