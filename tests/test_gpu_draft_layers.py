@@ -157,3 +157,83 @@ def test_the_kernels_that_are_meant_run_and_follow_the_oracle(name, n_seq):
         top = logits.max(axis=1, keepdims=True)
         want = logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
         assert np.abs(np.log(np.maximum(qg[s], 1e-30)) - want).max() <= LOG_TOL, s
+
+
+NEEDLE = 5
+
+
+def _needle_model(n_layers):
+    """Every query scores the token NEEDLE 14 (in the softmax's exponent) above all others, wherever it stands: feature 0 marks it, feature 1 is one for
+    every token, and both meet in the head's slowest rotary pair.  Its value is nearly the whole of the first layer's output; the other layers add nothing."""
+    dims = _m(n_layers, 128, 2, 128)
+    rng = np.random.default_rng(77)
+    w = synth.make_weights(dims, seed=3, model_index=1, dtype="f32")
+    w["embed"] = rng.standard_normal((V, 128), dtype=np.float32)
+    w["embed"][:, 0], w["embed"][:, 1] = 0.0, 1.0
+    w["embed"][NEEDLE, 0] = 8.0
+    w["lm_head"] = rng.standard_normal((V, 128), dtype=np.float32) * 0.2
+    for l in range(n_layers):
+        for name in ("wq", "wk", "wd", "wo"):
+            w[name][l] = np.zeros_like(w[name][l])
+    for h in range(2):
+        w["wq"][0][64 * h + 31, 1] = 4.2
+        w["wk"][0][64 * h + 31, 0] = 4.2
+    w["wv"][0] = rng.standard_normal(w["wv"][0].shape, dtype=np.float32) * 0.1
+    w["wo"][0] = rng.standard_normal(w["wo"][0].shape, dtype=np.float32) * 0.1
+    f32 = ("final_norm", "norm1", "norm2")
+    return dims, {k: v if k in f32 else [synth.f32_to_bf16_bits(a) for a in v] if isinstance(v, list) else synth.f32_to_bf16_bits(v) for k, v in w.items()}
+
+
+def _log_q(om, tokens, n):
+    logits = om.new_cache(len(tokens) + 1).forward(np.asarray(tokens, dtype=np.int32), 0)[-n:]
+    top = logits.max(axis=1, keepdims=True)
+    return logits - top - np.log(np.exp(logits - top).sum(axis=1, keepdims=True))
+
+
+# one position of every 16-key tile (of every fourth in the longest context); four contexts at once: every warp's share
+@pytest.mark.parametrize("lens", [[17], [33], [333], [513], [2049], [400, 15, 31, 333]], ids=str)
+def test_no_tile_of_the_cache_is_lost(lens):
+    from paper_2505_08600_b200 import binding
+    dims, wd = _needle_model(1 if len(lens) == 1 else 3)
+    target, gamma, n = _m(1, 64, 1, 64), 2, len(lens)
+    om = oracle.OracleModel(dims, wd)
+    stride = 64 if max(lens) > 1024 else 16
+    seqs = list(range(n))
+    ctx = binding.Context(target, [dims], "bf16", n, max(lens) + 8, gamma, 1.0, 7, stream=torch.cuda.Stream())
+    ctx.load_weights(0, synth.make_weights(target, seed=3, model_index=0, dtype="bf16")); ctx.load_weights(1, wd)
+    x, q = torch.zeros((n, gamma), dtype=torch.int32, device=DEV), torch.zeros((n, gamma, V), device=DEV)
+    torch.cuda.synchronize()
+    ctx.sd_launch_stamps(1)
+    rng = np.random.default_rng(3)
+    for k in range((max(lens) + stride - 1) // stride):
+        toks = []
+        for m in lens:
+            t = synth.make_prompt(V, m, seed=9, seq=k)
+            t[t == NEEDLE] = NEEDLE + 1
+            t[(k * stride + int(rng.integers(0, 16))) % m] = NEEDLE
+            toks.append(t)
+        for s in seqs:
+            ctx.sd_seq_begin(s, toks[s], s)
+        ctx.sd_route_prompt(seqs, forced_task=[0] * n)
+        ctx.sd_prefill(seqs)
+        ctx.sd_draft_steps(seqs, gamma, x, q)
+        torch.cuda.synchronize()
+        xg, got = x.cpu().numpy(), np.log(np.maximum(q.cpu().numpy().astype(np.float64), 1e-30))
+        for s in seqs:
+            whole = np.concatenate([toks[s], xg[s, :-1]])
+            assert np.abs(got[s] - _log_q(om, whole, gamma)).max() <= LOG_TOL, (k, s)
+    assert ctx.sd_launch_stamps_read()[1].tolist() == dims["n_layers"] * CLUSTER_LAYER + [3]
+    assert ctx.sd_device_status() == 0
+    ctx.close()
+
+
+def test_the_needle_is_seen_by_the_oracle():
+    """Without it the result is elsewhere by far more than the tolerance."""
+    dims, wd = _needle_model(1)
+    om = oracle.OracleModel(dims, wd)
+    for m in (17, 513):
+        t = synth.make_prompt(V, m, seed=9, seq=0)
+        t[t == NEEDLE] = NEEDLE + 1
+        with_it = t.copy()
+        with_it[m // 3] = NEEDLE
+        assert np.abs(_log_q(om, t, 1) - _log_q(om, with_it, 1)).max() > 10 * LOG_TOL
