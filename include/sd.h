@@ -463,7 +463,7 @@ size_t sd_op_attention_workspace(int rows, int n_heads, int head_dim, int max_ct
  * (d_conv taps, zeros before the prompt) + SiLU, input-dependent (dt, B, C) with dt = softplus(W_dt r + b_dt),
  * h_t = exp(dt_t A) h_{t-1} + dt_t v_t B_t with A = -exp(a_log), y_t = h_t C_t + d_skip v_t, gate silu(z_t), output
  * projection; no residual connection, no normalisation.  All weights fp32, row-major, DEVICE pointers owned by the
- * caller (read during the call only):
+ * caller:
  *   embed [vocab][d_model]   w_in [2*Di][d_model] (u rows first, then z), Di = expand * d_model
  *   w_conv [Di][d_conv]  b_conv [Di]   w_x [dt_rank + 2*d_state][Di] (r, B, C rows)   w_dt [Di][dt_rank]  b_dt [Di]
  *   a_log [Di][d_state]  d_skip [Di]   w_out [d_model][Di]   w_fc [n_classes][d_model]  b_fc [n_classes]
@@ -472,8 +472,10 @@ size_t sd_op_attention_workspace(int rows, int n_heads, int head_dim, int max_ct
  * fp32 and labels_dev [n_prompts] int32 (argmax, lowest index on ties) are device buffers, either may be NULL.
  * workspace_dev: sd_mamba_workspace(desc, sum of lengths, n_prompts) bytes of device memory at a multiple of 8 bytes
  * (at a multiple of 16 it is written by fours).  Long prompts are scanned in chunks side by side.  Limits: d_state <= 16, d_conv <= 8, d_model <= 512, Di <= 1024 (else SD_ERR_UNSUPPORTED).
- * Copies small host tables to the device and synchronises the stream once before launching; the launches are
- * asynchronous on cuda_stream. */
+ * Everything is asynchronous on cuda_stream and the call waits for nothing: desc, starts_host and lens_host have been read
+ * when it returns; weights, tokens, workspace and outputs have to stay as they are until the stream has passed the
+ * call.  On a stream that is being captured it returns SD_ERR_CUDA and launches nothing (the offsets and lengths are
+ * parameters of the launches: every replay would classify the prompts of this call). */
 typedef struct { int32_t vocab, d_model, d_state, d_conv, expand, n_classes, dt_rank; } sd_mamba_desc;
 typedef struct {
     const float *embed, *w_in, *w_conv, *b_conv, *w_x, *w_dt, *b_dt, *a_log, *d_skip, *w_out, *w_fc, *b_fc;

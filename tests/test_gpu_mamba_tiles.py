@@ -53,3 +53,21 @@ def test_a_capture_is_refused():
         with torch.cuda.graph(graph):
             clf.classify(tokens, [0], [8])
     torch.cuda.synchronize()
+
+
+def test_the_call_waits_for_nothing_and_has_read_its_host_tables():
+    """Offsets and lengths are overwritten as soon as the call returns, before the stream (held up for some ten milliseconds) has come to it."""
+    from paper_2505_08600_b200 import binding as sd
+    clf = sd.MambaClassifier(synth.make_mamba_classifier(90, d_model=32, d_state=4, d_conv=4, expand=1, n_classes=3, seed=2))
+    for n in (3, 40):                                            # a table of up to 32 prompts, a longer one
+        lens = np.array([5 + 31 * (i % 5) for i in range(n)], dtype=np.int32)
+        starts = np.concatenate([[0], np.cumsum(lens)[:-1]]).astype(np.int64)
+        tokens = torch.arange(int(lens.sum()), dtype=torch.int32, device=DEV) % 90
+        want, _ = clf.classify(tokens, starts, lens)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(20_000_000)
+        got, _ = clf.classify(tokens, starts, lens)
+        held = not torch.cuda.current_stream().query()
+        starts[:], lens[:] = 0, 1
+        assert held
+        assert torch.equal(got, want)
