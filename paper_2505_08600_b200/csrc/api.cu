@@ -799,6 +799,11 @@ sd_status draft_layers(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& 
     return SD_OK;
 }
 
+// Context bounds of a pass's sequences, for attention's launch order and form.
+void attention_hints(const sd_ctx* c, const int32_t* seqs, int n, int* hint) {
+    for (int i = 0; i < n && i < SD_MAX_BATCH; ++i) hint[i] = c->len_ub[seqs[i]];
+}
+
 // The same pass on the tensor-core path (bf16 models): per layer the QKV GEMM, attention, the Wo,
 // gate/up and down GEMMs, each GEMM followed by a small kernel that sums its split accumulators
 // and applies the step after it; every kernel is a programmatic dependent of the one before.
@@ -827,8 +832,8 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         e.lora_b = L.lora_b[mat]; e.lora_task = c->row_slot + SD_MAX_ROWS; e.lora_r = c->cfg.lora_rank; e.lora_n = c->cfg.lora_adapters;
         e.lora_scale = c->cfg.lora_scale; e.row_slot = c->row_slot;
     };
-    int len_hint[SD_MAX_BATCH];                                             // context bounds of the pass's sequences, for attention's launch order
-    for (int i = 0; i < list.n && i < SD_MAX_BATCH; ++i) len_hint[i] = c->len_ub[list.ids[i]];
+    int len_hint[SD_MAX_BATCH];
+    attention_hints(c, list.ids, list.n, len_hint);
     // The pass's first matrix kernel is launched in full stream order: it begins when the embedding kernel's stores are visible.
     // Every later kernel of the pass begins after it did, which is why they may read the row plan (slots, positions, rotary
     // factors, adapters) before they wait for the kernel before them; as the embedding kernel's programmatic dependent it could
@@ -1061,8 +1066,7 @@ sd_status forward_pass(sd_ctx* c, Model& M, const sd_ctx::CachedProgram& cp, con
 // Calls of the hot path repeat with the same shapes and buffers, and all state they depend on
 // lives on the device, so the launch sequence of a call is captured once into a CUDA graph
 // and replayed: one host call instead of hundreds of launches.  The key holds everything that
-// shapes the launches (sequences, gamma, buffers, context-length bucket); lengths below the bucket set the order of
-// attention's CTAs only, which no result depends on.
+// shapes the launches (sequences, gamma, buffers, context-length bucket, the form of attention).
 struct KeyBuilder {
     std::vector<uint8_t> bytes;
     template <typename T> KeyBuilder& add(const T& v) {
@@ -1074,6 +1078,15 @@ struct KeyBuilder {
 };
 
 int bound_bucket(int bound) { return (bound + 255) & ~255; }
+
+// The form that attention takes in a pass: it follows the lengths of all sequences, of which a key otherwise holds the longest one's bucket.
+void add_attention_form(KeyBuilder& key, const sd_ctx* c, const Model& M, const int32_t* seqs, int n, const RowPlan& plan, bool alone) {
+    if (!M.tc || n < 2) return;
+    int hint[SD_MAX_BATCH];
+    attention_hints(c, seqs, n, hint);
+    const AttnForm f = attention_split_form(n * plan.rows_per_seq, plan.rows_per_seq, M.d.n_heads, M.d.n_kv_heads, M.d.head_dim, std::min(plan.ctx_bound, c->cfg.max_ctx), hint, alone);
+    key.add(f.n_splits).add(f.warps).add(f.csize);
+}
 
 template <class Body>
 sd_status run_graphed(sd_ctx* c, const KeyBuilder& key, Body body) {
@@ -1509,24 +1522,21 @@ sd_status sd_draft_steps_replay(sd_ctx* c, const int32_t* seqs, int n_seq, int g
     // with low-rank adapters every task runs on the one base draft: a single group, adapters picked row by row
     const bool shared = c->cfg.lora_adapters > 0;
     const int n_groups = shared ? 1 : c->cfg.n_drafts;
+    std::vector<std::vector<int32_t>> members(n_groups);
+    for (int k = 0; k < n_groups; ++k)
+        for (int i = 0; i < n_seq; ++i) if (shared || c->draft_id[seqs[i]] == k) members[k].push_back(seqs[i]);
+    const int n_active = (int)std::count_if(members.begin(), members.end(), [](const std::vector<int32_t>& g) { return !g.empty(); });
     for (int k = 0; k < n_groups; ++k) {                    // programs of the persistent kernel exist before anything is captured
-        int n = 0;
-        for (int i = 0; i < n_seq; ++i) n += shared || c->draft_id[seqs[i]] == k;
-        if (n == 0) continue;
-        for (int s = 0; s < gamma; ++s) {
-            if (s == 0) { RowPlan plan{PLAN_DRAFT_FIRST, 2, 0, 0, gamma, x_in, bound}; SD_TRY(prepare_pass(c, 1 + k, plan, 2 * n, LOGITS_LAST)); }
-            else { RowPlan plan{PLAN_DRAFT_NEXT, 1, 0, s, gamma, x_in, bound + s}; SD_TRY(prepare_pass(c, 1 + k, plan, n, LOGITS_ALL)); }
+        const int n = (int)members[k].size();
+        for (int s = 0; n > 0 && s < gamma; ++s) {
+            const RowPlan plan = s == 0 ? RowPlan{PLAN_DRAFT_FIRST, 2, 0, 0, gamma, x_in, bound} : RowPlan{PLAN_DRAFT_NEXT, 1, 0, s, gamma, x_in, bound + s};
+            add_attention_form(key, c, c->models[1 + k], members[k].data(), n, plan, n_active == 1);
+            SD_TRY(prepare_pass(c, 1 + k, plan, n * plan.rows_per_seq, s == 0 ? LOGITS_LAST : LOGITS_ALL));
         }
     }
     return run_graphed(c, key, [&]() -> sd_status {
     // Groups of different draft models run side by side: every group after the first gets a stream and a scratch set of
     // its own, forked from and joined back to the context's stream (inside a capture these become parallel branches).
-    int n_active = 0;
-    for (int k = 0; k < n_groups; ++k) {
-        bool any = false;
-        for (int i = 0; i < n_seq; ++i) any |= shared || c->draft_id[seqs[i]] == k;
-        n_active += any;
-    }
     const bool side_by_side = c->groups_concurrent && n_active > 1 && !c->prof_on && !(c->pass_on && c->pass_drafts) &&
                               (int)c->sets.size() >= n_active;
     cudaStream_t main_st = c->st;
@@ -1584,6 +1594,7 @@ sd_status sd_verify(sd_ctx* c, const int32_t* seqs, int n_seq, int gamma, const 
     RowPlan plan{PLAN_VERIFY, gamma + 1, 0, 0, gamma, x_dev, bound_bucket(bound)};
     KeyBuilder key;
     key.add(2).add_list(seqs, n_seq).add(gamma).add(x_dev).add(logits_dev).add(plan.ctx_bound).add(c->force_plain).add(c->stamps_on).add(c->pass_on).add(c->pass_max_rows);
+    add_attention_form(key, c, c->models[0], seqs, n_seq, plan, true);
     SD_TRY(prepare_pass(c, 0, plan, n_seq * (gamma + 1), LOGITS_ALL));
     CostScope cost(c, 1, 1);
     return run_graphed(c, key, [&]() { return forward(c, c->models[0], list, plan, n_seq * (gamma + 1), LOGITS_ALL, logits_dev); });
@@ -1600,6 +1611,7 @@ sd_status sd_target_step(sd_ctx* c, const int32_t* seqs, int n_seq, float* logit
     RowPlan plan{PLAN_TARGET_STEP, 1, 0, 0, 0, nullptr, bound_bucket(bound)};
     KeyBuilder key;
     key.add(3).add_list(seqs, n_seq).add(logits_dev).add(plan.ctx_bound).add(c->force_plain).add(c->stamps_on).add(c->pass_on).add(c->pass_max_rows);
+    add_attention_form(key, c, c->models[0], seqs, n_seq, plan, true);
     SD_TRY(prepare_pass(c, 0, plan, n_seq, LOGITS_ALL));
     CostScope cost(c, 2, 1);
     return run_graphed(c, key, [&]() { return forward(c, c->models[0], list, plan, n_seq, LOGITS_ALL, logits_dev); });
@@ -1699,6 +1711,7 @@ sd_status sd_verify_accept(sd_ctx* c, const int32_t* seqs, int n_seq, int gamma,
     key.add(bound_bucket(bound));
     {
         RowPlan plan{PLAN_VERIFY, gamma + 1, 0, 0, gamma, x_dev, bound_bucket(bound)};
+        add_attention_form(key, c, c->models[0], seqs, n_seq, plan, true);
         SD_TRY(prepare_pass(c, 0, plan, n_seq * (gamma + 1), LOGITS_ALL));
     }
     std::vector<int> ub(c->len_ub);

@@ -10,6 +10,8 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <array>
+#include <functional>
 
 #include "gemm_tc.h"
 #include "kernels.h"
@@ -455,33 +457,48 @@ size_t attention_split_workspace(int rows, int H, int hd, int max_ctx) {
     return ATTN_COUNTER_BYTES + sizeof(float) * (size_t)rows * H * n_splits * (hd + 2);
 }
 
-// How a launch shares out its work: slices of the contexts, warps per CTA, CTAs per slice.  The results depend on it (keys are summed in another
-// order), and passes are captured into graphs, so it follows from what their keys hold: the shapes, the number of rows and ctx_bound.
-struct AttnForm { int n_splits, warps, csize; };
-static AttnForm attention_split_form(int n_blocks, int tile_queries, int Hkv, int hd, int ctx_bound, bool alone) {
+// How a launch shares out its work.  The results depend on it (keys are summed in another order), so whatever it is chosen by belongs into the
+// key of a captured graph, or the form itself does: the number of rows, ctx_bound, and the sequences' lengths one by one.
+AttnForm attention_split_form(int n_rows, int rows_per_seq, int H, int Hkv, int hd, int ctx_bound, const int* seq_len_hint, bool alone) {
+    const int n_seqs = n_rows / rows_per_seq, rows_per_block = std::max(1, std::min(rows_per_seq, NQ / (H / Hkv))), vectors = rows_per_block * (H / Hkv);
+    const int blocks = n_seqs * ((rows_per_seq + rows_per_block - 1) / rows_per_block);
     AttnForm f;
     // one slice while the context is short (no cross-CTA merge at all), SLICE_KEYS positions per slice beyond
     f.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS - 1) / SLICE_KEYS));
     int sm = 148;
     { int dev = 0; if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev); }
-    if (f.n_splits * Hkv * n_blocks > 2 * sm) f.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS_MANY - 1) / SLICE_KEYS_MANY));
+    if (f.n_splits * Hkv * blocks > 2 * sm) f.n_splits = std::max(1, std::min(32, (ctx_bound + SLICE_KEYS_MANY - 1) / SLICE_KEYS_MANY));
     // few (head, row block, slice) items: two or four CTAs of a cluster share each of them
-    const int items = f.n_splits * Hkv * n_blocks;
+    const int items = f.n_splits * Hkv * blocks;
     f.csize = items * 4 <= sm ? 4 : (items * 2 <= sm ? 2 : 1);
     f.warps = items > 2 * sm ? WARPS_MANY : WARPS_FEW;
-    // One CTA of eight warps per SM and a second wave that is partly empty, or three CTAs of four warps per SM: with heads of 128 the latter, in
-    // pairs up to one and a half items per SM, alone up to 512 positions.  Four layers of the 7B, us per pass, eight warps / chosen, one and six
-    // rows per sequence: five contexts of 1,000 positions 479 / 456 and 526 / 498, eight of 250 423 / 411 and 478 / 462; eight of 1,000 and 250
-    // mixed would take 447 / 468 and 503 / 510 with four (all of 1,000: 489 / 474 and 543 / 527; the bound does not tell them apart).  Within
-    // one wave eight are faster (four contexts of 250: 395 / 399 and 433 / 446).  With heads of 64, where a chunk is half as much work beside the same
-    // set-up and merge, eight are as fast or faster beyond one wave (1B, 16 contexts of 1,000: 265 / 264 and 325 / 339; 12-layer drafts of 12
-    // heads 1,470 / 1,471), and clusters of four where three CTAs per SM hold them and the contexts are long: nine sequences on such a
-    // draft, three passes, at 700 positions 1,290 / 1,253, at 1,000 1,370 / 1,292, but at 250 1,150 / 1,172.
-    // Measured for at most eight query vectors and without passes of other models beside it (16 sequences on four drafts: 7,423 against 7,051).
-    if (alone && f.csize == 1 && f.warps == WARPS_FEW && tile_queries <= 8) {
-        if (hd == 128 && items > sm && items * 2 <= 3 * sm) { f.warps = WARPS_MANY; f.csize = 2; }
-        else if (hd == 128 && items > sm && ctx_bound <= 512) f.warps = WARPS_MANY;
-        else if (hd == 64 && items * 4 <= 3 * sm && ctx_bound > 512) { f.warps = WARPS_MANY; f.csize = 4; }
+    // A CTA of eight warps per SM, or three of four warps?  Measured at 956 points (10 lengths, alike and mixed, 1...6 rows per sequence) without
+    // passes of other models beside it (16 sequences on four drafts: 7,423 us with four warps against 7,051) and for up to eight query vectors.
+    if (!alone || f.csize > 1 || f.warps == WARPS_MANY || vectors > 8) return f;
+    // Less than one wave of eight warps: clusters of four CTAs, if three CTAs per SM hold them and the contexts are long.  us, eight / chosen:
+    // nine sequences on a 12-layer draft with heads of 64, three passes, at 700 positions 1,290 / 1,253, at 1,000 1,370 / 1,292 (at 250 it would be
+    // 1,150 / 1,172); heads of 128 with one row: four layers of the 7B, three contexts of 1,000 426 / 428, of 1,000 and 250 414 / 408 (three rows at 700:
+    // 425 / 437); two layers of the 13B, one context of 2,000 327 / 322.
+    if (items * 4 <= 3 * sm && (hd == 64 ? ctx_bound > 512 : vectors == 1 && ctx_bound > 768)) { f.warps = WARPS_MANY; f.csize = 4; }
+    // More than one wave, heads of 128: by the longest chain of chunks, a CTA's set-up and merge counted as three of them and one of four warps'
+    // beside two others at 1.4; the second wave of eight warps begins where the shortest items of the first end.  Four layers of the 7B, one and
+    // six rows: five contexts of 1,000 479 / 456 and 526 / 498, eight of 250 423 / 411 and 478 / 462; the whole 7B, five of 131...777 stay with eight:
+    // 4,505, with four 4,631.  (With heads of 64 a chunk is half as much work beside the same set-up and merge: 1B, 16 contexts of 1,000, six rows
+    // 325 / 339, its 12-layer drafts 1,470 / 1,471.)
+    if (items > sm && hd == 128) {
+        const int per_seq = items / n_seqs;
+        std::array<int, 64> len;                                     // longest first; without hints: all as long as the bound
+        const bool known = seq_len_hint && n_seqs <= 64;
+        for (int i = 0; known && i < n_seqs; ++i) len[i] = std::max(1, std::min(seq_len_hint[i], ctx_bound));
+        if (known) std::sort(len.begin(), len.begin() + n_seqs, std::greater<int>());
+        auto chunks = [&](int item, int keys, int parts) {           // of the item'th longest
+            const int n = known ? len[std::min(item / per_seq, n_seqs - 1)] : ctx_bound;
+            return ((n + f.n_splits * parts - 1) / (f.n_splits * parts) + keys - 1) / keys;
+        };
+        const double setup = 3.0;
+        const double few = std::max(setup + chunks(0, 16 * WARPS_FEW, 1), 2 * setup + chunks(sm - 1, 16 * WARPS_FEW, 1) + chunks(sm, 16 * WARPS_FEW, 1));
+        const int c = items * 2 <= 3 * sm ? 2 : 1;
+        if (setup + 1.4 * chunks(0, 16 * WARPS_MANY, c) < few) { f.warps = WARPS_MANY; f.csize = c; }
     }
     return f;
 }
@@ -513,7 +530,7 @@ cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc
     P.rows_per_block = std::max(1, std::min(rows_per_seq, NQ / (H / Hkv)));
     const int bps = (rows_per_seq + P.rows_per_block - 1) / P.rows_per_block;
     const int n_blocks = (n_rows / rows_per_seq) * bps;
-    const AttnForm form = attention_split_form(n_blocks, P.rows_per_block * (H / Hkv), Hkv, hd, ctx_bound, alone);
+    const AttnForm form = attention_split_form(n_rows, rows_per_seq, H, Hkv, hd, ctx_bound, seq_len_hint, alone);
     P.n_splits = form.n_splits; P.csize = form.csize;
     const size_t need = ATTN_COUNTER_BYTES + sizeof(float) * (size_t)n_rows * H * P.n_splits * (hd + 2);
     if (need > workspace_bytes || (size_t)n_blocks * Hkv * sizeof(uint32_t) > ATTN_COUNTER_BYTES) return cudaErrorInvalidValue;

@@ -46,14 +46,17 @@ cudaError_t launch_attention(const void* q, const void* kcache_layer, const void
 // ---- attention_split.cu : split-KV kernel for bf16 caches with head_dim 64 / 128
 bool attention_split_supported(int dtype, int H, int Hkv, int hd);
 size_t attention_split_workspace(int rows, int H, int hd, int max_ctx);
+// How a launch with these arguments (ctx_bound at most max_ctx) shares out its work: slices of the contexts, warps per CTA, CTAs per slice.
+struct AttnForm { int n_splits, warps, csize; };
+AttnForm attention_split_form(int n_rows, int rows_per_seq, int H, int Hkv, int hd, int ctx_bound, const int* seq_len_hint, bool alone);
 cudaError_t launch_attention_split(const void* q, const void* kc, const void* vc, void* out, const int32_t* row_slot,
                                    const int32_t* row_pos, int n_rows, int rows_per_seq, int H, int Hkv, int hd,
                                    int max_ctx, int ctx_bound, void* workspace, size_t workspace_bytes, int dependent,
                                    cudaStream_t st, int lo_off = 0 /*> 0: also write out's second bf16 part, lo_off rows further down*/,
                                    unsigned long long* stamp = nullptr /*optional time stamps of the launch*/,
-                                   int force_warps = 0 /*4 or 8: warps per CTA; 0: by heads, positions and the number of work items*/,
+                                   int force_warps = 0 /*4 or 8: warps per CTA; 0: as attention_split_form says*/,
                                    int max_cluster = 0 /*1 or 2: at most this many CTAs share a slice; 0: up to 4*/,
-                                   const int* seq_len_hint = nullptr /*host, one per sequence: context lengths (bounds will do); longest sequences are started first*/,
+                                   const int* seq_len_hint = nullptr /*host, one per sequence: context lengths (bounds will do); longest sequences are started first, and the form follows them*/,
                                    bool alone = true /*no other pass runs beside this one*/);
 
 // ---- sampling.cu

@@ -77,16 +77,18 @@ def test_scores_that_grow_and_shrink_from_tile_to_tile():
             np.testing.assert_allclose(got[s, h], oracle.attention_head(qf[s, h], kf[s, h], vf[s, h]), rtol=0, atol=TOL)
 
 
-# Around one wave of CTAs: with heads of 128 pairs of four warps, four warps alone up to 512 positions, eight warps past that and with more than
-# eight query vectors; with heads of 64 four CTAs of four warps from 513 positions on, eight warps up to there.
+# Around one wave of CTAs (every launch of an operator counts all contexts as the longest): pairs of four warps, four warps alone, eight warps with
+# more than eight query vectors and with heads of 64; below it four CTAs of four warps from 513 positions on, with heads of 128 from 769.
 AROUND_ONE_WAVE = {
     "pairs": (40, 40, 128, 1, [1030, 15, 300, 1023]),                           # 320 items in two slices each: more than two per SM; the slices' merge
     "pairs_one_slice": (32, 32, 128, 8, [700, 31, 33, 512, 64]),                # 160 items
     "alone_512": (32, 32, 128, 6, [511, 64, 65, 127, 128, 500, 8, 300]),        # 256 items
-    "eight_513": (32, 32, 128, 6, [512, 64, 65, 127, 128, 500, 8, 300]),
+    "alone_513": (32, 32, 128, 6, [512, 64, 65, 127, 128, 500, 8, 300]),
     "nine_vectors": (32, 32, 128, 9, [200, 64, 65, 127, 128]),
     "fours_513": (12, 12, 64, 2, [512, 63, 64, 65, 300, 127, 128, 15, 256]),     # 108 items
     "eight_512": (12, 12, 64, 2, [511, 63, 64, 65, 300, 127, 128, 15, 256]),
+    "fours_769": (32, 32, 128, 1, [768, 63, 64]),                               # 96 items
+    "eight_768": (32, 32, 128, 1, [767, 63, 64]),
     "heads_of_64": (40, 40, 64, 1, [255, 254, 129, 128, 127, 200]),             # 240 items
 }
 
@@ -97,13 +99,14 @@ def test_forms_around_one_wave(name, monkeypatch):
     test_every_form_follows_the_oracle(name)
 
 
+@pytest.mark.parametrize("head_dim", [64, 128])
 @pytest.mark.parametrize("call", ["draft", "verify", "step", "verify_accept"])
-def test_what_a_call_returns_does_not_depend_on_the_lengths_that_its_graph_was_captured_at(call):
+def test_what_a_call_returns_does_not_depend_on_the_lengths_that_its_graph_was_captured_at(call, head_dim):
     """Attention's form follows the lengths of all sequences: the same five slots with one long context (eight warps), then with five (four warps in
     clusters of two), the longest alike.  The second call returns bit for bit what it returns in a context that never saw the first, and without graphs."""
     from paper_2505_08600_b200 import binding
     V, gamma, seqs = 512, 3, list(range(5))
-    target = dict(n_layers=2, d_model=256, n_heads=32, n_kv_heads=32, head_dim=64, d_ffn=256, vocab=V)      # 160 (head, sequence) items
+    target = dict(n_layers=2, d_model=256, n_heads=32, n_kv_heads=32, head_dim=head_dim, d_ffn=256, vocab=V)      # 160 (head, sequence) items
     weights = [synth.make_weights(target, seed=3, model_index=k, dtype="bf16") for k in range(2)]
 
     def results(ctx, lens):
