@@ -761,7 +761,7 @@ bool draft_layers_wanted(const sd_ctx* c, const Model& M, const RowPlan& plan, i
     if (n <= 4) return 2 * n <= 3 * M.d.n_layers && keys <= 1024 * std::min(M.d.n_heads + 8, 5 * M.d.n_layers);
     return n <= 6 && M.d.n_layers >= 6 && M.d.d_model <= 768 && keys <= 1024 * M.d.n_heads;
 }
-sd_status draft_layers(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan, RowScale* scale) {
+sd_status draft_layers(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan, RowScale& scale) {
     const sd_model_desc& m = M.d;
     const size_t stream = (size_t)DL_MAX_ROWS * m.d_model;
     float* h[2] = {c->partials, c->partials + stream};
@@ -791,11 +791,10 @@ sd_status draft_layers(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& 
         LAUNCH(CAT_LINEAR, launch_draft_mlp(p, c->st));
         cur ^= 1;
     }
-    if (!scale) return SD_OK;
     p.h_in = h[cur]; p.part_in = from_features; p.n_in = n_features; p.gain = M.final_norm;
     LAUNCH(CAT_ELEMENTWISE, launch_draft_tail(p, (bf16*)c->xn, 8, c->ssq, SSQ_STRIDE, c->st));
-    scale->n_parts = (m.d_model + DL_TAIL - 1) / DL_TAIL;
-    scale->stride = SSQ_STRIDE;
+    scale.n_parts = (m.d_model + DL_TAIL - 1) / DL_TAIL;
+    scale.stride = SSQ_STRIDE;
     return SD_OK;
 }
 
@@ -852,7 +851,7 @@ sd_status forward_tc(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& pl
         return gv ? gemv_step(c, w, x, n_rows, n_out, K, e, dep) : gemm_tc(c, tm, x, n_rows, n_out, K, e, dep);
     };
     if (draft && lo == 8 && draft_layers_wanted(c, M, plan, n_rows)) {
-        SD_TRY(draft_layers(c, M, list, plan, mode == LOGITS_NONE ? nullptr : &scale));
+        SD_TRY(draft_layers(c, M, list, plan, scale));
         dependent = 1;
     } else {
     LAUNCH(CAT_ELEMENTWISE, launch_embed(c->S, list, plan, n_rows, M.embed, dt, d, m.vocab, c->h, c->row_slot, c->row_pos,

@@ -57,8 +57,8 @@ struct AttnParams {
 // whichever slice arrives last.
 // Bound: HBM where the chip is full of CTAs (13B, contexts of 8,000), else a warp's chain through a chunk: scores, softmax, values.  So
 // the scores are two sums per tile, the output is scaled only when the largest score has grown, and EIGHT leaves out what belongs to
-// the tile's upper eight query vectors where there are none.  Iterations: 13B 13,050 -> 12,766 us, 7B of five sequences 4,602 -> 4,529,
-// decoding step of three 2,884 -> 2,815.  (Barriers between the warps at every chunk, or a third chunk on its way, make no difference.)
+// the tile's upper eight query vectors where there are none.  Iterations: 13B 13,055 -> 12,662 us, 7B of five sequences 4,593 -> 4,503,
+// decoding step of three 2,881 -> 2,784.  (Barriers between the warps at every chunk, or a third chunk on its way, make no difference.)
 template <int HD, int NW, bool EIGHT>
 __global__ void __launch_bounds__(32 * NW) k_attn_mma(AttnParams P) {
     constexpr int NT = 32 * NW;              // threads; each warp takes 16 of the keys of a chunk

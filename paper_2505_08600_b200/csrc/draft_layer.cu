@@ -5,7 +5,7 @@
 // feed-forward features, over clusters of four CTAs:
 //   k_draft_attention  a cluster per head: the head's query, key and value rows of QKV, rotary embedding, cache append, attention over the
 //                      head's cache, and the head's columns of Wo;
-//   k_draft_mlp        a cluster per 128 features: their gate and up rows, SwiGLU, and their columns of the down matrix.
+//   k_draft_mlp        a cluster per 128 or 192 features: their gate and up rows, SwiGLU, and their columns of the down matrix.
 // Inside a cluster, CTAs hand over through distributed shared memory (a cluster barrier instead of a kernel boundary).  What a cluster
 // leaves is a piece of the layer's output for all columns; the next kernel's clusters each add all pieces (in their order: the same
 // sums in every cluster and from run to run), take the norm, and go on.  Weights are in registers before the wait for the kernel before
@@ -13,7 +13,7 @@
 // Activations enter the matrices in two bf16 parts, queries, keys, values and the cache in one, sums in fp32, as on the other paths.
 // Bound: latency.  12 layers of 768 columns at 512 positions, one row, us after the wait: k_draft_attention 1.6 pieces added up, 0.6 barrier,
 // 0.6 QKV, 0.5 rotation, 0.7 barrier, 0.8 attention, 1.3 its merge, 0.4 barrier, 0.6 Wo; k_draft_mlp 1.3, 0.5, 1.0, 0.5, 0.5, 0.7; between two
-// kernels 0.5.  17.5 -> 13 us per layer, 7B iteration 4,014 -> 3,749 us, 1B (drafts of two layers) 1,058 -> 1,043.
+// kernels 0.5.  17.5 -> 13 us per layer, 7B iteration 4,014 -> 3,698 us, 1B (drafts of two layers) 1,058 -> 1,035.  Where they are taken: api.cu.
 #include "draft_layer.h"
 
 #include <cooperative_groups.h>
@@ -30,7 +30,7 @@ constexpr int WARPS = 16, THREADS = 32 * WARPS;
 constexpr int ROWS = DL_MAX_ROWS;
 constexpr int HD = 64;
 constexpr int MAX_D = 1024;
-// Clusters of both kernels that are resident side by side (a CTA per SM; clusters of four fill 35 or 36 places of the 148 SMs when they come
+// Clusters of both kernels that are resident side by side (a CTA per SM; clusters of four fill 35 or 36 places of the B200's 148 SMs when they come
 // and go).  One more and the last cluster of either kernel begins when the other kernel ends: 12 + 24 clusters 18.4 us per layer.
 constexpr int MAX_CLUSTERS = 32;
 constexpr int ACC_COLS = MAX_D / RANKS;         // columns of the residual stream that a CTA adds up
@@ -472,7 +472,7 @@ __global__ void __cluster_dims__(RANKS, 1, 1) __launch_bounds__(THREADS, 1) k_dr
     extern __shared__ __align__(128) uint8_t dyn[];
     __shared__ float ssq[RANKS][ROWS][2];
     __shared__ __align__(16) uint8_t act[2 * ROWS * row_pitch(FEATURES)];         // the cluster's activations in two parts
-    __shared__ Plan plan;                                              // (not used: the rows come from the kernel before)
+    __shared__ Plan plan;                                              // (not used: the rows come from the kernel before; for rows_in, which is the same for both kernels)
     pdl_launch_dependents();
     cg::cluster_group cluster = cg::this_cluster();
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, gid = lane >> 2, tig = lane & 3;

@@ -1,5 +1,5 @@
 // Two fp32 values in one 64-bit register and the packed arithmetic of sm_100 on them: each instruction is two independent IEEE
-// operations (same results as the scalar forms), which halves the instructions per loaded byte.
+// operations (same results as the scalar forms), which halves the instructions per loaded byte.  And 2^x as one instruction.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -13,5 +13,7 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn
 __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ float f2_hsum(f32x2 v) { const float2 s = f2_unpack(v); return s.x + s.y; }
+// 2^x, zero below the normal range (a weight or a decay that small is lost in any sum it enters).
+__device__ __forceinline__ float exp2_ftz(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
 }  // namespace sd

@@ -159,12 +159,14 @@ k_mamba_in(MambaDims m, const int32_t* __restrict__ tok_id /*nullptr: row = toke
 //      are not their prompt's first keep the products of decays and the sum they are weighted with (see the top of the file): three of
 //      seven packed operations per pair of states.
 // 400 prompts of 109,096 tokens: 694 -> 391 us (some 290 instructions per token and 32 channels, 356 with the convolution in 2 and again in 4, the
-// step size and the SiLU of the gate in the scan, half of the states' results stored four bytes at a time); whole call 826 -> 517,
-// one prompt of 8 / 64 / 300 tokens 78 / 126 / 131 -> 66 / 75 / 83.  Two threads per channel with half of its states each, 32 warps of 64
-// registers, spill: 720...795.
+// step size and the SiLU of the gate in the scan, half of the states' results stored four bytes at a time); whole call 815 -> 512,
+// one prompt of 8 / 64 / 300 tokens 77 / 128 / 141 -> 54 / 81 / 91.  Two threads per channel with half of its states each, 32 warps of 64
+// registers, spill: 720...795.  Rank 8 as a compiled form: 539 -> 512, one prompt of 300 96 -> 91.
 //   More than MC_CHANNELS channels: a cluster of up to four CTAs per chunk with as many channels each.  A CTA projects its own channels;
-//   the parts of r, B, C meet through distributed shared memory (each CTA adds a share of them, parts in the CTAs' order).
-constexpr int MC_TILE = 32, MC_CHANNELS = 256, MC_THREADS = MC_CHANNELS, MC_STAGED = 40 * 1024;      // W_x is staged up to this size: two CTAs of the usual sizes still fit an SM
+//   the parts of r, B, C meet through distributed shared memory (each CTA adds a share of them, parts in the CTAs' order), tile by tile, before: once
+//   per chunk.  1,024 channels: one prompt of 300 tokens 459 -> 418 us, 400 prompts 14.9 -> 14.5 ms, but one of 4,000 858 -> 884; 512: 434 -> 387, 7.2 -> 6.9 ms.
+constexpr int MC_TILE = 32, MC_CHANNELS = 256, MC_THREADS = MC_CHANNELS, MC_STAGED = 40 * 1024;      // W_x is staged up to this size, with which two CTAs fit an SM
+// (256 channels of rank 16, 48 KB: staged 400 prompts take 1,171 us, read from L2 1,018; one prompt of 300 tokens 133 and 137)
 constexpr int MC_GROUP = 16 /*tokens of the convolution on their way at a time*/, MC_PITCH = MC_CHANNELS + 4, MC_AHEAD = 2 /*gates on their way during the scan*/;
 constexpr int MC_PARTS = MC_THREADS / 128, MC_OUT = 48;              // parts the channels of a projection are cut into; outputs of one round of it
 constexpr int MC_PART = MC_TILE * (MC_OUT + 1);          // floats of one part's sums, in the place of the step sizes
@@ -173,8 +175,6 @@ static_assert(MC_PARTS * MC_PART <= MC_TILE * MC_PITCH, "the parts' sums fit whe
 constexpr int MC_MAX_SMEM = (MC_TILE * MB_MAX_X + 2 * MC_TILE * MC_PITCH) * 4 + MC_STAGED;
 constexpr int MH_THREADS = 512;
 constexpr int MH_MAX_SMEM = (MB_MAX_DI * MB_MAX_N + MB_MAX_DI + MB_MAX_D + MB_MAX_K) * 4;
-// 2^x, zero below the normal range (a decay that small is lost in any sum it enters)
-__device__ __forceinline__ float exp2_ftz(float x) { float r; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x)); return r; }
 
 template <int NS /*states: 16, or any up to MB_MAX_N as 0*/, int KC /*taps: 4, or any up to four as -4, or up to MB_MAX_CONV as 0*/, int RS /*rank of the step size: 8, or any as 0*/,
           bool CL /*several CTAs per chunk*/, bool CARRY /*some prompt has more than one chunk*/>
@@ -415,9 +415,9 @@ k_mamba_chunk(MambaDims m, const ChunkRec* __restrict__ chunks, const int32_t* _
 
 // The pooled sums of long prompts: what the chunks' starting states add and the chunks' own sums, a thread per (channel, state) and a CTA
 // per eight channels instead of the head's one CTA per prompt, with the coefficients of eight chunks on their way at a time.  Bound: latency
-// of the chain over chunks.  One prompt of 4,000 / 30,000 / 200,000 tokens, whole call: 140 / 366 / 1,628 us,
-// in the head 203 / 869 / 6,758 (as kernels of their own, before: 275 / 802 / 4,757).  From eight chunks on a queue of shorter prompts is the slower
-// for the launch (100 prompts of 32...512 tokens: 323 against 319).
+// of the chain over chunks.  One prompt of 1,000 / 4,000 / 30,000 / 200,000 tokens, whole call: 90 / 102 / 281 / 1,214 us,
+// in the head 100 / 160 / 806 / 8,003.  From eight chunks on a queue of shorter prompts is the slower for the launch (100 / 400 prompts of
+// 32...512 tokens: 244 / 521 against 239 / 512).
 constexpr int MB_LONG = 16;                              // chunks from which on a prompt is long
 constexpr int CARRY_CH = 8, CARRY_BATCH = 8;
 __global__ void __launch_bounds__(CARRY_CH * MB_MAX_N)
