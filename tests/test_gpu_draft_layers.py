@@ -1,4 +1,4 @@
-"""Draft passes whose layers run in two kernels (a cluster per head, a cluster per 128 features) against the CPU oracle: widths that do not
+"""Draft passes whose layers run in two kernels (a cluster per head, a cluster per 128 or 192 features) against the CPU oracle: widths that do not
 fill the kernels' k blocks and tiles, 1...8 sequences (one or two rows each; the first pass of more than four is beyond these kernels), and
 contexts that end at the edges of a warp's tiles of 16 keys or go around its ring of two."""
 import numpy as np
