@@ -743,23 +743,23 @@ sd_status gemv_step(sd_ctx* c, const void* w, const void* x, int rows, int n_out
 // the row plan and reads the embedding itself, and so does every later one what it needs of the plan.
 // Only where one draft model takes part in the call: these kernels' CTAs take whole SMs, and the passes of several models beside one another
 // share the SMs better in smaller ones (7B, 16 sequences on four drafts: iteration 7,684 against 7,112 us).
-// And by sequences n and positions, since the four CTAs of a head walk all its caches, while the few-rows path cuts them into slices for
-// every SM; by layers, since a pass ends with a kernel more (some 4 us, against 2...4 saved per layer); from five sequences on by width.
-// Four passes in us, few-rows path / these kernels:
-//   12 layers of 768, 12 heads: one sequence at 128 / 2,048 / 8,000 positions 919 / 740, 1,155 / 820, 1,342 / 1,024; two at 8,000 1,514 / 1,341;
-//     three at 4,096 / 8,000 1,420 / 1,271, (1,608 / 1,708); four at 512 / 4,096 1,024 / 943, 1,468 / 1,454, at 8,000 (1,872 / 2,030); five at 2,048 1,449 / 1,379;
-//     six at 512 1,157 / 1,136, (at 2,048 1,503 / 1,513); (eight at 512 / 2,048 1,223 / 1,238, 1,628 / 1,673)
-//   4 layers of 256, 4 heads: two at 4,096 / 8,000 386 / 364, (419 / 453); four at 2,048 386 / 382, (at 4,096 419 / 479); (five at 2,048 404 / 414)
-//   6 layers of 1,024, 16 heads: three at 8,000 1,065 / 1,029; four at 4,096 947 / 886, (at 8,000 1,159 / 1,192); (five at 512 697 / 715)
-//   768 columns, 3 layers: three at 4,096 452 / 434; (four at 4,096 468 / 484).  2 layers: one at 512 261 / 244; three at 128 / 512 267 / 262,
-//     272 / 272; (four at 512 279 / 283).  1 layer: one at 128 / 1,024 186 / 187, 204 / 200; (two at 512 195 / 202)
+// And only where they are the faster form, by the time they save per layer, in us: 4.6 of hand-overs, and 2 more where the few-rows path merges
+// slices of a context; less 0.8 per sequence and 1,024 columns (every cluster adds up all pieces) and 0.54 - 0.028 per head for every 1,024 positions
+// (a head's four CTAs walk the caches of all sequences, the few-rows path cuts them into slices for every SM).  The kernel that ends
+// such a pass costs 4.2.  Fitted to seven drafts of 1...12 layers, 256...1,024 columns and 4...16 heads, 1...8 sequences of 128...8,000 positions: nowhere
+// more than 0.4 % above the few-rows path, nowhere more than 1.9 % above the faster form.  Four passes in us, few-rows path / these kernels:
+//   12 layers of 768, 12 heads: one sequence at 128 / 2,048 / 8,000 positions 919 / 740, 1,155 / 820, 1,342 / 1,024; four at 512 1,024 / 943, at 8,000 (1,872 / 2,030);
+//     eight at 128 (1,135 / 1,123), at 8,000 (2,693 / 3,240)
+//   4 layers of 256, 4 heads: six at 128 333 / 312, at 2,048 (410 / 453); two at 4,096 386 / 364, at 8,000 (419 / 453)
+//   6 layers of 1,024, 16 heads: four at 4,096 947 / 886, at 8,000 (1,159 / 1,192); five at 1,024 812 / 783, at 512 (697 / 715)
+//   2 layers of 768: three at 512 272 / 269; four at 1,024 304 / 293, at 512 (279 / 283).  One layer: two at 512 (195 / 202)
 bool draft_layers_wanted(const sd_ctx* c, const Model& M, const RowPlan& plan, int n_rows) {
     if (!c->one_draft || (plan.kind != PLAN_DRAFT_FIRST && plan.kind != PLAN_DRAFT_NEXT) || M.lora || !draft_layer_fits(M.d, n_rows) ||
         draft_layer_scratch(M.d) > c->partials_bytes) return false;
     const int n = n_rows / plan.rows_per_seq;
-    const int64_t keys = (int64_t)n * plan.ctx_bound;
-    if (n <= 4) return 2 * n <= 3 * M.d.n_layers && keys <= 1024 * std::min(M.d.n_heads + 8, 5 * M.d.n_layers);
-    return n <= 6 && M.d.n_layers >= 6 && M.d.d_model <= 768 && keys <= 1024 * M.d.n_heads;
+    const double saved = (plan.ctx_bound > 1024 ? 6.6 : 4.6) - 0.8 * n * M.d.d_model / 1024.0 -
+                         n * (plan.ctx_bound / 1024.0) * std::max(0.54 - 0.028 * M.d.n_heads, 0.1);
+    return M.d.n_layers * saved > 4.2;
 }
 sd_status draft_layers(sd_ctx* c, Model& M, const SeqList& list, const RowPlan& plan, RowScale& scale) {
     const sd_model_desc& m = M.d;
